@@ -27,13 +27,19 @@ namespace ts {
 
 static constexpr int kAttnRows = 128;   // packed rows per unit
 static constexpr int kAttnBlk = 64;     // kv positions per block
-static constexpr int kKvStages = 6;     // K/V blocks in the ring (three are held by issued products, the rest are in flight)
+// K/V blocks in the ring (three are held by issued products, the rest are in flight): 192 KB of shared memory for
+// either head width.  More than half of an SM's shared memory on purpose: a CTA takes all 512 columns of tensor memory,
+// so a second one on the same SM would sit in its allocation until the first is done while other SMs stay idle.  With six
+// stages of 16 KB (head_dim 64) the 128 CTAs of a 1B-shaped step were placed two to an SM: 13.5 us per launch at 4096
+// tokens of context, 7 of them spent in that wait; with twelve stages 7.9 us (eight ragged sessions: 31.2 -> 15.3 us).
+__host__ __device__ constexpr int kv_stages(int hd) { return hd == 64 ? 12 : 6; }
+static constexpr int kMaxKvStages = 12;
 static constexpr int kTcThreads = 192;
 static constexpr int kWorkers = 128;
 static constexpr int kWorkerWarp0 = 2;
 
 struct __align__(16) AttnCtl {
-  uint64_t kv_full[kKvStages], kv_empty[kKvStages], q_full;
+  uint64_t kv_full[kMaxKvStages], kv_empty[kMaxKvStages], q_full;
   uint64_t s_full[2], s_empty[2], p_full[2], pv_done[2], o_free;
   uint32_t tmem_base;
 };
@@ -336,6 +342,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr uint32_t kKvBytes = 2u * kAttnBlk * HD * 2, kHalves = HD / 64;
+  constexpr int kKvStages = kv_stages(HD);
   AttnCtl *ctl = reinterpret_cast<AttnCtl *>(smem + kKvStages * kKvBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int *err = a.err;
@@ -627,7 +634,7 @@ cudaError_t launch_attention_tc_merge(const AttnTcArgs &a, cudaStream_t st) {
 }
 
 static size_t attn_tc_smem(int hd) {
-  return 1024 + (size_t)kKvStages * 2 * kAttnBlk * hd * 2 + sizeof(AttnCtl) + 64;
+  return 1024 + (size_t)kv_stages(hd) * 2 * kAttnBlk * hd * 2 + sizeof(AttnCtl) + 64;
 }
 
 cudaError_t launch_attention_tc(const AttnTcArgs &a, cudaStream_t st) {
