@@ -5,7 +5,7 @@
 // The weight matrix is stored as contiguous 128 x 64 blocks (one TMA box each).
 // Operands are swapped with respect to the usual layout so that the 128-row dimension of the
 // tensor-core instruction runs over output features: a CTA owns 128 rows of W (operand A, K-major,
-// 16 KB per 64-wide k-block) and a chunk of up to 128 activation rows (operand B).  Activations can
+// 16 KB per 64-wide k-block) and the step's activation rows, at most 64 (operand B).  Activations can
 // be fed as a (hi, lo) bf16 pair stacked along the instruction's N dimension, so one MMA multiplies
 // the weight tile with both halves; the epilogue adds the two column groups.  The accumulator lives
 // in tensor memory: lane = output feature, column = activation row.
@@ -29,6 +29,8 @@ struct __align__(8) GemmSmemCtl {
   uint32_t abort_flag;
 };
 
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
 template <int EPI>
 __global__ void __launch_bounds__(192, 1)
 gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_a,
@@ -43,7 +45,6 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * kTileN;
   const int split = blockIdx.y;
-  const int m0 = blockIdx.z * g.Mc;
   // balanced cut of the k-blocks into gridDim.y runs
   const int kb0 = (int)(((long long)split * g.n_kblocks) / (int)gridDim.y);
   const int kb1 = (int)(((long long)(split + 1) * g.n_kblocks) / (int)gridDim.y);
@@ -87,13 +88,13 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       for (int it = 0; it < pre; ++it) {
         uint32_t bar = smem_u32(&ctl->full[it]);
         mbar_expect_tx(bar, stage_bytes);
-        tma_load_2d(smem_u32(smem + (size_t)it * stage_bytes), &tmap_w, 0, w_block(blockIdx.x, kb0 + it, (g.N + kTileN - 1) / kTileN, g.n_kblocks) * kTileN, bar, pol_w);
+        tma_load_2d(smem_u32(smem + (size_t)it * stage_bytes), &tmap_w, 0, w_block(blockIdx.x, kb0 + it, g.N / kTileN, g.n_kblocks) * kTileN, bar, pol_w);
       }
       pdl_wait();
       stamp_waited(g.stamp);
       for (int it = 0; it < pre; ++it) {
         uint32_t bar = smem_u32(&ctl->full[it]);
-        tma_load_3d(smem_u32(smem + (size_t)it * stage_bytes + kWBytes), &tmap_a, (kb0 + it) * kBlockK, m0, 0,
+        tma_load_3d(smem_u32(smem + (size_t)it * stage_bytes + kWBytes), &tmap_a, (kb0 + it) * kBlockK, 0, 0,
                     bar, pol_a);
       }
       // slot and round parity are carried along: an integer division per k-block would be a large part of
@@ -108,8 +109,8 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         uint32_t bar = smem_u32(&ctl->full[s]);
         mbar_expect_tx(bar, stage_bytes);
         uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes);
-        tma_load_2d(dst, &tmap_w, 0, w_block(blockIdx.x, kb0 + it, (g.N + kTileN - 1) / kTileN, g.n_kblocks) * kTileN, bar, pol_w);
-        tma_load_3d(dst + kWBytes, &tmap_a, (kb0 + it) * kBlockK, m0, 0, bar, pol_a);
+        tma_load_2d(dst, &tmap_w, 0, w_block(blockIdx.x, kb0 + it, g.N / kTileN, g.n_kblocks) * kTileN, bar, pol_w);
+        tma_load_3d(dst + kWBytes, &tmap_a, (kb0 + it) * kBlockK, 0, 0, bar, pol_a);
         if (++s == g.stages) { s = 0; ph ^= 1; }
       }
     } else if (lane == 0) {
@@ -152,6 +153,12 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
+    // Two passes through the ring's shared memory (free by now: every load was consumed by a product that has
+    // completed).  First thread <-> feature: the accumulator's columns, both planes added, go to [row][128 features].
+    // Then a warp takes every fourth row with four consecutive features per lane, so that global stores are whole lines
+    // and the row maximum of the LM head is one reduction over the warp per row.  (With a thread keeping its one feature
+    // a row's argmax took ten shuffles per warp and row and its SwiGLU stores were 32-byte pieces: the LM head of the 8B
+    // shape took 286 us at 32 rows and 180 at one, same weights.)
     pdl_wait();   // outputs of this kernel may still be read by the previous one's consumers
     bool ok = true;
     if (nkb > 0) {
@@ -159,69 +166,56 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       if (!ok && lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
     }
     tc_fence_after();
-    ok = ok && (ctl->abort_flag == 0);
+    ok = ok && (*reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) == 0);
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
-    const int n = n0 + q * 32 + lane;
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+    const uint32_t stg = smem_u32(smem);
+    for (int c0 = 0; c0 < g.Mc; c0 += 8) {        // (columns past the step's last row are read too and never used)
+      uint32_t r[8], r2[8];
+      if (nkb > 0) {
+        tmem_ld8(taddr + c0, r);
+        if (g.planes == 2) tmem_ld8(taddr + g.Mc + c0, r2);
+        tmem_wait_ld();
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) r[j] = r2[j] = 0u;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        st_shared_f32(stg + ((c0 + j) * kTileN + q * 32 + lane) * 4,
+                      __uint_as_float(r[j]) + (g.planes == 2 ? __uint_as_float(r2[j]) : 0.f));
+    }
+    epilogue_sync();
+    const int n = n0 + lane * 4;                  // this lane's features n .. n + 3
     if (ok) {
-      for (int c0 = 0; c0 < g.Mc; c0 += 16) {
-        if (m0 + c0 >= g.M) break;
-        uint32_t r[16], r2[16];
-        float v[16];
-        if (nkb > 0) {
-          tmem_ld16(taddr + c0, r);
-          if (g.planes == 2) tmem_ld16(taddr + g.Mc + c0, r2);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            v[j] = __uint_as_float(r[j]) + (g.planes == 2 ? __uint_as_float(r2[j]) : 0.f);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = 0.f;
-        }
+      for (int m = warp - 2; m < g.M; m += 4) {
+        const uint4 raw = ld_shared_v4(stg + (m * kTileN + lane * 4) * 4);
+        const float v[4] = {__uint_as_float(raw.x), __uint_as_float(raw.y), __uint_as_float(raw.z), __uint_as_float(raw.w)};
         if constexpr (EPI == EPI_PARTIAL) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int m = m0 + c0 + j;
-            if (m < g.M && n < g.N) g.out[((size_t)split * g.out_rows + m) * g.N + n] = v[j];
-          }
+          *reinterpret_cast<uint4 *>(g.out + ((size_t)split * g.out_rows + m) * g.N + n) = raw;
         } else if constexpr (EPI == EPI_LOGITS) {
+          *reinterpret_cast<uint4 *>(g.out + (size_t)m * g.N + n) = raw;
+          // order-preserving map of the float to an unsigned word; ties resolve to the lowest id (lowest lane, then
+          // lowest of its four)
+          uint32_t best = 0;
+          int bi = 0;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int m = m0 + c0 + j;
-            if (m < g.M && n < g.N) g.out[(size_t)m * g.N + n] = v[j];
-            float bv = (n < g.N) ? v[j] : -INFINITY;
-            int bi = n;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-              int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-              if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-            }
-            if (lane == 0 && m < g.M) {
-              // order-preserving map of the float to an unsigned word; ties resolve to the lowest id
-              uint32_t u = __float_as_uint(bv);
-              u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-              atomicMax(g.amax + m, ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)bi));
-            }
+          for (int j = 0; j < 4; ++j) {
+            uint32_t u = __float_as_uint(v[j]);
+            u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+            if (u > best) { best = u; bi = j; }
           }
+          const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+          if (lane == __ffs(__ballot_sync(0xffffffffu, best == top)) - 1)
+            atomicMax(g.amax + m, ((unsigned long long)top << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)(n + bi)));
         } else {  // EPI_SWIGLU: even feature row = gate_f, odd = up_f, f = n / 2
-          const int f = n >> 1;
-          const int F = g.N >> 1;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int m = m0 + c0 + j;
-            const float other = __shfl_xor_sync(0xffffffffu, v[j], 1);
-            const float gate = (lane & 1) ? other : v[j];
-            const float up = (lane & 1) ? v[j] : other;
-            const float a = gate / (1.f + __expf(-gate)) * up;
-            __nv_bfloat16 hi, lo;
-            split_bf16(a, hi, lo);
-            if (m < g.M && n < g.N) {
-              if ((lane & 1) == 0) g.act_out[(size_t)m * F + f] = hi;
-              else if (g.out_planes == 2) g.act_out[((size_t)g.act_rows + m) * F + f] = lo;
-            }
-          }
+          __nv_bfloat16 h0, l0, h1, l1;
+          split_bf16(v[0] / (1.f + __expf(-v[0])) * v[1], h0, l0);
+          split_bf16(v[2] / (1.f + __expf(-v[2])) * v[3], h1, l1);
+          const int F = g.N >> 1, f = n >> 1;
+          *reinterpret_cast<__nv_bfloat162 *>(g.act_out + (size_t)m * F + f) = __halves2bfloat162(h0, h1);
+          if (g.out_planes == 2)
+            *reinterpret_cast<__nv_bfloat162 *>(g.act_out + ((size_t)g.act_rows + m) * F + f) = __halves2bfloat162(l0, l1);
         }
       }
     }
@@ -273,7 +267,9 @@ cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, G
                         size_t smem_budget, cudaStream_t st, bool pdl) {
   g.stages = gemm_pick_stages(g.planes, g.Mc, smem_budget);
   const size_t smem = gemm_smem_bytes(g.stages, g.planes, g.Mc);
-  dim3 grid((g.N + kTileN - 1) / kTileN, n_splits, (g.M + g.Mc - 1) / g.Mc);
+  if (g.N % kTileN || g.M > g.Mc || g.Mc % 8 || (g.planes * g.Mc) % 16 || (int)(smem - 1024 - sizeof(GemmSmemCtl)) < g.Mc * kTileN * 4)
+    return cudaErrorInvalidValue;
+  dim3 grid(g.N / kTileN, n_splits);
   switch (epi) {
     case EPI_PARTIAL: return launch_one<EPI_PARTIAL>(tw, ta, g, grid, smem, st, pdl);
     case EPI_SWIGLU: return launch_one<EPI_SWIGLU>(tw, ta, g, grid, smem, st, pdl);

@@ -41,7 +41,13 @@ inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 constexpr int kMaxSplits = 12;
 constexpr int kMaxToolCandidates = 8;   // tool names verified in parallel while the name is open
 constexpr int kMaxAttnSplits = ts::kAttnMaxSplits;
-constexpr int kMcOptions[4] = {16, 32, 64, 128};
+// activation rows per TMA box.  Weight-streaming kernel: the step's rows rounded up to 8 (16 with one plane of
+// activations: the tensor-core instruction's N, planes x rows, is a multiple of 16) -- a k-block of 33 rows in a box of
+// 64 takes as many bytes as its weights, which left three stages in the ring: gate-up of the 1B shape 24.5 us against
+// 14.9 at 8 rows.  Many-rows kernel: 128.
+constexpr int kMcOptions[9] = {8, 16, 24, 32, 40, 48, 56, 64, 128};
+constexpr int kMcRows = 8;                       // index of the many-rows kernel's box
+constexpr int kFusedMc[3] = {1, 3, 7};           // the persistent kernel's boxes: 16, 32, 64 rows
 constexpr int kMaxFusedCtas = 256;   // the fused kernel runs one CTA per SM
 constexpr int kFusedMaxRows = 64;    // most rows per step the fused kernel takes
 constexpr bool kAutoPrefersFused = false;   // path = 0 picks the faster of the two on the 8B batch-1 step
@@ -197,9 +203,9 @@ struct ts_model {
   cudaStream_t st = nullptr;
   int planes = 1, n_sms = 148;
   int leaf_len = 64;   // KV positions per attention leaf: a constant of the model (see AttnTcArgs), set by ts_init_model
-  size_t gemm_smem_budget = 100 * 1024;
+  size_t gemm_smem_budget = 113 * 1024;   // two CTAs of the weight-streaming kernel per SM
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_d;
-  CUtensorMap tm_lm{}, tm_h[4]{}, tm_attn[4]{}, tm_act[4]{};
+  CUtensorMap tm_lm{}, tm_h[9]{}, tm_attn[9]{}, tm_act[9]{};
   std::vector<int32_t> free_pages;
   std::vector<ts_session *> sessions;   // live sessions over this model (detached on destroy)
   // last staged step
@@ -288,20 +294,20 @@ ts_status weight_map(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t N
   return make_map(enc, out, base, 2, dims, box);
 }
 
-ts_status act_maps(EncodeTiledFn enc, CUtensorMap *out4, void *base, uint64_t K, uint64_t rows, int planes) {
-  for (int i = 0; i < 4; ++i) {
+ts_status act_maps(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t K, uint64_t rows, int planes) {
+  for (int i = 0; i < 9; ++i) {
     const uint64_t dims[3] = {K, rows, (uint64_t)planes};
     const uint32_t box[3] = {64, (uint32_t)kMcOptions[i], (uint32_t)planes};
-    ts_status s = make_map(enc, &out4[i], base, 3, dims, box);
+    ts_status s = make_map(enc, &out[i], base, 3, dims, box);
     if (s) return s;
   }
   return TS_OK;
 }
 
-int pick_mc_index(int M) {
-  for (int i = 0; i < 3; ++i)
-    if (M <= kMcOptions[i]) return i;
-  return 3;
+int pick_mc_index(int M, int planes) {
+  if (M > 64) return kMcRows;
+  const int i = (M + 7) / 8 - 1;
+  return planes == 1 ? (i | 1) : i;
 }
 
 // split-K factor: two CTAs fit on an SM, so the grid runs in waves of 2 * n_sms CTAs; take the smallest factor
@@ -343,9 +349,9 @@ int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks
 
 struct GemmPlan { int splits, kb_per_split; };
 
-ts_status run_gemm(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta4, int N, int K, int M,
+ts_status run_gemm(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M,
                    float *out, __nv_bfloat16 *act_out, unsigned long long *amax, GemmPlan *plan) {
-  const int mi = pick_mc_index(M);
+  const int mi = pick_mc_index(M, m->planes);
   ts::GemmArgs g{};
   g.N = N; g.K = K; g.M = M; g.Mc = kMcOptions[mi]; g.planes = m->planes;
   g.n_kblocks = K / 64;
@@ -363,9 +369,9 @@ ts_status run_gemm(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMa
   g.stamp = m->stamp_slot();
   if (plan) { plan->splits = splits; plan->kb_per_split = g.kb_per_split; }
   if (many_rows)
-    CU_TRY(ts::launch_gemm_rows(epi, tw, ta4[3], g, splits, m->smem_optin, m->n_sms, m->st, m->use_pdl && !m->profiling));
+    CU_TRY(ts::launch_gemm_rows(epi, tw, ta[kMcRows], g, splits, m->smem_optin, m->n_sms, m->st, m->use_pdl && !m->profiling));
   else
-    CU_TRY(ts::launch_gemm(epi, tw, ta4[mi], g, splits, m->gemm_smem_budget, m->st, m->use_pdl && !m->profiling));
+    CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, splits, m->gemm_smem_budget, m->st, m->use_pdl && !m->profiling));
   m->launched(0);
   return TS_OK;
 }
@@ -384,7 +390,7 @@ ts_status run_step_fused(ts_model *m) {
   a.in.parent = di + L.o_parent; a.in.anc = (const uint32_t *)(di + L.o_anc); a.in.slot = di + L.o_slot;
   a.in.row_leaves = di + L.o_row_leaves;
   a.in.B = m->last_B; a.in.M = m->last_M;
-  a.mc_index = pick_mc_index(m->last_M); a.Mc = kMcOptions[a.mc_index]; a.planes = m->planes;
+  a.mc_index = m->last_M <= 16 ? 0 : (m->last_M <= 32 ? 1 : 2); a.Mc = kMcOptions[kFusedMc[a.mc_index]]; a.planes = m->planes;
   a.n_ctas = m->n_sms; a.skip_lm = (m->last_flags & TS_FLAG_SKIP_LM_HEAD) ? 1 : 0;
   a.k_max = c.k_max;
   a.n_attn_tiles = m->last_tiles128;
@@ -842,9 +848,9 @@ ts_status ts_init_model(const ts_model_config *cfg, const ts_buffers *bufs, void
     }
     maps[4 * c.n_layers] = m->tm_lm;
     for (int i = 0; i < 3; ++i) {
-      maps[4 * c.n_layers + 1 + 3 * i + 0] = m->tm_h[i];
-      maps[4 * c.n_layers + 1 + 3 * i + 1] = m->tm_attn[i];
-      maps[4 * c.n_layers + 1 + 3 * i + 2] = m->tm_act[i];
+      maps[4 * c.n_layers + 1 + 3 * i + 0] = m->tm_h[kFusedMc[i]];
+      maps[4 * c.n_layers + 1 + 3 * i + 1] = m->tm_attn[kFusedMc[i]];
+      maps[4 * c.n_layers + 1 + 3 * i + 2] = m->tm_act[kFusedMc[i]];
     }
     {
       // paged KV pool as a 5-d tensor: 64-element half of a head row, 16 positions of a page, kv head, page,
