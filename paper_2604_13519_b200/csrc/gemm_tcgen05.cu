@@ -12,6 +12,8 @@
 //
 // Roles: warp 0 = TMA producer, warp 1 = TMEM allocation + MMA issue, warps 2..5 = epilogue.
 // Every wait is bounded; on expiry the CTA records an error word and leaves through the normal exit.
+#include <cuda_fp16.h>
+
 #include "kernels.h"
 
 namespace ts {
@@ -27,9 +29,23 @@ struct __align__(8) GemmSmemCtl {
   uint64_t tmem_full;
   uint32_t tmem_base;
   uint32_t abort_flag;
+  float rs[64];   // per activation row: 1 / rms of the input (1 where the input is normalised already)
 };
 
+__device__ __forceinline__ __half to_half_sat(float x) { return __float2half_rn(fminf(fmaxf(x, -65504.f), 65504.f)); }
+__device__ __forceinline__ __half2 to_half2_sat(float a, float b) { return __halves2half2(to_half_sat(a), to_half_sat(b)); }
+// rounding remainder of a value stored as fp16 (dropped where the value saturates)
+__device__ __forceinline__ float half_rest(float x, __half h) { return fabsf(x) <= 65504.f ? x - __half2float(h) : 0.f; }
+
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// where row m's K/V of `head` (counted over Q, K and V heads) go, in rows of hd elements of the layer's K or V pages
+__device__ __forceinline__ long long kv_place(const GemmArgs &g, int m, int head) {
+  const int kh = head < g.Hq + g.Hkv ? head - g.Hq : head - g.Hq - g.Hkv, slot = g.in.slot[m];
+  const int page = g.in.block_tab[(size_t)g.in.row_seq[m] * g.in.pages_per_seq + (slot >> 4)];
+  return ts_in_range(g.in.ck, CHK_PAGE_APPEND, page, g.in.ck.max_pages) ? ((long long)page * g.Hkv + kh) * 16 + (slot & 15) : -1;
+}
+__device__ __forceinline__ void add4(float4 &s, const float4 &v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
 
 template <int EPI>
 __global__ void __launch_bounds__(192, 1)
@@ -44,7 +60,8 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * kTileN;
-  const int split = blockIdx.y;
+  constexpr bool kCluster = EPI == EPI_QKV || EPI == EPI_RESID;
+  const int split = blockIdx.y;   // (with kCluster: the CTA's rank in its cluster, which spans the K slices of one tile)
   // balanced cut of the k-blocks into gridDim.y runs
   const int kb0 = (int)(((long long)split * g.n_kblocks) / (int)gridDim.y);
   const int kb1 = (int)(((long long)(split + 1) * g.n_kblocks) / (int)gridDim.y);
@@ -116,6 +133,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     } else if (lane == 0) {
       pdl_wait();
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issue
     // The whole warp walks the loop and the waits; one elected lane issues the instructions of a k-block and its
@@ -159,11 +177,74 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     // and the row maximum of the LM head is one reduction over the warp per row.  (With a thread keeping its one feature
     // a row's argmax took ten shuffles per warp and row and its SwiGLU stores were 32-byte pieces: the LM head of the 8B
     // shape took 286 us at 32 rows and 180 at one, same weights.)
+    // With the K slices of a tile in one cluster (QKV, O, down) the rows are dealt out between the two passes: CTA r of C
+    // finishes rows [r, r + 1) * ceil(M / C), adding the C slices' sums in slice order out of the other CTAs' shared memory
+    // -- the same order whatever the number of rows.  Before, the slices went to L2 as slabs that a norm or rotary kernel
+    // of its own folded: three launches and their boundaries more per layer (8B shape at 32 rows: QKV + rotary 12.8 -> 11.6
+    // us, O + norm 10.9 -> 9.8, down + norm 20.6 -> 19.0; 1B shape at 8 rows 38 -> 34 us per layer).  Of a launch's time the
+    // exchange costs about 2 us: 0.6 for the slowest CTA of the cluster, 0.4 - 1.0 for the reads, the rest stores.
     pdl_wait();   // outputs of this kernel may still be read by the previous one's consumers
+    if constexpr (EPI == EPI_QKV || EPI == EPI_SWIGLU) {
+      const int m = (int)threadIdx.x - 64;
+      if (m < g.M) {
+        float s = 0.f;
+        if (g.ss) {
+          const float *p = g.ss + (size_t)m * g.ss_tiles;
+#pragma unroll 8
+          for (int i = 0; i < g.ss_tiles; ++i) s += p[i];
+          s = rsqrtf(s * g.inv_d + g.eps);
+        } else {
+          s = 1.f;
+        }
+        ctl->rs[m] = s;
+      }
+    }
+    const int C = kCluster ? (int)gridDim.y : 1;
+    const int rows_per = (g.M + C - 1) / C, m_beg = kCluster ? split * rows_per : 0, m_end = min(g.M, m_beg + rows_per);
+    const int n = n0 + lane * 4;                  // this lane's features n .. n + 3 in the second pass
+    // what the second pass needs besides the sums is on its way before the sums are complete
+    constexpr int kPre = 2;
+    float4 pre[kPre], gn = make_float4(0.f, 0.f, 0.f, 0.f);
+    int head = 0, ei = 0, half = 0;
+    long long kv_row[kPre];                       // K/V heads: the row's place in the pages (in rows of hd elements), -1: none
+    if constexpr (EPI == EPI_RESID) {
+      gn = *reinterpret_cast<const float4 *>(g.gain + n);
+#pragma unroll
+      for (int i = 0; i < kPre; ++i) {
+        const int m = m_beg + (warp - 2) + 4 * i;
+        if (m < m_end) pre[i] = *reinterpret_cast<const float4 *>(g.x + (size_t)m * g.N + n);
+      }
+    } else if constexpr (EPI == EPI_QKV) {
+      // QKV weight rows are stored with rotary partners adjacent: feature 2e of a head = element e, 2e + 1 = element
+      // e + hd/2; this lane has the pairs ei and ei + 1 of one head
+      head = n / g.hd;
+      half = g.hd >> 1;
+      ei = (n - head * g.hd) >> 1;
+      if (head < g.Hq + g.Hkv) {
+#pragma unroll
+        for (int i = 0; i < kPre; ++i) {
+          const int m = m_beg + (warp - 2) + 4 * i;
+          if (m < m_end) {
+            const int pos = g.in.pos[m];
+            pre[i] = ts_in_range(g.in.ck, CHK_POSITION, pos, g.in.ck.max_ctx)
+                         ? *reinterpret_cast<const float4 *>(g.rope_tab + (size_t)pos * half + ei)
+                         : make_float4(1.f, 0.f, 1.f, 0.f);
+          }
+        }
+      }
+      if (head >= g.Hq) {
+#pragma unroll
+        for (int i = 0; i < kPre; ++i) {
+          const int m = m_beg + (warp - 2) + 4 * i;
+          kv_row[i] = m < m_end ? kv_place(g, m, head) : -1;
+        }
+      }
+    }
     bool ok = true;
     if (nkb > 0) {
       ok = mbar_wait(smem_u32(&ctl->tmem_full), 0);
       if (!ok && lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
+      ok = __all_sync(0xffffffffu, ok);
     }
     tc_fence_after();
     ok = ok && (*reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) == 0);
@@ -185,16 +266,112 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         st_shared_f32(stg + ((c0 + j) * kTileN + q * 32 + lane) * 4,
                       __uint_as_float(r[j]) + (g.planes == 2 ? __uint_as_float(r2[j]) : 0.f));
     }
-    epilogue_sync();
-    const int n = n0 + lane * 4;                  // this lane's features n .. n + 3
-    if (ok) {
-      for (int m = warp - 2; m < g.M; m += 4) {
-        const uint4 raw = ld_shared_v4(stg + (m * kTileN + lane * 4) * 4);
-        const float v[4] = {__uint_as_float(raw.x), __uint_as_float(raw.y), __uint_as_float(raw.z), __uint_as_float(raw.w)};
-        if constexpr (EPI == EPI_PARTIAL) {
-          *reinterpret_cast<uint4 *>(g.out + ((size_t)split * g.out_rows + m) * g.N + n) = raw;
+    if constexpr (kCluster) {
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+    } else {
+      epilogue_sync();
+    }
+    // (a warp's rows two at a time: all their partial sums are fetched before the first is worked on)
+    bool left = !kCluster;   // this CTA has read all that it needs from the others
+#pragma unroll 1
+    for (int mg = m_beg + warp - 2, i0 = 0; ok && mg < m_end; mg += 8, i0 += 2) {
+      float4 sum[2];
+      if constexpr (kCluster) {
+        float4 p[2][8];
+        const bool two = mg + 4 < m_end;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (c < C) p[0][c] = ld_cluster_v4(stg + (mg * kTileN + lane * 4) * 4, c);
+        if (two) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            if (c < C) p[1][c] = ld_cluster_v4(stg + ((mg + 4) * kTileN + lane * 4) * 4, c);
+        }
+        sum[0] = p[0][0];
+#pragma unroll
+        for (int c = 1; c < 8; ++c)
+          if (c < C) add4(sum[0], p[0][c]);
+        if (two) {
+          sum[1] = p[1][0];
+#pragma unroll
+          for (int c = 1; c < 8; ++c)
+            if (c < C) add4(sum[1], p[1][c]);
+        }
+        if (mg + 8 >= m_end) {   // (nothing is left to read: the others may go; they are waited for at the end)
+          __syncwarp();
+          cluster_arrive();
+          left = true;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int m = mg + 4 * i;
+        if (m >= m_end) break;
+        float v[4];
+        if constexpr (kCluster) {
+          v[0] = sum[i].x; v[1] = sum[i].y; v[2] = sum[i].z; v[3] = sum[i].w;
+        } else {
+          const uint4 raw = ld_shared_v4(stg + (m * kTileN + lane * 4) * 4);
+          v[0] = __uint_as_float(raw.x); v[1] = __uint_as_float(raw.y); v[2] = __uint_as_float(raw.z); v[3] = __uint_as_float(raw.w);
+        }
+        if constexpr (EPI == EPI_QKV || EPI == EPI_SWIGLU) {
+          const float s = ctl->rs[m];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] *= s;
+        }
+        if constexpr (EPI == EPI_RESID) {
+          float4 xv = i0 == 0 ? pre[i] : *reinterpret_cast<const float4 *>(g.x + (size_t)m * g.N + n);
+          xv.x += v[0]; xv.y += v[1]; xv.z += v[2]; xv.w += v[3];
+          *reinterpret_cast<float4 *>(g.x + (size_t)m * g.N + n) = xv;
+          const float sq = warp_sum(xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w);
+          if (lane == 0) g.ss_out[(size_t)m * gridDim.x + blockIdx.x] = sq;
+          if (g.h_out) {
+            __align__(8) __nv_bfloat16 hi[4], lo[4];
+            split_bf16(xv.x * gn.x, hi[0], lo[0]);
+            split_bf16(xv.y * gn.y, hi[1], lo[1]);
+            split_bf16(xv.z * gn.z, hi[2], lo[2]);
+            split_bf16(xv.w * gn.w, hi[3], lo[3]);
+            *reinterpret_cast<uint2 *>(g.h_out + (size_t)m * g.N + n) = *reinterpret_cast<const uint2 *>(hi);
+            if (g.out_planes == 2)
+              *reinterpret_cast<uint2 *>(g.h_out + ((size_t)g.act_rows + m) * g.N + n) = *reinterpret_cast<const uint2 *>(lo);
+          }
+        } else if constexpr (EPI == EPI_QKV) {
+          float a0 = v[0], b0 = v[1], a1 = v[2], b1 = v[3];   // elements ei, ei + hd/2, ei + 1, ei + 1 + hd/2
+          if (head < g.Hq + g.Hkv) {
+            float4 cs;
+            if (i0 == 0) {
+              cs = pre[i];
+            } else {
+              const int pos = g.in.pos[m];
+              cs = ts_in_range(g.in.ck, CHK_POSITION, pos, g.in.ck.max_ctx)
+                       ? *reinterpret_cast<const float4 *>(g.rope_tab + (size_t)pos * half + ei)
+                       : make_float4(1.f, 0.f, 1.f, 0.f);
+            }
+            const float ra0 = a0 * cs.x - b0 * cs.y, rb0 = b0 * cs.x + a0 * cs.y;
+            const float ra1 = a1 * cs.z - b1 * cs.w, rb1 = b1 * cs.z + a1 * cs.w;
+            a0 = ra0; b0 = rb0; a1 = ra1; b1 = rb1;
+          }
+          const __half2 ha = to_half2_sat(a0, a1), hb = to_half2_sat(b0, b1);
+          if (head < g.Hq) {
+            // the query as an fp16 pair (value, rounding remainder): the score product adds both, so the 11 bits of
+            // fp16 do not limit the scores
+            const size_t qo = ((size_t)m * g.Hq + head) * g.hd + ei;
+            *reinterpret_cast<__half2 *>(g.q_out + qo) = ha;
+            *reinterpret_cast<__half2 *>(g.q_out + qo + half) = hb;
+            *reinterpret_cast<__half2 *>(g.q_lo_out + qo) = __floats2half2_rn(half_rest(a0, __low2half(ha)), half_rest(a1, __high2half(ha)));
+            *reinterpret_cast<__half2 *>(g.q_lo_out + qo + half) = __floats2half2_rn(half_rest(b0, __low2half(hb)), half_rest(b1, __high2half(hb)));
+          } else {
+            const long long at = i0 == 0 ? kv_row[i] : kv_place(g, m, head);
+            if (at >= 0) {
+              __half *dst = (head < g.Hq + g.Hkv ? g.k_pages : g.v_pages) + at * g.hd + ei;
+              *reinterpret_cast<__half2 *>(dst) = ha;
+              *reinterpret_cast<__half2 *>(dst + half) = hb;
+            }
+          }
         } else if constexpr (EPI == EPI_LOGITS) {
-          *reinterpret_cast<uint4 *>(g.out + (size_t)m * g.N + n) = raw;
+          *reinterpret_cast<float4 *>(g.out + (size_t)m * g.N + n) = make_float4(v[0], v[1], v[2], v[3]);
           // order-preserving map of the float to an unsigned word; ties resolve to the lowest id (lowest lane, then
           // lowest of its four)
           uint32_t best = 0;
@@ -219,6 +396,23 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         }
       }
     }
+    if constexpr (kCluster) {
+      if (!left) {
+        __syncwarp();
+        cluster_arrive();
+      }
+    }
+  }
+  if constexpr (kCluster) {
+    // (every thread of the cluster takes part in both barriers: the sums are in shared memory, then: nobody reads mine
+    // any more; the waits inside the roles are bounded and all of them lead here)
+    __syncwarp();
+    if (warp < 2) {
+      cluster_arrive();
+      cluster_wait();
+      cluster_arrive();
+    }
+    cluster_wait();
   }
   tc_fence_before();
   __syncthreads();
@@ -255,25 +449,66 @@ static cudaError_t launch_one(const CUtensorMap &tw, const CUtensorMap &ta, cons
   cfg.blockDim = dim3(192);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (grid.y > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = 1;
+    at[n].val.clusterDim.y = grid.y;
+    at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
   cfg.attrs = at;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, gemm_ws_kernel<EPI>, tw, ta, g);
 }
 
-cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int n_splits,
+// (asked about a kernel without tensor memory: for one with it the occupancy call answers one CTA per SM)
+__global__ void __launch_bounds__(192) cluster_probe_kernel(float *p) {
+  extern __shared__ float s[];
+  if (p) p[threadIdx.x] = s[threadIdx.x];
+}
+int gemm_max_clusters(int cluster, size_t smem_budget) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(1, cluster);
+  cfg.blockDim = dim3(192);
+  cfg.dynamicSmemBytes = smem_budget;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = cluster;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(cluster_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, cluster_probe_kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int cluster,
                         size_t smem_budget, cudaStream_t st, bool pdl) {
   g.stages = gemm_pick_stages(g.planes, g.Mc, smem_budget);
   const size_t smem = gemm_smem_bytes(g.stages, g.planes, g.Mc);
-  if (g.N % kTileN || g.M > g.Mc || g.Mc % 8 || (g.planes * g.Mc) % 16 || (int)(smem - 1024 - sizeof(GemmSmemCtl)) < g.Mc * kTileN * 4)
+  const bool split = epi == EPI_QKV || epi == EPI_RESID;
+  if (g.N % kTileN || g.M > g.Mc || g.Mc % 8 || (g.planes * g.Mc) % 16 || cluster < 1 || cluster > (split ? 8 : 1) ||
+      cluster > g.n_kblocks || (int)(smem - 1024 - sizeof(GemmSmemCtl)) < g.Mc * kTileN * 4)
     return cudaErrorInvalidValue;
-  dim3 grid(g.N / kTileN, n_splits);
+  const dim3 grid(g.N / kTileN, cluster);
   switch (epi) {
-    case EPI_PARTIAL: return launch_one<EPI_PARTIAL>(tw, ta, g, grid, smem, st, pdl);
+    case EPI_QKV: return launch_one<EPI_QKV>(tw, ta, g, grid, smem, st, pdl);
+    case EPI_RESID: return launch_one<EPI_RESID>(tw, ta, g, grid, smem, st, pdl);
     case EPI_SWIGLU: return launch_one<EPI_SWIGLU>(tw, ta, g, grid, smem, st, pdl);
-    default: return launch_one<EPI_LOGITS>(tw, ta, g, grid, smem, st, pdl);
+    case EPI_LOGITS: return launch_one<EPI_LOGITS>(tw, ta, g, grid, smem, st, pdl);
+    default: return cudaErrorInvalidValue;
   }
 }
 

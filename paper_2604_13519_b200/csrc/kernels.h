@@ -25,36 +25,6 @@ struct PerDeviceOnce {
   void done(int dev) { if (dev >= 0) mask.fetch_or(1ull << dev, std::memory_order_release); }
 };
 
-enum : int { EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_LOGITS = 2 };
-
-struct GemmArgs {
-  int N, K, M;          // output features, reduction length, valid activation rows
-  int Mc;               // activation rows per CTA: the step's rows rounded up (weight-streaming kernel, at most 64), 128 (many rows)
-  int planes;           // 1 = bf16 activations, 2 = (hi, lo) pair
-  int n_kblocks;        // K / 64
-  int kb_per_split;     // k-blocks per split-K slice
-  int stages;           // filled in by the launcher
-  int n_wide;           // many-rows kernel: weight tiles of 256 rows (the tiles after them have 128); filled in by the launcher
-  float *out;           // EPI_PARTIAL: [splits][out_rows][N]; EPI_LOGITS: [M][N]
-  int out_rows;
-  __nv_bfloat16 *act_out;  // EPI_SWIGLU: [out_planes][act_rows][N/2]
-  int act_rows;
-  int out_planes;
-  unsigned long long *amax;  // EPI_LOGITS: [M] packed (ordered logit bits << 32 | ~token id), atomicMax
-  int *err;             // device status word
-  unsigned long long *stamp;   // optional clock stamps of this launch (null = none)
-};
-
-int gemm_pick_stages(int planes, int Mc, size_t smem_budget);
-cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int n_splits,
-                        size_t smem_budget, cudaStream_t st, bool pdl);
-
-// The same projections for many rows (gemm_rows_tcgen05.cu): 128 activation rows x 256 weight rows per CTA, one CTA
-// per SM.  `ta` must be the activation map whose box holds 128 rows; g.Mc and g.stages are set by the launcher.
-int gemm_rows_tiles(int N);
-cudaError_t launch_gemm_rows(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int n_splits,
-                             size_t smem_limit, int n_sms, cudaStream_t st, bool pdl);
-
 // Per-step inputs resident in device memory (all int32).
 struct StepIn {
   const int32_t *tokens;     // [M] chunk ids, rows of sequence i at cu_rows[i]..cu_rows[i+1]
@@ -73,6 +43,56 @@ struct StepIn {
   int B, M;
   BoundsCheck ck;            // ranges for the debug build's index checks
 };
+
+// What a projection does with its sums.  EPI_PARTIAL (many-rows kernel): split-K slabs for the next kernel to fold.
+// EPI_QKV and EPI_RESID (weight-streaming kernel): the sums are complete inside a thread-block cluster; QKV rotates, stores
+// the queries and appends K/V; RESID (O, down) adds to the residual stream and prepares the next projection's input.
+enum : int { EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_LOGITS = 2, EPI_QKV = 3, EPI_RESID = 4 };
+
+struct GemmArgs {
+  int N, K, M;          // output features, reduction length, valid activation rows
+  int Mc;               // activation rows per CTA: the step's rows rounded up (weight-streaming kernel, at most 64), 128 (many rows)
+  int planes;           // 1 = bf16 activations, 2 = (hi, lo) pair
+  int n_kblocks;        // K / 64
+  int kb_per_split;     // k-blocks per split-K slice
+  int stages;           // filled in by the launcher
+  int n_wide;           // many-rows kernel: weight tiles of 256 rows (the tiles after them have 128); filled in by the launcher
+  float *out;           // EPI_PARTIAL: [splits][out_rows][N]; EPI_LOGITS: [M][N]
+  int out_rows;
+  __nv_bfloat16 *act_out;  // EPI_SWIGLU: [out_planes][act_rows][N/2]
+  int act_rows;
+  int out_planes;
+  unsigned long long *amax;  // EPI_LOGITS: [M] packed (ordered logit bits << 32 | ~token id), atomicMax
+  int *err;             // device status word
+  unsigned long long *stamp;   // optional clock stamps of this launch (null = none)
+  // ---- weight-streaming kernel only ----
+  // The RMS norm is split between two projections: the one before stores x * gain (not normalised) and, per row and
+  // 128-feature tile, the sum of x squared; the one after multiplies its finished sums by rsqrt(mean + eps).
+  const float *ss;      // QKV, SWIGLU: [M][ss_tiles] sums of squares of this input's rows; null: the input is normalised
+  int ss_tiles;
+  float inv_d, eps;
+  float *x;             // RESID: [M][N] residual stream, updated in place
+  const float *gain;    // RESID: gain of the norm that follows
+  __nv_bfloat16 *h_out; // RESID: [out_planes][act_rows][N] x * gain; null: not wanted
+  float *ss_out;        // RESID: [M][N / 128]
+  StepIn in;            // QKV
+  const float2 *rope_tab;
+  __half *q_out, *q_lo_out, *k_pages, *v_pages;
+  int Hq, Hkv, hd;
+};
+
+int gemm_pick_stages(int planes, int Mc, size_t smem_budget);
+// clusters of this many CTAs that are resident at once on the current device, at this much shared memory per CTA
+int gemm_max_clusters(int cluster, size_t smem_budget);
+// cluster: CTAs along K that complete a tile's sums together (QKV, RESID; 1 for the others)
+cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int cluster,
+                        size_t smem_budget, cudaStream_t st, bool pdl);
+
+// The same projections for many rows (gemm_rows_tcgen05.cu): 128 activation rows x 256 weight rows per CTA, one CTA
+// per SM.  `ta` must be the activation map whose box holds 128 rows; g.Mc and g.stages are set by the launcher.
+int gemm_rows_tiles(int N);
+cudaError_t launch_gemm_rows(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int n_splits,
+                             size_t smem_limit, int n_sms, cudaStream_t st, bool pdl);
 
 // x[m] = E[tokens[m]]; h = rmsnorm(x) * gain -> bf16 (hi[, lo])
 cudaError_t launch_embed_norm(const StepIn &in, const __nv_bfloat16 *embed, const float *gain, float eps,

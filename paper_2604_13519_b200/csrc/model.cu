@@ -220,6 +220,7 @@ struct ts_model {
   bool last_sample = false;                    // the staged step accepts by speculative sampling
   float last_inv_t = 1.f;                      // 1 / temperature of that step
   size_t smem_optin = 0;
+  int max_clusters[9] = {};                    // [c] = clusters of c CTAs of the weight-streaming kernel that fit at once
   // per-kernel timing pass (ts_profile_step): one event after every launch
   bool profiling = false;
   std::vector<cudaEvent_t> prof_ev;
@@ -310,20 +311,16 @@ int pick_mc_index(int M, int planes) {
   return planes == 1 ? (i | 1) : i;
 }
 
-// split-K factor: two CTAs fit on an SM, so the grid runs in waves of 2 * n_sms CTAs; take the smallest factor
-// (at least 4 k-blocks per slice) whose last wave is at least 95% full, else the one that fills its waves best
-int pick_splits(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks, bool allow, int ctas_per_sm = 2) {
-  if (!allow) return 1;
-  const int ctas = std::max(1, n_tiles * m_chunks), slots = ctas_per_sm * m->n_sms;
-  const int s_max = std::max(1, std::min(kMaxSplits, n_kblocks / 4));
+// CTAs per cluster along K for a projection of the weight-streaming kernel whose sums are completed inside the cluster
+// (QKV, O, down): as many as run at once, two CTAs to an SM, since the bytes in flight are what streams the weights (8B
+// shape at 32 rows, down projection: four CTAs per tile 20.5 us, seven 17.8).  How many clusters fit depends on how the device's SMs
+// are grouped, and a tenth more than needed must fit: with 32 tiles on 33 places one cluster can find its place taken by
+// the neighbouring kernels and run as a second wave (eight per tile: 8.2 us for O on one occasion, 14.1 on others; seven:
+// 8.8).
+int pick_cluster(const ts_model *m, int n_tiles, int n_kblocks) {
   int best = 1;
-  double best_eff = 0.0;
-  for (int s = 1; s <= s_max; ++s) {
-    const int waves = (ctas * s + slots - 1) / slots;
-    const double eff = (double)(ctas * s) / ((double)waves * slots);
-    if (eff > best_eff + 1e-9) { best_eff = eff; best = s; }
-    if (eff >= 0.95) return s;
-  }
+  for (int c = 2; c <= 8 && c <= n_kblocks; ++c)
+    if (m->max_clusters[c] * 10 >= n_tiles * 11) best = c;
   return best;
 }
 
@@ -347,31 +344,35 @@ int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks
   return best;
 }
 
-struct GemmPlan { int splits, kb_per_split; };
-
-ts_status run_gemm(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M,
-                   float *out, __nv_bfloat16 *act_out, unsigned long long *amax, GemmPlan *plan) {
-  const int mi = pick_mc_index(M, m->planes);
+// A projection of the many-rows kernel (more than 64 rows: bound by the tensor cores and the bytes per flop an SM pulls
+// from L2).  n_splits_out: split-K slabs written (EPI_PARTIAL).
+ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M,
+                        float *out, __nv_bfloat16 *act_out, unsigned long long *amax, int *n_splits_out) {
   ts::GemmArgs g{};
-  g.N = N; g.K = K; g.M = M; g.Mc = kMcOptions[mi]; g.planes = m->planes;
+  g.N = N; g.K = K; g.M = M; g.planes = m->planes;
   g.n_kblocks = K / 64;
-  // Up to 64 rows the step is bound by streaming the weights (weight-major kernel, two CTAs per SM); beyond, by the
-  // tensor cores and the bytes per flop an SM pulls from L2 (row-major kernel, 256 weight rows per CTA, one CTA per SM)
-  const bool many_rows = M > 64;
-  const int m_chunks = (M + g.Mc - 1) / g.Mc;
-  int splits = many_rows ? pick_splits_rows(m, ts::gemm_rows_tiles(N), m_chunks, g.n_kblocks, epi == ts::EPI_PARTIAL)
-                         : pick_splits(m, N / 128, m_chunks, g.n_kblocks, epi == ts::EPI_PARTIAL);
-  g.kb_per_split = (g.n_kblocks + splits - 1) / splits;   // (the kernel cuts K into `splits` balanced runs)
+  const int splits = pick_splits_rows(m, ts::gemm_rows_tiles(N), (M + 127) / 128, g.n_kblocks, epi == ts::EPI_PARTIAL);
   g.out = out; g.out_rows = m->L.rows_alloc;
   g.act_out = act_out; g.act_rows = m->L.rows_alloc; g.out_planes = m->planes;
   g.amax = amax;
   g.err = m->d_out() + m->L.o_err;
   g.stamp = m->stamp_slot();
-  if (plan) { plan->splits = splits; plan->kb_per_split = g.kb_per_split; }
-  if (many_rows)
-    CU_TRY(ts::launch_gemm_rows(epi, tw, ta[kMcRows], g, splits, m->smem_optin, m->n_sms, m->st, m->use_pdl && !m->profiling));
-  else
-    CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, splits, m->gemm_smem_budget, m->st, m->use_pdl && !m->profiling));
+  if (n_splits_out) *n_splits_out = splits;
+  CU_TRY(ts::launch_gemm_rows(epi, tw, ta[kMcRows], g, splits, m->smem_optin, m->n_sms, m->st, m->use_pdl && !m->profiling));
+  m->launched(0);
+  return TS_OK;
+}
+
+// A projection of the weight-streaming kernel (at most 64 rows); `g` carries what its epilogue needs.
+ts_status run_gemm_ws(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M, ts::GemmArgs g) {
+  const int mi = pick_mc_index(M, m->planes);
+  g.N = N; g.K = K; g.M = M; g.Mc = kMcOptions[mi]; g.planes = m->planes;
+  g.n_kblocks = K / 64;
+  g.act_rows = m->L.rows_alloc; g.out_planes = m->planes;
+  g.err = m->d_out() + m->L.o_err;
+  g.stamp = m->stamp_slot();
+  const int cluster = (epi == ts::EPI_QKV || epi == ts::EPI_RESID) ? pick_cluster(m, N / 128, g.n_kblocks) : 1;
+  CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, cluster, m->gemm_smem_budget, m->st, m->use_pdl && !m->profiling));
   m->launched(0);
   return TS_OK;
 }
@@ -479,18 +480,36 @@ ts_status run_step(ts_model *m) {
   CU_TRY(ts::launch_embed_norm(in, (const __nv_bfloat16 *)m->W(L.embed), (const float *)m->W(L.g1[0]), c.rms_eps,
                                d, x, h, R, m->planes, (unsigned long long *)m->WS(L.amax), m->st));
   m->launched(3);
-  GemmPlan plan{};
+  // Up to 64 rows the weight-streaming kernel: QKV rotates and appends K/V itself, O and down update the residual stream
+  // and prepare the next projection's input (6 launches per layer); beyond, the many-rows kernel with its split-K slabs
+  // folded by a rotary and two norm kernels.
+  const bool few = M <= 64;
+  float *ss = (float *)m->WS(L.ss_part);
+  const bool skip_head = (m->last_flags & TS_FLAG_SKIP_LM_HEAD) != 0;
+  int splits = 0;
   for (int l = 0; l < c.n_layers; ++l) {
-    if (l > 0) {
-      CU_TRY(ts::launch_add_norm(M, d, part, plan.splits, R, (const float *)m->W(L.g1[l]), c.rms_eps, x, h, R,
-                                 m->planes, m->st, m->stamp_slot()));
-      m->launched(3);
+    ts_status s;
+    if (few) {
+      ts::GemmArgs g{};
+      g.ss = l > 0 ? ss : nullptr;   // (the embedding kernel's rows are normalised)
+      g.ss_tiles = d / 128; g.inv_d = 1.f / (float)d; g.eps = c.rms_eps;
+      g.in = in; g.rope_tab = rope; g.q_out = q; g.q_lo_out = q + (size_t)R * Nq;
+      g.k_pages = m->k_pages(l); g.v_pages = m->v_pages(l);
+      g.Hq = c.n_q_heads; g.Hkv = c.n_kv_heads; g.hd = c.head_dim;
+      s = run_gemm_ws(m, ts::EPI_QKV, m->tm_qkv[l], m->tm_h, L.Nqkv, d, M, g);
+      if (s) return s;
+    } else {
+      if (l > 0) {
+        CU_TRY(ts::launch_add_norm(M, d, part, splits, R, (const float *)m->W(L.g1[l]), c.rms_eps, x, h, R,
+                                   m->planes, m->st, m->stamp_slot()));
+        m->launched(3);
+      }
+      s = run_gemm_rows(m, ts::EPI_PARTIAL, m->tm_qkv[l], m->tm_h, L.Nqkv, d, M, part, nullptr, nullptr, &splits);
+      if (s) return s;
+      CU_TRY(ts::launch_rope_kv(in, part, splits, R, c.n_q_heads, c.n_kv_heads, c.head_dim, rope, q,
+                                q + (size_t)R * Nq, m->k_pages(l), m->v_pages(l), m->st, m->stamp_slot()));
+      m->launched(4);
     }
-    ts_status s = run_gemm(m, ts::EPI_PARTIAL, m->tm_qkv[l], m->tm_h, L.Nqkv, d, M, part, nullptr, nullptr, &plan);
-    if (s) return s;
-    CU_TRY(ts::launch_rope_kv(in, part, plan.splits, R, c.n_q_heads, c.n_kv_heads, c.head_dim, rope, q,
-                              q + (size_t)R * Nq, m->k_pages(l), m->v_pages(l), m->st, m->stamp_slot()));
-    m->launched(4);
     aa.k_pages = m->k_pages(l); aa.v_pages = m->v_pages(l);
     if (m->fused_ok) {   // tensor-memory attention (needs the same device features as the persistent kernel)
       at.layer = l;
@@ -505,25 +524,48 @@ ts_status run_step(ts_model *m) {
       CU_TRY(ts::launch_attention_combine(aa, m->st));
     }
     m->launched(2);
-    s = run_gemm(m, ts::EPI_PARTIAL, m->tm_o[l], m->tm_attn, d, Nq, M, part, nullptr, nullptr, &plan);
-    if (s) return s;
-    CU_TRY(ts::launch_add_norm(M, d, part, plan.splits, R, (const float *)m->W(L.g2[l]), c.rms_eps, x, h, R,
-                               m->planes, m->st, m->stamp_slot()));
-    m->launched(3);
-    // (gate-up keeps its SwiGLU epilogue and so cannot split K: 192 tiles run as 1.3 waves.  Splitting K
-    // three ways with a separate SwiGLU kernel filled the waves but cost as much as it saved.)
-    s = run_gemm(m, ts::EPI_SWIGLU, m->tm_gu[l], m->tm_h, 2 * F, d, M, nullptr, act, nullptr, nullptr);
-    if (s) return s;
-    s = run_gemm(m, ts::EPI_PARTIAL, m->tm_d[l], m->tm_act, d, F, M, part, nullptr, nullptr, &plan);
-    if (s) return s;
+    if (few) {
+      ts::GemmArgs g{};
+      g.x = x; g.h_out = h; g.ss_out = ss;
+      g.gain = (const float *)m->W(L.g2[l]);
+      s = run_gemm_ws(m, ts::EPI_RESID, m->tm_o[l], m->tm_attn, d, Nq, M, g);
+      if (s) return s;
+      ts::GemmArgs u{};
+      u.ss = ss; u.ss_tiles = d / 128; u.inv_d = 1.f / (float)d; u.eps = c.rms_eps;
+      u.act_out = act;
+      s = run_gemm_ws(m, ts::EPI_SWIGLU, m->tm_gu[l], m->tm_h, 2 * F, d, M, u);
+      if (s) return s;
+      const bool last = l + 1 == c.n_layers;   // (the LM head's input is normalised by a norm kernel: it is an output too)
+      g.h_out = last ? nullptr : h;
+      g.gain = (const float *)m->W(last ? L.gf : L.g1[l + 1]);
+      s = run_gemm_ws(m, ts::EPI_RESID, m->tm_d[l], m->tm_act, d, F, M, g);
+      if (s) return s;
+    } else {
+      s = run_gemm_rows(m, ts::EPI_PARTIAL, m->tm_o[l], m->tm_attn, d, Nq, M, part, nullptr, nullptr, &splits);
+      if (s) return s;
+      CU_TRY(ts::launch_add_norm(M, d, part, splits, R, (const float *)m->W(L.g2[l]), c.rms_eps, x, h, R,
+                                 m->planes, m->st, m->stamp_slot()));
+      m->launched(3);
+      // (gate-up keeps its SwiGLU epilogue and so cannot split K)
+      s = run_gemm_rows(m, ts::EPI_SWIGLU, m->tm_gu[l], m->tm_h, 2 * F, d, M, nullptr, act, nullptr, nullptr);
+      if (s) return s;
+      s = run_gemm_rows(m, ts::EPI_PARTIAL, m->tm_d[l], m->tm_act, d, F, M, part, nullptr, nullptr, &splits);
+      if (s) return s;
+    }
   }
-  if (m->last_flags & TS_FLAG_SKIP_LM_HEAD) return TS_OK;
-  CU_TRY(ts::launch_add_norm(M, d, part, plan.splits, R, (const float *)m->W(L.gf), c.rms_eps, x, h, R, m->planes,
+  if (skip_head) return TS_OK;
+  CU_TRY(ts::launch_add_norm(M, d, part, few ? 0 : splits, R, (const float *)m->W(L.gf), c.rms_eps, x, h, R, m->planes,
                              m->st, m->stamp_slot()));
   m->launched(3);
   unsigned long long *amax = (unsigned long long *)m->WS(L.amax);
-  ts_status s = run_gemm(m, ts::EPI_LOGITS, m->tm_lm, m->tm_h, c.vocab, d, M, (float *)m->WS(L.logits), nullptr,
-                         amax, nullptr);
+  ts_status s;
+  if (few) {
+    ts::GemmArgs g{};
+    g.out = (float *)m->WS(L.logits); g.amax = amax;
+    s = run_gemm_ws(m, ts::EPI_LOGITS, m->tm_lm, m->tm_h, c.vocab, d, M, g);
+  } else {
+    s = run_gemm_rows(m, ts::EPI_LOGITS, m->tm_lm, m->tm_h, c.vocab, d, M, (float *)m->WS(L.logits), nullptr, amax, nullptr);
+  }
   if (s) return s;
   int32_t *dout = m->d_out();
   if (m->last_flags & TS_FLAG_WANT_TOPK) {   // per-position Top-K of the logits, for the successor tables
@@ -875,6 +917,7 @@ ts_status ts_init_model(const ts_model_config *cfg, const ts_buffers *bufs, void
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     m->smem_optin = (size_t)optin;
+    for (int cl = 1; cl <= 8; ++cl) m->max_clusters[cl] = ts::gemm_max_clusters(cl, m->gemm_smem_budget);
     m->fused_ok = coop != 0 && m->n_sms <= kMaxFusedCtas &&
                   ts::fused_ring_stages(m->planes, kFusedMaxRows, c.head_dim, m->smem_optin) >= 2;
   }
