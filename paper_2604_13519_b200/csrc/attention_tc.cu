@@ -1,8 +1,7 @@
 // Paged grouped-query attention of the verify chunk on the 5th-generation tensor cores, as a kernel of its own.
 //
-// One unit = (128-row tile of packed (position, query head) rows, kv head, leaf of the KV positions); a CTA takes one
-// unit when the step has no more units than SMs, else it walks several (tensor memory, barriers and the K/V ring are
-// set up once and the ring keeps running across units).
+// One unit = (128-row tile of packed (position, query head) rows, kv head, run of KV positions); a CTA walks its units one
+// after the other (tensor memory, barriers and the K/V ring are set up once and the ring keeps running across units).
 //   warp 0   K/V producer: TMA loads of 64-position blocks straight from the pages (5-d tensor map over the pool)
 //   warp 1   tensor memory allocation + tcgen05.mma issue:  S = Q K^T  (the unit's queries sit in tensor memory as
 //            the row operand -- re-reading a 128-row query tile from shared memory for every 64-position block was
@@ -14,7 +13,7 @@
 //            bits of fp16 do not limit the weights (a single fp16 P was the largest error of the whole step).  The
 //            output sums stay in tensor memory (every P V adds to them); the reference maximum follows the running
 //            one in steps, and only then is the row of sums multiplied down
-// Each leaf writes an un-normalised partial output with its (max, sum); attn_merge_kernel adds a row's leaves.
+// Each unit writes an un-normalised partial output with its (max, sum); attn_merge_kernel adds a row's units.
 // Every wait is bounded; on expiry the CTA records an error word and leaves through the normal exit.
 #include <cuda_fp16.h>
 
@@ -71,38 +70,29 @@ __device__ __forceinline__ bool mbar_wait_err(uint32_t bar, uint32_t parity, con
   }
 }
 
-struct AttnUnit {
-  int tile, kh, leaf;
-  int seq, row0, rows_here, r_beg, len, G;
+// a unit with what follows from it
+struct UnitInfo {
+  int kh, slot, G;
+  int r_beg, row0, rows_here, len;
   int pos_beg, pos_end, nblk;
 };
-
-// The j-th unit of CTA c out of G: units are listed longest first and dealt out in rounds of G, every other round in
-// reverse CTA order, so that the CTA given the longest unit of one round gets the shortest of the next.
-__device__ __forceinline__ int attn_unit_of(int c, int j, int G) { return j * G + ((j & 1) ? G - 1 - c : c); }
-
-// Unit u works on pair u / Hkv (a row tile and one leaf of its sequence) for kv head u % Hkv.  The leaf's positions
-// are [leaf * leaf_len, (leaf + 1) * leaf_len), cut off at the end of the chunk: absolute positions, so the blocks a
-// row meets, and their order, do not depend on where the chunk starts or how long it is.
-__device__ __forceinline__ AttnUnit attn_unit_info(const AttnTcArgs &a, int u) {
-  AttnUnit t;
-  const int pair = u / a.Hkv;
-  t.kh = u - pair * a.Hkv;
-  t.tile = a.unit_tile[pair];
-  t.leaf = a.unit_leaf[pair];
+__device__ __forceinline__ UnitInfo attn_unit_info(const AttnTcArgs &a, int u) {
+  const int4 lo = *reinterpret_cast<const int4 *>(a.units + u), hi = *(reinterpret_cast<const int4 *>(a.units + u) + 1);
+  UnitInfo t;
+  t.r_beg = lo.y;
+  t.row0 = lo.z;
+  t.rows_here = lo.w;
+  t.kh = hi.x & 0xFFFF;
+  t.slot = hi.x >> 16;
+  t.pos_beg = hi.y;
+  t.pos_end = hi.z;
+  t.len = hi.w;
   t.G = a.Hq / a.Hkv;
-  t.seq = a.tile_seq[t.tile];
-  if (!ts_in_range(a.in.ck, CHK_UNIT, t.seq, a.in.B) || !ts_in_range(a.in.ck, CHK_UNIT, t.leaf, a.n_slots)) {
-    t.seq = 0;   // (debug build: the failed check is on record; go on with indices that are in range)
-    t.leaf = 0;
+  if (!ts_in_range(a.in.ck, CHK_UNIT, lo.x, a.in.B) || !ts_in_range(a.in.ck, CHK_UNIT, t.slot, a.n_slots) ||
+      !ts_in_range(a.in.ck, CHK_UNIT, t.kh, a.Hkv) || !ts_in_range(a.in.ck, CHK_UNIT, t.r_beg, a.in.M)) {
+    // (debug build: the failed check is on record; go on with indices that are in range)
+    t.slot = t.kh = t.r_beg = t.rows_here = 0;
   }
-  t.row0 = a.tile_row0[t.tile];
-  t.r_beg = a.in.cu_rows[t.seq];
-  const int k_i = a.in.cu_rows[t.seq + 1] - t.r_beg;
-  t.len = a.in.seq_len[t.seq];
-  t.rows_here = min(kAttnRows, k_i * t.G - t.row0);
-  t.pos_beg = t.leaf * a.leaf_len;
-  t.pos_end = min(t.pos_beg + a.leaf_len, t.len + k_i);
   t.nblk = t.pos_end > t.pos_beg ? (t.pos_end - t.pos_beg + kAttnBlk - 1) / kAttnBlk : 0;
   return t;
 }
@@ -135,13 +125,13 @@ __device__ __forceinline__ uint32_t pack_h2(float x, float y) {
 // block's 64 scores, writes the 64 probabilities back as fp16 and, rarely, rescales the row's output sums.
 // `blk` counts K/V blocks over all units of this CTA (buffer index and barrier parity come from it).
 template <int HD>
-__device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *ctl, const AttnUnit &t, uint32_t tmem_base,
+__device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *ctl, const UnitInfo &t, uint32_t tmem_base,
                                                   int q, int lane, int wtid, uint32_t &blk, bool &waited, const int *err) {
   const int row = q * 32 + lane;      // row of the tile
   const int pr = t.row0 + row;        // packed row of the sequence
   const bool valid = row < t.rows_here;
   const int j = valid ? pr / t.G : 0, gq = valid ? pr % t.G : 0;
-  const size_t ob = ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * a.n_slots + t.leaf;
+  const size_t ob = ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * a.n_slots + t.slot;
   // (a step input like the unit tables: read before the dependency wait)
   const unsigned long long anc = ((unsigned long long)a.in.anc[2 * (t.r_beg + j) + 1] << 32) | a.in.anc[2 * (t.r_beg + j)];
   // the rotated queries come from the previous kernel; everything above was on the device before the step began
@@ -150,7 +140,7 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
     waited = true;
     if (wtid == 0) stamp_waited(a.stamp);
   }
-  if (t.nblk == 0) {   // no position in this leaf: mark it empty
+  if (t.nblk == 0) {   // no position in this unit: mark its slot empty
     if (valid) a.attn_ml[ob] = make_float2(-INFINITY, 0.f);
     return true;
   }
@@ -373,9 +363,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
   if (threadIdx.x == 0) stamp_min(a.stamp);
   pdl_launch_dependents();   // (this CTA holds its tensor memory; the dependent waits for this kernel's end anyway)
   // The step's integer inputs were copied in before the step's first kernel started, so they may be read here.
-  // This CTA's units: attn_unit_of(blockIdx.x, 0, 1, 2, ...).  The three roles walk the units as three loops coupled only by the barriers, whose
-  // phases are counted over all blocks (`gb`) and units (`un`) of the CTA.
-  const int n_total = a.n_units * a.Hkv;
+  // The three roles walk this CTA's units as three loops coupled only by the barriers, whose phases are counted over all
+  // blocks (`gb`) and units (`un`) of the CTA.
+  const int u_beg = a.cta_unit[blockIdx.x], u_end = a.cta_unit[blockIdx.x + 1];
 
   if (warp == 0) {
     // ---------------------------------------------------------------- K/V producer
@@ -385,15 +375,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
       const uint64_t pol = policy_evict_first();
       uint32_t gb = 0;
       bool waited = false, ok = true;
-      for (int j = 0; j * (int)gridDim.x < n_total && ok; ++j) {
-        const int u = attn_unit_of((int)blockIdx.x, j, (int)gridDim.x);
-        if (u >= n_total) continue;
-        const AttnUnit t = attn_unit_info(a, u);
-        const int32_t *btab = a.in.block_tab + (size_t)t.seq * a.in.pages_per_seq;
+      for (int u = u_beg; u < u_end && ok; ++u) {
+        const UnitInfo t = attn_unit_info(a, u);
+        const int32_t *btab = a.in.block_tab + (size_t)a.units[u].seq * a.in.pages_per_seq;
+        const int ready = a.ready_len >= 0 ? a.ready_len : t.len;
         for (int b = 0; b < t.nblk; ++b, ++gb) {
           // blocks wholly inside the cache of earlier steps do not depend on the previous kernel: the ring is filled
           // with them before the dependency wait; the chunk's own K/V rows come from the previous kernel
-          if (!waited && (gb >= (uint32_t)kKvStages || t.pos_beg + (b + 1) * kAttnBlk > t.len)) { pdl_wait(); waited = true; }
+          if (!waited && (gb >= (uint32_t)kKvStages || t.pos_beg + (b + 1) * kAttnBlk > ready)) { pdl_wait(); waited = true; }
           const uint32_t st = gb % kKvStages;
           if (gb >= (uint32_t)kKvStages &&
               !__all_sync(0xffffffffu, mbar_wait_err(smem_u32(&ctl->kv_empty[st]), ((gb / kKvStages) & 1) ^ 1, err))) {
@@ -498,10 +487,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
       // Issue order within a unit: S(0), then for every block b: S(b + 1), O += P(b) V(b).  The scores run one block
       // ahead of the block the workers are on, so a worker finds its scores complete when it gets to them, and the
       // product of block b waits only for that block's probabilities.
-      for (int j = 0; j * (int)gridDim.x < n_total && ok; ++j) {
-        const int u = attn_unit_of((int)blockIdx.x, j, (int)gridDim.x);
-        if (u >= n_total) continue;
-        const AttnUnit t = attn_unit_info(a, u);
+      for (int u = u_beg; u < u_end && ok; ++u) {
+        const UnitInfo t = attn_unit_info(a, u);
         if (t.nblk == 0) continue;
         ok = wait_all(smem_u32(&ctl->q_full), un & 1);
         if (ok) ok = issue_qk(gb);
@@ -517,10 +504,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
     // ---------------------------------------------------------------- workers
     uint32_t blk = 0;
     bool ok = true, waited = false;
-    for (int j = 0; j * (int)gridDim.x < n_total && ok; ++j) {
-      const int u = attn_unit_of((int)blockIdx.x, j, (int)gridDim.x);
-      if (u >= n_total) continue;
-      const AttnUnit t = attn_unit_info(a, u);
+    for (int u = u_beg; u < u_end && ok; ++u) {
+      const UnitInfo t = attn_unit_info(a, u);
       ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp & 3, lane, (int)threadIdx.x - kWorkerWarp0 * 32, blk, waited, err);
     }
     if (!waited) pdl_wait();
@@ -534,17 +519,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
   if (threadIdx.x == 0 && a.stamp) stamp_max(a.stamp + 3);
 }
 
-// grid = (M, Hq / 4), 4 warps: a warp adds the leaves of one (row, query head) and emits the normalised row as bf16
-// (hi[, lo]); lane i owns hd / 32 consecutive elements.  The row's sequence has n_leaves = ceil((cached length +
-// chunk rows) / leaf_len) leaves, all of them written (a leaf the row cannot see carries sum 0 and gets weight 0).
-// Lane s turns leaf s's (max, sum) into a weight; every lane loads its elements of all leaves at once (one round trip
-// to L2, 16 bytes per lane and leaf) and adds them in leaf order.  NS = compile-time bound on the number of leaves.
+// grid = (M, Hq / 4), 4 warps: a warp adds the partial results of one (row, query head) and emits the normalised row as
+// bf16 (hi[, lo]); lane i owns hd / 32 consecutive elements.  The (tile, kv head) has tile_slots units, all of them
+// written (one the row sees nothing of carries sum 0 and gets weight 0).  Lane s turns slot s's (max, sum) into a weight;
+// every lane loads its elements of all slots at once (one round trip to L2, 16 bytes per lane and slot) and adds them in
+// slot order.  NS = compile-time bound on the number of slots.
 template <int NS, int VW>
 __global__ void attn_merge_kernel(const AttnTcArgs a) {
   if (threadIdx.x == 0) stamp_min(a.stamp_merge);
   pdl_launch_dependents();   // the dependent kernel waits for this one's end before touching its data
   const int m = blockIdx.x, h = blockIdx.y * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  int nl = a.in.row_leaves[m];   // (a step input, on the device before the step's first kernel)
+  // (step inputs, on the device before the step's first kernel)
+  const int G = a.Hq / a.Hkv, meta = a.in.row_tile[m];
+  int nl = 0;
+  if (h < a.Hq) nl = a.tile_slots[((meta >> 6) + ((meta & 63) * G + h % G) / kAttnRows) * a.Hkv + h / G];
   if (!ts_in_range(a.in.ck, CHK_LEAVES, nl, a.n_slots + 1)) nl = 0;
   pdl_wait();
   if (threadIdx.x == 0) stamp_waited(a.stamp_merge);
@@ -648,7 +636,7 @@ cudaError_t launch_attention_tc(const AttnTcArgs &a, cudaStream_t st) {
     once.done(dev_);
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(std::min(a.n_units * a.Hkv, a.max_ctas));
+  cfg.gridDim = dim3(a.n_ctas);
   cfg.blockDim = dim3(kTcThreads);
   cfg.dynamicSmemBytes = attn_tc_smem(a.hd);
   cfg.stream = st;

@@ -335,7 +335,7 @@ static int pick_wide_tiles(int blocks, int chunks, int n_sms) {
   int best_x = x_max;
   double best_t = 1e30;
   std::vector<double> sm(n_sms);
-  for (int x = x_max; x >= 0 && x >= x_max - 2 * n_sms; --x) {
+  for (int x = x_max; x >= 0 && x >= x_max - 2 * n_sms / chunks; --x) {
     std::fill(sm.begin(), sm.end(), 0.0);
     std::make_heap(sm.begin(), sm.end(), std::greater<double>());
     const int tiles = x + (blocks - 2 * x);

@@ -38,8 +38,8 @@ struct StepIn {
   const int32_t *parent;     // [M] parent of each row inside its chunk (row index relative to the chunk; -1 = root)
   const uint32_t *anc;       // [M][2] low / high word of the row's visibility mask over its chunk: bit i = row i of
                              // the chunk is the row itself or one of its ancestors (a chain: bits 0..j)
-  const int32_t *row_leaves; // [M] attention leaves of the row's sequence: ceil((cached length + chunk rows) / leaf length)
-  int pages_per_seq;
+  const int32_t *row_tile;   // [M] 64 x (first attention tile of the row's sequence) + the row's index in its chunk
+  int pages_per_seq;         // (0: all sequences of the step share one row of the block table, as the pieces of a prompt do)
   int B, M;
   BoundsCheck ck;            // ranges for the debug build's index checks
 };
@@ -128,23 +128,26 @@ struct AttnArgs {
 cudaError_t launch_attention_split(const AttnArgs &a, cudaStream_t st);
 cudaError_t launch_attention_combine(const AttnArgs &a, cudaStream_t st);
 
-// tcgen05 attention as a kernel of its own (attention_tc.cu): one CTA per (128-row tile, leaf, kv head).
-// A leaf is a run of leaf_len KV positions starting at an absolute multiple of leaf_len (a model constant, a
-// multiple of 64): leaf L of a sequence holds positions [L * leaf_len, (L + 1) * leaf_len), whatever the cached
-// length or the chunk length.  Every leaf yields one partial result per row, and the merge adds a row's leaves in
-// leaf order, so the bits of a row's attention output are a function of its position and its prefix only: the same
-// token gets the same logits whether it is verified alone (vanilla decoding) or as row j of a chunk.
+// tcgen05 attention as a kernel of its own (attention_tc.cu).  A unit of work is (128-row tile of packed rows, kv head,
+// run of KV positions); the host lists each CTA's units.  Every unit yields one partial result per row in a slot of its
+// own, and the merge adds a row's slots in order of position.
+struct AttnWork {
+  int32_t seq, r_beg;         // sequence, its first row in the step
+  int32_t row0, rows;         // first packed row (chunk row x group + query head of the group) of the tile, rows in it
+  int32_t kh_slot;            // kv head | slot << 16
+  int32_t pos_beg, pos_end;   // positions (pos_beg is a multiple of 64; an empty run writes an empty slot)
+  int32_t len;                // cached length of the sequence: every row sees every position below it
+};
 struct AttnTcArgs {
   StepIn in;
   int Hq, Hkv, hd, layer;
-  int leaf_len;                  // KV positions per leaf
-  int n_units;                   // (tile, leaf) pairs of this step: n_units * Hkv units of work
-  int max_ctas;                  // CTAs launched at most (one per SM); a CTA walks units blockIdx.x, + gridDim.x, ...
-  int n_slots;                   // partial results kept per (row, query head): the most leaves any sequence has
-  const int32_t *unit_tile;      // [n_units] tile of each pair
-  const int32_t *unit_leaf;      // [n_units] leaf of each pair
-  const int32_t *tile_seq;       // [tiles] sequence of each 128-row tile of packed rows
-  const int32_t *tile_row0;      // [tiles] first packed row of the tile
+  int n_ctas;                    // CTA c walks units cta_unit[c] .. cta_unit[c + 1]
+  int n_slots;                   // partial results kept per (row, query head): the most units any (tile, kv head) has
+  int ready_len;                 // >= 0: positions below it were cached before this step (a step over pieces of one prompt,
+                                 // whose `len`s lie inside the step); -1: those below each sequence's own `len` were
+  const AttnWork *units;
+  const int32_t *cta_unit;
+  const int32_t *tile_slots;     // [tiles][Hkv] units of each (tile, kv head)
   const __half *q, *q_lo;        // [M][Hq][hd] rotated queries as an fp16 pair: value and rounding remainder
   const CUtensorMap *map_kv;     // device copy of the 5-d map over the paged KV pool
   float *attn_o;                 // [M*Hq][n_slots][hd] unnormalised partial outputs

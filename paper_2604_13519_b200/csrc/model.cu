@@ -48,6 +48,9 @@ constexpr int kMaxAttnSplits = ts::kAttnMaxSplits;
 constexpr int kMcOptions[9] = {8, 16, 24, 32, 40, 48, 56, 64, 128};
 constexpr int kMcRows = 8;                       // index of the many-rows kernel's box
 constexpr int kFusedMc[3] = {1, 3, 7};           // the persistent kernel's boxes: 16, 32, 64 rows
+constexpr int kPrefillRows = 1024;   // rows of a prompt that go through in one step
+constexpr int kPrefillSplits = 3;    // split-K slabs of such a step at most
+constexpr int kPrefillSlots = 8;     // attention slots per row of such a step at most
 constexpr int kMaxFusedCtas = 256;   // the fused kernel runs one CTA per SM
 constexpr int kFusedMaxRows = 64;    // most rows per step the fused kernel takes
 constexpr bool kAutoPrefersFused = false;   // path = 0 picks the faster of the two on the 8B batch-1 step
@@ -65,14 +68,17 @@ struct Layout {
   uint64_t maps, slab, ss_part, sync, phase_t, stamps;
   int max_stamps;
   int n_maps, n_counters, n_phases, max_tiles128, o_tile128_seq, o_tile128_row0;
-  int max_units, o_unit_tile, o_unit_leaf, o_row_leaves;   // attention units (see AttnTcArgs)
+  int max_units, max_ctas, o_row_tile, o_tile_slots, o_cta_unit;   // attention units (see AttnTcArgs)
   // step io (int32 offsets inside d_in / h_in)
   int o_tokens, o_pos, o_rowseq, o_cu, o_len, o_tile_seq, o_tile_row0, o_btab, in_ints;
   int o_parent, o_anc, o_path, o_uni, o_topk, o_slot;
   uint64_t samp_stats, topk_cand;
   // step out (int32 offsets)
   int o_argmax, o_accept, o_emitted, o_newlen, o_newpend, o_err, out_ints;
-  int rows_alloc, pages_per_seq, max_tiles, Nqkv, n_vocab_tiles;
+  int rows_alloc;        // rows of the activation buffers: max_rows or a piece of a prompt, whichever is more
+  int step_rows_alloc;   // max_rows rounded up to 128: rows of the logits
+  int prefill_rows, part_rows, slot_rows;   // (see make_layout)
+  int pages_per_seq, max_tiles, Nqkv, n_vocab_tiles;
   uint64_t host_io_bytes;
 };
 
@@ -119,40 +125,53 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->kv_layer_stride = 2 * L->kv_v_offset;
   L->kv_bytes = (uint64_t)c.n_layers * L->kv_layer_stride * 2;
 
-  L->rows_alloc = (int)align_up(c.max_rows, 128);
+  // A prompt goes through in pieces of up to kPrefillRows rows, whatever k_max and max_rows are: the weights are read once
+  // per piece (8B shape, 1999 tokens: 32 steps of 64 rows streamed 483 GB).  The activation buffers hold a piece; the
+  // logits need not.
+  L->step_rows_alloc = (int)align_up(c.max_rows, 128);
+  L->prefill_rows = (int)std::min<uint64_t>(kPrefillRows, align_up(c.max_ctx, 64));
+  L->rows_alloc = std::max(L->step_rows_alloc, (int)align_up(L->prefill_rows, 128));
+  L->part_rows = std::max(kMaxSplits * L->step_rows_alloc, kPrefillSplits * L->rows_alloc);      // split-K slabs x rows
+  L->slot_rows = std::max(kMaxAttnSplits * L->step_rows_alloc, kPrefillSlots * L->rows_alloc);   // attention slots x rows
+  const int io_rows = std::max(c.max_rows, L->prefill_rows), io_seqs = std::max(c.max_batch, (L->prefill_rows + 63) / 64);
   L->pages_per_seq = (c.max_ctx + TS_PAGE_SIZE - 1) / TS_PAGE_SIZE;
   const int G = c.n_q_heads / c.n_kv_heads;
   L->max_tiles = c.max_batch * ((c.k_max * G + 63) / 64);
   L->n_vocab_tiles = c.vocab / 128;
-  const uint64_t R = L->rows_alloc, planes = c.act_split ? 2 : 1;
+  const uint64_t R = L->rows_alloc, Rs = L->step_rows_alloc, planes = c.act_split ? 2 : 1;
   o = 0;
   L->x = take(R * d * 4);
   L->h = take(planes * R * d * 2);
   const uint64_t part_cols = std::max<uint64_t>(L->Nqkv, d);
-  L->part = take((uint64_t)kMaxSplits * R * part_cols * 4);
+  L->part = take((uint64_t)L->part_rows * part_cols * 4);
   L->q = take(2 * R * Nq * 2);   // rotated queries, fp16: values [R][Nq], then their rounding remainders [R][Nq]
-  L->attn_o = take(R * c.n_q_heads * kMaxAttnSplits * hd * 4);
-  L->attn_ml = take(R * c.n_q_heads * kMaxAttnSplits * 8);
+  L->attn_o = take((uint64_t)L->slot_rows * c.n_q_heads * hd * 4);
+  L->attn_ml = take((uint64_t)L->slot_rows * c.n_q_heads * 8);
   L->attn = take(planes * R * Nq * 2);
   L->act = take(planes * R * F * 2);
-  L->logits = take(R * V * 4);
+  L->logits = take(Rs * V * 4);
   L->amax = take(R * 8);
-  L->samp_stats = take(R * 16 * 4);
-  L->topk_cand = take(R * (uint64_t)((c.vocab + 4095) / 4096) * TS_TOPK * 8);
+  L->samp_stats = take(Rs * 16 * 4);
+  L->topk_cand = take(Rs * (uint64_t)((c.vocab + 4095) / 4096) * TS_TOPK * 8);
   L->rope = take((uint64_t)c.max_ctx * (hd / 2) * 8);
   int io = 0;
   auto itake = [&](int n) { int r = io; io += (n + 3) / 4 * 4; return r; };
-  L->o_tokens = itake(c.max_rows); L->o_pos = itake(c.max_rows); L->o_rowseq = itake(c.max_rows);
-  L->o_cu = itake(c.max_batch + 1); L->o_len = itake(c.max_batch);
+  L->o_tokens = itake(io_rows); L->o_pos = itake(io_rows); L->o_rowseq = itake(io_rows);
+  L->o_cu = itake(io_seqs + 1); L->o_len = itake(io_seqs);
   L->o_tile_seq = itake(L->max_tiles); L->o_tile_row0 = itake(L->max_tiles);
-  L->max_tiles128 = c.max_batch * ((c.k_max * G + 127) / 128);
+  const int prefill_tiles = (L->prefill_rows + 63) / 64 * ((64 * G + 127) / 128);
+  L->max_tiles128 = std::max(c.max_batch * ((c.k_max * G + 127) / 128), prefill_tiles);
   L->o_tile128_seq = itake(L->max_tiles128); L->o_tile128_row0 = itake(L->max_tiles128);
-  L->max_units = L->max_tiles128 * kMaxAttnSplits;
-  L->o_unit_tile = itake(L->max_units); L->o_unit_leaf = itake(L->max_units);
-  L->o_row_leaves = itake(c.max_rows);
-  L->o_parent = itake(c.max_rows); L->o_anc = itake(2 * c.max_rows); L->o_uni = itake(c.max_rows);
-  L->o_slot = itake(c.max_rows);
-  L->o_btab = itake(c.max_batch * L->pages_per_seq);   // (last: only the used part is copied per step)
+  // (units: at most kMaxAttnSplits per tile and kv head, see build_attention)
+  L->max_units = L->max_tiles128 * c.n_kv_heads * kMaxAttnSplits;
+  L->max_ctas = kMaxFusedCtas;
+  L->o_row_tile = itake(io_rows);
+  L->o_tile_slots = itake(L->max_tiles128 * c.n_kv_heads);
+  L->o_cta_unit = itake(L->max_ctas + 1);
+  L->o_parent = itake(io_rows); L->o_anc = itake(2 * io_rows); L->o_uni = itake(io_rows);
+  L->o_slot = itake(io_rows);
+  // (last, only the used part is copied per step: the block table, and behind its used rows the attention units)
+  L->o_btab = itake(c.max_batch * L->pages_per_seq + L->max_units * (int)(sizeof(ts::AttnWork) / 4));
   L->in_ints = io;
   io = 0;
   L->o_argmax = itake(c.max_rows); L->o_accept = itake(c.max_batch); L->o_emitted = itake(c.max_batch * c.k_max);
@@ -209,7 +228,9 @@ struct ts_model {
   std::vector<int32_t> free_pages;
   std::vector<ts_session *> sessions;   // live sessions over this model (detached on destroy)
   // last staged step
-  int last_B = 0, last_M = 0, last_tiles = 0, last_tiles128 = 0, last_units = 0, last_slots = 1;
+  int last_B = 0, last_M = 0, last_tiles = 0, last_tiles128 = 0, last_ctas = 0, last_slots = 1;
+  int last_ready = -1;                         // pieces of a prompt: positions cached before the step (else -1)
+  size_t last_units_at = 0;                    // where the step's attention units lie in its inputs (int32 offset)
   uint32_t last_flags = 0;
   bool have_step = false;
   int64_t launches = 0, h2d = 0, d2h = 0;
@@ -330,10 +351,10 @@ int pick_cluster(const ts_model *m, int n_tiles, int n_kblocks) {
 //   waves * (k-blocks per CTA + 13) + 2.5 * slices
 // (measured on the 8B shape with 256 rows: 9 slices of 7 k-blocks in two waves took 29.5 us for the O projection,
 // 4 slices of 16 in one wave 21 us, and the norm after it reads 4 slabs instead of 9).
-int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks, bool allow) {
+int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks, bool allow, int room) {
   if (!allow) return 1;
   const int ctas = std::max(1, n_tiles * m_chunks);
-  const int s_max = std::max(1, std::min(kMaxSplits, n_kblocks / 4));
+  const int s_max = std::max(1, std::min(std::min(kMaxSplits, room), n_kblocks / 4));
   int best = 1;
   double best_cost = 1e30;
   for (int s = 1; s <= s_max; ++s) {
@@ -351,8 +372,9 @@ ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUten
   ts::GemmArgs g{};
   g.N = N; g.K = K; g.M = M; g.planes = m->planes;
   g.n_kblocks = K / 64;
-  const int splits = pick_splits_rows(m, ts::gemm_rows_tiles(N), (M + 127) / 128, g.n_kblocks, epi == ts::EPI_PARTIAL);
-  g.out = out; g.out_rows = m->L.rows_alloc;
+  const int Ma = (M + 127) / 128 * 128;
+  const int splits = pick_splits_rows(m, ts::gemm_rows_tiles(N), Ma / 128, g.n_kblocks, epi == ts::EPI_PARTIAL, m->L.part_rows / Ma);
+  g.out = out; g.out_rows = Ma;
   g.act_out = act_out; g.act_rows = m->L.rows_alloc; g.out_planes = m->planes;
   g.amax = amax;
   g.err = m->d_out() + m->L.o_err;
@@ -389,7 +411,7 @@ ts_status run_step_fused(ts_model *m) {
   a.in.tokens = di + L.o_tokens; a.in.pos = di + L.o_pos; a.in.row_seq = di + L.o_rowseq; a.in.cu_rows = di + L.o_cu;
   a.in.seq_len = di + L.o_len; a.in.block_tab = di + L.o_btab; a.in.pages_per_seq = L.pages_per_seq;
   a.in.parent = di + L.o_parent; a.in.anc = (const uint32_t *)(di + L.o_anc); a.in.slot = di + L.o_slot;
-  a.in.row_leaves = di + L.o_row_leaves;
+  a.in.row_tile = di + L.o_row_tile;
   a.in.B = m->last_B; a.in.M = m->last_M;
   a.mc_index = m->last_M <= 16 ? 0 : (m->last_M <= 32 ? 1 : 2); a.Mc = kMcOptions[kFusedMc[a.mc_index]]; a.planes = m->planes;
   a.n_ctas = m->n_sms; a.skip_lm = (m->last_flags & TS_FLAG_SKIP_LM_HEAD) ? 1 : 0;
@@ -438,9 +460,9 @@ ts_status run_step(ts_model *m) {
   ts::StepIn in{};
   int32_t *di = m->d_in();
   in.tokens = di + L.o_tokens; in.pos = di + L.o_pos; in.row_seq = di + L.o_rowseq; in.cu_rows = di + L.o_cu;
-  in.seq_len = di + L.o_len; in.block_tab = di + L.o_btab; in.pages_per_seq = L.pages_per_seq;
+  in.seq_len = di + L.o_len; in.block_tab = di + L.o_btab; in.pages_per_seq = m->last_ready >= 0 ? 0 : L.pages_per_seq;
   in.parent = di + L.o_parent; in.anc = (const uint32_t *)(di + L.o_anc); in.slot = di + L.o_slot;
-  in.row_leaves = di + L.o_row_leaves;
+  in.row_tile = di + L.o_row_tile;
   in.B = B; in.M = M;
   in.ck.err = m->d_out() + L.o_err; in.ck.vocab = c.vocab; in.ck.max_pages = c.max_pages; in.ck.max_ctx = c.max_ctx;
   float *x = (float *)m->WS(L.x);
@@ -450,7 +472,7 @@ ts_status run_step(ts_model *m) {
   __nv_bfloat16 *attn = (__nv_bfloat16 *)m->WS(L.attn);
   __nv_bfloat16 *act = (__nv_bfloat16 *)m->WS(L.act);
   const float2 *rope = (const float2 *)m->WS(L.rope);
-  const int R = L.rows_alloc;
+  const int R = L.rows_alloc, part_R = (M + 127) / 128 * 128;
 
   ts::AttnArgs aa{};
   aa.in = in; aa.q = q; aa.Hq = c.n_q_heads; aa.Hkv = c.n_kv_heads; aa.hd = c.head_dim;
@@ -471,9 +493,8 @@ ts_status run_step(ts_model *m) {
 
   ts::AttnTcArgs at{};
   at.in = in; at.Hq = c.n_q_heads; at.Hkv = c.n_kv_heads; at.hd = c.head_dim;
-  at.leaf_len = m->leaf_len; at.n_units = m->last_units; at.n_slots = m->last_slots; at.max_ctas = m->n_sms;
-  at.unit_tile = di + L.o_unit_tile; at.unit_leaf = di + L.o_unit_leaf;
-  at.tile_seq = di + L.o_tile128_seq; at.tile_row0 = di + L.o_tile128_row0;
+  at.n_ctas = m->last_ctas; at.n_slots = m->last_slots; at.ready_len = m->last_ready;
+  at.units = (const ts::AttnWork *)(di + m->last_units_at); at.cta_unit = di + L.o_cta_unit; at.tile_slots = di + L.o_tile_slots;
   at.q = q; at.q_lo = q + (size_t)R * Nq; at.map_kv = (const CUtensorMap *)m->WS(L.maps) + (L.n_maps - 1);
   at.attn_o = aa.part_o; at.attn_ml = aa.part_ml; at.err = m->d_out() + L.o_err;
   at.out = attn; at.out_rows = R; at.planes = m->planes;
@@ -500,16 +521,18 @@ ts_status run_step(ts_model *m) {
       if (s) return s;
     } else {
       if (l > 0) {
-        CU_TRY(ts::launch_add_norm(M, d, part, splits, R, (const float *)m->W(L.g1[l]), c.rms_eps, x, h, R,
+        CU_TRY(ts::launch_add_norm(M, d, part, splits, part_R, (const float *)m->W(L.g1[l]), c.rms_eps, x, h, R,
                                    m->planes, m->st, m->stamp_slot()));
         m->launched(3);
       }
       s = run_gemm_rows(m, ts::EPI_PARTIAL, m->tm_qkv[l], m->tm_h, L.Nqkv, d, M, part, nullptr, nullptr, &splits);
       if (s) return s;
-      CU_TRY(ts::launch_rope_kv(in, part, splits, R, c.n_q_heads, c.n_kv_heads, c.head_dim, rope, q,
+      CU_TRY(ts::launch_rope_kv(in, part, splits, part_R, c.n_q_heads, c.n_kv_heads, c.head_dim, rope, q,
                                 q + (size_t)R * Nq, m->k_pages(l), m->v_pages(l), m->st, m->stamp_slot()));
       m->launched(4);
     }
+    // (of a prompt's last layer only the K/V are used)
+    if (m->last_ready >= 0 && l + 1 == c.n_layers) return TS_OK;
     aa.k_pages = m->k_pages(l); aa.v_pages = m->v_pages(l);
     if (m->fused_ok) {   // tensor-memory attention (needs the same device features as the persistent kernel)
       at.layer = l;
@@ -543,7 +566,7 @@ ts_status run_step(ts_model *m) {
     } else {
       s = run_gemm_rows(m, ts::EPI_PARTIAL, m->tm_o[l], m->tm_attn, d, Nq, M, part, nullptr, nullptr, &splits);
       if (s) return s;
-      CU_TRY(ts::launch_add_norm(M, d, part, splits, R, (const float *)m->W(L.g2[l]), c.rms_eps, x, h, R,
+      CU_TRY(ts::launch_add_norm(M, d, part, splits, part_R, (const float *)m->W(L.g2[l]), c.rms_eps, x, h, R,
                                  m->planes, m->st, m->stamp_slot()));
       m->launched(3);
       // (gate-up keeps its SwiGLU epilogue and so cannot split K)
@@ -554,7 +577,7 @@ ts_status run_step(ts_model *m) {
     }
   }
   if (skip_head) return TS_OK;
-  CU_TRY(ts::launch_add_norm(M, d, part, few ? 0 : splits, R, (const float *)m->W(L.gf), c.rms_eps, x, h, R, m->planes,
+  CU_TRY(ts::launch_add_norm(M, d, part, few ? 0 : splits, part_R, (const float *)m->W(L.gf), c.rms_eps, x, h, R, m->planes,
                              m->st, m->stamp_slot()));
   m->launched(3);
   unsigned long long *amax = (unsigned long long *)m->WS(L.amax);
@@ -616,6 +639,166 @@ ts_status ensure_pages(ts_session *s, int tokens) {
   return TS_OK;
 }
 
+// The step inputs of row `r` of the step, a row of sequence i.
+void put_row(ts_model *m, int i, int r, int32_t token, int pos, int slot, int parent, uint64_t mask) {
+  const Layout &L = m->L;
+  int32_t *hi = m->h_in();
+  hi[L.o_tokens + r] = token;
+  hi[L.o_pos + r] = pos;
+  hi[L.o_rowseq + r] = i;
+  hi[L.o_slot + r] = slot;
+  hi[L.o_parent + r] = parent;
+  hi[L.o_anc + 2 * r] = (int32_t)(uint32_t)(mask & 0xFFFFFFFFull);
+  hi[L.o_anc + 2 * r + 1] = (int32_t)(uint32_t)(mask >> 32);
+}
+uint64_t chain_mask(int j) { return j >= 63 ? ~0ull : ((2ull << j) - 1ull); }
+
+// Tiles and units of the attention kernels (o_cu and o_len are filled in; tables = rows of the block table in use).
+//
+// Steps of at most 64 rows: a unit is a LEAF of the context, the positions [L, L + 1) * leaf_len: absolute, so the blocks
+// a row meets and the order its sums are taken in do not depend on where its chunk starts, how long it is or what is
+// verified beside it.  Whole leaves first, the shorter last leaves at the end, dealt out to the CTAs in rounds, every
+// other round in reverse CTA order.
+//
+// Larger steps (their projections sum in another order anyway): the (tile, kv head) pairs' blocks in one line, cut into
+// equal stretches, one per CTA, a unit's fixed cost counted as kUnitBlocks blocks -- leaves left the SMs unevenly loaded.
+constexpr int kUnitBlocks = 5;   // setting up and draining a unit takes about as long as five 64-position blocks
+ts_status build_attention(ts_model *m, int B, int M, int tables) {
+  const Layout &L = m->L;
+  const int Hkv = m->c.n_kv_heads, G = m->c.n_q_heads / Hkv;
+  int32_t *hi = m->h_in();
+  std::vector<int> order(B);
+  for (int i = 0; i < B; ++i) order[i] = i;
+  auto rows_of = [&](int i) { return hi[L.o_cu + i + 1] - hi[L.o_cu + i]; };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hi[L.o_len + a] + rows_of(a) > hi[L.o_len + b] + rows_of(b); });
+  m->last_units_at = align_up((uint64_t)L.o_btab + (uint64_t)tables * L.pages_per_seq, 4);
+  ts::AttnWork *units = (ts::AttnWork *)(hi + m->last_units_at);
+  const int cap = std::min(L.max_units, (int)((L.in_ints - m->last_units_at) / (sizeof(ts::AttnWork) / 4)));
+  const int max_ctas = std::min(m->n_sms, L.max_ctas);
+  struct Tile { int seq, row0, rows, blocks, end; };   // blocks: 64-position blocks its rows can see
+  std::vector<Tile> tiles;
+  for (int i : order) {
+    const int k = rows_of(i), len = hi[L.o_len + i];
+    for (int r = hi[L.o_cu + i]; r < hi[L.o_cu + i + 1]; ++r) hi[L.o_row_tile + r] = 64 * (int)tiles.size() + (r - hi[L.o_cu + i]);
+    for (int r0 = 0; r0 < k * G; r0 += 128) {
+      const int rows = std::min(128, k * G - r0), end = len + (r0 + rows - 1) / G + 1;
+      hi[L.o_tile128_seq + tiles.size()] = i;
+      hi[L.o_tile128_row0 + tiles.size()] = r0;
+      tiles.push_back({i, r0, rows, (end + 63) / 64, end});
+    }
+  }
+  const int n_tiles = (int)tiles.size();
+  m->last_tiles128 = n_tiles;
+  int n = 0, slots = 1;
+  auto put = [&](int tile, int kh, int slot, int beg, int end) {
+    const Tile &t = tiles[tile];
+    if (n < cap)
+      units[n] = {t.seq, hi[L.o_cu + t.seq], t.row0, t.rows, kh | (slot << 16), beg, end, hi[L.o_len + t.seq]};
+    ++n;
+    slots = std::max(slots, slot + 1);
+  };
+  if (M <= 64) {
+    struct Leaf { int tile, leaf, nblk; };
+    std::vector<Leaf> leaves;
+    for (int t = 0; t < n_tiles; ++t) {
+      const int total = hi[L.o_len + tiles[t].seq] + rows_of(tiles[t].seq), n_leaves = (total + m->leaf_len - 1) / m->leaf_len;
+      for (int kh = 0; kh < Hkv; ++kh) hi[L.o_tile_slots + t * Hkv + kh] = n_leaves;
+      for (int lf = 0; lf < n_leaves; ++lf) leaves.push_back({t, lf, (std::min(total, (lf + 1) * m->leaf_len) - lf * m->leaf_len + 63) / 64});
+    }
+    std::stable_sort(leaves.begin(), leaves.end(), [](const Leaf &a, const Leaf &b) { return a.nblk > b.nblk; });
+    const int total = (int)leaves.size() * Hkv, ctas = std::min(total, max_ctas);
+    for (int c = 0; c < ctas; ++c) {
+      hi[L.o_cta_unit + c] = n;
+      for (int j = 0; j * ctas < total; ++j) {
+        const int u = j * ctas + ((j & 1) ? ctas - 1 - c : c);
+        if (u >= total) continue;
+        const Leaf &lf = leaves[u / Hkv];
+        const int s = tiles[lf.tile].seq;
+        put(lf.tile, u % Hkv, lf.leaf, lf.leaf * m->leaf_len, std::min((lf.leaf + 1) * m->leaf_len, hi[L.o_len + s] + rows_of(s)));
+      }
+    }
+    hi[L.o_cta_unit + ctas] = n;
+    m->last_ctas = ctas;
+  } else {
+    const int slot_cap = std::min(kMaxAttnSplits, L.slot_rows / M);
+    long long total = 0;
+    int longest = 1;
+    for (const Tile &t : tiles) { total += (long long)t.blocks * Hkv; longest = std::max(longest, t.blocks); }
+    // a CTA's share in blocks: everything and the fixed cost of every unit, evenly; a cut leaves at least kUnitBlocks
+    // blocks on either side, and no tile gets more slots than there are
+    long long share = (total + (long long)kUnitBlocks * (n_tiles * Hkv + max_ctas) + max_ctas - 1) / max_ctas;
+    share = std::max(share, (long long)std::max(3 * kUnitBlocks, kUnitBlocks + (longest + slot_cap - 2) / std::max(1, slot_cap - 1)));
+    for (;; share += (share + 31) / 32) {
+      n = 0; slots = 1;
+      int c = 0;
+      long long left = share;
+      hi[L.o_cta_unit] = 0;
+      bool fits = true;
+      for (int t = 0; t < n_tiles && fits; ++t)
+        for (int kh = 0; kh < Hkv && fits; ++kh) {
+          int b = 0, slot = 0;
+          while (b < tiles[t].blocks) {
+            const int rest = tiles[t].blocks - b;
+            long long take = std::min<long long>(rest, left - kUnitBlocks);
+            if (take < rest && rest - take < kUnitBlocks) take = left >= rest ? rest : rest - kUnitBlocks;   // (no sliver after the cut)
+            if (take < rest && take < kUnitBlocks) {   // nor before it
+              if (++c >= max_ctas) { fits = false; break; }
+              hi[L.o_cta_unit + c] = n;
+              left = share;
+              continue;
+            }
+            put(t, kh, slot, b * 64, take == rest ? tiles[t].end : (b + (int)take) * 64);
+            ++slot;
+            b += (int)take;
+            left -= take + kUnitBlocks;
+          }
+          if (fits) hi[L.o_tile_slots + t * Hkv + kh] = slot;
+        }
+      if (fits && slots <= slot_cap) {
+        m->last_ctas = c + 1;
+        hi[L.o_cta_unit + c + 1] = n;
+        break;
+      }
+    }
+  }
+  if (n > cap) return fail(TS_ERR_ARG, "internal: %d attention units exceed %d", n, cap);
+  m->last_slots = slots;
+  return TS_OK;
+}
+
+// Copies the staged inputs in, runs the step, copies its results back and waits.
+ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
+  const ts_model_config &c = m->c;
+  const Layout &L = m->L;
+  m->last_B = B; m->last_M = M; m->last_flags = flags;
+  m->have_step = true;
+  const size_t in_bytes = (m->last_units_at + (size_t)m->h_in()[L.o_cta_unit + m->last_ctas] * (sizeof(ts::AttnWork) / 4)) * 4;
+  CU_TRY(cudaMemcpyAsync(m->d_in(), m->h_in(), in_bytes, cudaMemcpyHostToDevice, m->st));
+  m->h2d += (int64_t)in_bytes;
+  ts_status st = run_step(m);
+  if (st) return st;
+  if (m->inject_err) {
+    // test support (ts_debug_inject_device_error): after the step's last kernel, write the status word an expired
+    // device-side wait would have left; the code below must then treat the step as failed
+    m->h_out()[L.o_err + 1] = m->inject_err;
+    m->inject_err = 0;
+    CU_TRY(cudaMemcpyAsync(m->d_out() + L.o_err, m->h_out() + L.o_err + 1, 4, cudaMemcpyHostToDevice, m->st));
+  }
+  const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
+  CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
+  m->d2h += (int64_t)out_bytes;
+  CU_TRY(cudaStreamSynchronize(m->st));
+  const int dev_err = m->h_out()[L.o_err];
+  if (dev_err != 0) {
+    cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
+    cudaMemsetAsync(m->WS(L.sync), 0, (size_t)(8 + L.n_counters) * 4, m->st);   // the fused kernel left its counters mid-step
+    if (dev_err >= ts::DEV_BOUNDS)
+      return fail(TS_ERR_DEVICE_BOUNDS, "an index check of the debug build failed on the device (check %d)", dev_err - ts::DEV_BOUNDS);
+    return fail(TS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired (code %d)", dev_err);
+  }
+  return TS_OK;
+}
+
 // Stage one step: rows[i] = chunk ids of sequence i.  Copies inputs, runs, copies results back, syncs.
 // parents (optional): parents[i][j] = chunk row that row j of sequence i hangs from (-1 for row 0); a chain if null.
 ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::vector<std::vector<int32_t>> &rows,
@@ -625,7 +808,7 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
   const Layout &L = m->L;
   int32_t *hi = m->h_in();
   const int G = c.n_q_heads / c.n_kv_heads;
-  int M = 0, tiles = 0, tiles128 = 0;
+  int M = 0, tiles = 0;
   hi[L.o_cu] = 0;
   for (int i = 0; i < B; ++i) {
     ts_session *s = ss[i];
@@ -654,14 +837,8 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
             if ((*parents)[i][e] == par && rows[i][e] == rows[i][j])
               return fail(TS_ERR_ARG, "sequence %d: rows %d and %d are children of row %d with the same token", i, e, j, par);
       }
-      const uint64_t mask = parents ? anc[j] : (j >= 63 ? ~0ull : ((2ull << j) - 1ull));
-      hi[L.o_tokens + M + j] = rows[i][j];
-      hi[L.o_pos + M + j] = s->cache_len + (parents ? depth[j] : j);
-      hi[L.o_rowseq + M + j] = i;
-      hi[L.o_slot + M + j] = s->cache_len + j;
-      hi[L.o_parent + M + j] = par;
-      hi[L.o_anc + 2 * (M + j)] = (int32_t)(uint32_t)(mask & 0xFFFFFFFFull);
-      hi[L.o_anc + 2 * (M + j) + 1] = (int32_t)(uint32_t)(mask >> 32);
+      const uint64_t mask = parents ? anc[j] : chain_mask(j);
+      put_row(m, i, M + j, rows[i][j], s->cache_len + (parents ? depth[j] : j), s->cache_len + j, par, mask);
     }
     hi[L.o_len + i] = s->cache_len;
     for (int r0 = 0; r0 < k * G; r0 += 64) {
@@ -669,46 +846,13 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
       hi[L.o_tile_row0 + tiles] = r0;
       ++tiles;
     }
-    tiles128 += (k * G + 127) / 128;
     std::memcpy(hi + L.o_btab + (size_t)i * L.pages_per_seq, s->pages.data(), s->pages.size() * sizeof(int32_t));
     M += k;
     hi[L.o_cu + i + 1] = M;
   }
   {
-    // 128-row tiles, longest sequence first: the attention kernel's CTAs are handed out in tile order, so the long
-    // units start first and the short ones fill the tail
-    std::vector<int> order(B);
-    for (int i = 0; i < B; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-      return hi[L.o_len + a] + (hi[L.o_cu + a + 1] - hi[L.o_cu + a]) > hi[L.o_len + b] + (hi[L.o_cu + b + 1] - hi[L.o_cu + b]);
-    });
-    int t = 0;
-    // (tile, leaf) pairs of the attention kernel: leaf L of a sequence is the absolute positions [L, L + 1) * leaf_len
-    struct Unit { int tile, leaf, nblk; };
-    std::vector<Unit> units;
-    int slots = 1;
-    for (int i : order) {
-      const int k = hi[L.o_cu + i + 1] - hi[L.o_cu + i], total = hi[L.o_len + i] + k;
-      const int n_leaves = (total + m->leaf_len - 1) / m->leaf_len;
-      slots = std::max(slots, n_leaves);
-      for (int r = hi[L.o_cu + i]; r < hi[L.o_cu + i + 1]; ++r) hi[L.o_row_leaves + r] = n_leaves;
-      for (int r0 = 0; r0 < k * G; r0 += 128) {
-        hi[L.o_tile128_seq + t] = i;
-        hi[L.o_tile128_row0 + t] = r0;
-        for (int lf = 0; lf < n_leaves; ++lf)
-          units.push_back({t, lf, (std::min(total, (lf + 1) * m->leaf_len) - lf * m->leaf_len + 63) / 64});
-        ++t;
-      }
-    }
-    // whole leaves first, the shorter last leaves at the end, where they fill the tail of the last wave
-    std::stable_sort(units.begin(), units.end(), [](const Unit &a, const Unit &b) { return a.nblk > b.nblk; });
-    if ((int)units.size() > L.max_units) return fail(TS_ERR_ARG, "internal: %zu attention units exceed %d", units.size(), L.max_units);
-    for (size_t u = 0; u < units.size(); ++u) {
-      hi[L.o_unit_tile + u] = units[u].tile;
-      hi[L.o_unit_leaf + u] = units[u].leaf;
-    }
-    m->last_units = (int)units.size();
-    m->last_slots = slots;
+    ts_status st = build_attention(m, B, M, B);
+    if (st) return st;
   }
   const bool can_fuse = m->fused_ok && M <= kFusedMaxRows;
   if (c.path == 2 && !can_fuse)
@@ -739,33 +883,37 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
     return fail(TS_ERR_UNIMPLEMENTED, "the per-position Top-K needs the one-kernel-per-stage path");
   m->last_fused = !m->last_tree && !m->last_sample && !(flags & TS_FLAG_WANT_TOPK) && can_fuse &&
                   (c.path == 2 || (c.path == 0 && kAutoPrefersFused));
-  m->last_B = B; m->last_M = M; m->last_tiles = tiles; m->last_tiles128 = tiles128; m->last_flags = flags;
-  m->have_step = true;
-  const size_t in_bytes = (size_t)(L.o_btab + (size_t)B * L.pages_per_seq) * 4;
-  CU_TRY(cudaMemcpyAsync(m->d_in(), hi, in_bytes, cudaMemcpyHostToDevice, m->st));
-  m->h2d += (int64_t)in_bytes;
-  ts_status st = run_step(m);
+  m->last_tiles = tiles;
+  m->last_ready = -1;
+  return submit_step(m, B, M, flags);
+}
+
+// One step over `k` tokens of a prompt (k <= prefill_rows), cached length cache_len: the piece goes through as sequences of
+// 64 rows, each seeing the ones before it as its context.  All K/V of a layer are in the pages before its attention begins.
+ts_status prefill_step(ts_model *m, ts_session *s, const int32_t *tokens, int k) {
+  const ts_model_config &c = m->c;
+  const Layout &L = m->L;
+  int32_t *hi = m->h_in();
+  const int base = s->cache_len;
+  if (base + k > c.max_ctx) return fail(TS_ERR_ARG, "sequence 0 would exceed max_ctx");
+  for (int j = 0; j < k; ++j)
+    if (tokens[j] < 0 || tokens[j] >= c.vocab) return fail(TS_ERR_TOKEN_RANGE, "token id %d outside [0, %d)", tokens[j], c.vocab);
+  ts_status st = ensure_pages(s, base + k);
   if (st) return st;
-  if (m->inject_err) {
-    // test support (ts_debug_inject_device_error): after the step's last kernel, write the status word an expired
-    // device-side wait would have left; the code below must then treat the step as failed
-    m->h_out()[L.o_err + 1] = m->inject_err;
-    m->inject_err = 0;
-    CU_TRY(cudaMemcpyAsync(m->d_out() + L.o_err, m->h_out() + L.o_err + 1, 4, cudaMemcpyHostToDevice, m->st));
+  std::memcpy(hi + L.o_btab, s->pages.data(), s->pages.size() * sizeof(int32_t));
+  const int B = (k + 63) / 64;
+  for (int i = 0; i < B; ++i) {
+    hi[L.o_cu + i] = 64 * i;
+    hi[L.o_len + i] = base + 64 * i;
   }
-  const size_t out_bytes = (size_t)L.out_ints * 4;
-  CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
-  m->d2h += (int64_t)out_bytes;
-  CU_TRY(cudaStreamSynchronize(m->st));
-  const int dev_err = m->h_out()[L.o_err];
-  if (dev_err != 0) {
-    cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
-    cudaMemsetAsync(m->WS(L.sync), 0, (size_t)(8 + L.n_counters) * 4, m->st);   // the fused kernel left its counters mid-step
-    if (dev_err >= ts::DEV_BOUNDS)
-      return fail(TS_ERR_DEVICE_BOUNDS, "an index check of the debug build failed on the device (check %d)", dev_err - ts::DEV_BOUNDS);
-    return fail(TS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired (code %d)", dev_err);
-  }
-  return TS_OK;
+  hi[L.o_cu + B] = k;
+  for (int r = 0; r < k; ++r) put_row(m, r >> 6, r, tokens[r], base + r, base + r, (r & 63) - 1, chain_mask(r & 63));
+  st = build_attention(m, B, k, 1);
+  if (st) return st;
+  m->last_tree = m->last_sample = m->last_fused = false;
+  m->last_tiles = 1;   // (the 64-row tiles of the kernel without tensor memory are not made)
+  m->last_ready = base;
+  return submit_step(m, B, k, TS_FLAG_SKIP_LM_HEAD);
 }
 
 // y <- y (+) ids, delta per id, stop at the first finishing id.  Returns ids consumed.
@@ -995,7 +1143,7 @@ ts_status ts_load_tensor(ts_model *m, int32_t kind, int32_t layer, const void *h
   cudaPointerAttributes pa{};
   const bool on_device = cudaPointerGetAttributes(&pa, host) == cudaSuccess && pa.type == cudaMemoryTypeDevice;
   cudaGetLastError();
-  const size_t stage_bytes = (size_t)L.rows_alloc * (size_t)c.vocab * 4;   // the logits area doubles as staging
+  const size_t stage_bytes = (size_t)L.step_rows_alloc * (size_t)c.vocab * 4;   // the logits area doubles as staging
   const int64_t rows_per_chunk = on_device ? er : std::max<int64_t>(1, (int64_t)(stage_bytes / row_bytes));
   for (int64_t r0 = 0; r0 < er; r0 += rows_per_chunk) {
     const int64_t nr = std::min(rows_per_chunk, er - r0);
@@ -1190,11 +1338,14 @@ ts_status ts_prefill(ts_model *m, ts_session *s, const int32_t *tokens, int32_t 
   s->prompt.assign(tokens, tokens + n);
   s->cache_len = 0;
   if (m) {
+    // (the persistent kernel takes k_max rows at a time; so does a device without tensor-memory attention)
+    const bool pieces = m->fused_ok && m->c.path != 2;
+    const int piece = pieces ? m->L.prefill_rows : m->c.k_max;
     std::vector<std::vector<int32_t>> rows(1);
-    for (int i = 0; i < n - 1; i += m->c.k_max) {
-      const int k = std::min(m->c.k_max, n - 1 - i);
-      rows[0].assign(tokens + i, tokens + i + k);
-      ts_status st = stage_and_run(m, &s, 1, rows, TS_FLAG_SKIP_LM_HEAD);
+    for (int i = 0; i < n - 1; i += piece) {
+      const int k = std::min(piece, n - 1 - i);
+      if (!pieces) rows[0].assign(tokens + i, tokens + i + k);
+      ts_status st = pieces ? prefill_step(m, s, tokens + i, k) : stage_and_run(m, &s, 1, rows, TS_FLAG_SKIP_LM_HEAD);
       if (st) { s->cache_len = -1; return st; }
       s->cache_len += k;
     }
@@ -1684,18 +1835,20 @@ ts_status ts_session_retrieve(ts_model *m, ts_session *s, int32_t row, int32_t K
 ts_status ts_debug_read_buffer(ts_model *m, int32_t which, void *host_out, uint64_t bytes) {
   if (!m || !host_out) return fail(TS_ERR_ARG, "null argument");
   const Layout &L = m->L;
-  const uint64_t R = L.rows_alloc, P = m->planes, d = m->c.d_model, Nq = (uint64_t)m->c.n_q_heads * m->c.head_dim;
-  uint64_t off = 0, cap = 0;
+  const uint64_t R = L.step_rows_alloc, P = m->planes, d = m->c.d_model, Nq = (uint64_t)m->c.n_q_heads * m->c.head_dim;
+  uint64_t off = 0, plane = 0, n_planes = 1;   // plane = bytes of one plane's first R rows
   switch (which) {
-    case 0: off = L.x; cap = R * d * 4; break;
-    case 1: off = L.h; cap = P * R * d * 2; break;
-    case 2: off = L.q; cap = R * Nq * 2; break;
-    case 3: off = L.attn; cap = P * R * Nq * 2; break;
-    case 4: off = L.act; cap = P * R * (uint64_t)m->c.d_ffn * 2; break;
+    case 0: off = L.x; plane = R * d * 4; break;
+    case 1: off = L.h; plane = R * d * 2; n_planes = P; break;
+    case 2: off = L.q; plane = R * Nq * 2; break;
+    case 3: off = L.attn; plane = R * Nq * 2; n_planes = P; break;
+    case 4: off = L.act; plane = R * (uint64_t)m->c.d_ffn * 2; n_planes = P; break;
     default: return fail(TS_ERR_ARG, "unknown buffer %d", which);
   }
-  if (bytes > cap) return fail(TS_ERR_ARG, "buffer %d holds %llu bytes", which, (unsigned long long)cap);
-  CU_TRY(cudaMemcpyAsync(host_out, m->WS(off), bytes, cudaMemcpyDeviceToHost, m->st));
+  if (bytes > plane * n_planes) return fail(TS_ERR_ARG, "buffer %d holds %llu bytes", which, (unsigned long long)(plane * n_planes));
+  for (uint64_t at = 0, pl = 0; at < bytes; at += plane, ++pl)
+    CU_TRY(cudaMemcpyAsync((uint8_t *)host_out + at, m->WS(off + pl * (plane / R) * L.rows_alloc), std::min(plane, bytes - at),
+                           cudaMemcpyDeviceToHost, m->st));
   CU_TRY(cudaStreamSynchronize(m->st));
   return TS_OK;
 }
