@@ -2,17 +2,24 @@
 //
 // One unit = (128-row tile of packed (position, query head) rows, kv head, run of KV positions); a CTA walks its units one
 // after the other (tensor memory, barriers and the K/V ring are set up once and the ring keeps running across units).
-//   warp 0   K/V producer: TMA loads of 64-position blocks straight from the pages (5-d tensor map over the pool)
-//   warp 1   tensor memory allocation + tcgen05.mma issue:  S = Q K^T  (the unit's queries sit in tensor memory as
+//   warp 8   K/V producer: TMA loads of 64-position blocks straight from the pages (5-d tensor map over the pool)
+//   warp 9   tensor memory allocation + tcgen05.mma issue:  S = Q K^T  (the unit's queries sit in tensor memory as
 //            the row operand -- re-reading a 128-row query tile from shared memory for every 64-position block was
 //            what bounded the kernel -- the K block K-major in shared memory, 128 x 64 fp32 result in tensor
-//            memory), then  O_blk = P V  with P read from tensor memory (fp16) and the V block read MN-major from
+//            memory), then  O += P V  with P read from tensor memory (fp16) and the V block read MN-major from
 //            the same [position][64 elements] image K uses
-//   warps 2..5  one row per thread: maximum over the block's 64 scores, P = exp2(S - reference maximum) written back
-//            to tensor memory as an fp16 (value, rounding remainder) pair -- the second product adds both, so the 11
-//            bits of fp16 do not limit the weights (a single fp16 P was the largest error of the whole step).  The
-//            output sums stay in tensor memory (every P V adds to them); the reference maximum follows the running
-//            one in steps, and only then is the row of sums multiplied down
+//   warps 0..3, 4..7   two softmax groups, one row per thread: group 0 takes the unit's even blocks, group 1 the odd ones,
+//            each with a reference maximum, a sum and output sums in tensor memory of its own, put together at the unit's
+//            end.  Maximum over the block's 64 scores, P = exp2(S - reference maximum) written over the scores as an fp16
+//            (value, rounding remainder) pair -- the second product adds both, so the 11 bits of fp16 do not limit the
+//            weights (a single fp16 P was the largest error of the whole step).  The reference maximum follows the
+//            running one in steps, and only then is the row of sums multiplied down
+// A block is 1024 cycles of tensor-core work (24 instructions: both planes of Q and of P) and about 950 of softmax by one
+// warp per scheduler, latency on latency; with one group the two alternated and a block took 2000 cycles, with two the
+// one's softmax runs under the other's products: 1350.  What is left above 1024 is the issuing warp: an instruction is taken
+// only when the ones before it are nearly done, so all that the warp does between two blocks leaves the tensor cores idle.
+// Four sessions of 8192 tokens with 64 rows each: 81 -> 70 us per launch; sixteen ragged ones: 114 -> 92.  (Measured and
+// slower: an issuing warp per group, 86 and 114 us; exponentials before the block's maximum is known, 75 and 103.)
 // Each unit writes an un-normalised partial output with its (max, sum); attn_merge_kernel adds a row's units.
 // Every wait is bounded; on expiry the CTA records an error word and leaves through the normal exit.
 #include <cuda_fp16.h>
@@ -33,21 +40,20 @@ static constexpr int kAttnBlk = 64;     // kv positions per block
 // tokens of context, 7 of them spent in that wait; with twelve stages 7.9 us (eight ragged sessions: 31.2 -> 15.3 us).
 __host__ __device__ constexpr int kv_stages(int hd) { return hd == 64 ? 12 : 6; }
 static constexpr int kMaxKvStages = 12;
-static constexpr int kTcThreads = 192;
-static constexpr int kWorkers = 128;
-static constexpr int kWorkerWarp0 = 2;
+static constexpr int kTcThreads = 320;
+static constexpr int kWorkerWarps = 8, kProducerWarp = 8, kMmaWarp = 9;
 
 struct __align__(16) AttnCtl {
   uint64_t kv_full[kMaxKvStages], kv_empty[kMaxKvStages], q_full;
-  uint64_t s_full[2], s_empty[2], p_full[2], pv_done[2], o_free;
+  uint64_t s_full[2], p_full[2], pv_done[2];   // [2]: one per softmax group
   uint32_t tmem_base;
+  float2 ml[2][kAttnRows];   // (reference maximum, sum) of each group's part of a row
 };
 
-__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 __device__ __forceinline__ bool worker_all(bool ok) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
       : "r"((uint32_t)ok)
       : "memory");
@@ -97,12 +103,11 @@ __device__ __forceinline__ UnitInfo attn_unit_info(const AttnTcArgs &a, int u) {
   return t;
 }
 
-// tensor-memory columns of the attention phase (they lie over the projection accumulators, which are idle then)
-static constexpr int kColS = 0;      // two score buffers of 64 columns
-static constexpr int kColP = 128;    // two probability buffers of 32 columns (fp16, two per column)
-static constexpr int kColO = 192;    // the output sums: head_dim columns, accumulated over the unit's blocks
-static constexpr int kColPL = 448;   // the probabilities' rounding remainders: two buffers of 32 columns
-static constexpr int kColQ = 320;    // the unit's queries, fp16 pairs: head_dim / 2 columns of values, then as many of remainders
+// tensor-memory columns
+static constexpr int kColS = 0;      // one buffer of 64 columns per group: the scores, then in their place the probabilities as
+                                     // fp16 pairs -- 32 columns of values, 32 of rounding remainders
+static constexpr int kColQ = 128;    // the unit's queries, fp16 pairs: head_dim / 2 columns of values, then as many of remainders
+static constexpr int kColO = 256;    // the output sums: head_dim columns per group (the second group's at + 128)
 static constexpr float kRescaleStep = 8.f;   // the reference maximum follows the running one in steps of 2^8
 
 // 2^x for x <= 0 (and 0 for -inf); tiny results flush to zero
@@ -121,12 +126,30 @@ __device__ __forceinline__ uint32_t pack_h2(float x, float y) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// Worker side of one unit.  Thread <-> row (tensor-memory lane q*32 + lane): it takes the row maximum over the
-// block's 64 scores, writes the 64 probabilities back as fp16 and, rarely, rescales the row's output sums.
-// `blk` counts K/V blocks over all units of this CTA (buffer index and barrier parity come from it).
+// two fp32 operations in one instruction
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
+// Worker side of one unit.  Thread <-> row (tensor-memory lane q*32 + lane) of one of the two groups: it takes the row
+// maximum over a block's 64 scores, writes the 64 probabilities over them as fp16 pairs and, rarely, rescales the row's
+// output sums.  `cnt` counts this group's blocks over all units of this CTA (barrier parities come from it).
 template <int HD>
 __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *ctl, const UnitInfo &t, uint32_t tmem_base,
-                                                  int q, int lane, int wtid, uint32_t &blk, bool &waited, const int *err) {
+                                                  int grp, int q, int lane, uint32_t &cnt, bool &waited, const int *err) {
   const int row = q * 32 + lane;      // row of the tile
   const int pr = t.row0 + row;        // packed row of the sequence
   const bool valid = row < t.rows_here;
@@ -138,51 +161,44 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
   if (!waited) {
     pdl_wait();
     waited = true;
-    if (wtid == 0) stamp_waited(a.stamp);
+    if (threadIdx.x == 0) stamp_waited(a.stamp);
   }
   if (t.nblk == 0) {   // no position in this unit: mark its slot empty
-    if (valid) a.attn_ml[ob] = make_float2(-INFINITY, 0.f);
+    if (valid && grp == 0) a.attn_ml[ob] = make_float2(-INFINITY, 0.f);
     return true;
   }
   // ---- stage Q into tensor memory: the score product reads its row operand there (thread <-> row, an fp16 pair
-  // per column: head_dim / 2 columns of values, then as many of rounding remainders), so per block only the keys
-  // and values come through shared memory.  Every score product of the CTA's previous unit has completed (its
-  // last scores were read before that unit's sums were drained), so the columns may be overwritten.
+  // per column; group 0 the values, group 1 the rounding remainders), so per block only the keys and values come
+  // through shared memory.  Every score product of the CTA's previous unit has completed (both groups had read their last
+  // scores when they met at its end), so the columns may be overwritten.
   const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16);
   {
-    const size_t so = ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * HD;
-    // all loads of both planes are issued before the first use: one round trip to L2, where the previous kernel has
-    // just written the rows
-    // (32 bytes per lane and load: the lanes of a warp read 32 different rows)
-    uint32_t v[2][HD / 2];
+    const __half *src = (grp ? a.q_lo : a.q) + ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * HD;
+    // all loads are issued before the first use: one round trip to L2, where the previous kernel has just written the
+    // rows (32 bytes per lane and load: the lanes of a warp read 32 different rows)
+    uint32_t v[HD / 2];
     if (valid) {
 #pragma unroll
-      for (int c = 0; c < HD / 16; ++c) {
-        ld_global_v8(a.q + so + c * 16, &v[0][c * 8]);
-        ld_global_v8(a.q_lo + so + c * 16, &v[1][c * 8]);
-      }
+      for (int c = 0; c < HD / 16; ++c) ld_global_v8(src + c * 16, &v[c * 8]);
     } else {
 #pragma unroll
-      for (int c = 0; c < HD / 2; ++c) v[0][c] = v[1][c] = 0u;
+      for (int c = 0; c < HD / 2; ++c) v[c] = 0u;
     }
 #pragma unroll
-    for (int pl = 0; pl < 2; ++pl) {
+    for (int c4 = 0; c4 < HD / 32; ++c4) {
+      uint32_t r[16];
 #pragma unroll
-      for (int c4 = 0; c4 < HD / 32; ++c4) {
-        uint32_t r[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) r[e] = v[pl][c4 * 16 + e];
-        tmem_st16(tq + kColQ + pl * (HD / 2) + c4 * 16, r);
-      }
+      for (int e = 0; e < 16; ++e) r[e] = v[c4 * 16 + e];
+      tmem_st16(tq + kColQ + grp * (HD / 2) + c4 * 16, r);
     }
     tmem_wait_st();
   }
   tc_fence_before();
-  worker_sync();
-  if (wtid == 0) mbar_arrive(smem_u32(&ctl->q_full));
+  __syncwarp();
+  if (lane == 0) mbar_arrive(smem_u32(&ctl->q_full));
 
   // Visibility: the whole cache, and of the chunk the rows named by this row's mask (itself and its ancestors in
-  // the draft tree; in a chain, rows 0..j), up to the end of this split.
+  // the draft tree; in a chain, rows 0..j), up to the end of this unit.
   const int lim_all = min(t.len, t.pos_end) - 1;   // every row sees every position up to here
   const float scale = rsqrtf((float)HD) * 1.4426950408889634f;
   // The output sums stay in tensor memory: every product P V adds to them.  Probabilities are taken against a
@@ -192,19 +208,19 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
   // inside fp16, and the sums are fp32.
   float m_ref = -INFINITY, l_run = 0.f;
   bool ok = true;
+  const uint32_t colS = tq + kColS + grp * 64, colO = tq + kColO + grp * 128;
 
-  for (int b = 0; b < t.nblk; ++b, ++blk) {
-    const uint32_t buf = blk & 1;
-    if (ok && !mbar_wait_err(smem_u32(&ctl->s_full[buf]), (blk >> 1) & 1, err)) { ok = false; atomicCAS((int *)err, 0, DEV_TIMEOUT_TMEM); }
+  for (int b = grp; b < t.nblk; b += 2, ++cnt) {
+    if (ok && !mbar_wait_err(smem_u32(&ctl->s_full[grp]), cnt & 1, err)) { ok = false; atomicCAS((int *)err, 0, DEV_TIMEOUT_TMEM); }
     tc_fence_after();
     const int p_base = t.pos_beg + b * kAttnBlk;
     float sc[64];
     {
       uint32_t r0[16], r1[16], r2[16], r3[16];
-      tmem_ld16(tq + kColS + buf * 64, r0);
-      tmem_ld16(tq + kColS + buf * 64 + 16, r1);
-      tmem_ld16(tq + kColS + buf * 64 + 32, r2);
-      tmem_ld16(tq + kColS + buf * 64 + 48, r3);
+      tmem_ld16(colS, r0);
+      tmem_ld16(colS + 16, r1);
+      tmem_ld16(colS + 32, r2);
+      tmem_ld16(colS + 48, r3);
       tmem_wait_ld();
 #pragma unroll
       for (int e = 0; e < 16; ++e) {
@@ -212,19 +228,16 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
         sc[32 + e] = __uint_as_float(r2[e]); sc[48 + e] = __uint_as_float(r3[e]);
       }
     }
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&ctl->s_empty[buf]));
-    // a block every row sees whole needs no mask (all but the last blocks of a sequence's last split)
+    // a block every row sees whole needs no mask (all but the last blocks of a sequence's last unit)
     if (p_base + kAttnBlk - 1 > lim_all) {
       // bit e of `vis`: position p_base + e is visible to this row (cache positions all, chunk rows by the mask,
-      // nothing at or past the split's end)
+      // nothing at or past the unit's end)
       const int rel0 = p_base - t.len;                 // chunk row of the block's first position (negative: cache)
       unsigned long long vis;
       if (rel0 >= 0) vis = rel0 < 64 ? anc >> rel0 : 0ull;
       else if (rel0 > -64) vis = (anc << (-rel0)) | ((1ull << (-rel0)) - 1ull);
       else vis = ~0ull;
-      const int n_in = t.pos_end - p_base;             // positions of the block inside the split
+      const int n_in = t.pos_end - p_base;             // positions of the block inside the unit
       if (n_in < 64) vis &= n_in > 0 ? (1ull << n_in) - 1ull : 0ull;
       const uint32_t vlo = (uint32_t)vis, vhi = (uint32_t)(vis >> 32);
 #pragma unroll
@@ -245,85 +258,90 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
     const float m_old = m_ref;
     if (raise) m_ref = m_blk;
     const float ref = (m_ref == -INFINITY) ? 0.f : m_ref;
-    float sum0 = 0.f, sum1 = 0.f;
-    uint32_t pk0[16], pk1[16], pl0[16], pl1[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      const float e0 = ex2_approx(fmaf(sc[2 * e], scale, -ref));
-      const float e1 = ex2_approx(fmaf(sc[2 * e + 1], scale, -ref));
-      const float e2 = ex2_approx(fmaf(sc[32 + 2 * e], scale, -ref));
-      const float e3 = ex2_approx(fmaf(sc[32 + 2 * e + 1], scale, -ref));
-      sum0 += e0 + e2; sum1 += e1 + e3;
-      const __half2 h01 = __floats2half2_rn(e0, e1), h23 = __floats2half2_rn(e2, e3);
-      pk0[e] = *reinterpret_cast<const uint32_t *>(&h01);
-      pk1[e] = *reinterpret_cast<const uint32_t *>(&h23);
-      pl0[e] = pack_h2(e0 - __low2float(h01), e1 - __high2float(h01));
-      pl1[e] = pack_h2(e2 - __low2float(h23), e3 - __high2float(h23));
-    }
-    // This block's P buffer last fed product b - 2, which is complete: the scores of this block were committed after
-    // it by the same thread, and a commit covers everything issued before it.  Only multiplying the sums down needs
-    // more -- product b - 1 complete -- so that is the only case that waits.  The products of even and of odd blocks
-    // complete phases of barriers of their own: a waiter is then never more than one phase behind (product b - 3,
-    // the previous one on the same barrier, is known complete), which a parity wait needs.
+    // Multiplying the sums down needs the group's previous product complete, and it is: it was issued before this block's
+    // scores, whose commit covers everything issued before it.
     float f = 1.f;
-    if (b > 0 && __any_sync(0xffffffffu, raise)) {       // tensor-memory accesses are warp-wide: lanes that stay use f = 1
-      if (ok && !mbar_wait_err(smem_u32(&ctl->pv_done[(blk - 1) & 1u]), ((blk - 1) >> 1) & 1u, err)) { ok = false; atomicCAS((int *)err, 0, DEV_TIMEOUT_TMEM); }
-      tc_fence_after();
+    if (b > grp && __any_sync(0xffffffffu, raise)) {     // tensor-memory accesses are warp-wide: lanes that stay use f = 1
       if (raise) f = ex2_approx(m_old - ref);            // exp2(-inf) = 0: nothing was summed before the first finite maximum
 #pragma unroll
       for (int i = 0; i < HD / 32; ++i) {
         uint32_t r0[16], r1[16];
-        tmem_ld16(tq + kColO + i * 32, r0);
-        tmem_ld16(tq + kColO + i * 32 + 16, r1);
+        tmem_ld16(colO + i * 32, r0);
+        tmem_ld16(colO + i * 32 + 16, r1);
         tmem_wait_ld();
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           r0[e] = __float_as_uint(__uint_as_float(r0[e]) * f);
           r1[e] = __float_as_uint(__uint_as_float(r1[e]) * f);
         }
-        tmem_st16(tq + kColO + i * 32, r0);
-        tmem_st16(tq + kColO + i * 32 + 16, r1);
+        tmem_st16(colO + i * 32, r0);
+        tmem_st16(colO + i * 32 + 16, r1);
       }
     }
-    l_run = l_run * f + (sum0 + sum1);
-    tmem_st16(tq + kColP + buf * 32, pk0);
-    tmem_st16(tq + kColP + buf * 32 + 16, pk1);
-    tmem_st16(tq + kColPL + buf * 32, pl0);
-    tmem_st16(tq + kColPL + buf * 32 + 16, pl1);
+    const float2 scale2 = make_float2(scale, scale), nref2 = make_float2(-ref, -ref), minus1 = make_float2(-1.f, -1.f);
+    float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {   // 32 scores at a time: 16 columns of values, 16 of remainders
+      uint32_t pk[16], pl[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        float2 x = fma2(make_float2(sc[32 * hh + 2 * e], sc[32 * hh + 2 * e + 1]), scale2, nref2);
+        x.x = ex2_approx(x.x);
+        x.y = ex2_approx(x.y);
+        if (e & 1) sum1 = add2(sum1, x);
+        else sum0 = add2(sum0, x);
+        const __half2 h = __floats2half2_rn(x.x, x.y);
+        pk[e] = *reinterpret_cast<const uint32_t *>(&h);
+        const float2 rest = fma2(__half22float2(h), minus1, x);   // x - h, exact
+        pl[e] = pack_h2(rest.x, rest.y);
+      }
+      tmem_st16(colS + 16 * hh, pk);
+      tmem_st16(colS + 32 + 16 * hh, pl);
+    }
+    sum0 = add2(sum0, sum1);
+    l_run = l_run * f + (sum0.x + sum0.y);
     tmem_wait_st();
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&ctl->p_full[buf]));
+    if (lane == 0) mbar_arrive(smem_u32(&ctl->p_full[grp]));
     // (no CTA-wide barrier per block: a failed wait has set the error word, which ends every other wait)
   }
-  // the unit's last product (and with it every earlier one)
-  if (ok && !mbar_wait_err(smem_u32(&ctl->pv_done[(blk - 1) & 1u]), ((blk - 1) >> 1) & 1u, err)) { ok = false; atomicCAS((int *)err, 0, DEV_TIMEOUT_TMEM); }
+  // the group's last product; its earlier ones are known complete (see above), so a parity wait is enough
+  const bool any = t.nblk > grp;
+  if (any && ok && !mbar_wait_err(smem_u32(&ctl->pv_done[grp]), (cnt - 1) & 1, err)) { ok = false; atomicCAS((int *)err, 0, DEV_TIMEOUT_TMEM); }
   tc_fence_after();
+  ctl->ml[grp][row] = make_float2(m_ref, l_run);
+  tc_fence_before();
   if (!worker_all(ok)) return false;
+  tc_fence_after();
 
-  // ---- partial result of this split: un-normalised output, its reference maximum (log2 domain), sum -------
+  // ---- partial result of this unit: un-normalised output, its reference maximum (log2 domain), sum.  Each thread puts
+  // half of its row's output together from both groups' sums.
   {
-    float *dst = a.attn_o + ob * HD;
-    if (valid) a.attn_ml[ob] = make_float2(m_ref, l_run);
+    const float2 m0 = ctl->ml[0][row], m1 = ctl->ml[1][row];
+    const float m = fmaxf(m0.x, m1.x);
+    const float w0 = m0.x == -INFINITY ? 0.f : ex2_approx(m0.x - m), w1 = m1.x == -INFINITY ? 0.f : ex2_approx(m1.x - m);
+    float *dst = a.attn_o + ob * HD + grp * (HD / 2);
+    if (valid && grp == 0) a.attn_ml[ob] = make_float2(m, m0.y * w0 + m1.y * w1);
+    const uint32_t src = tq + kColO + grp * (HD / 2);
+    const bool both = t.nblk > 1;   // (else group 1's sums were never started)
 #pragma unroll
     for (int i = 0; i < HD / 32; ++i) {
       uint32_t r0[16], r1[16];
-      tmem_ld16(tq + kColO + i * 32, r0);      // (warp-wide: rows past the tile's end read too, and write nothing)
-      tmem_ld16(tq + kColO + i * 32 + 16, r1);
+      tmem_ld16(src + i * 16, r0);      // (warp-wide: rows past the tile's end read too, and write nothing)
+      if (both) tmem_ld16(src + 128 + i * 16, r1);
       tmem_wait_ld();
+#pragma unroll
+      for (int e = 0; e < 16; ++e)
+        r0[e] = __float_as_uint(__uint_as_float(r0[e]) * w0 + (both ? __uint_as_float(r1[e]) * w1 : 0.f));
       if (valid) {   // whole 32-byte sectors per lane: the lanes of a warp write 32 different rows
-        st_global_v8(dst + i * 32, r0);
-        st_global_v8(dst + i * 32 + 8, r0 + 8);
-        st_global_v8(dst + i * 32 + 16, r1);
-        st_global_v8(dst + i * 32 + 24, r1 + 8);
+        st_global_v8(dst + i * 16, r0);
+        st_global_v8(dst + i * 16 + 8, r0 + 8);
       }
     }
   }
-  // the output sums are in registers / on their way to memory: the next unit's first product may overwrite them, and
-  // its queries may be written over this unit's (every score product of this unit has completed)
-  tc_fence_before();
-  __syncwarp();
-  if (lane == 0) mbar_arrive(smem_u32(&ctl->o_free));
+  // (The output sums are in registers / on their way to memory; the next unit's first products, which overwrite them, wait
+  // for its queries, which this warp stages next.)
   return true;
 }
 
@@ -344,15 +362,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&ctl->s_full[b]), 1);
-      mbar_init(smem_u32(&ctl->s_empty[b]), 4);
       mbar_init(smem_u32(&ctl->p_full[b]), 4);
       mbar_init(smem_u32(&ctl->pv_done[b]), 1);
     }
-    mbar_init(smem_u32(&ctl->q_full), 1);
-    mbar_init(smem_u32(&ctl->o_free), 4);   // one arrival per worker warp
+    mbar_init(smem_u32(&ctl->q_full), kWorkerWarps);   // one arrival per worker warp
     fence_barrier_init();
   }
-  if (warp == 1) {
+  if (warp == kMmaWarp) {
     tmem_alloc(smem_u32(&ctl->tmem_base), 512);
     tmem_relinquish();
   }
@@ -367,7 +383,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
   // blocks (`gb`) and units (`un`) of the CTA.
   const int u_beg = a.cta_unit[blockIdx.x], u_end = a.cta_unit[blockIdx.x + 1];
 
-  if (warp == 0) {
+  if (warp == kProducerWarp) {
     // ---------------------------------------------------------------- K/V producer
     // (the whole warp walks the loops and the waits; an elected lane issues a block's sixteen copies -- a lone lane
     // in a divergent branch needs about 50 cycles per copy instruction, more than half of a block's time)
@@ -419,100 +435,99 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
         }
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == kMmaWarp) {
     // ---------------------------------------------------------------- MMA issue
-    // The whole warp walks the loops and the waits together; one elected lane issues each tensor-core instruction and
-    // each commit (the loop state is then the same in every lane, which lets the compiler keep descriptors and
-    // addresses in uniform registers: a lone lane issued an instruction every ~50 cycles, too slow for 20 small
-    // instructions per 64-position block).
+    // The whole warp walks the loops and the waits together; one elected lane issues a block's tensor-core instructions
+    // and commits (the loop state is then the same in every lane, which lets the compiler keep descriptors and addresses
+    // in uniform registers: a lone lane in a divergent branch issued an instruction every ~50 cycles).
     {
       const uint32_t idesc_qk = umma_idesc_f16(kAttnRows, kAttnBlk, 0);
       const uint32_t idesc_pv = umma_idesc_f16(kAttnRows, HD, 1);
       const uint32_t sKV = smem_u32(smem);
       bool ok = true;
-      uint32_t gb = 0, un = 0;
+      uint32_t gb = 0, un = 0, par = 0;   // par: bit g = parity of group g's blocks so far
       // a wait that ran out in one lane ends the loops of all lanes together (elect.sync names the full warp)
       auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, mbar_wait_err(bar, parity, err));
       };
-      // O (+)= P V for block bi; `first`: the unit's first block starts the sums afresh, which needs the workers to
-      // have read the previous unit's sums out
-      auto issue_pv = [&](uint32_t bi, bool first) -> bool {
-        const uint32_t pb = bi & 1, vst = bi % kKvStages;
-        if (!wait_all(smem_u32(&ctl->p_full[pb]), (bi >> 1) & 1)) return false;
-        if (first && un > 0 && !wait_all(smem_u32(&ctl->o_free), (un - 1) & 1)) return false;
-        tc_fence_after();
-        const uint32_t sV = sKV + vst * kKvBytes + kAttnBlk * HD * 2;
+      // S = Q K^T + Q_lo K^T for the CTA's block bi into group g's buffer: the remainder plane of the queries goes through
+      // the same keys into the same sums; the queries are read from tensor memory (8 columns = 16 elements per
+      // instruction).  The buffer is free: the product that read the group's previous probabilities was issued before.
+      auto qk = [&](uint32_t g, uint32_t bi) {
+        const uint64_t dk = umma_desc_sw128(sKV + (bi % kKvStages) * kKvBytes);
+        const uint32_t colS = tmem_base + kColS + g * 64;
 #pragma unroll
-        for (int ks = 0; ks < kAttnBlk / 16; ++ks) {   // 16 positions per instruction: values, then remainders
-          if (elect_one())
-            umma_f16_ts(tmem_base + kColO, tmem_base + kColP + pb * 32 + ks * 8,
-                        umma_desc_sw128_mn(sV + ks * 2048, kAttnBlk * 128), idesc_pv, (!first || ks != 0) ? 1u : 0u);
-          if (elect_one())
-            umma_f16_ts(tmem_base + kColO, tmem_base + kColPL + pb * 32 + ks * 8,
-                        umma_desc_sw128_mn(sV + ks * 2048, kAttnBlk * 128), idesc_pv, 1u);
-        }
-        if (elect_one()) {
-          umma_commit(smem_u32(&ctl->pv_done[pb]));
-          umma_commit(smem_u32(&ctl->kv_empty[vst]));
-        }
-        __syncwarp();
-        return true;
-      };
-      // S = Q K^T + Q_lo K^T for block g (counted over the CTA's blocks): the remainder plane of the queries goes
-      // through the same keys into the same sums; the queries are read from tensor memory (8 columns = 16 elements
-      // per instruction)
-      auto issue_qk = [&](uint32_t g) -> bool {
-        const uint32_t kst = g % kKvStages, st = g & 1;
-        if (!wait_all(smem_u32(&ctl->kv_full[kst]), (g / kKvStages) & 1)) return false;
-        if (!wait_all(smem_u32(&ctl->s_empty[st]), ((g >> 1) & 1) ^ 1)) return false;
-        tc_fence_after();
-        const uint32_t sK = sKV + kst * kKvBytes;
+        for (int pl = 0; pl < 2; ++pl)
 #pragma unroll
-        for (int pl = 0; pl < 2; ++pl) {
-#pragma unroll
-          for (int hh = 0; hh < (int)kHalves; ++hh) {
-            const uint64_t dk = umma_desc_sw128(sK + hh * (kAttnBlk * 128));
+          for (int hh = 0; hh < (int)kHalves; ++hh)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              if (elect_one())
-                umma_f16_ts(tmem_base + kColS + st * 64, tmem_base + kColQ + pl * (HD / 2) + hh * 32 + kk * 8, dk + 2 * kk,
-                            idesc_qk, (pl | hh | kk) != 0 ? 1u : 0u);
-          }
-        }
-        if (elect_one()) umma_commit(smem_u32(&ctl->s_full[st]));
-        __syncwarp();
-        return true;
+              umma_f16_ts(colS, tmem_base + kColQ + pl * (HD / 2) + hh * 32 + kk * 8, dk + hh * (kAttnBlk * 128 / 16) + 2 * kk,
+                          idesc_qk, (pl | hh | kk) != 0 ? 1u : 0u);
+        umma_commit(smem_u32(&ctl->s_full[g]));
       };
-      // Issue order within a unit: S(0), then for every block b: S(b + 1), O += P(b) V(b).  The scores run one block
-      // ahead of the block the workers are on, so a worker finds its scores complete when it gets to them, and the
-      // product of block b waits only for that block's probabilities.
+      // O (+)= P V for block b of the unit, the CTA's block bi; a group's first block of a unit starts its sums afresh
+      auto pv = [&](int b, uint32_t bi) {
+        const uint32_t vst = bi % kKvStages, g = b & 1;
+        const uint32_t colO = tmem_base + kColO + g * 128, colP = tmem_base + kColS + g * 64;
+        const uint64_t dv = umma_desc_sw128_mn(sKV + vst * kKvBytes + kAttnBlk * HD * 2, kAttnBlk * 128);
+#pragma unroll
+        for (int ks = 0; ks < kAttnBlk / 16; ++ks) {   // 16 positions per instruction: values, then remainders
+          umma_f16_ts(colO, colP + ks * 8, dv + ks * (2048 / 16), idesc_pv, (b > 1 || ks != 0) ? 1u : 0u);
+          umma_f16_ts(colO, colP + 32 + ks * 8, dv + ks * (2048 / 16), idesc_pv, 1u);
+        }
+        umma_commit(smem_u32(&ctl->pv_done[g]));
+        umma_commit(smem_u32(&ctl->kv_empty[vst]));
+      };
+      auto wait_kv = [&](uint32_t bi) { return wait_all(smem_u32(&ctl->kv_full[bi % kKvStages]), (bi / kKvStages) & 1); };
+      // Issue order within a unit: S(0), S(1), then for every block b: O += P(b) V(b), S(b + 2).  While one group works
+      // on its scores the other's products run.
       for (int u = u_beg; u < u_end && ok; ++u) {
         const UnitInfo t = attn_unit_info(a, u);
         if (t.nblk == 0) continue;
-        ok = wait_all(smem_u32(&ctl->q_full), un & 1);
-        if (ok) ok = issue_qk(gb);
-        for (int b = 0; ok && b < t.nblk; ++b, ++gb) {
-          if (b + 1 < t.nblk) ok = issue_qk(gb + 1);
-          if (ok) ok = issue_pv(gb, b == 0);
-        }
+        ok = wait_all(smem_u32(&ctl->q_full), un & 1) && wait_kv(gb);
         ++un;
+        tc_fence_after();
+        if (ok && elect_one()) qk(0, gb);
+        __syncwarp();
+        if (ok && t.nblk > 1) {
+          ok = wait_kv(gb + 1);
+          tc_fence_after();
+          if (ok && elect_one()) qk(1, gb + 1);
+          __syncwarp();
+        }
+        for (int b = 0; ok && b < t.nblk; ++b, ++gb) {
+          // (the keys of block b + 2 first: they are long there, and nothing comes between the block's products then)
+          const bool more = b + 2 < t.nblk;
+          // (both barriers are looked at together: what this warp does between two issues leaves the tensor cores idle)
+          const uint32_t kv2 = gb + (more ? 2 : 0), bar_kv = smem_u32(&ctl->kv_full[kv2 % kKvStages]), par_kv = (kv2 / kKvStages) & 1;
+          const uint32_t bar_p = smem_u32(&ctl->p_full[b & 1]), par_p = (par >> (b & 1)) & 1;
+          if (!__all_sync(0xffffffffu, mbar_try_wait(bar_kv, par_kv) & mbar_try_wait(bar_p, par_p)))
+            ok = wait_all(bar_kv, par_kv) && wait_all(bar_p, par_p);
+          par ^= 1u << (b & 1);
+          tc_fence_after();
+          if (ok && elect_one()) {
+            pv(b, gb);
+            if (more) qk(b & 1, gb + 2);
+          }
+          __syncwarp();
+        }
       }
       if (!ok && lane == 0) atomicCAS(a.err, 0, DEV_TIMEOUT_FULL);
     }
   } else {
     // ---------------------------------------------------------------- workers
-    uint32_t blk = 0;
+    uint32_t cnt = 0;
     bool ok = true, waited = false;
     for (int u = u_beg; u < u_end && ok; ++u) {
       const UnitInfo t = attn_unit_info(a, u);
-      ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp & 3, lane, (int)threadIdx.x - kWorkerWarp0 * 32, blk, waited, err);
+      ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp >> 2, warp & 3, lane, cnt, waited, err);
     }
     if (!waited) pdl_wait();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (warp == kMmaWarp) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }
