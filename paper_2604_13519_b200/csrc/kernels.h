@@ -191,11 +191,13 @@ cudaError_t launch_sample_accept(const SampleArgs &a, cudaStream_t st);
 // Cosine Top-K over datastore hidden states (retrieval.cu).  scores: [N + 2K] floats; the result pairs (index as int
 // bits, score), best first, follow the N scores.  The query is q_dev (fp32 [d]) or, if null, bf16 planes of a row.
 cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float *q_dev, const __nv_bfloat16 *q_planes,
-                               int plane_stride, int planes, int K, float *scores, cudaStream_t st);
+                               int plane_stride, int planes, int K, float *scores, int n_sms, float *out_host, int *err, cudaStream_t st);
 
 // Row-wise Top-K (topk.cu): out[r][j] = (column as int bits, value) of the j-th largest entry of row r, lowest column
 // on ties.  cand: scratch of n_rows * ceil(n_cols / 4096) * K pairs.
-cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, cudaStream_t st);
+// out_host (one row, may be null): the same pairs to host memory that the device can write, and behind them the status word *err.
+cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, float *out_host,
+                             const int *err, cudaStream_t st);
 
 // After a tree step: move the K/V rows of the accepted path to consecutive cache positions len, len+1, ...
 struct CompactArgs {

@@ -192,7 +192,7 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->max_stamps = 9 * c.n_layers + 16;
   L->stamps = take((uint64_t)L->max_stamps * 4 * 8);
   L->workspace_bytes = o;
-  L->host_io_bytes = align_up((uint64_t)(L->in_ints + L->out_ints) * 4, 4096);
+  L->host_io_bytes = align_up((uint64_t)(L->in_ints + L->out_ints + 2 * 64 + 1) * 4, 4096);   // (and a retrieval's result pairs and status)
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -235,6 +235,7 @@ struct ts_model {
   bool have_step = false;
   int64_t launches = 0, h2d = 0, d2h = 0;
   bool use_pdl = true;
+  int32_t *host_dev = nullptr;                 // the pinned block as the device sees it (null: it cannot write there)
   int32_t inject_err = 0;                      // test support: status code the next step is made to report
   bool fused_ok = false, last_fused = false;   // device can run the fused kernel; the staged step uses it
   bool last_tree = false;                      // the staged step verifies a draft tree (not a chain)
@@ -593,7 +594,7 @@ ts_status run_step(ts_model *m) {
   int32_t *dout = m->d_out();
   if (m->last_flags & TS_FLAG_WANT_TOPK) {   // per-position Top-K of the logits, for the successor tables
     CU_TRY(ts::launch_topk_rows((const float *)m->WS(L.logits), M, c.vocab, TS_TOPK, (float2 *)m->WS(L.topk_cand),
-                                (float *)(dout + L.o_topk), m->st));
+                                (float *)(dout + L.o_topk), nullptr, nullptr, m->st));
     m->launched(5);
     m->launched(5);
   }
@@ -995,6 +996,11 @@ ts_status ts_init_model(const ts_model_config *cfg, const ts_buffers *bufs, void
   m->planes = cfg->act_split ? 2 : 1;
   m->n_sms = prop.multiProcessorCount;
   make_layout(*cfg, &m->L);
+  {
+    void *p = nullptr;
+    if (cudaHostGetDevicePointer(&p, bufs->host_io, 0) == cudaSuccess) m->host_dev = (int32_t *)p;
+    cudaGetLastError();
+  }
   const Layout &L = m->L;
   const ts_model_config &c = m->c;
   auto bail = [&](ts_status s) { delete m; return s; };
@@ -1801,11 +1807,22 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
     if (row < 0 || row >= m->last_M) return fail(TS_ERR_ARG, "row outside the last step");
     planes = (const __nv_bfloat16 *)m->WS(m->L.h) + (size_t)row * m->c.d_model;
   }
+  // the result pairs go straight to the pinned block where the device can write it, else by a copy
+  float *res = (float *)(m->h_out() + m->L.out_ints);
+  float *res_dev = m->host_dev ? (float *)(m->host_dev + m->L.in_ints + m->L.out_ints) : nullptr;
   CU_TRY(ts::launch_topk_cosine((const __nv_bfloat16 *)hidden_dev, n_entries, m->c.d_model, query_dev, planes,
-                                (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->st));
-  std::vector<float> res(2 * (size_t)K);
-  CU_TRY(cudaMemcpyAsync(res.data(), scores_dev + n_entries, res.size() * 4, cudaMemcpyDeviceToHost, m->st));
+                                (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms, res_dev, m->d_out() + m->L.o_err, m->st));
+  if (!res_dev) {
+    CU_TRY(cudaMemcpyAsync(res, scores_dev + n_entries, 2 * (size_t)K * 4, cudaMemcpyDeviceToHost, m->st));
+    CU_TRY(cudaMemcpyAsync(res + 2 * K, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));
+  }
   CU_TRY(cudaStreamSynchronize(m->st));
+  int dev_err;
+  std::memcpy(&dev_err, res + 2 * K, 4);
+  if (dev_err != 0) {
+    cudaMemsetAsync(m->d_out() + m->L.o_err, 0, 4, m->st);
+    return fail(TS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired (code %d)", dev_err);
+  }
   for (int j = 0; j < K; ++j) {
     int32_t idx;
     std::memcpy(&idx, &res[2 * j], 4);

@@ -45,6 +45,28 @@ def test_topk_matches_oracle(n, d, K):
     gm.close()
 
 
+@pytest.mark.parametrize("n,d,K", [(1, 256, 1), (33, 4096, 33), (4095, 2048, 1), (4097, 256, 64), (9473, 4096, 64), (1050001, 256, 64)])
+def test_topk_at_the_edges_of_pieces_slices_and_lists(n, d, K):
+    """One entry; an odd last pair; one score less and one more than a slice of 4096; as many winners as a list holds;
+    more slices than the last kernel has threads.  Equal scores (copies of one entry, far apart) keep their order."""
+    shape = synth.SHAPES[{256: "tiny", 2048: "1b-2l", 4096: "8b-2l"}[d]]
+    g = torch.Generator().manual_seed(n)
+    H = torch.randn(n, d, generator=g).to(torch.bfloat16)
+    q = torch.randn(d, generator=g)
+    for j in (0, n // 2, n - 1):
+        H[j] = q.to(torch.bfloat16)
+    gm = ts.Model(shape, max_pages=8, max_batch=1, k_max=8, max_rows=8, max_ctx=64, act_split=True, path=1)
+    idx, sc = ts.ts_topk_cosine(gm, H.cuda(), K, query=q.cuda())
+    s_all = oracle.cosine_scores(H, q)
+    want = torch.topk(s_all, K).values.numpy()
+    # fp32 sums of d products of size about 1/d against float64: d^0.5 * 2^-24 of the norms, times a few
+    assert np.abs(np.array(sc) - want).max() < 2e-6
+    assert np.abs(s_all[torch.tensor(idx)].numpy() - want).max() < 4e-6 and len(set(idx)) == K
+    same = sorted({0, n // 2, n - 1})
+    assert idx[:min(K, len(same))] == same[:K]
+    gm.close()
+
+
 def test_query_from_the_last_step_is_the_final_hidden_state():
     shape = synth.SHAPES["8b-2l"]
     om, gm = make_pair(shape, k_max=8, max_ctx=256, path=1)
