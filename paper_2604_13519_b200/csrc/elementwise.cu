@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(64)
 accept_kernel(AcceptArgs a) {
   pdl_launch_dependents();   // the dependent kernel waits for this one's end before touching its data
   pdl_wait();
+  __shared__ int sh_l;
   const int seq = blockIdx.x;
   const int r0 = a.in.cu_rows[seq], r1 = a.in.cu_rows[seq + 1];
   for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
@@ -347,7 +348,10 @@ accept_kernel(AcceptArgs a) {
     em[l] = a.argmax[r0 + u];
     a.new_len[seq] = a.in.seq_len[seq] + l + 1;   // rejected rows stay in their pages, uncounted
     a.new_pending[seq] = a.argmax[r0 + u];
+    sh_l = l;
   }
+  __syncthreads();
+  publish(a, seq, r0, r1 - r0, sh_l);
 }
 
 // grid = (B, layers, kv heads), hd threads.  Path entry j (chunk row path[j]) moves from cache slot len + path[j]

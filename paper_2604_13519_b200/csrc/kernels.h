@@ -160,6 +160,15 @@ struct AttnTcArgs {
 cudaError_t launch_attention_tc(const AttnTcArgs &a, cudaStream_t st);
 cudaError_t launch_attention_tc_merge(const AttnTcArgs &a, cudaStream_t st);
 
+// A step's results straight to the host: the acceptance kernels write the words of the result block that the host reads to
+// pinned memory as well, so that no copy follows them (base: the block on the device, host: the same block as the device
+// sees the pinned one; host null: not wanted).
+struct HostOut {
+  const int32_t *base;
+  int32_t *host;
+  const int *err;   // status word, published too
+};
+
 // per-row argmax over the LM-head tiles, longest accepted prefix per sequence, new lengths
 struct AcceptArgs {
   StepIn in;
@@ -171,22 +180,45 @@ struct AcceptArgs {
   int32_t *new_pending;    // [B]
   int32_t *path;           // [B][k_max] chunk rows of the accepted path, root first (accept_len + 1 entries)
   int k_max;
+  HostOut ho;
 };
 cudaError_t launch_accept(const AcceptArgs &a, cudaStream_t st);
 
+constexpr int kSampleSlices = 32;   // slices of a row whose sums of weights are kept
 // Speculative-sampling acceptance (sampling.cu): per-row softmax statistics, accept tests, the step's one sample.
 struct SampleArgs {
   StepIn in;
   float *logits;                    // [M][V] (refused tokens are masked for the draw and restored)
   const unsigned long long *amax;   // [M] packed per-row maxima (argmax is still reported)
   const float *uni;                 // [M] uniforms in [0, 1): row c of a chunk decides node c, the root row's draws the sample
-  float *part;                      // [M][16] scratch: per-slice sums of exp((l - max) / T)
+  float *part;                      // [M][kSampleSlices] scratch: per-slice sums of exp((l - max) / T)
   int V;
   float inv_t;                      // 1 / temperature
   int32_t *argmax, *accept_len, *emitted, *new_len, *new_pending, *path;
   int k_max;
+  HostOut ho;
 };
 cudaError_t launch_sample_accept(const SampleArgs &a, cudaStream_t st);
+
+#ifdef __CUDACC__
+// the results of sequence `seq` (rows r0 .. r0 + k, accepted length l) by the whole CTA, after a barrier
+template <typename Args>
+__device__ __forceinline__ void publish(const Args &a, int seq, int r0, int k, int l) {
+  if (!a.ho.host) return;
+  auto put = [&](const int32_t *p) { a.ho.host[p - a.ho.base] = *p; };
+  for (int i = threadIdx.x; i < k; i += blockDim.x) put(a.argmax + r0 + i);
+  for (int i = threadIdx.x; i <= l; i += blockDim.x) {
+    put(a.emitted + (size_t)seq * a.k_max + i);
+    put(a.path + (size_t)seq * a.k_max + i);
+  }
+  if (threadIdx.x == 0) {
+    put(a.accept_len + seq);
+    put(a.new_len + seq);
+    put(a.new_pending + seq);
+    if (seq == 0) put(a.ho.err);
+  }
+}
+#endif
 
 // Cosine Top-K over datastore hidden states (retrieval.cu).  scores: [N + 2K] floats; the result pairs (index as int
 // bits, score), best first, follow the N scores.  The query is q_dev (fp32 [d]) or, if null, bf16 planes of a row.

@@ -151,7 +151,7 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->act = take(planes * R * F * 2);
   L->logits = take(Rs * V * 4);
   L->amax = take(R * 8);
-  L->samp_stats = take(Rs * 16 * 4);
+  L->samp_stats = take(Rs * ts::kSampleSlices * 4);
   L->topk_cand = take(Rs * (uint64_t)((c.vocab + 4095) / 4096) * TS_TOPK * 8);
   L->rope = take((uint64_t)c.max_ctx * (hd / 2) * 8);
   int io = 0;
@@ -235,6 +235,7 @@ struct ts_model {
   bool have_step = false;
   int64_t launches = 0, h2d = 0, d2h = 0;
   bool use_pdl = true;
+  bool publish = false;                        // the step being enqueued writes its results to the pinned block itself
   int32_t *host_dev = nullptr;                 // the pinned block as the device sees it (null: it cannot write there)
   int32_t inject_err = 0;                      // test support: status code the next step is made to report
   bool fused_ok = false, last_fused = false;   // device can run the fused kernel; the staged step uses it
@@ -598,6 +599,8 @@ ts_status run_step(ts_model *m) {
     m->launched(5);
     m->launched(5);
   }
+  ts::HostOut ho{};
+  if (m->publish) { ho.base = dout; ho.host = m->host_dev + L.in_ints; ho.err = dout + L.o_err; }
   if (m->last_sample) {
     ts::SampleArgs sa{};
     sa.in = in; sa.logits = (float *)m->WS(L.logits); sa.amax = amax;
@@ -605,6 +608,7 @@ ts_status run_step(ts_model *m) {
     sa.V = c.vocab; sa.inv_t = m->last_inv_t; sa.k_max = c.k_max;
     sa.argmax = dout + L.o_argmax; sa.accept_len = dout + L.o_accept; sa.emitted = dout + L.o_emitted;
     sa.new_len = dout + L.o_newlen; sa.new_pending = dout + L.o_newpend; sa.path = dout + L.o_path;
+    sa.ho = ho;
     CU_TRY(ts::launch_sample_accept(sa, m->st));
     m->launched(5);
     m->launched(5);
@@ -614,6 +618,7 @@ ts_status run_step(ts_model *m) {
     ac.argmax = dout + L.o_argmax; ac.accept_len = dout + L.o_accept; ac.emitted = dout + L.o_emitted;
     ac.new_len = dout + L.o_newlen; ac.new_pending = dout + L.o_newpend; ac.k_max = c.k_max;
     ac.path = dout + L.o_path;
+    ac.ho = ho;
     CU_TRY(ts::launch_accept(ac, m->st));
     m->launched(5);
   }
@@ -776,7 +781,17 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const size_t in_bytes = (m->last_units_at + (size_t)m->h_in()[L.o_cta_unit + m->last_ctas] * (sizeof(ts::AttnWork) / 4)) * 4;
   CU_TRY(cudaMemcpyAsync(m->d_in(), m->h_in(), in_bytes, cudaMemcpyHostToDevice, m->st));
   m->h2d += (int64_t)in_bytes;
+  // A step that ends in an acceptance kernel (and maybe the cache's compaction) publishes its results itself; prompts, the
+  // persistent kernel, per-position Top-K lists and an injected status word take a copy, as does the debug build, whose
+  // checks go on in the compaction.
+#ifdef TS_DEBUG_BOUNDS
+  const bool publishes = false;
+#else
+  const bool publishes = m->host_dev && !m->last_fused && !m->inject_err && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
+#endif
+  m->publish = publishes;
   ts_status st = run_step(m);
+  m->publish = false;
   if (st) return st;
   if (m->inject_err) {
     // test support (ts_debug_inject_device_error): after the step's last kernel, write the status word an expired
@@ -786,7 +801,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
     CU_TRY(cudaMemcpyAsync(m->d_out() + L.o_err, m->h_out() + L.o_err + 1, 4, cudaMemcpyHostToDevice, m->st));
   }
   const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
-  CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
+  if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
   m->d2h += (int64_t)out_bytes;
   CU_TRY(cudaStreamSynchronize(m->st));
   const int dev_err = m->h_out()[L.o_err];

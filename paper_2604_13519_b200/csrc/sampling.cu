@@ -11,13 +11,31 @@
 namespace ts {
 
 static constexpr int kStatThreads = 256;
-static constexpr int kStatSlices = 16;        // CTAs per row in the statistics kernel
-static constexpr int kSampleThreads = 1024;   // 32 warps: one contiguous stretch of the vocabulary each
+static constexpr int kStatSlices = kSampleSlices;   // slices a row's statistics are kept in, a warp's lane each in the draw
+static constexpr int kSampleThreads = 512;
+
+// ids per slice: a multiple of 128, like V
+__device__ __forceinline__ int slice_len(int V) { return (V / 128 + kStatSlices - 1) / kStatSlices * 128; }
 
 // the row maximum, from the packed (ordered value bits, ~id) word the LM-head epilogue reduced
 __device__ __forceinline__ float row_max_of(unsigned long long word) {
   const uint32_t u = (uint32_t)(word >> 32);
   return __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
+}
+
+__device__ __forceinline__ float4 weights4(const float *row, int i, float mx, float inv_t) {
+  const float4 v = __ldcg(reinterpret_cast<const float4 *>(row + i));
+  return make_float4(__expf((v.x - mx) * inv_t), __expf((v.y - mx) * inv_t), __expf((v.z - mx) * inv_t), __expf((v.w - mx) * inv_t));
+}
+
+// sum of v over a CTA of at most 32 warps, in every thread
+__device__ __forceinline__ float cta_sum(float v, float *red) {
+  v = warp_sum(v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  return warp_sum(lane < (int)(blockDim.x >> 5) ? red[lane] : 0.f);
 }
 
 // grid = (rows, slices): sum of exp((l - max) / T) over one slice of one row
@@ -29,35 +47,32 @@ row_expsum_kernel(const float *logits, const unsigned long long *amax, int V, fl
   const int r = blockIdx.x, sl = blockIdx.y;
   const float *row = logits + (size_t)r * V;
   const float mx = row_max_of(amax[r]);
-  const int per = (V + kStatSlices - 1) / kStatSlices;
-  const int i0 = sl * per, i1 = min(V, i0 + per);
+  const int per = slice_len(V), i0 = sl * per, i1 = min(V, i0 + per);
   float sum = 0.f;
-  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) sum += __expf((row[i] - mx) * inv_t);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < kStatThreads / 32; ++w) t += red[w];
-    part[(size_t)r * kStatSlices + sl] = t;
+#pragma unroll 4
+  for (int i = i0 + 4 * threadIdx.x; i < i1; i += 4 * kStatThreads) {
+    const float4 w = weights4(row, i, mx, inv_t);
+    sum += (w.x + w.y) + (w.z + w.w);
   }
+  sum = cta_sum(sum, red);
+  if (threadIdx.x == 0) part[(size_t)r * kStatSlices + sl] = sum;
 }
 
 // grid = sequences.  The chunk is a draft tree (a chain is the tree with parents j - 1).  Thread c < k computes the
 // weight of node c's token under its parent's row; thread 0 then walks from the root: the children of a node are
 // tried in node order against the residual (the parent's weights with the tokens of refused children removed),
 // child c accepted iff uni[c] * residual total < its weight.  Where the walk ends the block draws the step's one
-// sample from the residual with uni[root]: the refused tokens' logits are set to -inf for the draw and put back
-// afterwards; warp w owns ids [w * S, (w + 1) * S), read 32 at a time; the running sum goes warp by warp, then group
-// of 32 by group, then lane by lane, so it is non-decreasing in the id and the first id above the target is found.
+// sample from the residual with uni[root]: the refused tokens' logits are set to -inf for the draw (their slices' sums are
+// taken again) and put back afterwards.  The running sum goes slice by slice over the sums the statistics kernel left,
+// and through the one slice in which it passes the target id by id: only that slice of the row is read again (reading the
+// whole row twice with one CTA took 39 us of a step on 128 256 ids, this 14).
 __global__ void __launch_bounds__(kSampleThreads)
 sample_accept_kernel(SampleArgs a) {
-  __shared__ float seg_total[kSampleThreads / 32];
+  __shared__ float red[kSampleThreads / 32], slice_sum[kStatSlices], warp_tot[kSampleThreads / 32];
   __shared__ float w_node[64], tot_node[64];
   __shared__ int refused[64];
   __shared__ float refused_logit[64];
-  __shared__ int sh_l, sh_last, sh_nref, sh_tok;
+  __shared__ int sh_l, sh_last, sh_nref, sh_tok, sh_lastw;
   pdl_launch_dependents();
   pdl_wait();
   const int seq = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -65,12 +80,12 @@ sample_accept_kernel(SampleArgs a) {
   int32_t *path = a.path + (size_t)seq * a.k_max;
   for (int r = r0 + threadIdx.x; r < r0 + k; r += blockDim.x)
     a.argmax[r] = (int32_t)(0xFFFFFFFFu - (uint32_t)(a.amax[r] & 0xFFFFFFFFull));
+  for (int c = warp; c < k; c += kSampleThreads / 32) {
+    const float tot = warp_sum(a.part[(size_t)(r0 + c) * kStatSlices + lane]);   // total weight of node c's own row
+    if (lane == 0) tot_node[c] = tot;
+  }
   if ((int)threadIdx.x < k) {
-    const int c = threadIdx.x;
-    float tot = 0.f;
-    for (int s = 0; s < kStatSlices; ++s) tot += a.part[(size_t)(r0 + c) * kStatSlices + s];
-    tot_node[c] = tot;                                   // total weight of node c's own row
-    const int par = a.in.parent[r0 + c];
+    const int c = threadIdx.x, par = a.in.parent[r0 + c];
     w_node[c] = par < 0 ? 0.f
                         : __expf((a.logits[(size_t)(r0 + par) * a.V + a.in.tokens[r0 + c]] - row_max_of(a.amax[r0 + par])) * a.inv_t);
   }
@@ -92,58 +107,86 @@ sample_accept_kernel(SampleArgs a) {
       v = nxt;
       path[++l] = v;
     }
-    sh_l = l; sh_last = v; sh_nref = nref; sh_tok = -1;
+    sh_l = l; sh_last = v; sh_nref = nref; sh_tok = -1; sh_lastw = -1;
     // the refused tokens leave the row for the draw
     float *row_w = a.logits + (size_t)(r0 + v) * a.V;
     for (int i = 0; i < nref; ++i) { refused_logit[i] = row_w[refused[i]]; row_w[refused[i]] = -INFINITY; }
     __threadfence_block();
   }
   __syncthreads();
-  const int l = sh_l, last = sh_last;
+  const int l = sh_l, last = sh_last, nref = sh_nref;
   const float *row = a.logits + (size_t)(r0 + last) * a.V;
   const float mx = row_max_of(a.amax[r0 + last]);
-  const int S = ((a.V + kSampleThreads - 1) / kSampleThreads) * 32;   // ids per warp, a multiple of 32
-  const int i0 = warp * S, i1 = min(a.V, i0 + S);
-  auto weight = [&](int i) { return i < i1 ? __expf((__ldcg(row + i) - mx) * a.inv_t) : 0.f; };
-  float part = 0.f;
-  for (int i = i0 + lane; i < i1; i += 32) part += weight(i);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if (lane == 0) seg_total[warp] = part;
+  const int per = slice_len(a.V);
+  if (threadIdx.x < kStatSlices) slice_sum[threadIdx.x] = a.part[(size_t)(r0 + last) * kStatSlices + threadIdx.x];
   __syncthreads();
-  float before = 0.f, total = 0.f;
-  for (int w = 0; w < kSampleThreads / 32; ++w) {
-    if (w < warp) before += seg_total[w];
-    total += seg_total[w];
+  for (int i = 0; i < nref; ++i) {   // (a slice with several refused tokens is taken again for the first of them)
+    const int sl = refused[i] / per;
+    bool seen = false;
+    for (int e = 0; e < i; ++e) seen |= refused[e] / per == sl;
+    if (seen) continue;
+    float sum = 0.f;
+    for (int id = sl * per + 4 * threadIdx.x; id < min(a.V, (sl + 1) * per); id += 4 * kSampleThreads) {
+      const float4 w = weights4(row, id, mx, a.inv_t);
+      sum += (w.x + w.y) + (w.z + w.w);
+    }
+    sum = cta_sum(sum, red);
+    if (threadIdx.x == 0) slice_sum[sl] = sum;
+    __syncthreads();
   }
+  float total = 0.f;
+  for (int s = 0; s < kStatSlices; ++s) total += slice_sum[s];
   const float target = a.uni[r0] * total;
-  if (before + seg_total[warp] > target && !(before > target)) {   // the running sum passes the target in this stretch
+  // the slice in which the running sum passes the target (none: rounding, or no weight at all)
+  float before = 0.f;
+  int sl = 0;
+  while (sl < kStatSlices && !(before + slice_sum[sl] > target)) before += slice_sum[sl++];
+  if (sl < kStatSlices) {
+    const int i1 = min(a.V, (sl + 1) * per);
     float run = before;
-    int tok = -1, lastw = -1;                          // lastw: the last id of the stretch that carries weight
-    for (int g0 = i0; g0 < i1 && tok < 0; g0 += 32) {
-      const float w = weight(g0 + lane);
-      float inc = w;                                   // inclusive prefix over the group's 32 lanes
+    bool done = false;
+    for (int b0 = sl * per; b0 < i1 && !done; b0 += 4 * kSampleThreads) {   // 2048 ids at a time, four neighbours per thread
+      const int id = b0 + 4 * threadIdx.x;
+      const float4 w = id < i1 ? weights4(row, id, mx, a.inv_t) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float c0 = w.x, c1 = c0 + w.y, c2 = c1 + w.z, c3 = c2 + w.w;
+      float inc = c3;                                  // inclusive prefix over the warp's threads
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const float t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
       }
-      const unsigned hit = __ballot_sync(0xffffffffu, run + inc > target && w > 0.f);
-      const unsigned any = __ballot_sync(0xffffffffu, w > 0.f);
-      if (any) lastw = g0 + 31 - __clz(any);
-      if (hit) tok = g0 + __ffs(hit) - 1;
-      run += __shfl_sync(0xffffffffu, inc, 31);
+      __syncthreads();
+      if (lane == 31) warp_tot[warp] = inc;
+      __syncthreads();
+      float base = run, sum = 0.f;
+      for (int v = 0; v < kSampleThreads / 32; ++v) {
+        if (v < warp) base += warp_tot[v];
+        sum += warp_tot[v];
+      }
+      const float ex = base + (inc - c3);
+      // this thread's first id past the target, and the last id that carries weight (the two summation orders may round
+      // apart by an ulp: then that one is taken)
+      const int hit = (ex + c0 > target && w.x > 0.f) ? id : (ex + c1 > target && w.y > 0.f) ? id + 1
+                      : (ex + c2 > target && w.z > 0.f) ? id + 2 : (ex + c3 > target && w.w > 0.f) ? id + 3 : 0x7FFFFFFF;
+      const int lw = w.w > 0.f ? id + 3 : w.z > 0.f ? id + 2 : w.y > 0.f ? id + 1 : w.x > 0.f ? id : -1;
+      const int first = __reduce_min_sync(0xffffffffu, hit), lastw = __reduce_max_sync(0xffffffffu, lw);
+      if (lane == 0) {
+        if (first != 0x7FFFFFFF) atomicMin((unsigned int *)&sh_tok, (unsigned int)first);   // (-1 = none yet)
+        atomicMax(&sh_lastw, lastw);
+      }
+      __syncthreads();
+      done = sh_tok >= 0;
+      run += sum;
     }
-    if (lane == 0) sh_tok = tok >= 0 ? tok : lastw;    // (the two summation orders may round apart by an ulp)
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int tok = sh_tok;
+    int tok = sh_tok >= 0 ? sh_tok : sh_lastw;
     if (tok < 0) {   // rounding kept every partial sum at or below the target: the last id that carries weight
       for (tok = a.V - 1; tok > 0 && !(__expf((row[tok] - mx) * a.inv_t) > 0.f); --tok) {}
     }
     float *row_w = a.logits + (size_t)(r0 + last) * a.V;
-    for (int i = 0; i < sh_nref; ++i) row_w[refused[i]] = refused_logit[i];   // the logits are an output: put them back
+    for (int i = 0; i < nref; ++i) row_w[refused[i]] = refused_logit[i];   // the logits are an output: put them back
     int32_t *em = a.emitted + (size_t)seq * a.k_max;
     for (int j = 1; j <= l; ++j) em[j - 1] = a.in.tokens[r0 + path[j]];
     em[l] = tok;
@@ -151,6 +194,8 @@ sample_accept_kernel(SampleArgs a) {
     a.new_len[seq] = a.in.seq_len[seq] + l + 1;
     a.new_pending[seq] = tok;
   }
+  __syncthreads();
+  publish(a, seq, r0, k, l);
 }
 
 template <typename K, typename... Args>

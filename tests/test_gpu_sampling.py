@@ -163,3 +163,34 @@ def test_sampled_acceptance_over_a_tree(name, ctx, n_nodes):
                 d = (got[ctx:].double() - ref).abs()
                 assert bool((d <= 1e-2 + 1e-2 * ref.abs()).all())
     gm.close()
+
+
+@pytest.mark.parametrize("name,n_refused", [("tiny", 0), ("tiny", 5), ("8b-2l", 0), ("8b-2l", 12)])
+def test_draws_at_the_edges_of_the_vocabulary_and_its_slices(name, n_refused):
+    """The draw's running sum goes slice by slice and then id by id: uniforms at both ends, at the first id of the last
+    slice and around every fourth slice's boundary, without refused tokens and with several in one slice."""
+    shape = synth.SHAPES[name]
+    om, gm = make_pair(shape, k_max=16, max_ctx=128, path=1)
+    cache, s, pending = synthetic_context(shape, om, gm, 50)
+    ids = [700 + 3 * j for j in range(n_refused)]               # (all within one slice of the 8192-id vocabulary)
+    T = 4.0                                                     # nearly uniform: a child is refused by any u above 1e-2
+    ref = om.verify(pending, [], cache.clone(), want_logits=True)["logits"]
+    p = oracle.target_probs(ref[0], T).clone()
+    p[ids] = 0.0
+    cdf = (torch.cumsum(p, 0) / p.sum()).numpy()
+    per = (shape.vocab // 128 + 31) // 32 * 128
+    us = [0.0, 1e-6, 0.99999994] + [float(cdf[b - 1]) + d for b in range(per, shape.vocab, 4 * per) for d in (-2e-5, 2e-5)]
+    for u in us:
+        uni = [float(np.float32(min(max(u, 0.0), 0.99999994)))] + [0.99] * n_refused
+        if n_refused:
+            res = ts.ts_verify_tree_sampled(gm, [s], [ids], [[0] * n_refused], T, uni)[0][0]
+        else:
+            res = ts.ts_verify_sampled(gm, [s], [[]], T, uni)[0]
+        assert res.accept_len == 0
+        tok = res.emitted[0]
+        # logits differ by LOGIT_MAX_ABS at most, the running sum by that over T, relatively
+        slack = LOGIT_MAX_ABS / T / 4
+        assert tok not in ids and (cdf[tok - 1] if tok else 0.0) - slack <= u <= cdf[tok] + slack
+    a = gm.read_logits(0, 1)
+    assert np.isfinite(a).all()                                 # the refused tokens' logits were put back
+    gm.close()
