@@ -32,6 +32,7 @@
 namespace ts {
 
 static constexpr int kAttnRows = 128;   // packed rows per unit
+static constexpr long long kMergeManyRows = 8192;   // (row, query head) pairs from which the merge takes several rows per warp
 static constexpr int kAttnBlk = 64;     // kv positions per block
 // K/V blocks in the ring (three are held by issued products, the rest are in flight): 192 KB of shared memory for
 // either head width.  More than half of an SM's shared memory on purpose: a CTA takes all 512 columns of tensor memory,
@@ -516,82 +517,99 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
   if (threadIdx.x == 0 && a.stamp) stamp_max(a.stamp + 3);
 }
 
-// grid = (M, Hq / 4), 4 warps: a warp adds the partial results of one (row, query head) and emits the normalised row as
-// bf16 (hi[, lo]); lane i owns hd / 32 consecutive elements.  The (tile, kv head) has tile_slots units, all of them
+// grid = (M / RW, Hq / 4), 4 warps: a warp adds the partial results of RW rows of one query head and emits the normalised
+// rows as bf16 (hi[, lo]); lane i owns hd / 32 consecutive elements.  The (tile, kv head) has tile_slots units, all of them
 // written (one the row sees nothing of carries sum 0 and gets weight 0).  Lane s turns slot s's (max, sum) into a weight;
 // every lane loads its elements of all slots at once (one round trip to L2, 16 bytes per lane and slot) and adds them in
-// slot order.  NS = compile-time bound on the number of slots.
-template <int NS, int VW>
+// slot order.  NS = compile-time bound on the number of slots.  (RW > 1 for many rows, where a row at a time is several
+// waves of CTAs that each wait for a few round trips: 1024 rows of the 8B shape 29 us, four at a time 9.5.)
+template <int NS, int VW, int RW>
 __global__ void attn_merge_kernel(const AttnTcArgs a) {
   if (threadIdx.x == 0) stamp_min(a.stamp_merge);
   pdl_launch_dependents();   // the dependent kernel waits for this one's end before touching its data
-  const int m = blockIdx.x, h = blockIdx.y * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int m0 = blockIdx.x * RW, h = blockIdx.y * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   // (step inputs, on the device before the step's first kernel)
-  const int G = a.Hq / a.Hkv, meta = a.in.row_tile[m];
-  int nl = 0;
-  if (h < a.Hq) nl = a.tile_slots[((meta >> 6) + ((meta & 63) * G + h % G) / kAttnRows) * a.Hkv + h / G];
-  if (!ts_in_range(a.in.ck, CHK_LEAVES, nl, a.n_slots + 1)) nl = 0;
+  const int G = a.Hq / a.Hkv;
+  int nl[RW];
+#pragma unroll
+  for (int i = 0; i < RW; ++i) {
+    nl[i] = 0;
+    if (h < a.Hq && m0 + i < a.in.M) {
+      const int meta = a.in.row_tile[m0 + i];
+      nl[i] = a.tile_slots[((meta >> 6) + ((meta & 63) * G + h % G) / kAttnRows) * a.Hkv + h / G];
+    }
+    if (!ts_in_range(a.in.ck, CHK_LEAVES, nl[i], a.n_slots + 1)) nl[i] = 0;
+  }
   pdl_wait();
   if (threadIdx.x == 0) stamp_waited(a.stamp_merge);
   if (h >= a.Hq) return;
-  const size_t base = ((size_t)m * a.Hq + h) * a.n_slots;
-  const float2 ml = lane < nl ? a.attn_ml[base + lane] : make_float2(-INFINITY, 0.f);
-  float t[NS][VW];
+  float2 ml[RW];
+  float t[RW][NS][VW];
 #pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    if (s < nl) {
-      const float *src = a.attn_o + (base + s) * a.hd + lane * VW;
-      if constexpr (VW == 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(src);
-        t[s][0] = v.x; t[s][1] = v.y; t[s][2] = v.z; t[s][3] = v.w;
+  for (int i = 0; i < RW; ++i) {
+    const size_t base = ((size_t)(m0 + i) * a.Hq + h) * a.n_slots;
+    ml[i] = lane < nl[i] ? a.attn_ml[base + lane] : make_float2(-INFINITY, 0.f);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      if (s < nl[i]) {
+        const float *src = a.attn_o + (base + s) * a.hd + lane * VW;
+        if constexpr (VW == 4) {
+          const float4 v = *reinterpret_cast<const float4 *>(src);
+          t[i][s][0] = v.x; t[i][s][1] = v.y; t[i][s][2] = v.z; t[i][s][3] = v.w;
+        } else {
+          const float2 v = *reinterpret_cast<const float2 *>(src);
+          t[i][s][0] = v.x; t[i][s][1] = v.y;
+        }
       } else {
-        const float2 v = *reinterpret_cast<const float2 *>(src);
-        t[s][0] = v.x; t[s][1] = v.y;
+#pragma unroll
+        for (int e = 0; e < VW; ++e) t[i][s][e] = 0.f;
       }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < RW; ++i) {
+    const int m = m0 + i;
+    if (m >= a.in.M) break;
+    float mx = ml[i].y > 0.f ? ml[i].x : -INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float w = ml[i].y > 0.f ? exp2f(ml[i].x - mx) : 0.f;
+    // the denominator: slot by slot in slot order (a shuffle tree would pair lanes differently as slots are added)
+    float den = 0.f, num[VW];
+#pragma unroll
+    for (int e = 0; e < VW; ++e) num[e] = 0.f;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const float ws = __shfl_sync(0xffffffffu, w, s);
+      const float ls = __shfl_sync(0xffffffffu, ml[i].y, s);
+      if (ws != 0.f) {
+        den += ws * ls;
+#pragma unroll
+        for (int e = 0; e < VW; ++e) num[e] += ws * t[i][s][e];
+      }
+    }
+    const float inv = 1.f / den;
+    __align__(8) __nv_bfloat16 hi[VW], lo[VW];
+#pragma unroll
+    for (int e = 0; e < VW; ++e) split_bf16(num[e] * inv, hi[e], lo[e]);
+    const size_t col = (size_t)h * a.hd + lane * VW;
+    const size_t ld = (size_t)a.Hq * a.hd;
+    __nv_bfloat16 *o_hi = a.out + (size_t)m * ld + col, *o_lo = a.out + ((size_t)a.out_rows + m) * ld + col;
+    if constexpr (VW == 4) {
+      *reinterpret_cast<uint2 *>(o_hi) = *reinterpret_cast<const uint2 *>(hi);
+      if (a.planes == 2) *reinterpret_cast<uint2 *>(o_lo) = *reinterpret_cast<const uint2 *>(lo);
     } else {
-#pragma unroll
-      for (int e = 0; e < VW; ++e) t[s][e] = 0.f;
+      *reinterpret_cast<uint32_t *>(o_hi) = *reinterpret_cast<const uint32_t *>(hi);
+      if (a.planes == 2) *reinterpret_cast<uint32_t *>(o_lo) = *reinterpret_cast<const uint32_t *>(lo);
     }
-  }
-  float mx = ml.y > 0.f ? ml.x : -INFINITY;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  float w = ml.y > 0.f ? exp2f(ml.x - mx) : 0.f;
-  // the denominator: leaf by leaf in leaf order (a shuffle tree would pair lanes differently as leaves are added)
-  float den = 0.f, num[VW];
-#pragma unroll
-  for (int e = 0; e < VW; ++e) num[e] = 0.f;
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    const float ws = __shfl_sync(0xffffffffu, w, s);
-    const float ls = __shfl_sync(0xffffffffu, ml.y, s);
-    if (ws != 0.f) {
-      den += ws * ls;
-#pragma unroll
-      for (int e = 0; e < VW; ++e) num[e] += ws * t[s][e];
-    }
-  }
-  const float inv = 1.f / den;
-  __align__(8) __nv_bfloat16 hi[VW], lo[VW];
-#pragma unroll
-  for (int e = 0; e < VW; ++e) split_bf16(num[e] * inv, hi[e], lo[e]);
-  const size_t col = (size_t)h * a.hd + lane * VW;
-  const size_t ld = (size_t)a.Hq * a.hd;
-  __nv_bfloat16 *o_hi = a.out + (size_t)m * ld + col, *o_lo = a.out + ((size_t)a.out_rows + m) * ld + col;
-  if constexpr (VW == 4) {
-    *reinterpret_cast<uint2 *>(o_hi) = *reinterpret_cast<const uint2 *>(hi);
-    if (a.planes == 2) *reinterpret_cast<uint2 *>(o_lo) = *reinterpret_cast<const uint2 *>(lo);
-  } else {
-    *reinterpret_cast<uint32_t *>(o_hi) = *reinterpret_cast<const uint32_t *>(hi);
-    if (a.planes == 2) *reinterpret_cast<uint32_t *>(o_lo) = *reinterpret_cast<const uint32_t *>(lo);
   }
   if (threadIdx.x == 0 && a.stamp_merge) stamp_max(a.stamp_merge + 3);
 }
 
-template <typename K>
-static cudaError_t launch_merge_pdl(K kernel, const AttnTcArgs &a, cudaStream_t st) {
+template <int NS, int VW, int RW>
+static cudaError_t launch_merge_pdl(const AttnTcArgs &a, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(a.in.M, (a.Hq + 3) / 4);
+  cfg.gridDim = dim3((a.in.M + RW - 1) / RW, (a.Hq + 3) / 4);
   cfg.blockDim = dim3(128);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -599,23 +617,23 @@ static cudaError_t launch_merge_pdl(K kernel, const AttnTcArgs &a, cudaStream_t 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
+  return cudaLaunchKernelEx(&cfg, attn_merge_kernel<NS, VW, RW>, a);
+}
+
+template <int VW>
+static cudaError_t launch_merge(const AttnTcArgs &a, cudaStream_t st) {
+  // four rows per warp where that still fills the SMs' warps about once
+  const bool many = (long long)a.in.M * a.Hq >= kMergeManyRows;
+  if (a.n_slots <= 2) return many ? launch_merge_pdl<2, VW, 4>(a, st) : launch_merge_pdl<2, VW, 1>(a, st);
+  if (a.n_slots <= 4) return many ? launch_merge_pdl<4, VW, 4>(a, st) : launch_merge_pdl<4, VW, 1>(a, st);
+  if (a.n_slots <= 8) return many ? launch_merge_pdl<8, VW, 2>(a, st) : launch_merge_pdl<8, VW, 1>(a, st);
+  if (a.n_slots <= 16) return launch_merge_pdl<16, VW, 1>(a, st);
+  return launch_merge_pdl<32, VW, 1>(a, st);
 }
 
 cudaError_t launch_attention_tc_merge(const AttnTcArgs &a, cudaStream_t st) {
   if (a.n_slots < 1 || a.n_slots > kAttnMaxSplits) return cudaErrorInvalidValue;
-  if (a.hd == 128) {
-    if (a.n_slots <= 2) return launch_merge_pdl(attn_merge_kernel<2, 4>, a, st);
-    if (a.n_slots <= 4) return launch_merge_pdl(attn_merge_kernel<4, 4>, a, st);
-    if (a.n_slots <= 8) return launch_merge_pdl(attn_merge_kernel<8, 4>, a, st);
-    if (a.n_slots <= 16) return launch_merge_pdl(attn_merge_kernel<16, 4>, a, st);
-    return launch_merge_pdl(attn_merge_kernel<32, 4>, a, st);
-  }
-  if (a.n_slots <= 2) return launch_merge_pdl(attn_merge_kernel<2, 2>, a, st);
-  if (a.n_slots <= 4) return launch_merge_pdl(attn_merge_kernel<4, 2>, a, st);
-  if (a.n_slots <= 8) return launch_merge_pdl(attn_merge_kernel<8, 2>, a, st);
-  if (a.n_slots <= 16) return launch_merge_pdl(attn_merge_kernel<16, 2>, a, st);
-  return launch_merge_pdl(attn_merge_kernel<32, 2>, a, st);
+  return a.hd == 128 ? launch_merge<4>(a, st) : launch_merge<2>(a, st);
 }
 
 static size_t attn_tc_smem(int hd) {

@@ -99,6 +99,64 @@ norm_kernel(const int32_t *tokens, const __nv_bfloat16 *embed, const float *part
   if (stamp) { __syncthreads(); if (threadIdx.x == 0) stamp_max(stamp + 3); }
 }
 
+// The same (MODE 1) for steps of many rows: 256 threads per row, kNormChunks x 1024 elements in registers at most, so that
+// several rows share an SM (a 1024-thread CTA fills one alone: 1024 rows of the 8B shape took seven waves, 27 us; now
+// 14, and 256 rows with four slabs 5.8 instead of 7.3).
+static constexpr int kNormRowsThreads = 256;
+static constexpr int kNormChunks = 4;      // d <= 4096
+template <int NS>   // most slabs: all loads are issued before the first sum
+__global__ void __launch_bounds__(kNormRowsThreads, NS == 1 ? 5 : NS == 2 ? 4 : NS == 3 ? 3 : 2)
+norm_rows_kernel(const float *part, int n_splits, int part_rows, const float *gain, float eps, int d, float *x,
+                 __nv_bfloat16 *h, int h_rows, int planes, unsigned long long *stamp) {
+  __shared__ float red[32];
+  if (threadIdx.x == 0) stamp_min(stamp);
+  pdl_launch_dependents();   // the dependent kernel waits for this one's end before touching its data
+  const int m = blockIdx.x, c0 = threadIdx.x * 4;
+  pdl_wait();
+  if (threadIdx.x == 0) stamp_waited(stamp);
+  float *xr = x + (size_t)m * d;
+  float4 v[kNormChunks], p[NS][kNormChunks];
+#pragma unroll
+  for (int i = 0; i < kNormChunks; ++i) {
+    const int c = c0 + i * 4 * kNormRowsThreads;
+    if (c < d) {
+      v[i] = *reinterpret_cast<const float4 *>(xr + c);
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if (s < n_splits) p[s][i] = *reinterpret_cast<const float4 *>(part + ((size_t)s * part_rows + m) * d + c);
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s)   // (the sums in slab order, as everywhere)
+#pragma unroll
+    for (int i = 0; i < kNormChunks; ++i)
+      if (s < n_splits) { v[i].x += p[s][i].x; v[i].y += p[s][i].y; v[i].z += p[s][i].z; v[i].w += p[s][i].w; }
+  float ss = 0.f;
+#pragma unroll
+  for (int i = 0; i < kNormChunks; ++i) {
+    const int c = c0 + i * 4 * kNormRowsThreads;
+    if (c < d) {
+      *reinterpret_cast<float4 *>(xr + c) = v[i];
+      ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+    }
+  }
+  const float r = rsqrtf(block_sum(ss, red) / (float)d + eps);
+#pragma unroll
+  for (int i = 0; i < kNormChunks; ++i) {
+    const int c = c0 + i * 4 * kNormRowsThreads;
+    if (c < d) {
+      const float4 g = *reinterpret_cast<const float4 *>(gain + c);
+      const float o[4] = {v[i].x * r * g.x, v[i].y * r * g.y, v[i].z * r * g.z, v[i].w * r * g.w};
+      __align__(8) __nv_bfloat16 hi[4], lo[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) split_bf16(o[j], hi[j], lo[j]);
+      *reinterpret_cast<uint2 *>(h + (size_t)m * d + c) = *reinterpret_cast<uint2 *>(hi);
+      if (planes == 2) *reinterpret_cast<uint2 *>(h + ((size_t)h_rows + m) * d + c) = *reinterpret_cast<uint2 *>(lo);
+    }
+  }
+  if (stamp) { __syncthreads(); if (threadIdx.x == 0) stamp_max(stamp + 3); }
+}
+
 template <typename K, typename... Args>
 static cudaError_t launch_pdl(K kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg{};
@@ -114,6 +172,7 @@ static cudaError_t launch_pdl(K kernel, dim3 grid, dim3 block, size_t smem, cuda
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+static constexpr int kNormManyRows = 100;   // below, one CTA of 1024 threads per SM is a single wave and the quicker one
 static int norm_threads(int d) { return std::min(kNormMaxThreads, (d / 4 + 31) / 32 * 32); }
 
 cudaError_t launch_embed_norm(const StepIn &in, const __nv_bfloat16 *embed, const float *gain, float eps,
@@ -127,6 +186,9 @@ cudaError_t launch_add_norm(int M, int d, const float *part, int n_splits, int p
                             float eps, float *x, __nv_bfloat16 *h, int h_rows, int planes, cudaStream_t st,
                             unsigned long long *stamp) {
   if (n_splits > kNormMaxSplits) return cudaErrorInvalidValue;
+  if (M >= kNormManyRows && d <= kNormChunks * 4 * kNormRowsThreads && n_splits <= 4)
+    return launch_pdl(n_splits <= 1 ? norm_rows_kernel<1> : n_splits <= 2 ? norm_rows_kernel<2> : n_splits <= 3 ? norm_rows_kernel<3> : norm_rows_kernel<4>, dim3(M), dim3(kNormRowsThreads), 0, st, part, n_splits, part_rows, gain, eps, d, x,
+                      h, h_rows, planes, stamp);
   return launch_pdl(norm_kernel<1>, dim3(M), dim3(norm_threads(d)), 0, st, (const int32_t *)nullptr,
                     (const __nv_bfloat16 *)nullptr, part, n_splits, part_rows, gain, eps, d, x, h, h_rows,
                     planes, (unsigned long long *)nullptr, stamp, BoundsCheck{});
@@ -136,7 +198,7 @@ __device__ __forceinline__ __half to_half_sat(float x) {
   return __float2half_rn(fminf(fmaxf(x, -65504.f), 65504.f));
 }
 
-static constexpr int kRopeWideRows = 128;   // steps of at least this many rows take the wide kernel (no faster below)
+static constexpr int kRopeWideRows = 65;   // steps of at least this many rows take the wide kernel (smaller ones have none)
 
 // grid = (M, Hq + 2*Hkv); one CTA of hd/2 threads per (row, head).  Thread i handles the rotary pair
 // (i, i + hd/2) of q or k heads, or elements (i, i + hd/2) of a v head.  Every load is issued before the first use
@@ -196,7 +258,10 @@ __global__ void rope_kv_kernel(StepIn in, const float *part, int n_splits, int p
 // The same for steps of many rows: grid = (M, ceil(heads / 16)), block = (hd / 8, 16): a thread handles FOUR
 // neighbouring rotary pairs of one head (32 bytes per slab in one load, 8-byte stores), so a 256-row step is 768 CTAs
 // of 256 threads instead of 12 288 CTAs of 64 -- less than one wave of resident threads instead of nearly three.  The
-// sums are taken in the same order as above: the results are the same bits.
+// sums are taken in the same order as above: the results are the same bits.  NS = most slabs: with room for twelve slabs'
+// loads in registers only one or two CTAs fit on an SM (256 rows, three slabs: 12.5 us; 1024 rows, two slabs: 56), with room
+// for four or two all of them do (4.2 us; 15).
+template <int NS>
 __global__ void rope_kv_wide_kernel(StepIn in, const float *part, int n_splits, int part_rows, int Hq, int Hkv, int hd,
                                     const float2 *rope_tab, __half *q_out, __half *q_lo_out, __half *k_pages,
                                     __half *v_pages, unsigned long long *stamp) {
@@ -222,9 +287,9 @@ __global__ void rope_kv_wide_kernel(StepIn in, const float *part, int n_splits, 
   if (live) {
     // the QKV weight rows are stored with rotary partners adjacent: feature 2i = element i, 2i+1 = element i + hd/2
     const int col = head * hd + 2 * i0;
-    float4 p[kNormMaxSplits][2];
+    float4 p[NS][2];
 #pragma unroll
-    for (int s = 0; s < kNormMaxSplits; ++s)
+    for (int s = 0; s < NS; ++s)
       if (s < n_splits) {
         const float4 *src = reinterpret_cast<const float4 *>(part + ((size_t)s * part_rows + m) * N + col);
         p[s][0] = src[0];
@@ -232,7 +297,7 @@ __global__ void rope_kv_wide_kernel(StepIn in, const float *part, int n_splits, 
       }
     float a[4] = {0.f, 0.f, 0.f, 0.f}, b[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int s = 0; s < kNormMaxSplits; ++s)
+    for (int s = 0; s < NS; ++s)
       if (s < n_splits) {
         a[0] += p[s][0].x; b[0] += p[s][0].y; a[1] += p[s][0].z; b[1] += p[s][0].w;
         a[2] += p[s][1].x; b[2] += p[s][1].y; a[3] += p[s][1].z; b[3] += p[s][1].w;
@@ -278,7 +343,8 @@ cudaError_t launch_rope_kv(const StepIn &in, const float *part, int n_splits, in
                            int hd, const float2 *rope_tab, __half *q_out, __half *q_lo_out, __half *k_pages,
                            __half *v_pages, cudaStream_t st, unsigned long long *stamp) {
   if (in.M >= kRopeWideRows && hd % 8 == 0)
-    return launch_pdl(rope_kv_wide_kernel, dim3(in.M, (Hq + 2 * Hkv + 15) / 16), dim3(hd / 8, 16), 0, st, in, part,
+    return launch_pdl(n_splits <= 2 ? rope_kv_wide_kernel<2> : n_splits <= 4 ? rope_kv_wide_kernel<4> : rope_kv_wide_kernel<kNormMaxSplits>,
+                      dim3(in.M, (Hq + 2 * Hkv + 15) / 16), dim3(hd / 8, 16), 0, st, in, part,
                       n_splits, part_rows, Hq, Hkv, hd, rope_tab, q_out, q_lo_out, k_pages, v_pages, stamp);
   return launch_pdl(rope_kv_kernel, dim3(in.M, Hq + 2 * Hkv), dim3(hd / 2), 0, st, in, part, n_splits,
                     part_rows, Hq, Hkv, hd, rope_tab, q_out, q_lo_out, k_pages, v_pages, stamp);
