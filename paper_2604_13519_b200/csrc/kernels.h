@@ -51,7 +51,7 @@ enum : int { EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_LOGITS = 2, EPI_QKV = 3, EPI_R
 
 struct GemmArgs {
   int N, K, M;          // output features, reduction length, valid activation rows
-  int Mc;               // activation rows per CTA: the step's rows rounded up (weight-streaming kernel, at most 64), 128 (many rows)
+  int Mc;               // activation rows per CTA: the step's rows rounded up (weight-streaming kernel), 128 (many rows)
   int planes;           // 1 = bf16 activations, 2 = (hi, lo) pair
   int n_kblocks;        // K / 64
   int kb_per_split;     // k-blocks per split-K slice

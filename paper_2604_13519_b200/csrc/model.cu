@@ -45,8 +45,13 @@ constexpr int kMaxAttnSplits = ts::kAttnMaxSplits;
 // activations: the tensor-core instruction's N, planes x rows, is a multiple of 16) -- a k-block of 33 rows in a box of
 // 64 takes as many bytes as its weights, which left three stages in the ring: gate-up of the 1B shape 24.5 us against
 // 14.9 at 8 rows.  Many-rows kernel: 128.
-constexpr int kMcOptions[9] = {8, 16, 24, 32, 40, 48, 56, 64, 128};
-constexpr int kMcRows = 8;                       // index of the many-rows kernel's box
+constexpr int kMcOptions[13] = {8, 16, 24, 32, 40, 48, 56, 64, 72, 80, 88, 96, 128};
+constexpr int kMcRows = 12;                      // index of the many-rows kernel's box
+// Most rows of a step whose projections run on the weight-streaming kernel, with one and with two planes of activations.
+// With two planes a ring of three stages still fits twice on an SM at 80 rows and one of two at 88.  Measured, four sessions,
+// many-rows kernel against this one: 1B shape two planes 80 rows 1440 / 1281 us, 96 rows 1481 / 1518; 8B 5467 / 4684 and
+// 5511 / 5483; one plane 1B 96 rows 1267 / 1276, 112 rows 1297 / 1371, 8B 4547 / 4378 and 4672 / 4558.
+constexpr int kFewRows[2] = {96, 80};
 constexpr int kFusedMc[3] = {1, 3, 7};           // the persistent kernel's boxes: 16, 32, 64 rows
 constexpr int kPrefillRows = 1024;   // rows of a prompt that go through in one step
 constexpr int kPrefillSplits = 3;    // split-K slabs of such a step at most
@@ -224,7 +229,7 @@ struct ts_model {
   int leaf_len = 64;   // KV positions per attention leaf: a constant of the model (see AttnTcArgs), set by ts_init_model
   size_t gemm_smem_budget = 113 * 1024;   // two CTAs of the weight-streaming kernel per SM
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_d;
-  CUtensorMap tm_lm{}, tm_h[9]{}, tm_attn[9]{}, tm_act[9]{};
+  CUtensorMap tm_lm{}, tm_h[13]{}, tm_attn[13]{}, tm_act[13]{};
   std::vector<int32_t> free_pages;
   std::vector<ts_session *> sessions;   // live sessions over this model (detached on destroy)
   // last staged step
@@ -319,7 +324,7 @@ ts_status weight_map(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t N
 }
 
 ts_status act_maps(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t K, uint64_t rows, int planes) {
-  for (int i = 0; i < 9; ++i) {
+  for (int i = 0; i < 13; ++i) {
     const uint64_t dims[3] = {K, rows, (uint64_t)planes};
     const uint32_t box[3] = {64, (uint32_t)kMcOptions[i], (uint32_t)planes};
     ts_status s = make_map(enc, &out[i], base, 3, dims, box);
@@ -329,7 +334,6 @@ ts_status act_maps(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t K, 
 }
 
 int pick_mc_index(int M, int planes) {
-  if (M > 64) return kMcRows;
   const int i = (M + 7) / 8 - 1;
   return planes == 1 ? (i | 1) : i;
 }
@@ -367,7 +371,7 @@ int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks
   return best;
 }
 
-// A projection of the many-rows kernel (more than 64 rows: bound by the tensor cores and the bytes per flop an SM pulls
+// A projection of the many-rows kernel (more than kFewRows rows: bound by the tensor cores and the bytes per flop an SM pulls
 // from L2).  n_splits_out: split-K slabs written (EPI_PARTIAL).
 ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M,
                         float *out, __nv_bfloat16 *act_out, unsigned long long *amax, int *n_splits_out) {
@@ -387,7 +391,7 @@ ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUten
   return TS_OK;
 }
 
-// A projection of the weight-streaming kernel (at most 64 rows); `g` carries what its epilogue needs.
+// A projection of the weight-streaming kernel; `g` carries what its epilogue needs.
 ts_status run_gemm_ws(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M, ts::GemmArgs g) {
   const int mi = pick_mc_index(M, m->planes);
   g.N = N; g.K = K; g.M = M; g.Mc = kMcOptions[mi]; g.planes = m->planes;
@@ -503,10 +507,10 @@ ts_status run_step(ts_model *m) {
   CU_TRY(ts::launch_embed_norm(in, (const __nv_bfloat16 *)m->W(L.embed), (const float *)m->W(L.g1[0]), c.rms_eps,
                                d, x, h, R, m->planes, (unsigned long long *)m->WS(L.amax), m->st));
   m->launched(3);
-  // Up to 64 rows the weight-streaming kernel: QKV rotates and appends K/V itself, O and down update the residual stream
+  // Up to kFewRows rows the weight-streaming kernel: QKV rotates and appends K/V itself, O and down update the residual stream
   // and prepare the next projection's input (6 launches per layer); beyond, the many-rows kernel with its split-K slabs
   // folded by a rotary and two norm kernels.
-  const bool few = M <= 64;
+  const bool few = M <= kFewRows[m->planes - 1];
   float *ss = (float *)m->WS(L.ss_part);
   const bool skip_head = (m->last_flags & TS_FLAG_SKIP_LM_HEAD) != 0;
   int splits = 0;

@@ -175,6 +175,49 @@ def test_row_counts_around_the_projection_kernels_switch(name, ks):
     gm.close()
 
 
+@pytest.mark.parametrize("name,ks", [("8b-2l", [40, 32]), ("8b-2l", [40, 33]), ("1b-2l", [40, 40]), ("1b-2l", [41, 40]), ("tiny", [33, 47])],
+                         ids=lambda v: v if isinstance(v, str) else f"{sum(v)}rows")
+def test_row_counts_at_the_end_of_the_weight_streaming_kernel(name, ks):
+    """72, 73, 80 and 81 rows: the largest activation boxes of the weight-streaming projections, a partly filled one, the
+    last size before and the first size after the switch to the many-rows kernel."""
+    shape = synth.SHAPES[name]
+    lens = [333, 70]
+    om, gm = make_pair(shape, max_batch=2, k_max=64, max_rows=sum(ks), max_ctx=512)
+    sess, drafts, refs = [], [], []
+    for i, (n, k) in enumerate(zip(lens, ks)):
+        cache, s, pending = synthetic_context(shape, om, gm, n, stream=i, pending=300 + i)
+        draft = _rand_draft(shape.vocab, k - 1, 70 + i)
+        sess.append(s); drafts.append(draft)
+        refs.append(om.verify(pending, draft, cache, want_logits=True))
+    row = 0
+    for i, (res, ref) in enumerate(zip(ts.ts_verify(gm, sess, drafts), refs)):
+        check_step(res, gm.read_logits(row, res.k), ref, f"{name}, {sum(ks)} rows, seq {i}")
+        row += res.k
+    gm.close()
+
+
+@pytest.mark.parametrize("ks", [[49, 47], [49, 48]], ids=lambda ks: f"{sum(ks)}rows")
+def test_row_counts_at_the_switch_with_one_plane(ks):
+    """One plane of activations, 96 and 97 rows: each session's logits against the same rows verified alone.  The two
+    differ by summation orders, which move single activations across a bf16 rounding (2^-9 relative each, thousands of
+    them independent in every sum): 2.4e-2 of the logits' norm, four times what 16 and 36 layers showed."""
+    shape = synth.SHAPES["1b-2l"]
+    om, gm = make_pair(shape, max_batch=2, k_max=64, max_rows=sum(ks), max_ctx=512, act_split=False)
+    sess, drafts = [], []
+    for i, (n, k) in enumerate(zip([333, 70], ks)):
+        _, s, _ = synthetic_context(shape, om, gm, n, stream=i, pending=300 + i)
+        sess.append(s); drafts.append(_rand_draft(shape.vocab, k - 1, 70 + i))
+    ts.ts_verify(gm, sess, drafts)
+    both = gm.read_logits(0, sum(ks)).copy()
+    row = 0
+    for s, d, k in zip(sess, drafts, ks):
+        ts.ts_verify(gm, [s], [d])
+        alone = gm.read_logits(0, k)
+        assert np.linalg.norm(both[row:row + k] - alone) <= 2.4e-2 * np.linalg.norm(alone)
+        row += k
+    gm.close()
+
+
 def test_sixteen_sessions_512_rows():
     """The largest step of the batched configuration: 16 sessions x k = 32 = 512 rows (four 128-row chunks in every
     projection, 16 attention row tiles), ragged contexts from a few tokens to two thousand."""
