@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
 // slot order.  NS = compile-time bound on the number of slots.  (RW > 1 for many rows, where a row at a time is several
 // waves of CTAs that each wait for a few round trips: 1024 rows of the 8B shape 29 us, four at a time 9.5.)
 template <int NS, int VW, int RW>
-__global__ void attn_merge_kernel(const AttnTcArgs a) {
+__global__ void __launch_bounds__(128) attn_merge_kernel(const AttnTcArgs a) {
   if (threadIdx.x == 0) stamp_min(a.stamp_merge);
   pdl_launch_dependents();   // the dependent kernel waits for this one's end before touching its data
   const int m0 = blockIdx.x * RW, h = blockIdx.y * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -551,21 +551,17 @@ __global__ void attn_merge_kernel(const AttnTcArgs a) {
     ml[i] = lane < nl[i] ? a.attn_ml[base + lane] : make_float2(-INFINITY, 0.f);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-      if (s < nl[i]) {
-        const float *src = a.attn_o + (base + s) * a.hd + lane * VW;
-        if constexpr (VW == 4) {
-          const float4 v = *reinterpret_cast<const float4 *>(src);
-          t[i][s][0] = v.x; t[i][s][1] = v.y; t[i][s][2] = v.z; t[i][s][3] = v.w;
-        } else {
-          const float2 v = *reinterpret_cast<const float2 *>(src);
-          t[i][s][0] = v.x; t[i][s][1] = v.y;
-        }
+      const float *src = a.attn_o + (base + s) * a.hd + lane * VW;
+      if constexpr (VW == 4) {
+        const float4 v = ld_global_v4_if(src, s < nl[i]);
+        t[i][s][0] = v.x; t[i][s][1] = v.y; t[i][s][2] = v.z; t[i][s][3] = v.w;
       } else {
-#pragma unroll
-        for (int e = 0; e < VW; ++e) t[i][s][e] = 0.f;
+        const float2 v = ld_global_v2_if(src, s < nl[i]);
+        t[i][s][0] = v.x; t[i][s][1] = v.y;
       }
     }
   }
+  __syncwarp();   // (no load may move past it: left to itself the compiler puts every load next to its use)
 #pragma unroll
   for (int i = 0; i < RW; ++i) {
     const int m = m0 + i;
@@ -582,11 +578,9 @@ __global__ void attn_merge_kernel(const AttnTcArgs a) {
     for (int s = 0; s < NS; ++s) {
       const float ws = __shfl_sync(0xffffffffu, w, s);
       const float ls = __shfl_sync(0xffffffffu, ml[i].y, s);
-      if (ws != 0.f) {
-        den += ws * ls;
+      den += ws * ls;
 #pragma unroll
-        for (int e = 0; e < VW; ++e) num[e] += ws * t[i][s][e];
-      }
+      for (int e = 0; e < VW; ++e) num[e] += ws * (ws != 0.f ? t[i][s][e] : 0.f);
     }
     const float inv = 1.f / den;
     __align__(8) __nv_bfloat16 hi[VW], lo[VW];

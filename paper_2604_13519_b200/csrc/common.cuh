@@ -158,6 +158,29 @@ __device__ __forceinline__ void ld_global_v8(const void *p, uint32_t *r) {
                : "memory");
 }
 
+// 16 / 8 bytes, or zeros where `p` is false.  (A statement of its own, so that a run of them is issued as written: under a
+// branch each the compiler made every load wait for the one before.)
+__device__ __forceinline__ float4 ld_global_v4_if(const float *src, bool p) {
+  float4 v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
+      "mov.f32 %2, 0f00000000;\n\tmov.f32 %3, 0f00000000;\n\t@p ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "l"(src), "r"((int)p)
+      : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_global_v2_if(const float *src, bool p) {
+  float2 v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
+      "@p ld.global.v2.f32 {%0, %1}, [%2];\n\t}"
+      : "=f"(v.x), "=f"(v.y)
+      : "l"(src), "r"((int)p)
+      : "memory");
+  return v;
+}
+
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
