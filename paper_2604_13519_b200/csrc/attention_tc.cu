@@ -60,9 +60,6 @@ __device__ __forceinline__ bool worker_all(bool ok) {
       : "memory");
   return r != 0;
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ bool mbar_wait_err(uint32_t bar, uint32_t parity, const int *err) {
   uint64_t t0 = 0;
   for (uint32_t it = 0;; ++it) {

@@ -83,9 +83,6 @@ __device__ __forceinline__ bool worker_all(bool ok) {
       : "memory");
   return r != 0;
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
 // Bounded mbarrier wait that also gives up when another CTA has reported an error.

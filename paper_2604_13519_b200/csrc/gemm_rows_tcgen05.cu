@@ -7,17 +7,19 @@
 // into the SAME accumulator, so per 64-wide k-block a CTA brings in 32 KB of activations and 32 KB of weights for
 // 8.4 MFLOP -- two thirds of the bytes per flop of the weight-streaming kernel (gemm_tcgen05.cu), which at these sizes
 // is what sets the pace.  The weight matrix keeps its storage (contiguous 128 x 64 blocks, one TMA box each): a CTA's
-// 256 weight rows are two such boxes.  One CTA per SM (three 64 KB stages).
+// 256 weight rows are two such boxes.  One CTA per SM (three 64 KB stages), and the launch has no more CTAs than SMs: a CTA
+// walks its tiles one after the other with two accumulators in tensor memory, so that the loads of the next tile and its
+// products run under the epilogue of this one.  (A CTA per tile paid 8 to 10 us for set-up, first loads and epilogue each
+// time, against 40 of main loop for the longest tiles; 1024 rows of the 8B shape: gate-up 328 -> 300 us, 1.37 PFLOP/s of issued
+// work, the rate a sustained cuBLAS product reaches under the power cap.)
 //
 // Roles: warp 0 = TMA producer, warp 1 = TMEM allocation + MMA issue, warps 2..9 = epilogue (thread <-> row, two
 // warps per row quarter, half of the columns each).
 // Every wait is bounded; on expiry the CTA records an error word and leaves through the normal exit.
 #include <algorithm>
-#include <functional>
 #include <map>
 #include <mutex>
 #include <tuple>
-#include <vector>
 
 #include "kernels.h"
 
@@ -33,10 +35,45 @@ static constexpr int kMaxStages = 4;
 struct __align__(8) RowsSmemCtl {
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
-  uint64_t tmem_full;
+  uint64_t acc_full[2];    // [accumulator]
+  uint64_t acc_empty[2];
   uint32_t tmem_base;
   uint32_t abort_flag;
 };
+static constexpr int kStagingBytes = 8 * 4096;   // per epilogue warp 32 rows x 128 bytes
+
+// One output tile of a launch: rows [m0, m0 + 128), stored weight blocks blk0 (and blk0 + 1 if nb = 256), k-blocks [kb0, kb1).
+struct RowsTile {
+  int m0, blk0, nb, split, kb0, nkb;
+};
+// The tiles of CTA c out of G.  Wide tiles (two weight blocks) are dealt out in turn; of the narrow ones the first
+// g.narrow_short go in turn to the CTAs that got one wide tile less (all of them, if it came out even), the others to the
+// rest: the launcher has chosen the counts.  Row chunks are neighbours in the order: they run at the same time and all but
+// the first find the weight blocks in L2.  j = how many tiles this CTA has had; false: no more.
+__device__ __forceinline__ bool rows_tile(const GemmArgs &g, int c, int G, int j, RowsTile &t) {
+  const int blocks = g.N / kBoxN, n_narrow = blocks - 2 * g.n_wide;
+  const int nW = g.n_wide * g.chunks * g.n_splits, nN = n_narrow * g.chunks * g.n_splits;
+  const int r = nW % G, wides = nW / G + (c < r ? 1 : 0);
+  int u, n_tiles;
+  if (j < wides) {
+    u = c + j * G;
+    n_tiles = g.n_wide;
+    t.nb = kTileN;
+  } else {
+    const bool is_long = c < r;
+    u = is_long ? g.narrow_short + c + (j - wides) * r : (c - r) + (j - wides) * (G - r);
+    if (u >= (is_long ? nN : g.narrow_short)) return false;
+    n_tiles = n_narrow;
+    t.nb = kBoxN;
+  }
+  t.m0 = (u % g.chunks) * kRowsM;
+  const int v = u / g.chunks, tile = v % n_tiles;
+  t.split = v / n_tiles;
+  t.blk0 = t.nb == kTileN ? 2 * tile : 2 * g.n_wide + tile;
+  t.kb0 = (int)(((long long)t.split * g.n_kblocks) / g.n_splits);   // balanced cut of the k-blocks
+  t.nkb = (int)(((long long)(t.split + 1) * g.n_kblocks) / g.n_splits) - t.kb0;
+  return true;
+}
 
 template <int EPI>
 __global__ void __launch_bounds__(320, 1)
@@ -47,24 +84,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int a_bytes = g.planes * kRowsM * kBlockK * 2;
   const int stage_bytes = a_bytes + 2 * kBoxBytes;
-  RowsSmemCtl *ctl = reinterpret_cast<RowsSmemCtl *>(smem + (size_t)g.stages * stage_bytes);
+  uint8_t *staging = smem + (size_t)g.stages * stage_bytes;
+  RowsSmemCtl *ctl = reinterpret_cast<RowsSmemCtl *>(staging + kStagingBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // grid = (row chunks, weight tiles, K slices): the row chunks of one (tile, slice) are neighbours in launch order, so
-  // they run at the same time and all but the first find the weight blocks in L2
-  // the first n_wide tiles hold two stored 128-row weight blocks, the tiles after them one (the launcher mixes the
-  // widths so that the last wave of CTAs is short instead of nearly empty)
-  const int tile = blockIdx.y;
-  const int blk0 = tile < g.n_wide ? 2 * tile : g.n_wide + tile;   // the tile's first weight block
-  const int n0 = blk0 * kBoxN;
-  const int nb = tile < g.n_wide ? kTileN : kBoxN;
-  const int split = blockIdx.z;
-  const int m0 = blockIdx.x * kRowsM;
-  // balanced cut of the k-blocks into gridDim.z runs
-  const int kb0 = (int)(((long long)split * g.n_kblocks) / (int)gridDim.z);
-  const int kb1 = (int)(((long long)(split + 1) * g.n_kblocks) / (int)gridDim.z);
-  const int nkb = kb1 - kb0;
-  const int tx_bytes = a_bytes + (nb / kBoxN) * kBoxBytes;
+  const int cta = blockIdx.x, G = gridDim.x;
 
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmap_w);
@@ -73,12 +97,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       mbar_init(smem_u32(&ctl->full[s]), 1);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
     }
-    mbar_init(smem_u32(&ctl->tmem_full), 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(smem_u32(&ctl->acc_full[s]), 1);
+      mbar_init(smem_u32(&ctl->acc_empty[s]), 8);   // one arrival per epilogue warp
+    }
     ctl->abort_flag = 0;
     fence_barrier_init();
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&ctl->tmem_base), kTileN);
+    tmem_alloc(smem_u32(&ctl->tmem_base), 2 * kTileN);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -91,51 +118,65 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0 && nkb > 0) {
+    if (lane == 0) {
       const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
       // block (128-row block j, k-block kb) of the stored matrix = rows w_block(j, kb) * 128 .. of a [.][64] array
-      auto load_w = [&](int s, int kb) {
+      auto load_w = [&](const RowsTile &t, int s, int kb) {
         const uint32_t bar = smem_u32(&ctl->full[s]);
         const uint32_t dst = smem_u32(smem + (size_t)s * stage_bytes + a_bytes);
-        for (int j = 0; j < nb / kBoxN; ++j)
-          tma_load_2d(dst + j * kBoxBytes, &tmap_w, 0, w_block(blk0 + j, kb, g.N / kBoxN, g.n_kblocks) * kBoxN, bar, pol_w);
+        mbar_expect_tx(bar, a_bytes + (t.nb / kBoxN) * kBoxBytes);
+        for (int j = 0; j < t.nb / kBoxN; ++j)
+          tma_load_2d(dst + j * kBoxBytes, &tmap_w, 0, w_block(t.blk0 + j, kb, g.N / kBoxN, g.n_kblocks) * kBoxN, bar, pol_w);
       };
-      const int pre = min(g.stages, nkb);
-      // weights do not depend on the previous kernel: start them before the programmatic-dependency wait
-      for (int it = 0; it < pre; ++it) {
-        mbar_expect_tx(smem_u32(&ctl->full[it]), tx_bytes);
-        load_w(it, kb0 + it);
-      }
-      pdl_wait();
-      stamp_waited(g.stamp);
-      for (int it = 0; it < pre; ++it)
-        tma_load_3d(smem_u32(smem + (size_t)it * stage_bytes), &tmap_a, (kb0 + it) * kBlockK, m0, 0,
-                    smem_u32(&ctl->full[it]), pol_a);
-      int s = (pre == g.stages) ? 0 : pre;
-      uint32_t ph = (pre == g.stages) ? 1 : 0;
-      for (int it = pre; it < nkb; ++it) {
-        if (!mbar_wait(smem_u32(&ctl->empty[s]), ph ^ 1)) {
-          atomicExch(g.err, DEV_TIMEOUT_EMPTY);
-          break;
+      auto load_a = [&](const RowsTile &t, int s, int kb) {
+        tma_load_3d(smem_u32(smem + (size_t)s * stage_bytes), &tmap_a, kb * kBlockK, t.m0, 0, smem_u32(&ctl->full[s]), pol_a);
+      };
+      RowsTile t;
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int j = 0; ok && rows_tile(g, cta, G, j, t); ++j) {
+        int it = 0;
+        if (j == 0) {
+          // weights do not depend on the previous kernel: start them before the programmatic-dependency wait
+          const int pre = min(g.stages, t.nkb);
+          for (int i = 0; i < pre; ++i) load_w(t, i, t.kb0 + i);
+          pdl_wait();
+          stamp_waited(g.stamp);
+          for (int i = 0; i < pre; ++i) load_a(t, i, t.kb0 + i);
+          it = pre;
+          s = pre == g.stages ? 0 : pre;
+          ph = pre == g.stages ? 1 : 0;
         }
-        mbar_expect_tx(smem_u32(&ctl->full[s]), tx_bytes);
-        load_w(s, kb0 + it);
-        tma_load_3d(smem_u32(smem + (size_t)s * stage_bytes), &tmap_a, (kb0 + it) * kBlockK, m0, 0,
-                    smem_u32(&ctl->full[s]), pol_a);
-        if (++s == g.stages) { s = 0; ph ^= 1; }
+        for (; it < t.nkb; ++it) {
+          if (!mbar_wait(smem_u32(&ctl->empty[s]), ph ^ 1)) {
+            atomicExch(g.err, DEV_TIMEOUT_EMPTY);
+            ok = false;
+            break;
+          }
+          load_w(t, s, t.kb0 + it);
+          load_a(t, s, t.kb0 + it);
+          if (++s == g.stages) { s = 0; ph ^= 1; }
+        }
       }
-    } else if (lane == 0) {
-      pdl_wait();
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issue
     // The whole warp walks the loop and the waits; one elected lane issues the instructions of a k-block and its commit.
-    {
-      const uint32_t idesc = umma_idesc_bf16(kRowsM, (uint32_t)nb);
-      bool ok = true;
-      int s = 0;
-      uint32_t ph = 0;
-      for (int it = 0; it < nkb; ++it) {
+    RowsTile t;
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int j = 0; ok && rows_tile(g, cta, G, j, t); ++j) {
+      const int b = j & 1;
+      const uint32_t idesc = umma_idesc_bf16(kRowsM, (uint32_t)t.nb), d = tmem_base + b * kTileN;
+      // the accumulator's previous tile has been read out
+      if (j >= 2 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->acc_empty[b]), ((j >> 1) - 1) & 1))) {
+        if (lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
+        ok = false;
+      }
+      for (int it = 0; ok && it < t.nkb; ++it) {
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->full[s]), ph))) {   // (all lanes leave together)
           if (lane == 0) atomicExch(g.err, DEV_TIMEOUT_FULL);
           ok = false;
@@ -150,7 +191,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             const uint64_t da = umma_desc_sw128(sa + pl * (kRowsM * kBlockK * 2));
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk)   // 16 bf16 along K = 32 bytes = 2 descriptor address units
-              umma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, idesc, (it | kk | pl) != 0);
+              umma_bf16(d, da + 2 * kk, db + 2 * kk, idesc, (it | kk | pl) != 0);
           }
           umma_commit(smem_u32(&ctl->empty[s]));
         }
@@ -158,49 +199,54 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         if (++s == g.stages) { s = 0; ph ^= 1; }
       }
       if (elect_one()) {
-        if (!ok) ctl->abort_flag = 1;
-        umma_commit(smem_u32(&ctl->tmem_full));
+        if (!ok) *reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) = 1;
+        umma_commit(smem_u32(&ctl->acc_full[b]));
       }
       __syncwarp();
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..9): thread <-> row
     pdl_wait();   // outputs of this kernel may still be read by the previous one's consumers
-    bool ok = true;
-    if (nkb > 0) {
-      ok = mbar_wait(smem_u32(&ctl->tmem_full), 0);
-      if (!ok && lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
-    }
-    tc_fence_after();
-    ok = ok && (*reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) == 0);
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
-    const int m = m0 + q * 32 + lane;             // this thread's row
-    const bool row_ok = m < g.M;
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
-    float best = -INFINITY;
-    int best_n = 0;
     // Results leave through shared memory so that global stores are whole lines: a thread owns a ROW of the
     // accumulator, so storing from registers makes the 32 lanes of a warp write 32 different lines per instruction
     // (4 us for the 128 KB of a tile).  Each warp stages 32 rows x 128 bytes (16-byte chunks, slot = chunk ^ (row & 7):
-    // conflict-free both ways) in the ring's shared memory -- free by now: every load was consumed by a product that
-    // has completed -- and writes them back 4 rows x 128 bytes per instruction.
+    // conflict-free both ways) in a buffer of its own and writes them back 4 rows x 128 bytes per instruction.
     // Eight epilogue warps: warps 2..5 take the first half of the tile's columns, warps 6..9 the second (two warps
     // per tensor-memory lane quarter).
-    const int eh = (warp - 2) >> 2, c_beg = eh * (nb >> 1), c_end = c_beg + (nb >> 1);
-    const uint32_t stg = smem_u32(smem) + (warp - 2) * 4096;
+    const int eh = (warp - 2) >> 2;
+    const uint32_t stg = smem_u32(staging) + (warp - 2) * 4096;
     const int rr = lane >> 3, slot = lane & 7;   // read-back: rows rr, rr + 4, ...; 16-byte slot of the row
-    if (ok) {
+    RowsTile t;
+    for (int j = 0; rows_tile(g, cta, G, j, t); ++j) {
+      const int b = j & 1;
+      bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ctl->acc_full[b]), (j >> 1) & 1));
+      if (!ok && lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
+      tc_fence_after();
+      ok = ok && (*reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) == 0);
+      if (!ok) break;
+      const int m0 = t.m0, n0 = t.blk0 * kBoxN, split = t.split;
+      const int m = m0 + q * 32 + lane;             // this thread's row
+      const bool row_ok = m < g.M;
+      const uint32_t tacc = taddr + b * kTileN;
+      float best = -INFINITY;
+      int best_n = 0;
+      const int c_beg = eh * (t.nb >> 1), c_end = c_beg + (t.nb >> 1);
+      // (the sums are out of tensor memory when a warp has read its last columns)
+      auto read_done = [&](int c_next) {
+        if (c_next < c_end) return;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+      };
       if constexpr (EPI != EPI_SWIGLU) {
         for (int c0 = c_beg; c0 < c_end; c0 += 32) {
           uint32_t r[32];
-          if (nkb > 0) {
-            tmem_ld16(taddr + c0, *reinterpret_cast<uint32_t(*)[16]>(r));     // (warp-wide: rows past the end read too)
-            tmem_ld16(taddr + c0 + 16, *reinterpret_cast<uint32_t(*)[16]>(r + 16));
-            tmem_wait_ld();
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) r[j] = 0u;
-          }
+          tmem_ld16(tacc + c0, *reinterpret_cast<uint32_t(*)[16]>(r));     // (warp-wide: rows past the end read too)
+          tmem_ld16(tacc + c0 + 16, *reinterpret_cast<uint32_t(*)[16]>(r + 16));
+          tmem_wait_ld();
+          read_done(c0 + 32);
           const int n = n0 + c0;
           if constexpr (EPI == EPI_LOGITS) {
             if (row_ok) {
@@ -235,13 +281,9 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
 #pragma unroll
           for (int part = 0; part < 4; ++part) {
             uint32_t r[16];
-            if (nkb > 0) {
-              tmem_ld16(taddr + c0 + part * 16, r);
-              tmem_wait_ld();
-            } else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) r[j] = 0u;
-            }
+            tmem_ld16(tacc + c0 + part * 16, r);
+            tmem_wait_ld();
+            if (part == 3) read_done(c0 + 64);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               __nv_bfloat16 h0, l0, h1, l1;
@@ -286,13 +328,13 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTileN);
+    tmem_dealloc(tmem_base, 2 * kTileN);
   }
   if (threadIdx.x == 0 && g.stamp) stamp_max(g.stamp + 3);
 }
 
 static size_t rows_smem_bytes(int stages, int planes) {
-  return (size_t)stages * (planes * kRowsM * kBlockK * 2 + 2 * kBoxBytes) + sizeof(RowsSmemCtl) + 1024;
+  return (size_t)stages * (planes * kRowsM * kBlockK * 2 + 2 * kBoxBytes) + kStagingBytes + sizeof(RowsSmemCtl) + 1024;
 }
 
 template <int EPI>
@@ -320,36 +362,36 @@ static cudaError_t launch_rows_one(const CUtensorMap &tw, const CUtensorMap &ta,
 
 int gemm_rows_tiles(int N) { return (N + kTileN - 1) / kTileN; }
 
-// How many of a projection's `blocks` stored weight blocks go into 256-row tiles (two blocks) when the launch has
-// `chunks` row chunks and one CTA per SM: the rest become 128-row tiles, launched last.  A 128-row tile costs about
-// 0.6 of a 256-row one (half the flops, three quarters of the bytes through shared memory).  The CTAs start in launch
-// order on whichever SM frees up first; the count with the shortest finish wins, ties go to fewer narrow tiles.
-static int pick_wide_tiles(int blocks, int chunks, int n_sms) {
+// How a launch's tiles are dealt out (see rows_tile).  A launch that is not cut along K mixes tile widths: a narrow tile
+// costs about 0.6 of a wide one (half the flops, three quarters of the bytes through shared memory), and with the last
+// tiles narrow the CTAs end closer together.  The count of wide tiles, and how many narrow ones go to the CTAs that have
+// one wide tile less, with the earliest finish win; ties go to fewer narrow tiles.
+static constexpr double kNarrowCost = 0.6;
+struct Deal { int n_wide, narrow_short; };
+static Deal pick_deal(int blocks, int chunks, int splits, int G, bool mix) {
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int>, int> memo;
+  static std::map<std::tuple<int, int, int, int, bool>, Deal> memo;   // (a pure function of its key: shapes and SM count)
   std::lock_guard<std::mutex> lk(mu);
-  const auto key = std::make_tuple(blocks, chunks, n_sms);
+  const auto key = std::make_tuple(blocks, chunks, splits, G, mix);
   auto it = memo.find(key);
   if (it != memo.end()) return it->second;
-  const int x_max = blocks / 2;
-  int best_x = x_max;
+  Deal best{blocks / 2, 0};
   double best_t = 1e30;
-  std::vector<double> sm(n_sms);
-  for (int x = x_max; x >= 0 && x >= x_max - 2 * n_sms / chunks; --x) {
-    std::fill(sm.begin(), sm.end(), 0.0);
-    std::make_heap(sm.begin(), sm.end(), std::greater<double>());
-    const int tiles = x + (blocks - 2 * x);
-    for (int t = 0; t < tiles; ++t)
-      for (int c = 0; c < chunks; ++c) {
-        std::pop_heap(sm.begin(), sm.end(), std::greater<double>());
-        sm.back() += t < x ? 1.0 : 0.6;
-        std::push_heap(sm.begin(), sm.end(), std::greater<double>());
-      }
-    const double finish = *std::max_element(sm.begin(), sm.end());
-    if (finish < best_t - 1e-9) { best_t = finish; best_x = x; }
+  const int x_max = blocks / 2, x_min = mix ? std::max(0, x_max - 2 * G / chunks) : x_max;
+  for (int x = x_max; x >= x_min; --x) {
+    const int nW = x * chunks * splits, nN = (blocks - 2 * x) * chunks * splits, r = nW % G, S = G - r;
+    // ns narrow tiles over S CTAs from the start of the last round, the others over r CTAs one wide tile later
+    double t_x = 1e30;
+    int ns_x = nN;
+    for (int ns = r ? 0 : nN; ns <= nN; ++ns) {
+      const double t = std::max(kNarrowCost * ((ns + S - 1) / S), r ? 1.0 + kNarrowCost * ((nN - ns + r - 1) / r) : 0.0);
+      if (t < t_x - 1e-9) { t_x = t; ns_x = ns; }
+    }
+    t_x += nW / G;
+    if (t_x < best_t - 1e-9) { best_t = t_x; best = {x, ns_x}; }
   }
-  memo[key] = best_x;
-  return best_x;
+  memo[key] = best;
+  return best;
 }
 
 // `ta` must be the activation map whose box holds 128 rows.  N must be a multiple of 128.
@@ -361,10 +403,16 @@ cudaError_t launch_gemm_rows(int epi, const CUtensorMap &tw, const CUtensorMap &
   while (g.stages > 2 && rows_smem_bytes(g.stages, g.planes) > smem_limit) --g.stages;
   const size_t smem = rows_smem_bytes(g.stages, g.planes);
   if (smem > smem_limit) return cudaErrorInvalidConfiguration;
-  const int blocks = g.N / kBoxN, chunks = (g.M + kRowsM - 1) / kRowsM;
-  // split-K launches are already cut to fill their waves; the others may mix tile widths
-  g.n_wide = n_splits > 1 ? blocks / 2 : pick_wide_tiles(blocks, chunks, n_sms);
-  dim3 grid(chunks, g.n_wide + (blocks - 2 * g.n_wide), n_splits);
+  const int blocks = g.N / kBoxN;
+  g.chunks = (g.M + kRowsM - 1) / kRowsM;
+  g.n_splits = n_splits;
+  // split-K launches are already cut to fill their rounds; the others may mix tile widths
+  const bool mix = n_splits == 1;
+  const int G = mix ? n_sms : std::min(n_sms, (blocks + 1) / 2 * g.chunks * n_splits);
+  const Deal deal = pick_deal(blocks, g.chunks, n_splits, G, mix);
+  g.n_wide = deal.n_wide;
+  g.narrow_short = deal.narrow_short;
+  dim3 grid(G);
   switch (epi) {
     case EPI_PARTIAL: return launch_rows_one<EPI_PARTIAL>(tw, ta, g, grid, smem, st, pdl);
     case EPI_SWIGLU: return launch_rows_one<EPI_SWIGLU>(tw, ta, g, grid, smem, st, pdl);

@@ -56,7 +56,9 @@ struct GemmArgs {
   int n_kblocks;        // K / 64
   int kb_per_split;     // k-blocks per split-K slice
   int stages;           // filled in by the launcher
-  int n_wide;           // many-rows kernel: weight tiles of 256 rows (the tiles after them have 128); filled in by the launcher
+  // many-rows kernel, filled in by the launcher: weight tiles of 256 rows (the tiles after them have 128), narrow tiles of the
+  // CTAs with one wide tile less, row chunks, K slices
+  int n_wide, narrow_short, chunks, n_splits;
   float *out;           // EPI_PARTIAL: [splits][out_rows][N]; EPI_LOGITS: [M][N]
   int out_rows;
   __nv_bfloat16 *act_out;  // EPI_SWIGLU: [out_planes][act_rows][N/2]

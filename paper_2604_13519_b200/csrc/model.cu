@@ -351,12 +351,10 @@ int pick_cluster(const ts_model *m, int n_tiles, int n_kblocks) {
   return best;
 }
 
-// split-K factor of the many-rows kernel (one CTA per SM, 128 x 256 output tile per CTA).  A CTA there costs about
-// 13 k-blocks' worth of time besides its k-blocks (set-up, the first loads, 128 KB of partial sums written out), and
+// split-K factor of the many-rows kernel (128 x 256 output tiles dealt out to one CTA per SM).  Besides its k-blocks a launch
+// costs about 11 k-blocks' worth of time (set-up, first loads, the last tile's epilogue), every further tile of a CTA two, and
 // every slice adds a slab of partial sums that the next kernel reads back: take the factor with the smallest
-//   waves * (k-blocks per CTA + 13) + 2.5 * slices
-// (measured on the 8B shape with 256 rows: 9 slices of 7 k-blocks in two waves took 29.5 us for the O projection,
-// 4 slices of 16 in one wave 21 us, and the norm after it reads 4 slabs instead of 9).
+//   rounds * (k-blocks per tile + 2) + 2.5 * slices
 int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks, bool allow, int room) {
   if (!allow) return 1;
   const int ctas = std::max(1, n_tiles * m_chunks);
@@ -365,7 +363,7 @@ int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks
   double best_cost = 1e30;
   for (int s = 1; s <= s_max; ++s) {
     const int waves = (ctas * s + m->n_sms - 1) / m->n_sms;
-    const double cost = waves * ((double)n_kblocks / s + 13.0) + 2.5 * s;
+    const double cost = waves * ((double)n_kblocks / s + 2.0) + 2.5 * s;
     if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
   }
   return best;
