@@ -251,20 +251,26 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t stg = smem_u32(smem);
-    for (int c0 = 0; c0 < g.Mc; c0 += 8) {        // (columns past the step's last row are read too and never used)
+    // (columns past the step's last row are read too and never used)
+    auto put = [&](int c, uint32_t lo, uint32_t hi) {
+      st_shared_f32(stg + (c * kTileN + q * 32 + lane) * 4, __uint_as_float(lo) + (g.planes == 2 ? __uint_as_float(hi) : 0.f));
+    };
+    int c0 = 0;
+    for (; c0 + 16 <= g.Mc; c0 += 16) {
+      uint32_t r[16], r2[16];
+      tmem_ld16(taddr + c0, r);
+      if (g.planes == 2) tmem_ld16(taddr + g.Mc + c0, r2);
+      tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < 16; ++j) put(c0 + j, r[j], r2[j]);
+    }
+    if (c0 < g.Mc) {
       uint32_t r[8], r2[8];
-      if (nkb > 0) {
-        tmem_ld8(taddr + c0, r);
-        if (g.planes == 2) tmem_ld8(taddr + g.Mc + c0, r2);
-        tmem_wait_ld();
-      } else {
+      tmem_ld8(taddr + c0, r);
+      if (g.planes == 2) tmem_ld8(taddr + g.Mc + c0, r2);
+      tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) r[j] = r2[j] = 0u;
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        st_shared_f32(stg + ((c0 + j) * kTileN + q * 32 + lane) * 4,
-                      __uint_as_float(r[j]) + (g.planes == 2 ? __uint_as_float(r2[j]) : 0.f));
+      for (int j = 0; j < 8; ++j) put(c0 + j, r[j], r2[j]);
     }
     if constexpr (kCluster) {
       __syncwarp();
