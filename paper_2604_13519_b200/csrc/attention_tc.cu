@@ -42,6 +42,7 @@ static constexpr int kAttnBlk = 64;     // kv positions per block
 __host__ __device__ constexpr int kv_stages(int hd) { return hd == 64 ? 12 : 6; }
 static constexpr int kMaxKvStages = 12;
 static constexpr int kTcThreads = 320;
+static constexpr int kStageBytes = 2048;   // per worker warp: 32 query rows x 64 bytes on their way to a row per thread (head_dim 64)
 static constexpr int kWorkerWarps = 8, kProducerWarp = 8, kMmaWarp = 9;
 
 struct __align__(16) AttnCtl {
@@ -129,7 +130,7 @@ __device__ __forceinline__ uint32_t pack_h2(float x, float y) {
 // output sums.  `cnt` counts this group's blocks over all units of this CTA (barrier parities come from it).
 template <int HD>
 __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *ctl, const UnitInfo &t, uint32_t tmem_base,
-                                                  int grp, int q, int lane, uint32_t &cnt, bool &waited, const int *err) {
+                                                  int grp, int q, int lane, uint32_t stg, uint32_t &cnt, bool &waited, const int *err) {
   const int row = q * 32 + lane;      // row of the tile
   const int pr = t.row0 + row;        // packed row of the sequence
   const bool valid = row < t.rows_here;
@@ -137,6 +138,20 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
   const size_t ob = ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * a.n_slots + t.slot;
   // (a step input like the unit tables: read before the dependency wait)
   const unsigned long long anc = ((unsigned long long)a.in.anc[2 * (t.r_beg + j) + 1] << 32) | a.in.anc[2 * (t.r_beg + j)];
+  // head_dim 64: the queries come through a staging buffer per warp, 64 bytes of each of 32 rows at a time, so that a load
+  // instruction touches eight rows in 64-byte pieces instead of 32 rows in 32-byte ones (1B shape, steps of 8 and 33 rows:
+  // 748 -> 739 us, 967 -> 951; at head_dim 128 the loads of a thread's own row are as quick, and the staging's registers
+  // spill).  This lane's part: rows 8 p + lane / 4 of the warp's 32 (their (row, query head) number, or -1), 16-byte piece
+  // lane % 4.  Row r's piece s lies at slot s ^ (r / 2 % 4): no bank conflicts either way.
+  constexpr bool kStaged = HD == 64;
+  int rq[4];
+  if constexpr (kStaged) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const int R = q * 32 + 8 * p + (lane >> 2), x = t.row0 + R;
+      rq[p] = R < t.rows_here ? (t.r_beg + x / t.G) * a.Hq + t.kh * t.G + x % t.G : -1;
+    }
+  }
   // the rotated queries come from the previous kernel; everything above was on the device before the step began
   if (!waited) {
     pdl_wait();
@@ -153,23 +168,53 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
   // scores when they met at its end), so the columns may be overwritten.
   const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16);
   {
-    const __half *src = (grp ? a.q_lo : a.q) + ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * HD;
-    // all loads are issued before the first use: one round trip to L2, where the previous kernel has just written the
-    // rows (32 bytes per lane and load: the lanes of a warp read 32 different rows)
-    uint32_t v[HD / 2];
-    if (valid) {
+    // (either way all loads are issued before the first use: one round trip to L2)
+    if constexpr (kStaged) {
+      const __half *src = grp ? a.q_lo : a.q;
+      const int piece = lane & 3;
+      auto slot_of = [&](int r, int s) { return (uint32_t)((s ^ ((r >> 1) & 3)) << 4); };
+      uint4 v[HD / 32][4];
 #pragma unroll
-      for (int c = 0; c < HD / 16; ++c) ld_global_v8(src + c * 16, &v[c * 8]);
+      for (int c = 0; c < HD / 32; ++c)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+          v[c][p] = rq[p] >= 0 ? *reinterpret_cast<const uint4 *>(src + (size_t)rq[p] * HD + c * 32 + piece * 8) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int c = 0; c < HD / 32; ++c) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const int R = 8 * p + (lane >> 2);
+          st_shared_v4(stg + R * 64 + slot_of(R, piece), v[c][p].x, v[c][p].y, v[c][p].z, v[c][p].w);
+        }
+        __syncwarp();
+        uint32_t r[16];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const uint4 w = ld_shared_v4(stg + lane * 64 + slot_of(lane, s));
+          r[4 * s] = w.x; r[4 * s + 1] = w.y; r[4 * s + 2] = w.z; r[4 * s + 3] = w.w;
+        }
+        __syncwarp();
+        tmem_st16(tq + kColQ + grp * (HD / 2) + c * 16, r);
+      }
     } else {
+      const __half *src = (grp ? a.q_lo : a.q) + ((size_t)(t.r_beg + j) * a.Hq + t.kh * t.G + gq) * HD;
+      // all loads are issued before the first use: one round trip to L2, where the previous kernel has just written the
+      // rows (32 bytes per lane and load: the lanes of a warp read 32 different rows)
+      uint32_t v[HD / 2];
+      if (valid) {
 #pragma unroll
-      for (int c = 0; c < HD / 2; ++c) v[c] = 0u;
-    }
+        for (int c = 0; c < HD / 16; ++c) ld_global_v8(src + c * 16, &v[c * 8]);
+      } else {
 #pragma unroll
-    for (int c4 = 0; c4 < HD / 32; ++c4) {
-      uint32_t r[16];
+        for (int c = 0; c < HD / 2; ++c) v[c] = 0u;
+      }
 #pragma unroll
-      for (int e = 0; e < 16; ++e) r[e] = v[c4 * 16 + e];
-      tmem_st16(tq + kColQ + grp * (HD / 2) + c4 * 16, r);
+      for (int c4 = 0; c4 < HD / 32; ++c4) {
+        uint32_t r[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) r[e] = v[c4 * 16 + e];
+        tmem_st16(tq + kColQ + grp * (HD / 2) + c4 * 16, r);
+      }
     }
     tmem_wait_st();
   }
@@ -501,7 +546,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
     bool ok = true, waited = false;
     for (int u = u_beg; u < u_end && ok; ++u) {
       const UnitInfo t = attn_unit_info(a, u);
-      ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp >> 2, warp & 3, lane, cnt, waited, err);
+      ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp >> 2, warp & 3, lane, smem_u32(ctl + 1) + warp * kStageBytes, cnt, waited, err);
     }
     if (!waited) pdl_wait();
   }
@@ -628,7 +673,7 @@ cudaError_t launch_attention_tc_merge(const AttnTcArgs &a, cudaStream_t st) {
 }
 
 static size_t attn_tc_smem(int hd) {
-  return 1024 + (size_t)kv_stages(hd) * 2 * kAttnBlk * hd * 2 + sizeof(AttnCtl) + 64;
+  return 1024 + (size_t)kv_stages(hd) * 2 * kAttnBlk * hd * 2 + sizeof(AttnCtl) + (hd == 64 ? kWorkerWarps * kStageBytes : 0) + 64;
 }
 
 cudaError_t launch_attention_tc(const AttnTcArgs &a, cudaStream_t st) {
