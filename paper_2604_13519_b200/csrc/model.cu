@@ -60,6 +60,15 @@ constexpr int kMaxFusedCtas = 256;   // the fused kernel runs one CTA per SM
 constexpr int kFusedMaxRows = 64;    // most rows per step the fused kernel takes
 constexpr bool kAutoPrefersFused = false;   // path = 0 picks the faster of the two on the 8B batch-1 step
 
+// Where a step's integer inputs lie (int32 offsets inside d_in / h_in).  Sized by what kind of step it is, since all up to the
+// used part of the block table is copied every time: with 1024-row arrays in every step that was 45 KB to copy instead of 3
+// (two-layer shape 78.9 -> 78.0 us a step, 1B shape 8 rows 769.7 -> 766.1).
+struct StepIo {
+  int o_tokens, o_pos, o_rowseq, o_cu, o_len, o_tile_seq, o_tile_row0, o_tile128_seq, o_tile128_row0, o_row_tile, o_tile_slots,
+      o_cta_unit, o_parent, o_anc, o_uni, o_slot, o_btab;
+  int max_units, ints;
+};
+
 struct Layout {
   // weights buffer (byte offsets)
   uint64_t embed, lm_head, gf;
@@ -72,11 +81,9 @@ struct Layout {
   // fused single-kernel path
   uint64_t maps, slab, ss_part, sync, phase_t, stamps;
   int max_stamps;
-  int n_maps, n_counters, n_phases, max_tiles128, o_tile128_seq, o_tile128_row0;
-  int max_units, max_ctas, o_row_tile, o_tile_slots, o_cta_unit;   // attention units (see AttnTcArgs)
-  // step io (int32 offsets inside d_in / h_in)
-  int o_tokens, o_pos, o_rowseq, o_cu, o_len, o_tile_seq, o_tile_row0, o_btab, in_ints;
-  int o_parent, o_anc, o_path, o_uni, o_topk, o_slot;
+  int n_maps, n_counters, n_phases;
+  StepIo step_io, prompt_io;   // of a verification step, of a piece of a prompt
+  int in_ints, o_path, o_topk;
   uint64_t samp_stats, topk_cand;
   // step out (int32 offsets)
   int o_argmax, o_accept, o_emitted, o_newlen, o_newpend, o_err, out_ints;
@@ -138,7 +145,6 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->rows_alloc = std::max(L->step_rows_alloc, (int)align_up(L->prefill_rows, 128));
   L->part_rows = std::max(kMaxSplits * L->step_rows_alloc, kPrefillSplits * L->rows_alloc);      // split-K slabs x rows
   L->slot_rows = std::max(kMaxAttnSplits * L->step_rows_alloc, kPrefillSlots * L->rows_alloc);   // attention slots x rows
-  const int io_rows = std::max(c.max_rows, L->prefill_rows), io_seqs = std::max(c.max_batch, (L->prefill_rows + 63) / 64);
   L->pages_per_seq = (c.max_ctx + TS_PAGE_SIZE - 1) / TS_PAGE_SIZE;
   const int G = c.n_q_heads / c.n_kv_heads;
   L->max_tiles = c.max_batch * ((c.k_max * G + 63) / 64);
@@ -161,23 +167,29 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->rope = take((uint64_t)c.max_ctx * (hd / 2) * 8);
   int io = 0;
   auto itake = [&](int n) { int r = io; io += (n + 3) / 4 * 4; return r; };
-  L->o_tokens = itake(io_rows); L->o_pos = itake(io_rows); L->o_rowseq = itake(io_rows);
-  L->o_cu = itake(io_seqs + 1); L->o_len = itake(io_seqs);
-  L->o_tile_seq = itake(L->max_tiles); L->o_tile_row0 = itake(L->max_tiles);
-  const int prefill_tiles = (L->prefill_rows + 63) / 64 * ((64 * G + 127) / 128);
-  L->max_tiles128 = std::max(c.max_batch * ((c.k_max * G + 127) / 128), prefill_tiles);
-  L->o_tile128_seq = itake(L->max_tiles128); L->o_tile128_row0 = itake(L->max_tiles128);
-  // (units: at most kMaxAttnSplits per tile and kv head, see build_attention)
-  L->max_units = L->max_tiles128 * c.n_kv_heads * kMaxAttnSplits;
-  L->max_ctas = kMaxFusedCtas;
-  L->o_row_tile = itake(io_rows);
-  L->o_tile_slots = itake(L->max_tiles128 * c.n_kv_heads);
-  L->o_cta_unit = itake(L->max_ctas + 1);
-  L->o_parent = itake(io_rows); L->o_anc = itake(2 * io_rows); L->o_uni = itake(io_rows);
-  L->o_slot = itake(io_rows);
-  // (last, only the used part is copied per step: the block table, and behind its used rows the attention units)
-  L->o_btab = itake(c.max_batch * L->pages_per_seq + L->max_units * (int)(sizeof(ts::AttnWork) / 4));
-  L->in_ints = io;
+  auto lay_out = [&](StepIo &I, int rows, int seqs, int tables, int tiles64, int tiles128) {
+    io = 0;
+    I.o_tokens = itake(rows); I.o_pos = itake(rows); I.o_rowseq = itake(rows);
+    I.o_cu = itake(seqs + 1); I.o_len = itake(seqs);
+    I.o_tile_seq = itake(tiles64); I.o_tile_row0 = itake(tiles64);
+    I.o_tile128_seq = itake(tiles128); I.o_tile128_row0 = itake(tiles128);
+    // units (see build_attention): steps of at most 64 rows have at most kMaxAttnSplits per tile and kv head, and few tiles;
+    // larger ones one per tile and kv head and one more per CTA
+    const int few_tiles = std::min(tiles128, 64 * G / 128 + 1 + std::min(seqs, 64));
+    I.max_units = std::max(few_tiles * kMaxAttnSplits, tiles128 + kMaxFusedCtas / c.n_kv_heads + 1) * c.n_kv_heads;
+    I.o_row_tile = itake(rows);
+    I.o_tile_slots = itake(tiles128 * c.n_kv_heads);
+    I.o_cta_unit = itake(kMaxFusedCtas + 1);
+    I.o_parent = itake(rows); I.o_anc = itake(2 * rows); I.o_uni = itake(rows);
+    I.o_slot = itake(rows);
+    // (last, only the used part is copied per step: the block table, and behind its used rows the attention units)
+    I.o_btab = itake(tables * L->pages_per_seq + I.max_units * (int)(sizeof(ts::AttnWork) / 4));
+    I.ints = io;
+  };
+  lay_out(L->step_io, c.max_rows, c.max_batch, c.max_batch, L->max_tiles, c.max_batch * ((c.k_max * G + 127) / 128));
+  const int pieces = (L->prefill_rows + 63) / 64;
+  lay_out(L->prompt_io, L->prefill_rows, pieces, 1, 1, pieces * ((64 * G + 127) / 128));
+  L->in_ints = std::max(L->step_io.ints, L->prompt_io.ints);
   io = 0;
   L->o_argmax = itake(c.max_rows); L->o_accept = itake(c.max_batch); L->o_emitted = itake(c.max_batch * c.k_max);
   L->o_newlen = itake(c.max_batch); L->o_newpend = itake(c.max_batch); L->o_err = itake(4);
@@ -275,6 +287,7 @@ struct ts_model {
 
   uint8_t *W(uint64_t off) const { return (uint8_t *)b.weights + off; }
   uint8_t *WS(uint64_t off) const { return (uint8_t *)b.workspace + off; }
+  const StepIo &io() const { return last_ready >= 0 ? L.prompt_io : L.step_io; }   // of the last step
   int32_t *h_in() const { return (int32_t *)b.host_io; }
   int32_t *h_out() const { return (int32_t *)b.host_io + L.in_ints; }
   int32_t *d_in() const { return (int32_t *)WS(L.d_in); }
@@ -405,6 +418,7 @@ ts_status run_gemm_ws(ts_model *m, int epi, const CUtensorMap &tw, const CUtenso
 
 // The staged step as one persistent kernel (fused.cu).
 ts_status run_step_fused(ts_model *m) {
+  const StepIo &I = m->io();
   const ts_model_config &c = m->c;
   const Layout &L = m->L;
   int32_t *di = m->d_in();
@@ -412,10 +426,10 @@ ts_status run_step_fused(ts_model *m) {
   ts::FusedArgs a{};
   a.n_layers = c.n_layers; a.d = c.d_model; a.Nqkv = L.Nqkv; a.Nq = c.n_q_heads * c.head_dim; a.F = c.d_ffn;
   a.V = c.vocab; a.Hq = c.n_q_heads; a.Hkv = c.n_kv_heads; a.hd = c.head_dim; a.eps = c.rms_eps;
-  a.in.tokens = di + L.o_tokens; a.in.pos = di + L.o_pos; a.in.row_seq = di + L.o_rowseq; a.in.cu_rows = di + L.o_cu;
-  a.in.seq_len = di + L.o_len; a.in.block_tab = di + L.o_btab; a.in.pages_per_seq = L.pages_per_seq;
-  a.in.parent = di + L.o_parent; a.in.anc = (const uint32_t *)(di + L.o_anc); a.in.slot = di + L.o_slot;
-  a.in.row_tile = di + L.o_row_tile;
+  a.in.tokens = di + I.o_tokens; a.in.pos = di + I.o_pos; a.in.row_seq = di + I.o_rowseq; a.in.cu_rows = di + I.o_cu;
+  a.in.seq_len = di + I.o_len; a.in.block_tab = di + I.o_btab; a.in.pages_per_seq = L.pages_per_seq;
+  a.in.parent = di + I.o_parent; a.in.anc = (const uint32_t *)(di + I.o_anc); a.in.slot = di + I.o_slot;
+  a.in.row_tile = di + I.o_row_tile;
   a.in.B = m->last_B; a.in.M = m->last_M;
   a.mc_index = m->last_M <= 16 ? 0 : (m->last_M <= 32 ? 1 : 2); a.Mc = kMcOptions[kFusedMc[a.mc_index]]; a.planes = m->planes;
   a.n_ctas = m->n_sms; a.skip_lm = (m->last_flags & TS_FLAG_SKIP_LM_HEAD) ? 1 : 0;
@@ -426,13 +440,13 @@ ts_status run_step_fused(ts_model *m) {
     // number of rows verified)
     int max_total = 0;
     const int32_t *hi = m->h_in();
-    for (int i = 0; i < m->last_B; ++i) max_total = std::max(max_total, hi[L.o_len + i] + c.k_max);
+    for (int i = 0; i < m->last_B; ++i) max_total = std::max(max_total, hi[I.o_len + i] + c.k_max);
     const int nblk = (max_total + 63) / 64;
     const int G = c.n_q_heads / c.n_kv_heads;
     const int s = m->n_sms / std::max(1, c.n_kv_heads * m->last_B * ((c.k_max * G + 127) / 128));
     a.attn_splits = std::max(1, std::min(std::min(s, kMaxAttnSplits), nblk));
   }
-  a.tile_seq = di + L.o_tile128_seq; a.tile_row0 = di + L.o_tile128_row0;
+  a.tile_seq = di + I.o_tile128_seq; a.tile_row0 = di + I.o_tile128_row0;
   a.maps = (const CUtensorMap *)m->WS(L.maps);
   a.map_kv = L.n_maps - 1;
   a.embed = (const __nv_bfloat16 *)m->W(L.embed);
@@ -456,6 +470,7 @@ ts_status run_step_fused(ts_model *m) {
 }
 
 ts_status run_step(ts_model *m) {
+  const StepIo &I = m->io();
   if (m->last_fused) return run_step_fused(m);
   const ts_model_config &c = m->c;
   const Layout &L = m->L;
@@ -463,10 +478,10 @@ ts_status run_step(ts_model *m) {
   const int d = c.d_model, F = c.d_ffn, Nq = c.n_q_heads * c.head_dim;
   ts::StepIn in{};
   int32_t *di = m->d_in();
-  in.tokens = di + L.o_tokens; in.pos = di + L.o_pos; in.row_seq = di + L.o_rowseq; in.cu_rows = di + L.o_cu;
-  in.seq_len = di + L.o_len; in.block_tab = di + L.o_btab; in.pages_per_seq = m->last_ready >= 0 ? 0 : L.pages_per_seq;
-  in.parent = di + L.o_parent; in.anc = (const uint32_t *)(di + L.o_anc); in.slot = di + L.o_slot;
-  in.row_tile = di + L.o_row_tile;
+  in.tokens = di + I.o_tokens; in.pos = di + I.o_pos; in.row_seq = di + I.o_rowseq; in.cu_rows = di + I.o_cu;
+  in.seq_len = di + I.o_len; in.block_tab = di + I.o_btab; in.pages_per_seq = m->last_ready >= 0 ? 0 : L.pages_per_seq;
+  in.parent = di + I.o_parent; in.anc = (const uint32_t *)(di + I.o_anc); in.slot = di + I.o_slot;
+  in.row_tile = di + I.o_row_tile;
   in.B = B; in.M = M;
   in.ck.err = m->d_out() + L.o_err; in.ck.vocab = c.vocab; in.ck.max_pages = c.max_pages; in.ck.max_ctx = c.max_ctx;
   float *x = (float *)m->WS(L.x);
@@ -481,7 +496,7 @@ ts_status run_step(ts_model *m) {
   ts::AttnArgs aa{};
   aa.in = in; aa.q = q; aa.Hq = c.n_q_heads; aa.Hkv = c.n_kv_heads; aa.hd = c.head_dim;
   aa.n_row_tiles_total = m->last_tiles;
-  aa.tile_seq = di + L.o_tile_seq; aa.tile_row0 = di + L.o_tile_row0;
+  aa.tile_seq = di + I.o_tile_seq; aa.tile_row0 = di + I.o_tile_row0;
   aa.part_o = (float *)m->WS(L.attn_o); aa.part_ml = (float2 *)m->WS(L.attn_ml);
   aa.out = attn; aa.out_rows = R; aa.planes = m->planes;
   {
@@ -489,7 +504,7 @@ ts_status run_step(ts_model *m) {
     int max_total = 0;
     const int32_t *hi = m->h_in();
     for (int i = 0; i < B; ++i)
-      max_total = std::max(max_total, hi[L.o_len + i] + (hi[L.o_cu + i + 1] - hi[L.o_cu + i]));
+      max_total = std::max(max_total, hi[I.o_len + i] + (hi[I.o_cu + i + 1] - hi[I.o_cu + i]));
     const int nblk = (max_total + 63) / 64;
     int s = (2 * m->n_sms + c.n_kv_heads * m->last_tiles - 1) / (c.n_kv_heads * m->last_tiles);
     aa.n_splits = std::max(1, std::min(std::min(s, kMaxAttnSplits), nblk));
@@ -498,7 +513,7 @@ ts_status run_step(ts_model *m) {
   ts::AttnTcArgs at{};
   at.in = in; at.Hq = c.n_q_heads; at.Hkv = c.n_kv_heads; at.hd = c.head_dim;
   at.n_ctas = m->last_ctas; at.n_slots = m->last_slots; at.ready_len = m->last_ready;
-  at.units = (const ts::AttnWork *)(di + m->last_units_at); at.cta_unit = di + L.o_cta_unit; at.tile_slots = di + L.o_tile_slots;
+  at.units = (const ts::AttnWork *)(di + m->last_units_at); at.cta_unit = di + I.o_cta_unit; at.tile_slots = di + I.o_tile_slots;
   at.q = q; at.q_lo = q + (size_t)R * Nq; at.map_kv = (const CUtensorMap *)m->WS(L.maps) + (L.n_maps - 1);
   at.attn_o = aa.part_o; at.attn_ml = aa.part_ml; at.err = m->d_out() + L.o_err;
   at.out = attn; at.out_rows = R; at.planes = m->planes;
@@ -606,7 +621,7 @@ ts_status run_step(ts_model *m) {
   if (m->last_sample) {
     ts::SampleArgs sa{};
     sa.in = in; sa.logits = (float *)m->WS(L.logits); sa.amax = amax;
-    sa.uni = (const float *)(di + L.o_uni); sa.part = (float *)m->WS(L.samp_stats);
+    sa.uni = (const float *)(di + I.o_uni); sa.part = (float *)m->WS(L.samp_stats);
     sa.V = c.vocab; sa.inv_t = m->last_inv_t; sa.k_max = c.k_max;
     sa.argmax = dout + L.o_argmax; sa.accept_len = dout + L.o_accept; sa.emitted = dout + L.o_emitted;
     sa.new_len = dout + L.o_newlen; sa.new_pending = dout + L.o_newpend; sa.path = dout + L.o_path;
@@ -648,16 +663,15 @@ ts_status ensure_pages(ts_session *s, int tokens) {
 }
 
 // The step inputs of row `r` of the step, a row of sequence i.
-void put_row(ts_model *m, int i, int r, int32_t token, int pos, int slot, int parent, uint64_t mask) {
-  const Layout &L = m->L;
+void put_row(ts_model *m, const StepIo &I, int i, int r, int32_t token, int pos, int slot, int parent, uint64_t mask) {
   int32_t *hi = m->h_in();
-  hi[L.o_tokens + r] = token;
-  hi[L.o_pos + r] = pos;
-  hi[L.o_rowseq + r] = i;
-  hi[L.o_slot + r] = slot;
-  hi[L.o_parent + r] = parent;
-  hi[L.o_anc + 2 * r] = (int32_t)(uint32_t)(mask & 0xFFFFFFFFull);
-  hi[L.o_anc + 2 * r + 1] = (int32_t)(uint32_t)(mask >> 32);
+  hi[I.o_tokens + r] = token;
+  hi[I.o_pos + r] = pos;
+  hi[I.o_rowseq + r] = i;
+  hi[I.o_slot + r] = slot;
+  hi[I.o_parent + r] = parent;
+  hi[I.o_anc + 2 * r] = (int32_t)(uint32_t)(mask & 0xFFFFFFFFull);
+  hi[I.o_anc + 2 * r + 1] = (int32_t)(uint32_t)(mask >> 32);
 }
 uint64_t chain_mask(int j) { return j >= 63 ? ~0ull : ((2ull << j) - 1ull); }
 
@@ -671,27 +685,27 @@ uint64_t chain_mask(int j) { return j >= 63 ? ~0ull : ((2ull << j) - 1ull); }
 // Larger steps (their projections sum in another order anyway): the (tile, kv head) pairs' blocks in one line, cut into
 // equal stretches, one per CTA, a unit's fixed cost counted as kUnitBlocks blocks -- leaves left the SMs unevenly loaded.
 constexpr int kUnitBlocks = 5;   // setting up and draining a unit takes about as long as five 64-position blocks
-ts_status build_attention(ts_model *m, int B, int M, int tables) {
+ts_status build_attention(ts_model *m, const StepIo &I, int B, int M, int tables) {
   const Layout &L = m->L;
   const int Hkv = m->c.n_kv_heads, G = m->c.n_q_heads / Hkv;
   int32_t *hi = m->h_in();
   std::vector<int> order(B);
   for (int i = 0; i < B; ++i) order[i] = i;
-  auto rows_of = [&](int i) { return hi[L.o_cu + i + 1] - hi[L.o_cu + i]; };
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hi[L.o_len + a] + rows_of(a) > hi[L.o_len + b] + rows_of(b); });
-  m->last_units_at = align_up((uint64_t)L.o_btab + (uint64_t)tables * L.pages_per_seq, 4);
+  auto rows_of = [&](int i) { return hi[I.o_cu + i + 1] - hi[I.o_cu + i]; };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hi[I.o_len + a] + rows_of(a) > hi[I.o_len + b] + rows_of(b); });
+  m->last_units_at = align_up((uint64_t)I.o_btab + (uint64_t)tables * L.pages_per_seq, 4);
   ts::AttnWork *units = (ts::AttnWork *)(hi + m->last_units_at);
-  const int cap = std::min(L.max_units, (int)((L.in_ints - m->last_units_at) / (sizeof(ts::AttnWork) / 4)));
-  const int max_ctas = std::min(m->n_sms, L.max_ctas);
+  const int cap = std::min(I.max_units, (int)((L.in_ints - m->last_units_at) / (sizeof(ts::AttnWork) / 4)));
+  const int max_ctas = std::min(m->n_sms, kMaxFusedCtas);
   struct Tile { int seq, row0, rows, blocks, end; };   // blocks: 64-position blocks its rows can see
   std::vector<Tile> tiles;
   for (int i : order) {
-    const int k = rows_of(i), len = hi[L.o_len + i];
-    for (int r = hi[L.o_cu + i]; r < hi[L.o_cu + i + 1]; ++r) hi[L.o_row_tile + r] = 64 * (int)tiles.size() + (r - hi[L.o_cu + i]);
+    const int k = rows_of(i), len = hi[I.o_len + i];
+    for (int r = hi[I.o_cu + i]; r < hi[I.o_cu + i + 1]; ++r) hi[I.o_row_tile + r] = 64 * (int)tiles.size() + (r - hi[I.o_cu + i]);
     for (int r0 = 0; r0 < k * G; r0 += 128) {
       const int rows = std::min(128, k * G - r0), end = len + (r0 + rows - 1) / G + 1;
-      hi[L.o_tile128_seq + tiles.size()] = i;
-      hi[L.o_tile128_row0 + tiles.size()] = r0;
+      hi[I.o_tile128_seq + tiles.size()] = i;
+      hi[I.o_tile128_row0 + tiles.size()] = r0;
       tiles.push_back({i, r0, rows, (end + 63) / 64, end});
     }
   }
@@ -701,7 +715,7 @@ ts_status build_attention(ts_model *m, int B, int M, int tables) {
   auto put = [&](int tile, int kh, int slot, int beg, int end) {
     const Tile &t = tiles[tile];
     if (n < cap)
-      units[n] = {t.seq, hi[L.o_cu + t.seq], t.row0, t.rows, kh | (slot << 16), beg, end, hi[L.o_len + t.seq]};
+      units[n] = {t.seq, hi[I.o_cu + t.seq], t.row0, t.rows, kh | (slot << 16), beg, end, hi[I.o_len + t.seq]};
     ++n;
     slots = std::max(slots, slot + 1);
   };
@@ -709,23 +723,23 @@ ts_status build_attention(ts_model *m, int B, int M, int tables) {
     struct Leaf { int tile, leaf, nblk; };
     std::vector<Leaf> leaves;
     for (int t = 0; t < n_tiles; ++t) {
-      const int total = hi[L.o_len + tiles[t].seq] + rows_of(tiles[t].seq), n_leaves = (total + m->leaf_len - 1) / m->leaf_len;
-      for (int kh = 0; kh < Hkv; ++kh) hi[L.o_tile_slots + t * Hkv + kh] = n_leaves;
+      const int total = hi[I.o_len + tiles[t].seq] + rows_of(tiles[t].seq), n_leaves = (total + m->leaf_len - 1) / m->leaf_len;
+      for (int kh = 0; kh < Hkv; ++kh) hi[I.o_tile_slots + t * Hkv + kh] = n_leaves;
       for (int lf = 0; lf < n_leaves; ++lf) leaves.push_back({t, lf, (std::min(total, (lf + 1) * m->leaf_len) - lf * m->leaf_len + 63) / 64});
     }
     std::stable_sort(leaves.begin(), leaves.end(), [](const Leaf &a, const Leaf &b) { return a.nblk > b.nblk; });
     const int total = (int)leaves.size() * Hkv, ctas = std::min(total, max_ctas);
     for (int c = 0; c < ctas; ++c) {
-      hi[L.o_cta_unit + c] = n;
+      hi[I.o_cta_unit + c] = n;
       for (int j = 0; j * ctas < total; ++j) {
         const int u = j * ctas + ((j & 1) ? ctas - 1 - c : c);
         if (u >= total) continue;
         const Leaf &lf = leaves[u / Hkv];
         const int s = tiles[lf.tile].seq;
-        put(lf.tile, u % Hkv, lf.leaf, lf.leaf * m->leaf_len, std::min((lf.leaf + 1) * m->leaf_len, hi[L.o_len + s] + rows_of(s)));
+        put(lf.tile, u % Hkv, lf.leaf, lf.leaf * m->leaf_len, std::min((lf.leaf + 1) * m->leaf_len, hi[I.o_len + s] + rows_of(s)));
       }
     }
-    hi[L.o_cta_unit + ctas] = n;
+    hi[I.o_cta_unit + ctas] = n;
     m->last_ctas = ctas;
   } else {
     const int slot_cap = std::min(kMaxAttnSplits, L.slot_rows / M);
@@ -740,7 +754,7 @@ ts_status build_attention(ts_model *m, int B, int M, int tables) {
       n = 0; slots = 1;
       int c = 0;
       long long left = share;
-      hi[L.o_cta_unit] = 0;
+      hi[I.o_cta_unit] = 0;
       bool fits = true;
       for (int t = 0; t < n_tiles && fits; ++t)
         for (int kh = 0; kh < Hkv && fits; ++kh) {
@@ -751,7 +765,7 @@ ts_status build_attention(ts_model *m, int B, int M, int tables) {
             if (take < rest && rest - take < kUnitBlocks) take = left >= rest ? rest : rest - kUnitBlocks;   // (no sliver after the cut)
             if (take < rest && take < kUnitBlocks) {   // nor before it
               if (++c >= max_ctas) { fits = false; break; }
-              hi[L.o_cta_unit + c] = n;
+              hi[I.o_cta_unit + c] = n;
               left = share;
               continue;
             }
@@ -760,11 +774,11 @@ ts_status build_attention(ts_model *m, int B, int M, int tables) {
             b += (int)take;
             left -= take + kUnitBlocks;
           }
-          if (fits) hi[L.o_tile_slots + t * Hkv + kh] = slot;
+          if (fits) hi[I.o_tile_slots + t * Hkv + kh] = slot;
         }
       if (fits && slots <= slot_cap) {
         m->last_ctas = c + 1;
-        hi[L.o_cta_unit + c + 1] = n;
+        hi[I.o_cta_unit + c + 1] = n;
         break;
       }
     }
@@ -776,11 +790,12 @@ ts_status build_attention(ts_model *m, int B, int M, int tables) {
 
 // Copies the staged inputs in, runs the step, copies its results back and waits.
 ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
+  const StepIo &I = m->io();
   const ts_model_config &c = m->c;
   const Layout &L = m->L;
   m->last_B = B; m->last_M = M; m->last_flags = flags;
   m->have_step = true;
-  const size_t in_bytes = (m->last_units_at + (size_t)m->h_in()[L.o_cta_unit + m->last_ctas] * (sizeof(ts::AttnWork) / 4)) * 4;
+  const size_t in_bytes = (m->last_units_at + (size_t)m->h_in()[I.o_cta_unit + m->last_ctas] * (sizeof(ts::AttnWork) / 4)) * 4;
   CU_TRY(cudaMemcpyAsync(m->d_in(), m->h_in(), in_bytes, cudaMemcpyHostToDevice, m->st));
   m->h2d += (int64_t)in_bytes;
   // A step that ends in an acceptance kernel (and maybe the cache's compaction) publishes its results itself; prompts, the
@@ -824,10 +839,11 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
                         const float *uniforms = nullptr, float temperature = 0.f) {
   const ts_model_config &c = m->c;
   const Layout &L = m->L;
+  const StepIo &I = L.step_io;
   int32_t *hi = m->h_in();
   const int G = c.n_q_heads / c.n_kv_heads;
   int M = 0, tiles = 0;
-  hi[L.o_cu] = 0;
+  hi[I.o_cu] = 0;
   for (int i = 0; i < B; ++i) {
     ts_session *s = ss[i];
     const int k = (int)rows[i].size();
@@ -856,20 +872,20 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
               return fail(TS_ERR_ARG, "sequence %d: rows %d and %d are children of row %d with the same token", i, e, j, par);
       }
       const uint64_t mask = parents ? anc[j] : chain_mask(j);
-      put_row(m, i, M + j, rows[i][j], s->cache_len + (parents ? depth[j] : j), s->cache_len + j, par, mask);
+      put_row(m, I, i, M + j, rows[i][j], s->cache_len + (parents ? depth[j] : j), s->cache_len + j, par, mask);
     }
-    hi[L.o_len + i] = s->cache_len;
+    hi[I.o_len + i] = s->cache_len;
     for (int r0 = 0; r0 < k * G; r0 += 64) {
-      hi[L.o_tile_seq + tiles] = i;
-      hi[L.o_tile_row0 + tiles] = r0;
+      hi[I.o_tile_seq + tiles] = i;
+      hi[I.o_tile_row0 + tiles] = r0;
       ++tiles;
     }
-    std::memcpy(hi + L.o_btab + (size_t)i * L.pages_per_seq, s->pages.data(), s->pages.size() * sizeof(int32_t));
+    std::memcpy(hi + I.o_btab + (size_t)i * L.pages_per_seq, s->pages.data(), s->pages.size() * sizeof(int32_t));
     M += k;
-    hi[L.o_cu + i + 1] = M;
+    hi[I.o_cu + i + 1] = M;
   }
   {
-    ts_status st = build_attention(m, B, M, B);
+    ts_status st = build_attention(m, I, B, M, B);
     if (st) return st;
   }
   const bool can_fuse = m->fused_ok && M <= kFusedMaxRows;
@@ -885,12 +901,12 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
     m->last_inv_t = 1.f / temperature;
     // the kernel reads uni[node c] for node c and the root's for the draw; a chain's caller gives value j for draft
     // j + 1 and its chunk's last value for the draw
-    float *un = reinterpret_cast<float *>(hi + L.o_uni);
+    float *un = reinterpret_cast<float *>(hi + I.o_uni);
     if (m->last_tree) {
       std::memcpy(un, uniforms, sizeof(float) * M);
     } else {
       for (int i = 0, r = 0; i < B; ++i) {
-        const int k = hi[L.o_cu + i + 1] - hi[L.o_cu + i];
+        const int k = hi[I.o_cu + i + 1] - hi[I.o_cu + i];
         un[r] = uniforms[r + k - 1];
         for (int j = 1; j < k; ++j) un[r + j] = uniforms[r + j - 1];
         r += k;
@@ -911,22 +927,23 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
 ts_status prefill_step(ts_model *m, ts_session *s, const int32_t *tokens, int k) {
   const ts_model_config &c = m->c;
   const Layout &L = m->L;
-  int32_t *hi = m->h_in();
+  const StepIo &I = L.prompt_io;
   const int base = s->cache_len;
+  int32_t *hi = m->h_in();
   if (base + k > c.max_ctx) return fail(TS_ERR_ARG, "sequence 0 would exceed max_ctx");
   for (int j = 0; j < k; ++j)
     if (tokens[j] < 0 || tokens[j] >= c.vocab) return fail(TS_ERR_TOKEN_RANGE, "token id %d outside [0, %d)", tokens[j], c.vocab);
   ts_status st = ensure_pages(s, base + k);
   if (st) return st;
-  std::memcpy(hi + L.o_btab, s->pages.data(), s->pages.size() * sizeof(int32_t));
+  std::memcpy(hi + I.o_btab, s->pages.data(), s->pages.size() * sizeof(int32_t));
   const int B = (k + 63) / 64;
   for (int i = 0; i < B; ++i) {
-    hi[L.o_cu + i] = 64 * i;
-    hi[L.o_len + i] = base + 64 * i;
+    hi[I.o_cu + i] = 64 * i;
+    hi[I.o_len + i] = base + 64 * i;
   }
-  hi[L.o_cu + B] = k;
-  for (int r = 0; r < k; ++r) put_row(m, r >> 6, r, tokens[r], base + r, base + r, (r & 63) - 1, chain_mask(r & 63));
-  st = build_attention(m, B, k, 1);
+  hi[I.o_cu + B] = k;
+  for (int r = 0; r < k; ++r) put_row(m, I, r >> 6, r, tokens[r], base + r, base + r, (r & 63) - 1, chain_mask(r & 63));
+  st = build_attention(m, I, B, k, 1);
   if (st) return st;
   m->last_tree = m->last_sample = m->last_fused = false;
   m->last_tiles = 1;   // (the 64-row tiles of the kernel without tensor memory are not made)
