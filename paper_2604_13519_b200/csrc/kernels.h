@@ -164,11 +164,13 @@ cudaError_t launch_attention_tc_merge(const AttnTcArgs &a, cudaStream_t st);
 
 // A step's results straight to the host: the acceptance kernels write the words of the result block that the host reads to
 // pinned memory as well, so that no copy follows them (base: the block on the device, host: the same block as the device
-// sees the pinned one; host null: not wanted).
+// sees the pinned one; host null: not wanted).  done: a word per sequence in the pinned block, raised when its results are there
+// (null: the host waits for the stream instead).
 struct HostOut {
   const int32_t *base;
   int32_t *host;
   const int *err;   // status word, published too
+  int32_t *done;
 };
 
 // per-row argmax over the LM-head tiles, longest accepted prefix per sequence, new lengths
@@ -203,6 +205,12 @@ struct SampleArgs {
 cudaError_t launch_sample_accept(const SampleArgs &a, cudaStream_t st);
 
 #ifdef __CUDACC__
+// tells the host that what the CTA wrote (before a barrier), and all kernels that it waited for, can be read
+__device__ __forceinline__ void raise_flag(int32_t *flag) {
+  __threadfence_system();
+  *reinterpret_cast<volatile int32_t *>(flag) = 1;
+}
+
 // the results of sequence `seq` (rows r0 .. r0 + k, accepted length l) by the whole CTA, after a barrier
 template <typename Args>
 __device__ __forceinline__ void publish(const Args &a, int seq, int r0, int k, int l) {
@@ -219,6 +227,9 @@ __device__ __forceinline__ void publish(const Args &a, int seq, int r0, int k, i
     put(a.new_pending + seq);
     if (seq == 0) put(a.ho.err);
   }
+  if (!a.ho.done) return;
+  __syncthreads();
+  if (threadIdx.x == 0) raise_flag(a.ho.done + seq);
 }
 #endif
 
@@ -229,7 +240,8 @@ cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float
 
 // Row-wise Top-K (topk.cu): out[r][j] = (column as int bits, value) of the j-th largest entry of row r, lowest column
 // on ties.  cand: scratch of n_rows * ceil(n_cols / 4096) * K pairs.
-// out_host (one row, may be null): the same pairs to host memory that the device can write, and behind them the status word *err.
+// out_host (one row, may be null): the same pairs to host memory that the device can write, and behind them the
+// status word *err and a word that is raised when all of it is there.
 cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, float *out_host,
                              const int *err, cudaStream_t st);
 

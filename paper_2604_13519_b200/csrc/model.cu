@@ -1,6 +1,7 @@
 // Host side of the library: handles, buffer layout, weight upload, the verify step's kernel sequence,
 // sessions (page lists, drafter state) and every extern "C" entry point declared in toolspec.h.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -86,7 +87,7 @@ struct Layout {
   int in_ints, o_path, o_topk;
   uint64_t samp_stats, topk_cand;
   // step out (int32 offsets)
-  int o_argmax, o_accept, o_emitted, o_newlen, o_newpend, o_err, out_ints;
+  int o_argmax, o_accept, o_emitted, o_newlen, o_newpend, o_err, o_done, out_ints;
   int rows_alloc;        // rows of the activation buffers: max_rows or a piece of a prompt, whichever is more
   int step_rows_alloc;   // max_rows rounded up to 128: rows of the logits
   int prefill_rows, part_rows, slot_rows;   // (see make_layout)
@@ -194,6 +195,7 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->o_argmax = itake(c.max_rows); L->o_accept = itake(c.max_batch); L->o_emitted = itake(c.max_batch * c.k_max);
   L->o_newlen = itake(c.max_batch); L->o_newpend = itake(c.max_batch); L->o_err = itake(4);
   L->o_path = itake(c.max_batch * c.k_max);
+  L->o_done = itake(c.max_batch);   // (pinned block only, see wait_results)
   L->o_topk = itake(c.max_rows * TS_TOPK * 2);   // (id bits, value) pairs, written by the Top-K kernel
   L->out_ints = io;
   L->d_in = take((uint64_t)L->in_ints * 4);
@@ -209,7 +211,7 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->max_stamps = 9 * c.n_layers + 16;
   L->stamps = take((uint64_t)L->max_stamps * 4 * 8);
   L->workspace_bytes = o;
-  L->host_io_bytes = align_up((uint64_t)(L->in_ints + L->out_ints + 2 * 64 + 1) * 4, 4096);   // (and a retrieval's result pairs and status)
+  L->host_io_bytes = align_up((uint64_t)(L->in_ints + L->out_ints + 2 * 64 + 2) * 4, 4096);   // (and a retrieval's result pairs, status and flag)
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -617,7 +619,10 @@ ts_status run_step(ts_model *m) {
     m->launched(5);
   }
   ts::HostOut ho{};
-  if (m->publish) { ho.base = dout; ho.host = m->host_dev + L.in_ints; ho.err = dout + L.o_err; }
+  if (m->publish) {
+    ho.base = dout; ho.host = m->host_dev + L.in_ints; ho.err = dout + L.o_err;
+    ho.done = m->last_tree ? nullptr : ho.host + L.o_done;   // (a tree's step ends with the compaction, which publishes nothing)
+  }
   if (m->last_sample) {
     ts::SampleArgs sa{};
     sa.in = in; sa.logits = (float *)m->WS(L.logits); sa.amax = amax;
@@ -788,6 +793,28 @@ ts_status build_attention(ts_model *m, const StepIo &I, int B, int M, int tables
   return TS_OK;
 }
 
+// Waits for n words of the pinned block, cleared before the launches, that the last kernel on the stream raises behind its
+// results; by then all kernels before it are complete and it has nothing left to do.  3.5 us sooner than the stream's own
+// synchronisation, which learns of the kernel's end by way of the driver (ten small kernels in a row: 52.1 -> 48.8 us; the
+// two-layer shape's step 77.1 -> 75.1, a retrieval over 100 000 entries 149.2 -> 147.7).  The stream is still asked from time to time, so that a failed launch or kernel ends the wait with its error.
+cudaError_t wait_results(const int32_t *words, int n, cudaStream_t st) {
+  const volatile int32_t *w = words;
+  for (uint32_t it = 1;; ++it) {
+    while (n > 0 && w[n - 1]) --n;
+    if (n == 0) break;
+    if ((it & 4095u) == 0) {
+      const cudaError_t e = cudaStreamQuery(st);
+      if (e == cudaErrorNotReady) cudaGetLastError();   // (it is kept as the thread's last error)
+      else return e;
+    }
+#if defined(__x86_64__)
+    __builtin_ia32_pause();
+#endif
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  return cudaSuccess;
+}
+
 // Copies the staged inputs in, runs the step, copies its results back and waits.
 ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const StepIo &I = m->io();
@@ -807,6 +834,8 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const bool publishes = m->host_dev && !m->last_fused && !m->inject_err && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
 #endif
   m->publish = publishes;
+  const bool flagged = publishes && !m->last_tree;
+  if (flagged) std::memset(m->h_out() + L.o_done, 0, sizeof(int32_t) * B);
   ts_status st = run_step(m);
   m->publish = false;
   if (st) return st;
@@ -820,7 +849,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
   if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
   m->d2h += (int64_t)out_bytes;
-  CU_TRY(cudaStreamSynchronize(m->st));
+  CU_TRY(flagged ? wait_results(m->h_out() + L.o_done, B, m->st) : cudaStreamSynchronize(m->st));
   const int dev_err = m->h_out()[L.o_err];
   if (dev_err != 0) {
     cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
@@ -1844,13 +1873,14 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
   // the result pairs go straight to the pinned block where the device can write it, else by a copy
   float *res = (float *)(m->h_out() + m->L.out_ints);
   float *res_dev = m->host_dev ? (float *)(m->host_dev + m->L.in_ints + m->L.out_ints) : nullptr;
+  if (res_dev) std::memset(res + 2 * K + 1, 0, 4);
   CU_TRY(ts::launch_topk_cosine((const __nv_bfloat16 *)hidden_dev, n_entries, m->c.d_model, query_dev, planes,
                                 (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms, res_dev, m->d_out() + m->L.o_err, m->st));
   if (!res_dev) {
     CU_TRY(cudaMemcpyAsync(res, scores_dev + n_entries, 2 * (size_t)K * 4, cudaMemcpyDeviceToHost, m->st));
     CU_TRY(cudaMemcpyAsync(res + 2 * K, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));
   }
-  CU_TRY(cudaStreamSynchronize(m->st));
+  CU_TRY(res_dev ? wait_results((const int32_t *)(res + 2 * K + 1), 1, m->st) : cudaStreamSynchronize(m->st));
   int dev_err;
   std::memcpy(&dev_err, res + 2 * K, 4);
   if (dev_err != 0) {

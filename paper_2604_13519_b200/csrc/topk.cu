@@ -134,7 +134,10 @@ topk_final_kernel(const float2 *cand, int n_lists, int K, float *out, float *out
     out[2 * threadIdx.x + 1] = r.y;
     if (out_host) { out_host[2 * threadIdx.x] = r.x; out_host[2 * threadIdx.x + 1] = r.y; }
   }
-  if (out_host && threadIdx.x == 0) out_host[2 * K] = __int_as_float(*err);
+  if (!out_host) return;
+  if (threadIdx.x == 0) out_host[2 * K] = __int_as_float(*err);
+  __syncthreads();
+  if (threadIdx.x == 0) raise_flag(reinterpret_cast<int32_t *>(out_host) + 2 * K + 1);
 }
 
 cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, float *out_host,
