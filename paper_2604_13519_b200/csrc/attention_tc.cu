@@ -49,7 +49,10 @@ struct __align__(16) AttnCtl {
   uint64_t kv_full[kMaxKvStages], kv_empty[kMaxKvStages], q_full;
   uint64_t s_full[2], p_full[2], pv_done[2];   // [2]: one per softmax group
   uint32_t tmem_base;
-  float2 ml[2][kAttnRows];   // (reference maximum, sum) of each group's part of a row
+  // (reference maximum, sum) of each group's part of a row.  Two sets, for the CTA's units in turn: in a unit of one block
+  // group 1 waits for nothing before it writes its (nothing), so a set may be written again only after the meeting of the
+  // unit in between, which group 0 comes to when it has read this one.
+  float2 ml[2][2][kAttnRows];
 };
 
 __device__ __forceinline__ bool worker_all(bool ok) {
@@ -127,10 +130,12 @@ __device__ __forceinline__ uint32_t pack_h2(float x, float y) {
 
 // Worker side of one unit.  Thread <-> row (tensor-memory lane q*32 + lane) of one of the two groups: it takes the row
 // maximum over a block's 64 scores, writes the 64 probabilities over them as fp16 pairs and, rarely, rescales the row's
-// output sums.  `cnt` counts this group's blocks over all units of this CTA (barrier parities come from it).
+// output sums.  `cnt` counts this group's blocks over all units of this CTA (barrier parities come from it), `set` alternates
+// over the CTA's units that have blocks (see AttnCtl::ml).
 template <int HD>
 __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *ctl, const UnitInfo &t, uint32_t tmem_base,
-                                                  int grp, int q, int lane, uint32_t stg, uint32_t &cnt, bool &waited, const int *err) {
+                                                  int grp, int q, int lane, uint32_t stg, uint32_t &cnt, uint32_t &set, bool &waited,
+                                                  const int *err) {
   const int row = q * 32 + lane;      // row of the tile
   const int pr = t.row0 + row;        // packed row of the sequence
   const bool valid = row < t.rows_here;
@@ -335,7 +340,9 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
   const bool any = t.nblk > grp;
   if (any && ok && !mbar_wait_err(smem_u32(&ctl->pv_done[grp]), (cnt - 1) & 1, err)) { ok = false; atomicCAS((int *)err, 0, DEV_TIMEOUT_TMEM); }
   tc_fence_after();
-  ctl->ml[grp][row] = make_float2(m_ref, l_run);
+  float2(*ml)[kAttnRows] = ctl->ml[set];
+  set ^= 1u;
+  ml[grp][row] = make_float2(m_ref, l_run);
   tc_fence_before();
   if (!worker_all(ok)) return false;
   tc_fence_after();
@@ -343,7 +350,7 @@ __device__ __forceinline__ bool attn_unit_workers(const AttnTcArgs &a, AttnCtl *
   // ---- partial result of this unit: un-normalised output, its reference maximum (log2 domain), sum.  Each thread puts
   // half of its row's output together from both groups' sums.
   {
-    const float2 m0 = ctl->ml[0][row], m1 = ctl->ml[1][row];
+    const float2 m0 = ml[0][row], m1 = ml[1][row];
     const float m = fmaxf(m0.x, m1.x);
     const float w0 = m0.x == -INFINITY ? 0.f : ex2_approx(m0.x - m), w1 = m1.x == -INFINITY ? 0.f : ex2_approx(m1.x - m);
     float *dst = a.attn_o + ob * HD + grp * (HD / 2);
@@ -542,11 +549,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
     }
   } else {
     // ---------------------------------------------------------------- workers
-    uint32_t cnt = 0;
+    uint32_t cnt = 0, set = 0;
     bool ok = true, waited = false;
     for (int u = u_beg; u < u_end && ok; ++u) {
       const UnitInfo t = attn_unit_info(a, u);
-      ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp >> 2, warp & 3, lane, smem_u32(ctl + 1) + warp * kStageBytes, cnt, waited, err);
+      ok = attn_unit_workers<HD>(a, ctl, t, tmem_base, warp >> 2, warp & 3, lane, smem_u32(ctl + 1) + warp * kStageBytes, cnt, set, waited, err);
     }
     if (!waited) pdl_wait();
   }

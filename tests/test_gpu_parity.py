@@ -239,6 +239,30 @@ def test_sixteen_sessions_512_rows():
     gm.close()
 
 
+@pytest.mark.parametrize("name", ["1b-2l", "8b-2l"])
+def test_units_of_many_blocks_before_units_of_one(name):
+    """Sixteen sessions just past 512 cached positions, four rows each: with leaves of 512 positions every (session, kv
+    head) has a unit of eight blocks and one of a single block, which the attention kernel's CTAs walk one after the
+    other.  In the second only one of the two softmax groups has work, and the other must not touch what the first
+    unit's groups still have to read of each other.  Against the oracle, and every repetition the same bits."""
+    shape = synth.SHAPES[name]
+    lens = [513 + 3 * i for i in range(16)]
+    om, gm = make_pair(shape, max_batch=16, k_max=4, max_ctx=2048, max_pages=16 * 36)
+    sess, drafts, refs = [], [], []
+    for i, n in enumerate(lens):
+        cache, s, pending = synthetic_context(shape, om, gm, n, stream=i, pending=300 + i)
+        draft = _rand_draft(shape.vocab, 3, 90 + i)
+        sess.append(s); drafts.append(draft)
+        refs.append(om.verify(pending, draft, cache, want_logits=True))
+    for i, (res, ref) in enumerate(zip(ts.ts_verify(gm, sess, drafts), refs)):
+        check_step(res, gm.read_logits(4 * i, 4), ref, f"{name}, seq {i}")
+    first = gm.read_logits(0, 64).copy()
+    for _ in range(50):
+        ts.ts_verify_replay(gm)
+        assert np.array_equal(first, gm.read_logits(0, 64))
+    gm.close()
+
+
 def test_retrieval_heavy_batch():
     """Config-5-like: batch 4, long retrieved drafts (k = 64) from a large store searched through
     the n-gram index; drafts bit-exact with the oracle's linear scan."""
