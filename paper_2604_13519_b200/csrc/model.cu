@@ -248,6 +248,7 @@ struct ts_model {
   std::vector<ts_session *> sessions;   // live sessions over this model (detached on destroy)
   // last staged step
   int last_B = 0, last_M = 0, last_tiles = 0, last_tiles128 = 0, last_ctas = 0, last_slots = 1;
+  int last_max_len = 0, last_max_total = 0;    // longest cached length, longest with the chunk's rows
   int last_ready = -1;                         // pieces of a prompt: positions cached before the step (else -1)
   size_t last_units_at = 0;                    // where the step's attention units lie in its inputs (int32 offset)
   uint32_t last_flags = 0;
@@ -440,10 +441,7 @@ ts_status run_step_fused(ts_model *m) {
   {
     // (from the cached lengths and the model's k_max, not from this step's k, so that the cut does not change with the
     // number of rows verified)
-    int max_total = 0;
-    const int32_t *hi = m->h_in();
-    for (int i = 0; i < m->last_B; ++i) max_total = std::max(max_total, hi[I.o_len + i] + c.k_max);
-    const int nblk = (max_total + 63) / 64;
+    const int nblk = (m->last_max_len + c.k_max + 63) / 64;
     const int G = c.n_q_heads / c.n_kv_heads;
     const int s = m->n_sms / std::max(1, c.n_kv_heads * m->last_B * ((c.k_max * G + 127) / 128));
     a.attn_splits = std::max(1, std::min(std::min(s, kMaxAttnSplits), nblk));
@@ -503,11 +501,7 @@ ts_status run_step(ts_model *m) {
   aa.out = attn; aa.out_rows = R; aa.planes = m->planes;
   {
     // enough CTAs for about two per SM, each split at least one 64-position block
-    int max_total = 0;
-    const int32_t *hi = m->h_in();
-    for (int i = 0; i < B; ++i)
-      max_total = std::max(max_total, hi[I.o_len + i] + (hi[I.o_cu + i + 1] - hi[I.o_cu + i]));
-    const int nblk = (max_total + 63) / 64;
+    const int nblk = (m->last_max_total + 63) / 64;
     int s = (2 * m->n_sms + c.n_kv_heads * m->last_tiles - 1) / (c.n_kv_heads * m->last_tiles);
     aa.n_splits = std::max(1, std::min(std::min(s, kMaxAttnSplits), nblk));
   }
@@ -821,6 +815,12 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const ts_model_config &c = m->c;
   const Layout &L = m->L;
   m->last_B = B; m->last_M = M; m->last_flags = flags;
+  m->last_max_len = m->last_max_total = 0;
+  for (int i = 0; i < B; ++i) {
+    const int32_t *hi = m->h_in();
+    m->last_max_len = std::max(m->last_max_len, hi[I.o_len + i]);
+    m->last_max_total = std::max(m->last_max_total, hi[I.o_len + i] + hi[I.o_cu + i + 1] - hi[I.o_cu + i]);
+  }
   m->have_step = true;
   const size_t in_bytes = (m->last_units_at + (size_t)m->h_in()[I.o_cta_unit + m->last_ctas] * (sizeof(ts::AttnWork) / 4)) * 4;
   CU_TRY(cudaMemcpyAsync(m->d_in(), m->h_in(), in_bytes, cudaMemcpyHostToDevice, m->st));
@@ -913,20 +913,24 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
     M += k;
     hi[I.o_cu + i + 1] = M;
   }
-  {
-    ts_status st = build_attention(m, I, B, M, B);
-    if (st) return st;
-  }
+  // All refusals come before the first word of the staged step's own state (last_*) changes: a replay after a refused call
+  // runs the step that was staged last.
   const bool can_fuse = m->fused_ok && M <= kFusedMaxRows;
   if (c.path == 2 && !can_fuse)
     return fail(TS_ERR_K_TOO_LARGE, "the fused kernel takes at most %d rows on a device that supports it (step has %d)",
                 kFusedMaxRows, M);
-  m->last_tree = parents != nullptr;
-  if (m->last_tree && (c.path == 2 || !m->fused_ok))
+  if (parents && (c.path == 2 || !m->fused_ok))
     return fail(TS_ERR_UNIMPLEMENTED, "draft trees need the one-kernel-per-stage path with tensor-memory attention");
+  if (uniforms && c.path == 2) return fail(TS_ERR_UNIMPLEMENTED, "sampling acceptance needs the one-kernel-per-stage path");
+  if ((flags & TS_FLAG_WANT_TOPK) && c.path == 2)
+    return fail(TS_ERR_UNIMPLEMENTED, "the per-position Top-K needs the one-kernel-per-stage path");
+  {
+    ts_status st = build_attention(m, I, B, M, B);
+    if (st) return st;
+  }
+  m->last_tree = parents != nullptr;
   m->last_sample = uniforms != nullptr;
   if (m->last_sample) {
-    if (c.path == 2) return fail(TS_ERR_UNIMPLEMENTED, "sampling acceptance needs the one-kernel-per-stage path");
     m->last_inv_t = 1.f / temperature;
     // the kernel reads uni[node c] for node c and the root's for the draw; a chain's caller gives value j for draft
     // j + 1 and its chunk's last value for the draw
@@ -942,8 +946,6 @@ ts_status stage_and_run(ts_model *m, ts_session *const *ss, int B, const std::ve
       }
     }
   }
-  if ((flags & TS_FLAG_WANT_TOPK) && c.path == 2)
-    return fail(TS_ERR_UNIMPLEMENTED, "the per-position Top-K needs the one-kernel-per-stage path");
   m->last_fused = !m->last_tree && !m->last_sample && !(flags & TS_FLAG_WANT_TOPK) && can_fuse &&
                   (c.path == 2 || (c.path == 0 && kAutoPrefersFused));
   m->last_tiles = tiles;

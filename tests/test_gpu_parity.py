@@ -323,6 +323,32 @@ def test_argument_and_capacity_errors():
     gm.close()
 
 
+@pytest.mark.parametrize("path", PATHS)
+def test_refused_calls_leave_the_staged_step(path):
+    """Calls that are refused -- for their rows, their ids, or (persistent kernel) their kind -- stage nothing: a replay
+    after them runs the step verified before, bit for bit."""
+    shape = synth.SHAPES["tiny"]
+    om, gm = make_pair(shape, max_batch=2, k_max=40, max_rows=80, max_ctx=512, path=path)
+    _, a, _ = synthetic_context(shape, om, gm, 300)
+    _, b, _ = synthetic_context(shape, om, gm, 30, stream=1)
+    ts.ts_verify(gm, [b], [_rand_draft(shape.vocab, 7, 3)])
+    first = gm.read_logits(0, 8).copy()
+    long = _rand_draft(shape.vocab, 39, 4)
+    refused = [(-5, lambda: ts.ts_verify(gm, [a, b], [long, [shape.vocab]])), (-4, lambda: ts.ts_verify(gm, [b, a], [long, long + [70]]))]
+    if path == 2:
+        chain = [list(range(39))]
+        refused += [(-4, lambda: ts.ts_verify(gm, [a, b], [long, long])), (-8, lambda: ts.ts_verify_tree(gm, [a], [long], chain)),
+                    (-8, lambda: ts.ts_verify_sampled(gm, [a], [long], 1.0, [0.5] * 40)),
+                    (-8, lambda: ts.ts_verify(gm, [a], [long], ts.TS_FLAG_WANT_TOPK))]
+    for code, call in refused:
+        with pytest.raises(ts.TsError) as e:
+            call()
+        assert e.value.code == code
+        ts.ts_verify_replay(gm)
+        assert np.array_equal(first, gm.read_logits(0, 8))
+    gm.close()
+
+
 def test_commit_is_checked_against_the_verified_chunk():
     """A commit moves the cache length over rows the last verification wrote: it is refused without one, twice for
     the same one, for more ids than rows, and for ids other than the ones those rows were computed from."""
