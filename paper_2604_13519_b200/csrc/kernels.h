@@ -164,13 +164,14 @@ cudaError_t launch_attention_tc_merge(const AttnTcArgs &a, cudaStream_t st);
 
 // A step's results straight to the host: the acceptance kernels write the words of the result block that the host reads to
 // pinned memory as well, so that no copy follows them (base: the block on the device, host: the same block as the device
-// sees the pinned one; host null: not wanted).  done: a word per sequence in the pinned block, raised when its results are there
-// (null: the host waits for the stream instead).
+// sees the pinned one; host null: not wanted).  done: a word per sequence in the pinned block that takes the call's number when
+// the sequence's results are there (null: the host waits for the stream instead).
 struct HostOut {
   const int32_t *base;
   int32_t *host;
   const int *err;   // status word, published too
   int32_t *done;
+  int32_t number;
 };
 
 // per-row argmax over the LM-head tiles, longest accepted prefix per sequence, new lengths
@@ -206,9 +207,9 @@ cudaError_t launch_sample_accept(const SampleArgs &a, cudaStream_t st);
 
 #ifdef __CUDACC__
 // tells the host that what the CTA wrote (before a barrier), and all kernels that it waited for, can be read
-__device__ __forceinline__ void raise_flag(int32_t *flag) {
+__device__ __forceinline__ void raise_flag(int32_t *flag, int32_t number) {
   __threadfence_system();
-  *reinterpret_cast<volatile int32_t *>(flag) = 1;
+  *reinterpret_cast<volatile int32_t *>(flag) = number;
 }
 
 // the results of sequence `seq` (rows r0 .. r0 + k, accepted length l) by the whole CTA, after a barrier
@@ -229,20 +230,27 @@ __device__ __forceinline__ void publish(const Args &a, int seq, int r0, int k, i
   }
   if (!a.ho.done) return;
   __syncthreads();
-  if (threadIdx.x == 0) raise_flag(a.ho.done + seq);
+  if (threadIdx.x == 0) raise_flag(a.ho.done + seq, a.ho.number);
 }
 #endif
+
+// A row's Top-K straight to the host: kTopMax pairs, then the status word and a word that takes the call's number when all of
+// it is there, in pinned memory as the device sees it (null: not wanted).
+constexpr int kTopMax = 64;
+struct PairsOut {
+  float *host;
+  int32_t number;
+};
 
 // Cosine Top-K over datastore hidden states (retrieval.cu).  scores: [N + 2K] floats; the result pairs (index as int
 // bits, score), best first, follow the N scores.  The query is q_dev (fp32 [d]) or, if null, bf16 planes of a row.
 cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float *q_dev, const __nv_bfloat16 *q_planes,
-                               int plane_stride, int planes, int K, float *scores, int n_sms, float *out_host, int *err, cudaStream_t st);
+                               int plane_stride, int planes, int K, float *scores, int n_sms, PairsOut po, int *err, cudaStream_t st);
 
 // Row-wise Top-K (topk.cu): out[r][j] = (column as int bits, value) of the j-th largest entry of row r, lowest column
 // on ties.  cand: scratch of n_rows * ceil(n_cols / 4096) * K pairs.
-// out_host (one row, may be null): the same pairs to host memory that the device can write, and behind them the
-// status word *err and a word that is raised when all of it is there.
-cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, float *out_host,
+// po: one row only; err is published with it.
+cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, PairsOut po,
                              const int *err, cudaStream_t st);
 
 // After a tree step: move the K/V rows of the accepted path to consecutive cache positions len, len+1, ...

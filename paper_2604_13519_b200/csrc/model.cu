@@ -211,7 +211,7 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->max_stamps = 9 * c.n_layers + 16;
   L->stamps = take((uint64_t)L->max_stamps * 4 * 8);
   L->workspace_bytes = o;
-  L->host_io_bytes = align_up((uint64_t)(L->in_ints + L->out_ints + 2 * 64 + 2) * 4, 4096);   // (and a retrieval's result pairs, status and flag)
+  L->host_io_bytes = align_up((uint64_t)(L->in_ints + L->out_ints + 2 * ts::kTopMax + 2) * 4, 4096);   // (and a retrieval's result pairs, status and number)
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -256,6 +256,7 @@ struct ts_model {
   int64_t launches = 0, h2d = 0, d2h = 0;
   bool use_pdl = true;
   bool publish = false;                        // the step being enqueued writes its results to the pinned block itself
+  int32_t call_no = 0;                         // number that the call being waited for ends with (see wait_results)
   int32_t *host_dev = nullptr;                 // the pinned block as the device sees it (null: it cannot write there)
   int32_t inject_err = 0;                      // test support: status code the next step is made to report
   bool fused_ok = false, last_fused = false;   // device can run the fused kernel; the staged step uses it
@@ -288,6 +289,7 @@ struct ts_model {
     }
   }
 
+  void next_call() { call_no = call_no == INT32_MAX ? 1 : call_no + 1; }   // (never 0: the words start with it)
   uint8_t *W(uint64_t off) const { return (uint8_t *)b.weights + off; }
   uint8_t *WS(uint64_t off) const { return (uint8_t *)b.workspace + off; }
   const StepIo &io() const { return last_ready >= 0 ? L.prompt_io : L.step_io; }   // of the last step
@@ -608,13 +610,14 @@ ts_status run_step(ts_model *m) {
   int32_t *dout = m->d_out();
   if (m->last_flags & TS_FLAG_WANT_TOPK) {   // per-position Top-K of the logits, for the successor tables
     CU_TRY(ts::launch_topk_rows((const float *)m->WS(L.logits), M, c.vocab, TS_TOPK, (float2 *)m->WS(L.topk_cand),
-                                (float *)(dout + L.o_topk), nullptr, nullptr, m->st));
+                                (float *)(dout + L.o_topk), ts::PairsOut{}, nullptr, m->st));
     m->launched(5);
     m->launched(5);
   }
   ts::HostOut ho{};
   if (m->publish) {
     ho.base = dout; ho.host = m->host_dev + L.in_ints; ho.err = dout + L.o_err;
+    ho.number = m->call_no;
     ho.done = m->last_tree ? nullptr : ho.host + L.o_done;   // (a tree's step ends with the compaction, which publishes nothing)
   }
   if (m->last_sample) {
@@ -812,14 +815,14 @@ ts_status build_attention(ts_model *m, const StepIo &I, int B, int M, int tables
   return TS_OK;
 }
 
-// Waits for n words of the pinned block, cleared before the launches, that the last kernel on the stream raises behind its
-// results; by then all kernels before it are complete and it has nothing left to do.  3.5 us sooner than the stream's own
+// Waits for n words of the pinned block that take the call's number when the last kernel on the stream has written its results
+// (a number of the call's own: a kernel left over from a call that ended early cannot end a later one); by then all kernels before it are complete and it has nothing left to do.  3.5 us sooner than the stream's own
 // synchronisation, which learns of the kernel's end by way of the driver (ten small kernels in a row: 52.1 -> 48.8 us; the
 // two-layer shape's step 77.1 -> 75.1, a retrieval over 100 000 entries 149.2 -> 147.7).  The stream is still asked from time to time, so that a failed launch or kernel ends the wait with its error.
-cudaError_t wait_results(const int32_t *words, int n, cudaStream_t st) {
+cudaError_t wait_results(const int32_t *words, int n, int32_t number, cudaStream_t st) {
   const volatile int32_t *w = words;
   for (uint32_t it = 1;; ++it) {
-    while (n > 0 && w[n - 1]) --n;
+    while (n > 0 && w[n - 1] == number) --n;
     if (n == 0) break;
     if ((it & 4095u) == 0) {
       const cudaError_t e = cudaStreamQuery(st);
@@ -860,7 +863,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
 #endif
   m->publish = publishes;
   const bool flagged = publishes && !m->last_tree;
-  if (flagged) std::memset(m->h_out() + L.o_done, 0, sizeof(int32_t) * B);
+  m->next_call();
   ts_status st = run_step(m);
   m->publish = false;
   if (st) return st;
@@ -874,7 +877,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
   if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
   m->d2h += (int64_t)out_bytes;
-  CU_TRY(flagged ? wait_results(m->h_out() + L.o_done, B, m->st) : cudaStreamSynchronize(m->st));
+  CU_TRY(flagged ? wait_results(m->h_out() + L.o_done, B, m->call_no, m->st) : cudaStreamSynchronize(m->st));
   const int dev_err = m->h_out()[L.o_err];
   if (dev_err != 0) {
     cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
@@ -1090,6 +1093,8 @@ ts_status ts_init_model(const ts_model_config *cfg, const ts_buffers *bufs, void
     void *p = nullptr;
     if (cudaHostGetDevicePointer(&p, bufs->host_io, 0) == cudaSuccess) m->host_dev = (int32_t *)p;
     cudaGetLastError();
+    std::memset(m->h_out() + m->L.o_done, 0, sizeof(int32_t) * cfg->max_batch);
+    m->h_out()[m->L.out_ints + 2 * ts::kTopMax + 1] = 0;
   }
   const Layout &L = m->L;
   const ts_model_config &c = m->c;
@@ -1900,16 +1905,16 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
   // the result pairs go straight to the pinned block where the device can write it, else by a copy
   float *res = (float *)(m->h_out() + m->L.out_ints);
   float *res_dev = m->host_dev ? (float *)(m->host_dev + m->L.in_ints + m->L.out_ints) : nullptr;
-  if (res_dev) std::memset(res + 2 * K + 1, 0, 4);
+  m->next_call();
   CU_TRY(ts::launch_topk_cosine((const __nv_bfloat16 *)hidden_dev, n_entries, m->c.d_model, query_dev, planes,
-                                (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms, res_dev, m->d_out() + m->L.o_err, m->st));
+                                (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms, ts::PairsOut{res_dev, m->call_no}, m->d_out() + m->L.o_err, m->st));
   if (!res_dev) {
     CU_TRY(cudaMemcpyAsync(res, scores_dev + n_entries, 2 * (size_t)K * 4, cudaMemcpyDeviceToHost, m->st));
-    CU_TRY(cudaMemcpyAsync(res + 2 * K, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));
+    CU_TRY(cudaMemcpyAsync(res + 2 * ts::kTopMax, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));
   }
-  CU_TRY(res_dev ? wait_results((const int32_t *)(res + 2 * K + 1), 1, m->st) : cudaStreamSynchronize(m->st));
+  CU_TRY(res_dev ? wait_results((const int32_t *)(res + 2 * ts::kTopMax + 1), 1, m->call_no, m->st) : cudaStreamSynchronize(m->st));
   int dev_err;
-  std::memcpy(&dev_err, res + 2 * K, 4);
+  std::memcpy(&dev_err, res + 2 * ts::kTopMax, 4);
   if (dev_err != 0) {
     cudaMemsetAsync(m->d_out() + m->L.o_err, 0, 4, m->st);
     return fail(TS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired (code %d)", dev_err);

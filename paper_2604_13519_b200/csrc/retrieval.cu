@@ -108,7 +108,7 @@ cosine_scores_kernel(const __nv_bfloat16 *H, int N, int d, int piece, const floa
 }
 
 cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float *q_dev, const __nv_bfloat16 *q_planes,
-                               int plane_stride, int planes, int K, float *scores, int n_sms, float *out_host, int *err,
+                               int plane_stride, int planes, int K, float *scores, int n_sms, PairsOut po, int *err,
                                cudaStream_t st) {
   static PerDeviceOnce once;
   int dev_ = -1;
@@ -131,7 +131,7 @@ cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float
   if (e != cudaSuccess) return e;
   // candidates live behind the K result pairs: scores[N + 2K ...], 2 floats per candidate
   float2 *cand = reinterpret_cast<float2 *>(scores + N + 2 * K + ((N + 2 * K) & 1));
-  return launch_topk_rows(scores, 1, N, K, cand, scores + N, out_host, err, st);
+  return launch_topk_rows(scores, 1, N, K, cand, scores + N, po, err, st);
 }
 
 }  // namespace ts

@@ -15,7 +15,6 @@ static constexpr int kSlice = 4096;
 static constexpr int kSelThreads = 256;
 static constexpr int kSelWarps = kSelThreads / 32;
 static constexpr int kPer = kSlice / kSelThreads;   // entries per thread
-static constexpr int kTopMax = 64;
 
 // An entry as one word that orders like (score, then lower index): order-preserving map of the score above the index's
 // complement; 0 = no entry (also for NaN and -inf, which are never taken).
@@ -106,7 +105,7 @@ topk_slice_kernel(const float *x, int N, int K, float2 *cand) {
 }
 
 __global__ void __launch_bounds__(kSelThreads)
-topk_final_kernel(const float2 *cand, int n_lists, int K, float *out, float *out_host, const int *err) {
+topk_final_kernel(const float2 *cand, int n_lists, int K, float *out, PairsOut po, const int *err) {
   __shared__ Entry lists[kSelWarps + 1][kTopMax], best[kTopMax];
   cand += (size_t)blockIdx.x * n_lists * K;
   out += (size_t)blockIdx.x * 2 * K;
@@ -132,15 +131,16 @@ topk_final_kernel(const float2 *cand, int n_lists, int K, float *out, float *out
     const float2 r = pair_of(lists[kSelWarps][threadIdx.x]);
     out[2 * threadIdx.x] = r.x;
     out[2 * threadIdx.x + 1] = r.y;
-    if (out_host) { out_host[2 * threadIdx.x] = r.x; out_host[2 * threadIdx.x + 1] = r.y; }
+    if (po.host) { po.host[2 * threadIdx.x] = r.x; po.host[2 * threadIdx.x + 1] = r.y; }
   }
-  if (!out_host) return;
-  if (threadIdx.x == 0) out_host[2 * K] = __int_as_float(*err);
+  if (!po.host) return;
+  int32_t *tail = reinterpret_cast<int32_t *>(po.host) + 2 * kTopMax;
+  if (threadIdx.x == 0) tail[0] = *err;
   __syncthreads();
-  if (threadIdx.x == 0) raise_flag(reinterpret_cast<int32_t *>(out_host) + 2 * K + 1);
+  if (threadIdx.x == 0) raise_flag(tail + 1, po.number);
 }
 
-cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, float *out_host,
+cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, PairsOut po,
                              const int *err, cudaStream_t st) {
   if (K < 1 || K > kTopMax || n_rows < 1 || n_cols < 1) return cudaErrorInvalidValue;
   const int slices = (n_cols + kSlice - 1) / kSlice;
@@ -156,7 +156,7 @@ cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, floa
   cudaError_t e = cudaLaunchKernelEx(&cfg, topk_slice_kernel, x, n_cols, K, cand);
   if (e != cudaSuccess) return e;
   cfg.gridDim = dim3(n_rows);
-  return cudaLaunchKernelEx(&cfg, topk_final_kernel, (const float2 *)cand, slices, K, out, out_host, err);
+  return cudaLaunchKernelEx(&cfg, topk_final_kernel, (const float2 *)cand, slices, K, out, po, err);
 }
 
 }  // namespace ts

@@ -1,6 +1,8 @@
 """GPU parity tests: the CUDA verify path, called through the C ABI, against the CPU oracle on the
 same seeded inputs.  Logits within max-abs 3e-2 / mean-abs 3e-3; drafts bit-exact; accepted lengths,
 argmax and emitted ids exact except at positions where the oracle's top-2 logit gap is below 0.05."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -320,6 +322,48 @@ def test_argument_and_capacity_errors():
     assert e.value.code == -3
     res = ts.ts_verify(gm, [s], [[70]])[0]                 # the context is still usable
     assert res.k == 2
+    gm.close()
+
+
+def _counting_word(gm, call):
+    """Index of the one word of the pinned block that differs, by one, between two equal calls: the number a call ends with."""
+    words = gm._host.view(torch.int32).numpy()
+    call()
+    first = words.copy()
+    call()
+    at = np.flatnonzero(words != first)
+    assert len(at) == 1 and words[at[0]] == first[at[0]] + 1
+    return words, int(at[0])
+
+
+def test_a_late_end_of_an_earlier_call_does_not_end_the_next():
+    """A call returns when the last kernel has written the call's number to the pinned block.  Earlier numbers that turn up
+    there meanwhile (a thread keeps writing one, as a kernel left over from a call that ended early would) end nothing:
+    every step and every retrieval returns its own results."""
+    shape = synth.SHAPES["1b-2l"]
+    om, gm = make_pair(shape, k_max=8, max_ctx=512)
+    _, s, _ = synthetic_context(shape, om, gm, 200)
+    H = torch.randn(5000, shape.d_model, generator=torch.Generator().manual_seed(3)).to(torch.bfloat16).cuda()
+    drafts, queries = [_rand_draft(shape.vocab, 7, i) for i in range(4)], [H[100 * i + 7].float() for i in range(4)]
+    step = lambda i: list(ts.ts_verify(gm, [s], [drafts[i]])[0].argmax[:8])
+    find = lambda i: ts.ts_topk_cosine(gm, H, 3, query=queries[i])[0]
+    for call in (step, find):
+        want = [call(i) for i in range(4)]
+        assert len({tuple(w) for w in want}) == 4
+        words, at = _counting_word(gm, lambda: call(0))
+        old, stop = int(words[at]), threading.Event()
+
+        def late():
+            while not stop.is_set():
+                words[at] = old
+        t = threading.Thread(target=late)
+        t.start()
+        try:
+            got = [call(i % 4) for i in range(200)]
+        finally:
+            stop.set()
+            t.join()
+        assert got == [want[i % 4] for i in range(200)]
     gm.close()
 
 
