@@ -392,11 +392,12 @@ ts_status ts_debug_schedule(int32_t n_tiles, int32_t n_kblocks, int32_t n_ctas, 
  * ts_profile_step; at most cap launches are written, *n_launches receives their number.  A launch without stamps
  * (acceptance, Top-K, sampling) reports ~0, ~0, 0, 0.  One-kernel-per-stage path only.  Synchronises the stream. */
 ts_status ts_debug_timeline(ts_model *m, uint64_t *stamps, int32_t *classes, int32_t cap, int32_t *n_launches);
-/* Make the NEXT step (ts_verify*, ts_prefill chunk) report `code` (> 0) in its device status word, as a bounded
- * device-side wait that expired would: the word is written on the model's stream after the step's last kernel and
- * before the results are read back, so no kernel sees it and nothing is left waiting.  That step then fails with
- * TS_ERR_DEVICE_TIMEOUT (codes below 64) or TS_ERR_DEVICE_BOUNDS (64 + the number of a debug-build index check), the
- * library clears the word and the persistent kernel's counters, and later steps run normally.  For testing the
+/* Make the NEXT step or retrieval (ts_verify*, ts_prefill, ts_topk_cosine) report `code` (> 0) in its device status word,
+ * as a bounded device-side wait that expired would: the word is written on the model's stream behind the step's last
+ * kernel that waits for anything -- ahead of the acceptance kernel, which hands it to the host with its results; after the
+ * last kernel where there is none; ahead of a retrieval's kernels, which do not read it -- so nothing is left waiting.  The
+ * call then fails with TS_ERR_DEVICE_TIMEOUT (codes below 64) or TS_ERR_DEVICE_BOUNDS (64 + the number of a debug-build
+ * index check; steps only), the library clears the word and the persistent kernel's counters, and later calls run normally.  For testing the
  * host's handling of a device timeout, or of a failed index check, without making a GPU wait or go out of range. */
 ts_status ts_debug_inject_device_error(ts_model *m, int32_t code);
 /* Counters: kernels launched since ts_init_model, bytes copied host->device and device->host by

@@ -258,7 +258,8 @@ struct ts_model {
   bool publish = false;                        // the step being enqueued writes its results to the pinned block itself
   int32_t call_no = 0;                         // number that the call being waited for ends with (see wait_results)
   int32_t *host_dev = nullptr;                 // the pinned block as the device sees it (null: it cannot write there)
-  int32_t inject_err = 0;                      // test support: status code the next step is made to report
+  int32_t inject_err = 0;                      // test support: status code the next step or retrieval is made to report
+  bool staging = false;                        // the step being enqueued is a new one, not a replay
   bool fused_ok = false, last_fused = false;   // device can run the fused kernel; the staged step uses it
   bool last_tree = false;                      // the staged step verifies a draft tree (not a chain)
   bool last_sample = false;                    // the staged step accepts by speculative sampling
@@ -471,6 +472,16 @@ ts_status run_step_fused(ts_model *m) {
   return TS_OK;
 }
 
+// Test support (ts_debug_inject_device_error): leaves the status word that an expired device-side wait would have left.  In
+// the stream behind the last kernel that waits for anything and ahead of the acceptance kernel, which publishes the word with
+// the step's results as it would a real one.
+cudaError_t write_injected(ts_model *m) {
+  int32_t *word = m->h_out() + m->L.o_err + 1;
+  *word = m->inject_err;
+  m->inject_err = 0;
+  return cudaMemcpyAsync(m->d_out() + m->L.o_err, word, 4, cudaMemcpyHostToDevice, m->st);
+}
+
 ts_status run_step(ts_model *m) {
   const StepIo &I = m->io();
   if (m->last_fused) return run_step_fused(m);
@@ -620,6 +631,7 @@ ts_status run_step(ts_model *m) {
     ho.number = m->call_no;
     ho.done = m->last_tree ? nullptr : ho.host + L.o_done;   // (a tree's step ends with the compaction, which publishes nothing)
   }
+  if (m->staging && m->inject_err) CU_TRY(write_injected(m));
   if (m->last_sample) {
     ts::SampleArgs sa{};
     sa.in = in; sa.logits = (float *)m->WS(L.logits); sa.amax = amax;
@@ -837,7 +849,7 @@ cudaError_t wait_results(const int32_t *words, int n, int32_t number, cudaStream
   return cudaSuccess;
 }
 
-// Copies the staged inputs in, runs the step, copies its results back and waits.
+// Copies the staged inputs in, runs the step and waits for its results.
 ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const StepIo &I = m->io();
   const ts_model_config &c = m->c;
@@ -854,26 +866,21 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   CU_TRY(cudaMemcpyAsync(m->d_in(), m->h_in(), in_bytes, cudaMemcpyHostToDevice, m->st));
   m->h2d += (int64_t)in_bytes;
   // A step that ends in an acceptance kernel (and maybe the cache's compaction) publishes its results itself; prompts, the
-  // persistent kernel, per-position Top-K lists and an injected status word take a copy, as does the debug build, whose
-  // checks go on in the compaction.
+  // persistent kernel and per-position Top-K lists take a copy, as does the debug build, whose checks go on in the
+  // acceptance kernel's other blocks and in the compaction.
 #ifdef TS_DEBUG_BOUNDS
   const bool publishes = false;
 #else
-  const bool publishes = m->host_dev && !m->last_fused && !m->inject_err && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
+  const bool publishes = m->host_dev && !m->last_fused && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
 #endif
   m->publish = publishes;
   const bool flagged = publishes && !m->last_tree;
   m->next_call();
+  m->staging = true;
   ts_status st = run_step(m);
-  m->publish = false;
+  m->publish = m->staging = false;
   if (st) return st;
-  if (m->inject_err) {
-    // test support (ts_debug_inject_device_error): after the step's last kernel, write the status word an expired
-    // device-side wait would have left; the code below must then treat the step as failed
-    m->h_out()[L.o_err + 1] = m->inject_err;
-    m->inject_err = 0;
-    CU_TRY(cudaMemcpyAsync(m->d_out() + L.o_err, m->h_out() + L.o_err + 1, 4, cudaMemcpyHostToDevice, m->st));
-  }
+  if (m->inject_err) CU_TRY(write_injected(m));   // (a step without an acceptance kernel of its own)
   const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
   if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
   m->d2h += (int64_t)out_bytes;
@@ -1906,6 +1913,7 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
   float *res = (float *)(m->h_out() + m->L.out_ints);
   float *res_dev = m->host_dev ? (float *)(m->host_dev + m->L.in_ints + m->L.out_ints) : nullptr;
   m->next_call();
+  if (m->inject_err) CU_TRY(write_injected(m));
   CU_TRY(ts::launch_topk_cosine((const __nv_bfloat16 *)hidden_dev, n_entries, m->c.d_model, query_dev, planes,
                                 (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms, ts::PairsOut{res_dev, m->call_no}, m->d_out() + m->L.o_err, m->st));
   if (!res_dev) {

@@ -470,6 +470,33 @@ def test_device_index_check_is_reported_and_survived():
     gm.close()
 
 
+def test_every_way_results_reach_the_host_carries_the_status():
+    """A status word left on the device reaches the host with the results that the last kernel writes to the pinned block:
+    greedy and sampled acceptance, of one session and of three, chains and trees, and a retrieval.  The call fails with the
+    code, and the same call again succeeds with the results of before."""
+    shape = synth.SHAPES["tiny"]
+    om, gm = make_pair(shape, max_batch=3, k_max=8, max_ctx=256)
+    ss = [synthetic_context(shape, om, gm, n, stream=i)[1] for i, n in enumerate([100, 33, 7])]
+    drafts = [_rand_draft(shape.vocab, k, 50 + k) for k in (7, 4, 0)]
+    parents = [[0, 0, 1, 2, 2, 3, 4], [0, 0, 1, 1], []]
+    uni = [0.25 + 0.03 * i for i in range(14)]
+    H = torch.randn(300, shape.d_model, generator=torch.Generator().manual_seed(3)).to(torch.bfloat16).cuda()
+    seen = lambda res: [(r.accept_len, list(r.emitted[:r.n_emitted]), list(r.argmax[:r.k])) for r in res]
+    calls = [lambda: seen(ts.ts_verify(gm, ss[:1], drafts[:1])), lambda: seen(ts.ts_verify(gm, ss, drafts)),
+             lambda: seen(ts.ts_verify_sampled(gm, ss[:1], drafts[:1], 0.9, uni[:8])), lambda: seen(ts.ts_verify_sampled(gm, ss, drafts, 0.9, uni)),
+             lambda: ts.ts_topk_cosine(gm, H, 5, query=H[9].float()),
+             lambda: seen(ts.ts_verify_tree(gm, ss, drafts, parents)[0]), lambda: seen(ts.ts_verify_tree_sampled(gm, ss, drafts, parents, 0.9, uni)[0]),
+             lambda: seen(ts.ts_verify(gm, ss, drafts, ts.TS_FLAG_WANT_TOPK))]
+    for call in calls:
+        want = call()
+        gm.inject_device_error(2)
+        with pytest.raises(ts.TsError) as e:
+            call()
+        assert e.value.code == -6 and "code 2" in str(e.value)
+        assert call() == want
+    gm.close()
+
+
 def test_small_batch_fused():
     """Several short sequences in one step of the persistent kernel (ragged k, ragged contexts)."""
     shape = synth.SHAPES["1b-2l"]
