@@ -17,11 +17,11 @@ static constexpr int kSelWarps = kSelThreads / 32;
 static constexpr int kPer = kSlice / kSelThreads;   // entries per thread
 
 // An entry as one word that orders like (score, then lower index): order-preserving map of the score above the index's
-// complement; 0 = no entry (also for NaN and -inf, which are never taken).
+// complement; 0 = no entry (also for NaN and -inf, which are never taken).  Both zeros are the same score: -0 + 0 = +0.
 typedef unsigned long long Entry;
 __device__ __forceinline__ Entry entry_of(float v, int idx) {
   if (!(v > -INFINITY)) return 0ull;
-  uint32_t u = __float_as_uint(v);
+  uint32_t u = __float_as_uint(v + 0.f);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   return ((Entry)u << 32) | (uint32_t)~idx;
 }

@@ -67,6 +67,29 @@ def test_topk_at_the_edges_of_pieces_slices_and_lists(n, d, K):
     gm.close()
 
 
+def test_zeros_of_either_sign_tie():
+    """Scores of -0 (a negative product that underflows) and +0 (orthogonal entries) are equal: the lower index first, in
+    one list and across the lists of two slices; above negative scores, below positive ones."""
+    shape = synth.SHAPES["tiny"]
+    d, n = shape.d_model, 4200
+    H = torch.zeros(n, d)
+    H[:, 2] = 1.0                                    # orthogonal to the query: +0
+    minus = [0, 3, 7, 4150]
+    for j in minus:
+        H[j, 0], H[j, 2] = -1e-18, 1e18              # dot product -1e-38, norm 1e18: -1e-56
+    H[5, 1], H[2, 1] = 1.0, -1.0                     # a positive score, a negative one
+    q = torch.zeros(d)
+    q[0], q[1] = 1e-20, 1.0
+    gm = ts.Model(shape, max_pages=8, max_batch=1, k_max=8, max_rows=8, max_ctx=64, act_split=True, path=1)
+    idx, sc = ts.ts_topk_cosine(gm, H.to(torch.bfloat16).cuda(), 64, query=q.cuda())
+    assert idx == [5] + [j for j in range(n) if j not in (5, 2)][:63]
+    assert sc[0] > 0.7 and all(v == 0.0 for v in sc[1:])
+    only = [0, 3, 5, 2, 4150]
+    idx, sc = ts.ts_topk_cosine(gm, H[only].to(torch.bfloat16).cuda(), 5, query=q.cuda())
+    assert idx == [2, 0, 1, 4, 3] and sc[-1] < 0
+    gm.close()
+
+
 def test_query_from_the_last_step_is_the_final_hidden_state():
     shape = synth.SHAPES["8b-2l"]
     om, gm = make_pair(shape, k_max=8, max_ctx=256, path=1)
