@@ -400,8 +400,8 @@ ts_status ts_debug_timeline(ts_model *m, uint64_t *stamps, int32_t *classes, int
  * index check; steps only), the library clears the word and the persistent kernel's counters, and later calls run normally.  For testing the
  * host's handling of a device timeout, or of a failed index check, without making a GPU wait or go out of range. */
 ts_status ts_debug_inject_device_error(ts_model *m, int32_t code);
-/* Counters: kernels launched since ts_init_model, bytes copied host->device and device->host by
- * ts_verify since then. */
+/* Counters: kernels launched since ts_init_model, bytes that steps have moved host->device and device->host since then
+ * (by copies, or written to the pinned block by the step's last kernel). */
 ts_status ts_model_counters(const ts_model *m, int64_t *launches, int64_t *h2d_bytes,
                             int64_t *d2h_bytes);
 

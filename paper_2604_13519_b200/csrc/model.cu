@@ -883,9 +883,17 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   if (m->inject_err) CU_TRY(write_injected(m));   // (a step without an acceptance kernel of its own)
   const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
   if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
-  m->d2h += (int64_t)out_bytes;
   CU_TRY(flagged ? wait_results(m->h_out() + L.o_done, B, m->call_no, m->st) : cudaStreamSynchronize(m->st));
-  const int dev_err = m->h_out()[L.o_err];
+  const int32_t *ho = m->h_out();
+  if (publishes) {   // (see ts::publish: the status; per sequence length, pending id, accepted drafts, maybe the call's number; a row's
+                     // argmax; emitted ids and path)
+    int64_t words = 1 + (3 + flagged) * (int64_t)B + M;
+    for (int i = 0; i < B; ++i) words += 2 * (ho[L.o_accept + i] + 1);
+    m->d2h += 4 * words;
+  } else {
+    m->d2h += (int64_t)out_bytes;
+  }
+  const int dev_err = ho[L.o_err];
   if (dev_err != 0) {
     cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
     cudaMemsetAsync(m->WS(L.sync), 0, (size_t)(8 + L.n_counters) * 4, m->st);   // the fused kernel left its counters mid-step

@@ -497,6 +497,21 @@ def test_every_way_results_reach_the_host_carries_the_status():
     gm.close()
 
 
+def test_counted_bytes_are_the_ones_moved():
+    """Device to host a step counts the words its last kernel writes to the pinned block: status, four per sequence, an
+    argmax per row, emitted ids and path of the accepted ones; a tree's step, which the stream's end is waited for, one
+    less per sequence."""
+    shape = synth.SHAPES["tiny"]
+    om, gm = make_pair(shape, max_batch=3, k_max=8, max_ctx=256)
+    ss = [synthetic_context(shape, om, gm, n, stream=i)[1] for i, n in enumerate([100, 33, 7])]
+    drafts = [_rand_draft(shape.vocab, k, 50 + k) for k in (7, 4, 0)]
+    for per_seq, call in ((4, lambda: ts.ts_verify(gm, ss, drafts)), (3, lambda: ts.ts_verify_tree(gm, ss, drafts, [[0] * 7, [0] * 4, []])[0])):
+        before = gm.counters()[2]
+        res = call()
+        assert gm.counters()[2] - before == 4 * (1 + 3 * per_seq + 14 + sum(2 * (r.accept_len + 1) for r in res))
+    gm.close()
+
+
 def test_small_batch_fused():
     """Several short sequences in one step of the persistent kernel (ragged k, ragged contexts)."""
     shape = synth.SHAPES["1b-2l"]
