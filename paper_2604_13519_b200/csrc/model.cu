@@ -256,6 +256,7 @@ struct ts_model {
   int64_t launches = 0, h2d = 0, d2h = 0;
   bool use_pdl = true;
   bool publish = false;                        // the step being enqueued writes its results to the pinned block itself
+  bool flagged = false;                        // ... and raises its sequences' words there
   int32_t call_no = 0;                         // number that the call being waited for ends with (see wait_results)
   int32_t *host_dev = nullptr;                 // the pinned block as the device sees it (null: it cannot write there)
   int32_t inject_err = 0;                      // test support: status code the next step or retrieval is made to report
@@ -629,7 +630,7 @@ ts_status run_step(ts_model *m) {
   if (m->publish) {
     ho.base = dout; ho.host = m->host_dev + L.in_ints; ho.err = dout + L.o_err;
     ho.number = m->call_no;
-    ho.done = m->last_tree ? nullptr : ho.host + L.o_done;   // (a tree's step ends with the compaction, which publishes nothing)
+    ho.done = m->flagged ? ho.host + L.o_done : nullptr;
   }
   if (m->staging && m->inject_err) CU_TRY(write_injected(m));
   if (m->last_sample) {
@@ -849,6 +850,18 @@ cudaError_t wait_results(const int32_t *words, int n, int32_t number, cudaStream
   return cudaSuccess;
 }
 
+// Whether a wait may spin on the pinned block: not where the caller has the device's waits block or yield the processor
+// (cudaSetDeviceFlags; the stream's own synchronisation keeps to that).
+bool may_spin() {
+  unsigned flags = 0;
+  if (cudaGetDeviceFlags(&flags) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  flags &= cudaDeviceScheduleMask;
+  return flags != cudaDeviceScheduleBlockingSync && flags != cudaDeviceScheduleYield;
+}
+
 // Copies the staged inputs in, runs the step and waits for its results.
 ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const StepIo &I = m->io();
@@ -874,7 +887,8 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const bool publishes = m->host_dev && !m->last_fused && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
 #endif
   m->publish = publishes;
-  const bool flagged = publishes && !m->last_tree;
+  const bool flagged = publishes && !m->last_tree && may_spin();   // (a tree's step ends with the compaction, which publishes nothing)
+  m->flagged = flagged;
   m->next_call();
   m->staging = true;
   ts_status st = run_step(m);
@@ -1928,7 +1942,7 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
     CU_TRY(cudaMemcpyAsync(res, scores_dev + n_entries, 2 * (size_t)K * 4, cudaMemcpyDeviceToHost, m->st));
     CU_TRY(cudaMemcpyAsync(res + 2 * ts::kTopMax, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));
   }
-  CU_TRY(res_dev ? wait_results((const int32_t *)(res + 2 * ts::kTopMax + 1), 1, m->call_no, m->st) : cudaStreamSynchronize(m->st));
+  CU_TRY(res_dev && may_spin() ? wait_results((const int32_t *)(res + 2 * ts::kTopMax + 1), 1, m->call_no, m->st) : cudaStreamSynchronize(m->st));
   int dev_err;
   std::memcpy(&dev_err, res + 2 * ts::kTopMax, 4);
   if (dev_err != 0) {

@@ -1,5 +1,9 @@
 """ts_topk_cosine against the oracle's Top-K (Eq. 3), and the hidden state it takes as the query against the
 oracle's final-norm hidden state of the same row."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -65,6 +69,35 @@ def test_topk_at_the_edges_of_pieces_slices_and_lists(n, d, K):
     same = sorted({0, n // 2, n - 1})
     assert idx[:min(K, len(same))] == same[:K]
     gm.close()
+
+
+BLOCKING = r"""
+import ctypes, sys, time
+sys.path.insert(0, {root!r})
+cu = ctypes.CDLL("libcuda.so.1")   # CU_CTX_SCHED_BLOCKING_SYNC for the device's primary context, before anything makes it
+assert cu.cuInit(0) == 0 and cu.cuDevicePrimaryCtxSetFlags_v2(0, 4) == 0
+import torch, synth
+import paper_2604_13519_b200 as ts
+gm = ts.Model(synth.SHAPES["8b-2l"], max_pages=8, max_batch=1, k_max=8, max_rows=8, max_ctx=64, path=1)
+H = torch.ones(300000, 4096, device="cuda", dtype=torch.bfloat16)   # 2.5 GB: about 400 us a call
+H[7] = 0
+q = torch.ones(4096, device="cuda")
+want = ts.ts_topk_cosine(gm, H, 10, query=q)
+assert want[0] == [0, 1, 2, 3, 4, 5, 6, 8, 9, 10]
+cpu, wall = time.process_time(), time.perf_counter()
+for _ in range(500):
+    assert ts.ts_topk_cosine(gm, H, 10, query=q) == want
+print("share", (time.process_time() - cpu) / (time.perf_counter() - wall))
+"""
+
+
+def test_waits_keep_to_the_callers_choice_of_blocking():
+    """With the device set to blocking synchronisation a call's wait leaves the processor: a row of long calls takes 0.18 of
+    one; a wait that spins takes all of it."""
+    code = BLOCKING.format(root=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    assert float(r.stdout.split("share")[1]) < 0.6
 
 
 def test_zeros_of_either_sign_tie():
