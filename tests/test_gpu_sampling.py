@@ -3,6 +3,8 @@ uniforms on both sides: accepted length and emitted ids, trial after trial on on
 taken on floating point may differ only where the oracle's own margin is within the logit tolerance: an accept
 test with |u - p(x)| small, or a sample whose uniform lies next to the boundary of the GPU's id in the
 oracle's CDF."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -162,6 +164,23 @@ def test_sampled_acceptance_over_a_tree(name, ctx, n_nodes):
                 ref = want[torch.tensor(path)]
                 d = (got[ctx:].double() - ref).abs()
                 assert bool((d <= 1e-2 + 1e-2 * ref.abs()).all())
+    gm.close()
+
+
+@pytest.mark.parametrize("vocab", [128, 4224, 16384, 16512, 40064])
+def test_draws_at_vocabularies_around_the_widths_of_a_slice(vocab):
+    """Vocabularies of one slice, of slices that end early, of the longest slices that a warp takes the statistics of and the
+    shortest that a CTA does, and of several loads per thread: each draw against the oracle's running sum."""
+    shape = dataclasses.replace(synth.SHAPES["tiny"], name=f"v{vocab}", vocab=vocab)
+    om, gm = make_pair(shape, k_max=8, max_ctx=64, path=1)
+    cache, s, pending = synthetic_context(shape, om, gm, 20, pending=70)
+    T = 4.0
+    ref = om.verify(pending, [71, 72], cache.clone(), want_logits=True)["logits"]
+    cdf = torch.cumsum(oracle.target_probs(ref[0], T), 0).numpy()
+    for u in (0.0, 0.004, 0.13, 0.26, 0.51, 0.77, 0.96, 0.99999994):
+        res = ts.ts_verify_sampled(gm, [s], [[]], T, [u])[0]
+        tok, slack = res.emitted[0], LOGIT_MAX_ABS / T / 4
+        assert (cdf[tok - 1] if tok else 0.0) - slack <= u <= cdf[tok] + slack
     gm.close()
 
 
