@@ -31,22 +31,23 @@ __device__ __forceinline__ void cos_add(const uint4 &raw, const float4 &q0, cons
 }
 
 // q_dev != nullptr: the query as fp32 [d]; else the bf16 (hi[, lo]) planes of a row of the last step's hidden state.
-// piece = entries per stage (even); shared memory: the query (elements 8c .. 8c + 3 of all c, then 8c + 4 .. 8c + 7: reads
-// without bank conflicts), then a piece per warp.
+// piece = entries per stage; shared memory: the query (elements 8c .. 8c + 3 of all c, then 8c + 4 .. 8c + 7: reads
+// without bank conflicts), then a piece each for the first `bufs` warps (wide entries leave room for fewer than eight; all
+// warps bring the query in: with two warps doing it a store of one entry of 16384 took 15 us longer).
 __global__ void __launch_bounds__(32 * kCosWarps)
-cosine_scores_kernel(const __nv_bfloat16 *H, int N, int d, int piece, const float *q_dev, const __nv_bfloat16 *q_planes,
+cosine_scores_kernel(const __nv_bfloat16 *H, int N, int d, int piece, int bufs, const float *q_dev, const __nv_bfloat16 *q_planes,
                      int plane_stride, int planes, float *scores, int *err) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ float red[kCosWarps];
   __shared__ uint64_t bars[kCosWarps];
   pdl_launch_dependents();   // (the Top-K kernel waits for this one's end)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n_chunks = d / 8;                       // 8 bf16 = 16 bytes
   float4 *qa = reinterpret_cast<float4 *>(smem), *qb = qa + n_chunks;
   const uint32_t row_bytes = 2u * d, piece_bytes = piece * row_bytes;
   const uint8_t *src = smem + (size_t)d * 4 + (size_t)warp * piece_bytes;
   const uint32_t bar = smem_u32(&bars[warp]);
-  const int n_pieces = (N + piece - 1) / piece, step = gridDim.x * n_warps, p0 = blockIdx.x * n_warps + warp;
+  const int n_pieces = (N + piece - 1) / piece, step = gridDim.x * bufs, p0 = warp < bufs ? blockIdx.x * bufs + warp : n_pieces;
   const uint64_t pol = policy_evict_first();
   auto fetch = [&](int p) {   // (one lane)
     const uint32_t bytes = min(piece, N - p * piece) * row_bytes;
@@ -70,7 +71,7 @@ cosine_scores_kernel(const __nv_bfloat16 *H, int N, int d, int piece, const floa
   if (lane == 0) red[warp] = qq;
   __syncthreads();
   qq = 0.f;
-  for (int w = 0; w < n_warps; ++w) qq += red[w];
+  for (int w = 0; w < kCosWarps; ++w) qq += red[w];
   uint32_t ph = 0;
   for (int p = p0; p < n_pieces; p += step, ph ^= 1u) {
     if (!__all_sync(0xffffffffu, mbar_wait(bar, ph))) {
@@ -79,7 +80,7 @@ cosine_scores_kernel(const __nv_bfloat16 *H, int N, int d, int piece, const floa
     }
     const int e0 = p * piece, rows = min(piece, N - e0);
     for (int r = 0; r < rows; r += 2) {
-      // (the second of an odd last pair reads what an earlier piece left there, or nothing that counts)
+      // (the odd last entry of a piece is its pair's second too; nothing is kept of that)
       const uint4 *r0 = reinterpret_cast<const uint4 *>(src + (size_t)r * row_bytes);
       const uint4 *r1 = r + 1 < rows ? r0 + n_chunks : r0;
       float2 d0 = make_float2(0.f, 0.f), d1 = d0, n0 = d0, n1 = d0;
@@ -118,15 +119,15 @@ cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float
     if (e != cudaSuccess) return e;
     once.done(dev_);
   }
-  // entries per piece: about 16 KB, an even number
+  // entries per piece: about 16 KB, an even number (a single entry where a pair does not fit beside the query)
   int piece = std::max(2, kCosPieceBytes / (2 * d) / 2 * 2);
   while (piece > 1 && (size_t)d * 4 + (size_t)piece * 2 * d > kSmem) piece /= 2;
   const size_t piece_bytes = (size_t)piece * 2 * d;
   if ((size_t)d * 4 + piece_bytes > kSmem) return cudaErrorInvalidValue;
-  const int warps = (int)std::min<size_t>(kCosWarps, (kSmem - (size_t)d * 4) / piece_bytes);
+  const int bufs = (int)std::min<size_t>(kCosWarps, (kSmem - (size_t)d * 4) / piece_bytes);
   const int n_pieces = (N + piece - 1) / piece;
-  cosine_scores_kernel<<<std::min((n_pieces + warps - 1) / warps, n_sms), 32 * warps, (size_t)d * 4 + warps * piece_bytes, st>>>(
-      H, N, d, piece, q_dev, q_planes, plane_stride, planes, scores, err);
+  cosine_scores_kernel<<<std::min((n_pieces + bufs - 1) / bufs, n_sms), 32 * kCosWarps, (size_t)d * 4 + bufs * piece_bytes, st>>>(
+      H, N, d, piece, bufs, q_dev, q_planes, plane_stride, planes, scores, err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // candidates live behind the K result pairs: scores[N + 2K ...], 2 floats per candidate

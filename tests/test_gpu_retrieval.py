@@ -71,6 +71,26 @@ def test_topk_at_the_edges_of_pieces_slices_and_lists(n, d, K):
     gm.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 5, 601])
+@pytest.mark.parametrize("d", [5120, 16384])
+def test_wide_entries_leave_room_for_fewer_buffers(n, d):
+    """Entries of which the shared memory holds pieces for eight warps, and for two: one entry, odd counts, more than a
+    round of all SMs."""
+    shape = synth.ModelShape("wide", 1, d, 4, 4, 64, 256, 1024, 10000.0, 1e-5)
+    g = torch.Generator().manual_seed(n)
+    H = torch.randn(n, d, generator=g).to(torch.bfloat16)
+    q = torch.randn(d, generator=g)
+    H[n // 2] = q.to(torch.bfloat16)
+    gm = ts.Model(shape, max_pages=8, max_batch=1, k_max=8, max_rows=8, max_ctx=64, act_split=True, path=1)
+    K = min(n, 5)
+    idx, sc = ts.ts_topk_cosine(gm, H.cuda(), K, query=q.cuda())
+    s_all = oracle.cosine_scores(H, q)
+    want = torch.topk(s_all, K)
+    assert idx[0] == n // 2 and np.abs(np.array(sc) - want.values.numpy()).max() < 2e-6   # (fp32 sums, as above)
+    assert np.abs(s_all[torch.tensor(idx)].numpy() - want.values.numpy()).max() < 4e-6 and len(set(idx)) == K
+    gm.close()
+
+
 BLOCKING = r"""
 import ctypes, sys, time
 sys.path.insert(0, {root!r})
