@@ -20,12 +20,14 @@ sys.path.insert(0, {root!r}); sys.path.insert(0, {tests!r})
 from paper_2604_13519_b200 import build, binding
 build.build(debug_bounds=True)
 binding.use_debug_library()
-import test_gpu_parity as P, test_gpu_tree as T
+import test_gpu_parity as P, test_gpu_tree as T, test_gpu_prompts as Q
 P.test_c1_decode_loop_parity(1)
 P.test_synthetic_kv_single("8b-2l", 700, 64, 1)
 P.test_ragged_batch()
 P.test_row_counts_around_the_projection_kernels_switch("8b-2l", [33, 64, 64, 64, 64, 11])
 P.test_row_counts_around_the_projection_kernels_switch("1b-2l", [40, 33, 30])
+Q.check_prompt("tiny", 66, True)
+Q.check_prompt("tiny", 1090, True)
 for name in dir(T):
     if name.startswith("test_") and getattr(T, name).__code__.co_argcount == 0:
         getattr(T, name)()
