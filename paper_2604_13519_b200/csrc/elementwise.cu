@@ -198,71 +198,15 @@ __device__ __forceinline__ __half to_half_sat(float x) {
   return __float2half_rn(fminf(fmaxf(x, -65504.f), 65504.f));
 }
 
-static constexpr int kRopeWideRows = 65;   // steps of at least this many rows take the wide kernel (smaller ones have none)
-
-// grid = (M, Hq + 2*Hkv); one CTA of hd/2 threads per (row, head).  Thread i handles the rotary pair
-// (i, i + hd/2) of q or k heads, or elements (i, i + hd/2) of a v head.  Every load is issued before the first use
-// (the slabs, the row's position, sequence and slot): the kernel is two round trips to L2, not one per slab.
-__global__ void rope_kv_kernel(StepIn in, const float *part, int n_splits, int part_rows, int Hq, int Hkv, int hd,
-                               const float2 *rope_tab, __half *q_out, __half *q_lo_out, __half *k_pages, __half *v_pages,
-                               unsigned long long *stamp) {
-  if (threadIdx.x == 0) stamp_min(stamp);
-  pdl_launch_dependents();   // the dependent kernel waits for this one's end before touching its data
-  const int m = blockIdx.x, head = blockIdx.y, i = threadIdx.x, half = hd >> 1;
-  const int N = (Hq + 2 * Hkv) * hd;
-  // the step's integer inputs were copied in before the step's first kernel: they may be read before the wait
-  const int pos = in.pos[m], seq = in.row_seq[m], slot = in.slot[m];
-  const int page = (head >= Hq) ? in.block_tab[(size_t)seq * in.pages_per_seq + (slot >> 4)] : 0;
-  const bool pos_ok = ts_in_range(in.ck, CHK_POSITION, pos, in.ck.max_ctx);
-  const bool page_ok = ts_in_range(in.ck, CHK_PAGE_APPEND, page, in.ck.max_pages);
-  float2 cs = make_float2(1.f, 0.f);
-  if (head < Hq + Hkv && pos_ok) cs = rope_tab[(size_t)pos * half + i];
-  pdl_wait();
-  if (threadIdx.x == 0) stamp_waited(stamp);
-  // the QKV weight rows are stored with rotary partners adjacent: feature 2i = element i, 2i+1 = element i + hd/2
-  const int col = head * hd + 2 * i;
-  float2 p[kNormMaxSplits];
-#pragma unroll
-  for (int s = 0; s < kNormMaxSplits; ++s)
-    if (s < n_splits) p[s] = *reinterpret_cast<const float2 *>(part + ((size_t)s * part_rows + m) * N + col);
-  float a = 0.f, b = 0.f;
-#pragma unroll
-  for (int s = 0; s < kNormMaxSplits; ++s)
-    if (s < n_splits) { a += p[s].x; b += p[s].y; }
-  if (head < Hq + Hkv) {
-    const float ra = a * cs.x - b * cs.y;
-    const float rb = b * cs.x + a * cs.y;
-    a = ra; b = rb;
-  }
-  if (head < Hq) {
-    // the query as an fp16 pair (value, rounding remainder): the score product adds both, so the 11 bits of fp16
-    // do not limit the scores (the remainder of a saturated value is dropped)
-    const size_t qo = ((size_t)m * Hq + head) * hd;
-    const __half ha = to_half_sat(a), hb = to_half_sat(b);
-    q_out[qo + i] = ha;
-    q_out[qo + i + half] = hb;
-    if (q_lo_out) {
-      q_lo_out[qo + i] = __float2half_rn(fabsf(a) <= 65504.f ? a - __half2float(ha) : 0.f);
-      q_lo_out[qo + i + half] = __float2half_rn(fabsf(b) <= 65504.f ? b - __half2float(hb) : 0.f);
-    }
-  } else if (page_ok) {
-    const bool is_k = head < Hq + Hkv;
-    const int kh = is_k ? head - Hq : head - Hq - Hkv;
-    __half *dst = (is_k ? k_pages : v_pages) + (((size_t)page * Hkv + kh) * 16 + (slot & 15)) * hd;
-    dst[i] = to_half_sat(a);
-    dst[i + half] = to_half_sat(b);
-  }
-  if (threadIdx.x == 0) stamp_max(stamp ? stamp + 3 : nullptr);
-}
-
-// The same for steps of many rows: grid = (M, ceil(heads / 16)), block = (hd / 8, 16): a thread handles FOUR
+// After the many-rows projections: folds the QKV slabs in slab order, rotates q and k, writes q as an fp16 (value, remainder)
+// pair and k, v to their pages.  grid = (M, ceil(heads / 16)), block = (hd / 8, 16): a thread handles FOUR
 // neighbouring rotary pairs of one head (32 bytes per slab in one load, 8-byte stores), so a 256-row step is 768 CTAs
-// of 256 threads instead of 12 288 CTAs of 64 -- less than one wave of resident threads instead of nearly three.  The
-// sums are taken in the same order as above: the results are the same bits.  NS = most slabs: with room for twelve slabs'
+// of 256 threads -- less than one wave of resident threads, where a CTA per (row, head) is nearly three.  Every load is issued
+// before the first use (the row's position, sequence and slot before the wait, the slabs behind it).  NS = most slabs: with room for twelve slabs'
 // loads in registers only one or two CTAs fit on an SM (256 rows, three slabs: 12.5 us; 1024 rows, two slabs: 56), with room
 // for four or two all of them do (4.2 us; 15).
 template <int NS>
-__global__ void rope_kv_wide_kernel(StepIn in, const float *part, int n_splits, int part_rows, int Hq, int Hkv, int hd,
+__global__ void rope_kv_kernel(StepIn in, const float *part, int n_splits, int part_rows, int Hq, int Hkv, int hd,
                                     const float2 *rope_tab, __half *q_out, __half *q_lo_out, __half *k_pages,
                                     __half *v_pages, unsigned long long *stamp) {
   if (threadIdx.x == 0 && threadIdx.y == 0) stamp_min(stamp);
@@ -314,20 +258,19 @@ __global__ void rope_kv_wide_kernel(StepIn in, const float *part, int n_splits, 
 #pragma unroll
     for (int j = 0; j < 4; ++j) { ha[j] = to_half_sat(a[j]); hb[j] = to_half_sat(b[j]); }
     if (head < Hq) {
-      // the query as an fp16 pair (value, rounding remainder), as in rope_kv_kernel
+      // the score product adds both halves of a query's pair, so the 11 bits of fp16 do not limit the scores (the remainder of a
+      // saturated value is dropped)
       const size_t qo = ((size_t)m * Hq + head) * hd + i0;
       *reinterpret_cast<uint2 *>(q_out + qo) = *reinterpret_cast<const uint2 *>(ha);
       *reinterpret_cast<uint2 *>(q_out + qo + half) = *reinterpret_cast<const uint2 *>(hb);
-      if (q_lo_out) {
-        __align__(8) __half la[4], lb[4];
+      __align__(8) __half la[4], lb[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          la[j] = __float2half_rn(fabsf(a[j]) <= 65504.f ? a[j] - __half2float(ha[j]) : 0.f);
-          lb[j] = __float2half_rn(fabsf(b[j]) <= 65504.f ? b[j] - __half2float(hb[j]) : 0.f);
-        }
-        *reinterpret_cast<uint2 *>(q_lo_out + qo) = *reinterpret_cast<const uint2 *>(la);
-        *reinterpret_cast<uint2 *>(q_lo_out + qo + half) = *reinterpret_cast<const uint2 *>(lb);
+      for (int j = 0; j < 4; ++j) {
+        la[j] = __float2half_rn(fabsf(a[j]) <= 65504.f ? a[j] - __half2float(ha[j]) : 0.f);
+        lb[j] = __float2half_rn(fabsf(b[j]) <= 65504.f ? b[j] - __half2float(hb[j]) : 0.f);
       }
+      *reinterpret_cast<uint2 *>(q_lo_out + qo) = *reinterpret_cast<const uint2 *>(la);
+      *reinterpret_cast<uint2 *>(q_lo_out + qo + half) = *reinterpret_cast<const uint2 *>(lb);
     } else if (page_ok) {
       const bool is_k = head < Hq + Hkv;
       const int kh = is_k ? head - Hq : head - Hq - Hkv;
@@ -342,12 +285,10 @@ __global__ void rope_kv_wide_kernel(StepIn in, const float *part, int n_splits, 
 cudaError_t launch_rope_kv(const StepIn &in, const float *part, int n_splits, int part_rows, int Hq, int Hkv,
                            int hd, const float2 *rope_tab, __half *q_out, __half *q_lo_out, __half *k_pages,
                            __half *v_pages, cudaStream_t st, unsigned long long *stamp) {
-  if (in.M >= kRopeWideRows && hd % 8 == 0)
-    return launch_pdl(n_splits <= 2 ? rope_kv_wide_kernel<2> : n_splits <= 4 ? rope_kv_wide_kernel<4> : rope_kv_wide_kernel<kNormMaxSplits>,
-                      dim3(in.M, (Hq + 2 * Hkv + 15) / 16), dim3(hd / 8, 16), 0, st, in, part,
-                      n_splits, part_rows, Hq, Hkv, hd, rope_tab, q_out, q_lo_out, k_pages, v_pages, stamp);
-  return launch_pdl(rope_kv_kernel, dim3(in.M, Hq + 2 * Hkv), dim3(hd / 2), 0, st, in, part, n_splits,
-                    part_rows, Hq, Hkv, hd, rope_tab, q_out, q_lo_out, k_pages, v_pages, stamp);
+  if (hd % 8 || hd > 512 || n_splits > kNormMaxSplits) return cudaErrorInvalidValue;
+  return launch_pdl(n_splits <= 2 ? rope_kv_kernel<2> : n_splits <= 4 ? rope_kv_kernel<4> : rope_kv_kernel<kNormMaxSplits>,
+                    dim3(in.M, (Hq + 2 * Hkv + 15) / 16), dim3(hd / 8, 16), 0, st, in, part, n_splits, part_rows, Hq, Hkv, hd,
+                    rope_tab, q_out, q_lo_out, k_pages, v_pages, stamp);
 }
 
 // One CTA per source row; thread i moves 16 bytes.  Block (tile, kb) of the stored matrix starts at row

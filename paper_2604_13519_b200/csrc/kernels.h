@@ -54,7 +54,6 @@ struct GemmArgs {
   int Mc;               // activation rows per CTA: the step's rows rounded up (weight-streaming kernel), 128 (many rows)
   int planes;           // 1 = bf16 activations, 2 = (hi, lo) pair
   int n_kblocks;        // K / 64
-  int kb_per_split;     // k-blocks per split-K slice
   int stages;           // filled in by the launcher
   // many-rows kernel, filled in by the launcher: weight tiles of 256 rows (the tiles after them have 128), narrow tiles of the
   // CTAs with one wide tile less, row chunks, K slices
@@ -104,8 +103,8 @@ cudaError_t launch_embed_norm(const StepIn &in, const __nv_bfloat16 *embed, cons
 cudaError_t launch_add_norm(int M, int d, const float *part, int n_splits, int part_rows, const float *gain,
                             float eps, float *x, __nv_bfloat16 *h, int h_rows, int planes, cudaStream_t st,
                             unsigned long long *stamp = nullptr);
-// qkv = sum of split-K partials; rotary on q and k; q -> fp16 [M][Hq][hd] (and, if q_lo_out is given, the rounding
-// remainder of every element as a second fp16 array of the same shape); k, v -> fp16 pages
+// qkv = sum of split-K partials; rotary on q and k; q -> fp16 [M][Hq][hd] and the rounding remainder of
+// every element as a second array of the same shape; k, v -> fp16 pages
 cudaError_t launch_rope_kv(const StepIn &in, const float *part, int n_splits, int part_rows, int Hq, int Hkv,
                            int hd, const float2 *rope_tab, __half *q_out, __half *q_lo_out, __half *k_pages,
                            __half *v_pages, cudaStream_t st, unsigned long long *stamp = nullptr);
