@@ -256,7 +256,6 @@ struct ts_model {
   int64_t launches = 0, h2d = 0, d2h = 0;
   bool use_pdl = true;
   bool publish = false;                        // the step being enqueued writes its results to the pinned block itself
-  bool flagged = false;                        // ... and raises its sequences' words there
   int32_t call_no = 0;                         // number that the call being waited for ends with (see wait_results)
   int32_t *host_dev = nullptr;                 // the pinned block as the device sees it (null: it cannot write there)
   int32_t inject_err = 0;                      // test support: status code the next step or retrieval is made to report
@@ -630,7 +629,7 @@ ts_status run_step(ts_model *m) {
   if (m->publish) {
     ho.base = dout; ho.host = m->host_dev + L.in_ints; ho.err = dout + L.o_err;
     ho.number = m->call_no;
-    ho.done = m->flagged ? ho.host + L.o_done : nullptr;
+    ho.done = m->last_tree ? nullptr : ho.host + L.o_done;   // (a tree's step ends with the compaction, which publishes nothing)
   }
   if (m->staging && m->inject_err) CU_TRY(write_injected(m));
   if (m->last_sample) {
@@ -851,7 +850,7 @@ cudaError_t wait_results(const int32_t *words, int n, int32_t number, cudaStream
 }
 
 // Whether a wait may spin on the pinned block: not where the caller has the device's waits block or yield the processor
-// (cudaSetDeviceFlags; the stream's own synchronisation keeps to that).
+// (cudaSetDeviceFlags; the stream's own synchronisation keeps to that).  Asked when all is launched: it takes 0.1 us or more.
 bool may_spin() {
   unsigned flags = 0;
   if (cudaGetDeviceFlags(&flags) != cudaSuccess) {
@@ -887,8 +886,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const bool publishes = m->host_dev && !m->last_fused && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
 #endif
   m->publish = publishes;
-  const bool flagged = publishes && !m->last_tree && may_spin();   // (a tree's step ends with the compaction, which publishes nothing)
-  m->flagged = flagged;
+  const bool flagged = publishes && !m->last_tree;   // (a tree's step ends with the compaction, which publishes nothing)
   m->next_call();
   m->staging = true;
   ts_status st = run_step(m);
@@ -897,7 +895,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   if (m->inject_err) CU_TRY(write_injected(m));   // (a step without an acceptance kernel of its own)
   const size_t out_bytes = (size_t)((flags & TS_FLAG_WANT_TOPK) ? L.out_ints : L.o_topk) * 4;   // (the Top-K lists come last)
   if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
-  CU_TRY(flagged ? wait_results(m->h_out() + L.o_done, B, m->call_no, m->st) : cudaStreamSynchronize(m->st));
+  CU_TRY(flagged && may_spin() ? wait_results(m->h_out() + L.o_done, B, m->call_no, m->st) : cudaStreamSynchronize(m->st));
   const int32_t *ho = m->h_out();
   if (publishes) {   // (see ts::publish: the status; per sequence length, pending id, accepted drafts, maybe the call's number; a row's
                      // argmax; emitted ids and path)
