@@ -167,9 +167,13 @@ ts_status ts_session_create(ts_model *model, const ts_schema *schema, const ts_d
 ts_status ts_session_set_ranks(ts_session *s, const int32_t *ranks, int32_t n);
 ts_status ts_session_destroy(ts_session *s);
 
-/* Feed the prompt: the KV of tokens[0..n-2] is computed with the verify kernels (chunks of k_max,
- * LM head skipped) and tokens[n-1] becomes the pending token; every prompt id also passes through
- * the FSM's delta.  With a host-only session only the FSM part happens. */
+/* Feed the prompt: the KV of tokens[0..n-2] is computed with the verify kernels (LM head skipped) and
+ * tokens[n-1] becomes the pending token; every prompt id also passes through the FSM's delta.  With a
+ * host-only session only the FSM part happens.  The prompt goes through in pieces of up to 1024 rows
+ * (with the persistent kernel: of k_max).  Like any step of more than 64 rows a piece sums in an order of
+ * its own: the cached K/V agree to rounding, not bit for bit, with those of the same tokens fed through
+ * ts_verify, so a session re-opened with its prompt and output may differ in the last bits from the
+ * session that decoded them. */
 ts_status ts_prefill(ts_model *m, ts_session *s, const int32_t *tokens, int32_t n);
 
 /* ts_draft — drafting part of Algorithm 1's loop body.  Retrieval first (Eq. 4: suffix lengths
@@ -196,8 +200,10 @@ typedef struct {
 /* ts_verify — Verification + SelectLongestAcceptedPrefix for B sequences in one batched forward.
  * Sequence i's chunk is [pending_i, draft_tokens[draft_offsets[i] .. draft_offsets[i+1])], k_i rows
  * at positions len_i .. len_i+k_i-1.  Allocates KV pages as needed, copies the step's inputs to the
- * device, enqueues every kernel of the step, copies the result back and synchronises the stream.
- * The sessions are not advanced: ts_commit does that.  out: host, B entries.
+ * device, enqueues every kernel of the step and waits for its results.  On return they are complete, and
+ * so is all that the step wrote on the device; the stream itself may still count the last kernel as
+ * running for some microseconds (cudaStreamQuery).  The wait spins unless the device is set to blocking or yielding
+ * waits (cudaSetDeviceFlags), which it then uses.  The sessions are not advanced: ts_commit does that.  out: host, B entries.
  * Errors: TS_ERR_K_TOO_LARGE, TS_ERR_TOKEN_RANGE, TS_ERR_OOM_PAGES, TS_ERR_STATE (finished or
  * unprefilled session), TS_ERR_DEVICE_TIMEOUT, TS_ERR_CUDA. */
 ts_status ts_verify(ts_model *m, ts_session *const *sessions, int32_t B,
@@ -288,8 +294,8 @@ ts_status ts_verify_tree_sampled(ts_model *m, ts_session *const *sessions, int32
 ts_status ts_verify_replay(ts_model *m);
 
 /* Run the last step once more and return, per class, the summed milliseconds and a count:
- * 0 projection GEMM, 1 attention, 2 attention merge, 3 norm / residual, 4 rotary + KV append,
- * 5 acceptance, 6 the persistent kernel as a whole.  n_classes >= 6 (class 6 is written if
+ * 0 projection GEMM (up to 80 rows, 96 with one plane, with norm, residual, rotary and KV append in it), 1 attention,
+ * 2 attention merge, 3 norm / residual, 4 rotary + KV append, 5 acceptance, 6 the persistent kernel as a whole.  n_classes >= 6 (class 6 is written if
  * n_classes > 6).  With separate kernels an event follows every launch (no overlap between
  * kernels) and the count is the launches; with the persistent kernel classes 0..2 are sums of
  * its phases (time between the grid-wide ends of consecutive phases, read from device-side
@@ -328,8 +334,9 @@ ts_status ts_session_output(const ts_session *s, int32_t *out, int32_t cap, int3
  * query_dev: device fp32 [d_model], or NULL to use the final-norm hidden state of row `row` of the last step (row 0
  * of a session's first step is its question's last token).  scores_dev: device scratch of
  * TS_TOPK_SCRATCH_FLOATS(n_entries, K) floats, 8-byte aligned, owned by the caller, overwritten.  out_index / out_score: host, K entries (out_score may be NULL).  Ties go to the
- * lower index; an entry or query of zero norm scores -2 (ranks last).  Synchronises the model's stream.
- * Errors: TS_ERR_ARG (K outside [1, min(64, n_entries)], bad row), TS_ERR_STATE (no hidden state available). */
+ * lower index; an entry or query of zero norm scores -2 (ranks last).  Waits for the result as ts_verify does.
+ * Errors: TS_ERR_ARG (K outside [1, min(64, n_entries)], bad row), TS_ERR_STATE (no hidden state available),
+ * TS_ERR_DEVICE_TIMEOUT. */
 #define TS_TOPK_SCRATCH_FLOATS(n, k) ((n) + 2 * (k) + 1 + 2 * (k) * (((n) + 4095) / 4096))
 ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries, const float *query_dev,
                          int32_t row, int32_t K, float *scores_dev, int32_t *out_index, float *out_score);
@@ -366,11 +373,12 @@ ts_status ts_debug_restart(ts_session *s, int32_t cache_len, int32_t pending);
 ts_status ts_read_logits(ts_model *m, int32_t row0, int32_t n_rows, float *host_out);
 /* Copy the first `bytes` bytes of an internal activation buffer of the last step to host memory:
  * 0 residual stream x (float32 [rows_alloc][d_model]); 1 projection input activations (bf16
- * [planes][rows_alloc][d_model]; normalised with separate kernels, x times gain before the
- * row scale with the persistent kernel); 2 rotated queries (fp16 [rows_alloc][n_q_heads*head_dim], rounded values;
+ * [planes][rows_alloc][d_model]: the LM head's input, normalised; after a step that skipped the LM head, and with the
+ * persistent kernel, x times gain before the row scale, or normalised in steps of more than 80 rows, 96 with one plane); 2 rotated queries (fp16 [rows_alloc][n_q_heads*head_dim], rounded values;
  * the rounding remainders the attention kernel adds to them are kept beside them and are not returned);
  * 3 attention output (bf16 [planes][rows_alloc][n_q_heads*head_dim]); 4 SwiGLU output (bf16
- * [planes][rows_alloc][d_ffn]).  rows_alloc = max_rows rounded up to 128; planes = 1 + act_split. */
+ * [planes][rows_alloc][d_ffn]).  rows_alloc = max_rows rounded up to 128; planes = 1 + act_split.  After a prompt the
+ * buffers hold its last piece, as far as its last layer's K/V. */
 ts_status ts_debug_read_buffer(ts_model *m, int32_t which, void *host_out, uint64_t bytes);
 /* Device-side clocks (nanoseconds of the GPU's global timer, latest over the CTAs) that the
  * persistent kernel left during the last ts_profile_step: three rows of *n_phases entries —

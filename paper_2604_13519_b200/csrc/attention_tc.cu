@@ -16,9 +16,12 @@
 //            running one in steps, and only then is the row of sums multiplied down
 // A block is 1024 cycles of tensor-core work (24 instructions: both planes of Q and of P) and about 950 of softmax by one
 // warp per scheduler, latency on latency; with one group the two alternated and a block took 2000 cycles, with two the
-// one's softmax runs under the other's products: 1350.  What is left above 1024 is the issuing warp: an instruction is taken
+// one's softmax runs under the other's products: 1440 (four sessions with 64 rows each: from 8192 to 16384 tokens 62.1 -> 110.1
+// us for 55.3 blocks more per SM, at the 1660 MHz that the power cap left beside it; at head_dim 64 37.5 -> 67.4 at 1965 MHz,
+// 1060 cycles).  The rest of a launch, 14 us (7 at head_dim 64), is its CTAs' one or two units' set-up, first loads and way
+// out.  What is left above 1024 is the issuing warp: an instruction is taken
 // only when the ones before it are nearly done, so all that the warp does between two blocks leaves the tensor cores idle.
-// Four sessions of 8192 tokens with 64 rows each: 81 -> 70 us per launch; sixteen ragged ones: 114 -> 92.  (Measured and
+// Four sessions of 8192 tokens with 64 rows each: 81 -> 70 us per launch when the groups came; sixteen ragged ones: 114 -> 92.  (Measured and
 // slower: an issuing warp per group, 86 and 114 us; exponentials before the block's maximum is known, 75 and 103.)
 // Each unit writes an un-normalised partial output with its (max, sum); attn_merge_kernel adds a row's units.
 // Every wait is bounded; on expiry the CTA records an error word and leaves through the normal exit.

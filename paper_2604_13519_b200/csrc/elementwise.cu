@@ -103,7 +103,8 @@ norm_kernel(const int32_t *tokens, const __nv_bfloat16 *embed, const float *part
 // several rows share an SM (a 1024-thread CTA fills one alone: 1024 rows of the 8B shape took seven waves, 27 us; now
 // 14, and 256 rows with four slabs 5.8 instead of 7.3).
 static constexpr int kNormRowsThreads = 256;
-static constexpr int kNormChunks = 4;      // d <= 4096
+static constexpr int kNormChunks = 4;      // d <= 4096; a wider row and its slabs would not fit the registers of two CTAs per SM, and takes
+                                           // the form above (not tried otherwise)
 template <int NS>   // most slabs: all loads are issued before the first sum
 __global__ void __launch_bounds__(kNormRowsThreads, NS == 1 ? 5 : NS == 2 ? 4 : NS == 3 ? 3 : 2)
 norm_rows_kernel(const float *part, int n_splits, int part_rows, const float *gain, float eps, int d, float *x,

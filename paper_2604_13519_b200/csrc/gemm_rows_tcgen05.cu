@@ -1,4 +1,5 @@
-// The dense projections of the verify step for MANY rows (batched steps: more than 64 rows), where the work is bound by
+// The dense projections of the verify step for MANY rows (batched steps and prompts: more than the weight-streaming kernel
+// takes, 80 rows or 96 with one plane of activations), where the work is bound by
 // the tensor cores and by the bytes an SM pulls from L2 per flop, no longer by streaming the weights:
 //     out[m][n] = sum_k act[m][k] * W[n][k]
 // Orientation: a CTA owns a chunk of 128 activation rows (operand A of the tensor-core instruction, its 128-row

@@ -5,7 +5,7 @@
 // The weight matrix is stored as contiguous 128 x 64 blocks (one TMA box each).
 // Operands are swapped with respect to the usual layout so that the 128-row dimension of the
 // tensor-core instruction runs over output features: a CTA owns 128 rows of W (operand A, K-major,
-// 16 KB per 64-wide k-block) and the step's activation rows, at most 128 (operand B).  Activations can
+// 16 KB per 64-wide k-block) and the step's activation rows, at most 80 or, with one plane, 96 (operand B).  Activations can
 // be fed as a (hi, lo) bf16 pair stacked along the instruction's N dimension, so one MMA multiplies
 // the weight tile with both halves; the epilogue adds the two column groups.  The accumulator lives
 // in tensor memory: lane = output feature, column = activation row.

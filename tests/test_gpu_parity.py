@@ -433,7 +433,7 @@ def test_commit_is_checked_against_the_verified_chunk():
 @pytest.mark.parametrize("path", PATHS)
 def test_device_timeout_is_reported_and_survived(path):
     """The host's handling of an expired device-side wait, without making the GPU wait: the status word is written on
-    the stream after the step's last kernel (no kernel sees it).  The step fails with TS_ERR_DEVICE_TIMEOUT, the
+    the stream behind the last kernel that waits for anything.  The step fails with TS_ERR_DEVICE_TIMEOUT, the
     session is untouched, and the next step is parity-green again."""
     shape = synth.SHAPES["1b-2l"]
     om, gm = make_pair(shape, k_max=16, max_ctx=512, path=path)
@@ -457,7 +457,7 @@ def test_device_timeout_is_reported_and_survived(path):
 
 def test_device_index_check_is_reported_and_survived():
     """The host's handling of a failed index check of the debug build, exercised the same way (a status word written
-    after the step's last kernel; the release build's kernels contain no checks): TS_ERR_DEVICE_BOUNDS with the check's
+    ahead of the acceptance kernel; the release build's kernels contain no checks): TS_ERR_DEVICE_BOUNDS with the check's
     number, session untouched, next step clean."""
     shape = synth.SHAPES["1b-2l"]
     om, gm = make_pair(shape, k_max=16, max_ctx=512)
