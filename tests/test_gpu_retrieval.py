@@ -98,26 +98,35 @@ cu = ctypes.CDLL("libcuda.so.1")   # CU_CTX_SCHED_BLOCKING_SYNC for the device's
 assert cu.cuInit(0) == 0 and cu.cuDevicePrimaryCtxSetFlags_v2(0, 4) == 0
 import torch, synth
 import paper_2604_13519_b200 as ts
-gm = ts.Model(synth.SHAPES["8b-2l"], max_pages=8, max_batch=1, k_max=8, max_rows=8, max_ctx=64, path=1)
+gm = ts.Model(synth.SHAPES["8b-2l"], max_pages=160, max_batch=16, k_max=64, max_rows=1024, max_ctx=160, path=1)
+gm._raw[0].zero_()
 H = torch.ones(300000, 4096, device="cuda", dtype=torch.bfloat16)   # 2.5 GB: about 400 us a call
 H[7] = 0
 q = torch.ones(4096, device="cuda")
 want = ts.ts_topk_cosine(gm, H, 10, query=q)
 assert want[0] == [0, 1, 2, 3, 4, 5, 6, 8, 9, 10]
-cpu, wall = time.process_time(), time.perf_counter()
-for _ in range(500):
-    assert ts.ts_topk_cosine(gm, H, 10, query=q) == want
-print("share", (time.process_time() - cpu) / (time.perf_counter() - wall))
+ss = [ts.Session(gm, None, None) for _ in range(16)]
+for s in ss:
+    s.set_cache(64, 70)
+drafts = [list(range(100, 163))] * 16   # 1024 rows: about 1.5 ms a call
+assert all(r.argmax[0] == 0 for r in ts.ts_verify(gm, ss, drafts))   # (weights of zero: a tie of all ids)
+for call in (lambda: ts.ts_topk_cosine(gm, H, 10, query=q) == want, lambda: ts.ts_verify(gm, ss, drafts)):
+    cpu, wall = time.process_time(), time.perf_counter()
+    for _ in range(300):
+        assert call()
+    print("share", (time.process_time() - cpu) / (time.perf_counter() - wall))
 """
 
 
 def test_waits_keep_to_the_callers_choice_of_blocking():
-    """With the device set to blocking synchronisation a call's wait leaves the processor: a row of long calls takes 0.18 of
-    one; a wait that spins takes all of it."""
+    """With the device set to blocking synchronisation a call's wait leaves the processor: a row of long retrievals takes 0.18
+    of one, of long steps (which this process prepares, too) more; a wait that spins takes all of it."""
     code = BLOCKING.format(root=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
-    assert float(r.stdout.split("share")[1]) < 0.6
+    shares = [float(x) for x in r.stdout.split("share")[1:]]
+    print(shares)
+    assert len(shares) == 2 and shares[0] < 0.5 and shares[1] < 0.8
 
 
 def test_zeros_of_either_sign_tie():
