@@ -828,9 +828,11 @@ ts_status build_attention(ts_model *m, const StepIo &I, int B, int M, int tables
 }
 
 // Waits for n words of the pinned block that take the call's number when the last kernel on the stream has written its results
-// (a number of the call's own: a kernel left over from a call that ended early cannot end a later one); by then all kernels before it are complete and it has nothing left to do.  3.5 us sooner than the stream's own
-// synchronisation, which learns of the kernel's end by way of the driver (ten small kernels in a row: 52.1 -> 48.8 us; the
-// two-layer shape's step 77.1 -> 75.1, a retrieval over 100 000 entries 149.2 -> 147.7).  The stream is still asked from time to time, so that a failed launch or kernel ends the wait with its error.
+// (a number of the call's own: a kernel left over from a call that ended early cannot end a later one); by then all kernels
+// before it are complete and it has nothing left to do.  3.5 us sooner than the stream's own synchronisation, which learns of
+// the kernel's end by way of the driver (ten small kernels in a row: 52.1 -> 48.8 us; the two-layer shape's step 77.1 -> 75.1, a
+// retrieval over 100 000 entries 149.2 -> 147.7).  The stream is still asked from time to time, so that a failed launch or
+// kernel ends the wait with its error.
 cudaError_t wait_results(const int32_t *words, int n, int32_t number, cudaStream_t st) {
   const volatile int32_t *w = words;
   for (uint32_t it = 1;; ++it) {
@@ -897,8 +899,9 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   if (!publishes) CU_TRY(cudaMemcpyAsync(m->h_out(), m->d_out(), out_bytes, cudaMemcpyDeviceToHost, m->st));
   CU_TRY(flagged && may_spin() ? wait_results(m->h_out() + L.o_done, B, m->call_no, m->st) : cudaStreamSynchronize(m->st));
   const int32_t *ho = m->h_out();
-  if (publishes) {   // (see ts::publish: the status; per sequence length, pending id, accepted drafts, maybe the call's number; a row's
-                     // argmax; emitted ids and path)
+  if (publishes) {
+    // (see ts::publish: the status; per sequence length, pending id, accepted drafts and maybe the call's number; a row's
+    // argmax; emitted ids and path)
     int64_t words = 1 + (3 + flagged) * (int64_t)B + M;
     for (int i = 0; i < B; ++i) words += 2 * (ho[L.o_accept + i] + 1);
     m->d2h += 4 * words;
@@ -1935,12 +1938,14 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
   m->next_call();
   if (m->inject_err) CU_TRY(write_injected(m));
   CU_TRY(ts::launch_topk_cosine((const __nv_bfloat16 *)hidden_dev, n_entries, m->c.d_model, query_dev, planes,
-                                (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms, ts::PairsOut{res_dev, m->call_no}, m->d_out() + m->L.o_err, m->st));
+                                (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms,
+                                ts::PairsOut{res_dev, m->call_no}, m->d_out() + m->L.o_err, m->st));
   if (!res_dev) {
     CU_TRY(cudaMemcpyAsync(res, scores_dev + n_entries, 2 * (size_t)K * 4, cudaMemcpyDeviceToHost, m->st));
     CU_TRY(cudaMemcpyAsync(res + 2 * ts::kTopMax, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));
   }
-  CU_TRY(res_dev && may_spin() ? wait_results((const int32_t *)(res + 2 * ts::kTopMax + 1), 1, m->call_no, m->st) : cudaStreamSynchronize(m->st));
+  CU_TRY(res_dev && may_spin() ? wait_results((const int32_t *)(res + 2 * ts::kTopMax + 1), 1, m->call_no, m->st)
+                               : cudaStreamSynchronize(m->st));
   int dev_err;
   std::memcpy(&dev_err, res + 2 * ts::kTopMax, 4);
   if (dev_err != 0) {
