@@ -1,0 +1,43 @@
+"""Steps whose projections run on the kernel of CTA pairs, against the oracle, at the row counts where its cut changes: a chunk of
+rows that is a whole number of sixteens and one row more, one chunk and two, chunks of different length, and tiles that are left
+over and cut along K (8B layers: 96 gate-up tiles on 74 pairs); also on a shape all of whose matrices have an odd number of
+128-row blocks, so that a pair's second CTA has none in the last tile."""
+import pytest
+
+import synth
+import paper_2604_13519_b200 as ts
+from gpu_util import check_step, make_pair, synthetic_context
+from synth.shapes import ModelShape
+from test_gpu_parity import _rand_draft
+
+pytestmark = pytest.mark.gpu
+
+ODD = ModelShape("odd", 2, 384, 3, 3, 128, 1088, 33 * 128, 10000.0, 1e-5)   # 9, 3, 17, 3 and 33 blocks
+
+
+@pytest.mark.parametrize("name,rows", [("odd", 97), ("odd", 113), ("odd", 257), ("odd", 530), ("tiny", 112), ("tiny", 273),
+                                       ("1b-2l", 97), ("1b-2l", 144), ("1b-2l", 145), ("1b-2l", 272), ("1b-2l", 400),
+                                       ("8b-2l", 113), ("8b-2l", 200), ("8b-2l", 257)])
+@pytest.mark.parametrize("act_split", [True, False], ids=["two_planes", "one_plane"])
+def test_rows_of_a_pair(name, rows, act_split):
+    shape = ODD if name == "odd" else synth.SHAPES[name]
+    n = (rows + 63) // 64
+    ks = [rows // n + (i < rows % n) for i in range(n)]
+    om, gm = make_pair(shape, max_batch=n, k_max=64, max_rows=rows, max_ctx=512, act_split=act_split)
+    sess, drafts, refs = [], [], []
+    for i, k in enumerate(ks):
+        cache, s, pending = synthetic_context(shape, om, gm, 40 + 37 * i, stream=i, pending=300 + i)
+        sess.append(s)
+        drafts.append(_rand_draft(shape.vocab, k - 1, 70 + i))
+        refs.append(om.verify(pending, drafts[-1], cache, want_logits=True))
+    row = 0
+    for i, (res, ref) in enumerate(zip(ts.ts_verify(gm, sess, drafts), refs)):
+        logits = gm.read_logits(row, res.k)
+        if act_split:
+            check_step(res, logits, ref, f"{name}, {rows} rows, seq {i}")
+        else:
+            # (bf16 roundings of all activations: 1e-2 of the logits' norm seen on these depths, four times that allowed)
+            lo = ref["logits"].numpy()
+            assert ((logits - lo) ** 2).sum() <= 4e-2 ** 2 * (lo ** 2).sum(), (name, rows, i)
+        row += res.k
+    gm.close()
