@@ -22,11 +22,13 @@ static constexpr int kBlockK = 64;                 // k-block: 64 bf16 = 128 byt
 static constexpr int kTileN = 128;                 // weight rows per CTA
 static constexpr int kWBytes = kTileN * kBlockK * 2;
 static constexpr int kMaxStages = 8;
+static constexpr int kPushRows = 16;               // most rows whose sums are sent (see launch_gemm)
 
-struct __align__(8) GemmSmemCtl {
+struct __align__(16) GemmSmemCtl {
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
   uint64_t tmem_full;
+  uint64_t got;            // clusters that send their sums: those of this CTA's rows are here, from all K slices
   uint32_t tmem_base;
   uint32_t abort_flag;
   float rs[128];  // per activation row: 1 / rms of the input (1 where the input is normalised already)
@@ -47,13 +49,14 @@ __device__ __forceinline__ long long kv_place(const GemmArgs &g, int m, int head
 }
 __device__ __forceinline__ void add4(float4 &s, const float4 &v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
 
-template <int EPI>
+// PUSH (QKV, RESID): sums are sent to the CTAs that finish the rows, see launch_gemm.  (A template argument: a branch at each load
+// of a sum keeps the loads from being issued together, 0.7 to 1.2 us per launch.)
+template <int EPI, bool PUSH>
 __global__ void __launch_bounds__(192, 1)
 gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_a,
                const GemmArgs g) {
-  extern __shared__ uint8_t smem_raw[];
   // 1024-byte alignment is required by the 128-byte swizzle pattern
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem[];
   const int a_bytes = g.planes * g.Mc * kBlockK * 2;
   const int stage_bytes = kWBytes + a_bytes;
   GemmSmemCtl *ctl = reinterpret_cast<GemmSmemCtl *>(smem + (size_t)g.stages * stage_bytes);
@@ -79,7 +82,12 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     }
     mbar_init(smem_u32(&ctl->tmem_full), 1);
     ctl->abort_flag = 0;
+    if constexpr (kCluster) mbar_init(smem_u32(&ctl->got), 1);
     fence_barrier_init();
+    if constexpr (kCluster) {
+      const int C = (int)gridDim.y, per = (g.M + C - 1) / C;
+      if constexpr (PUSH) mbar_expect_tx(smem_u32(&ctl->got), C * min(per, max(0, g.M - split * per)) * kTileN * 4);
+    }
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&ctl->tmem_base), alloc_cols);
@@ -88,6 +96,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if constexpr (PUSH) cluster_arrive();   // (this CTA's barrier is set up: waited for before the first sums are sent)
   const uint32_t tmem_base = ctl->tmem_base;
   if (threadIdx.x == 0) stamp_min(g.stamp);
   // Let the next kernel launch now: it waits (griddepcontrol.wait) for this one to finish before it touches
@@ -251,9 +260,29 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t stg = smem_u32(smem);
+    // Sums sent (see launch_gemm): [slice][row of the CTA's][128 features] behind the control block of the CTA that finishes the rows.
+    const uint32_t inbox = smem_u32(ctl + 1), got = smem_u32(&ctl->got);
+    int to_row = 0, to = 0;    // the next row is row `to_row` of CTA `to`
+    uint32_t to_box = 0, to_bar = 0;
+    auto send_to = [&](int r) {
+      to = r;
+      to_row = 0;
+      to_box = cluster_addr(inbox + (split * rows_per * kTileN + q * 32 + lane) * 4, r);
+      to_bar = cluster_addr(got, r);
+    };
+    if constexpr (PUSH) {
+      cluster_wait();   // (all CTAs of the cluster are set up: long since)
+      send_to(0);
+    }
     // (columns past the step's last row are read too and never used)
     auto put = [&](int c, uint32_t lo, uint32_t hi) {
-      st_shared_f32(stg + (c * kTileN + q * 32 + lane) * 4, __uint_as_float(lo) + (g.planes == 2 ? __uint_as_float(hi) : 0.f));
+      const float v = __uint_as_float(lo) + (g.planes == 2 ? __uint_as_float(hi) : 0.f);
+      if constexpr (!PUSH) {
+        st_shared_f32(stg + (c * kTileN + q * 32 + lane) * 4, v);
+      } else if (c < g.M && ok) {
+        st_async_f32(to_box + to_row * kTileN * 4, v, to_bar);
+        if (++to_row == rows_per && c + 1 < g.M) send_to(to + 1);
+      }
     };
     int c0 = 0;
     for (; c0 + 16 <= g.Mc; c0 += 16) {
@@ -272,7 +301,16 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 #pragma unroll
       for (int j = 0; j < 8; ++j) put(c0 + j, r[j], r2[j]);
     }
-    if constexpr (kCluster) {
+    if constexpr (PUSH) {
+      if (m_beg < m_end) {
+        const bool here = __all_sync(0xffffffffu, mbar_wait_cluster(got, 0));
+        if (!here) {
+          if (lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
+          *reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) = 1;
+        }
+        ok = ok && here;
+      }
+    } else if constexpr (kCluster) {
       __syncwarp();
       cluster_arrive();
       cluster_wait();
@@ -280,20 +318,28 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
       epilogue_sync();
     }
     // (a warp's rows two at a time: all their partial sums are fetched before the first is worked on)
-    bool left = !kCluster;   // this CTA has read all that it needs from the others
+    bool left = !kCluster || PUSH;   // this CTA has read all that it needs from the others
 #pragma unroll 1
     for (int mg = m_beg + warp - 2, i0 = 0; ok && mg < m_end; mg += 8, i0 += 2) {
       float4 sum[2];
       if constexpr (kCluster) {
         float4 p[2][8];
         const bool two = mg + 4 < m_end;
+        auto part = [&](int m, int c) {
+          if constexpr (PUSH) {
+            const uint4 v = ld_shared_v4(inbox + ((c * rows_per + m - m_beg) * kTileN + lane * 4) * 4);
+            return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+          } else {
+            return ld_cluster_v4(stg + (m * kTileN + lane * 4) * 4, c);
+          }
+        };
 #pragma unroll
         for (int c = 0; c < 8; ++c)
-          if (c < C) p[0][c] = ld_cluster_v4(stg + (mg * kTileN + lane * 4) * 4, c);
+          if (c < C) p[0][c] = part(mg, c);
         if (two) {
 #pragma unroll
           for (int c = 0; c < 8; ++c)
-            if (c < C) p[1][c] = ld_cluster_v4(stg + ((mg + 4) * kTileN + lane * 4) * 4, c);
+            if (c < C) p[1][c] = part(mg + 4, c);
         }
         sum[0] = p[0][0];
 #pragma unroll
@@ -305,7 +351,7 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
           for (int c = 1; c < 8; ++c)
             if (c < C) add4(sum[1], p[1][c]);
         }
-        if (mg + 8 >= m_end) {   // (nothing is left to read: the others may go; they are waited for at the end)
+        if (!PUSH && mg + 8 >= m_end) {   // (nothing is left to read: the others may go; they are waited for at the end)
           __syncwarp();
           cluster_arrive();
           left = true;
@@ -411,14 +457,18 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
   }
   if constexpr (kCluster) {
     // (every thread of the cluster takes part in both barriers: the sums are in shared memory, then: nobody reads mine
-    // any more; the waits inside the roles are bounded and all of them lead here)
+    // any more; the waits inside the roles are bounded and all of them lead here.  Where sums are sent: everybody is set up.)
     __syncwarp();
-    if (warp < 2) {
-      cluster_arrive();
+    if constexpr (PUSH) {
+      if (warp < 2) cluster_wait();
+    } else {
+      if (warp < 2) {
+        cluster_arrive();
+        cluster_wait();
+        cluster_arrive();
+      }
       cluster_wait();
-      cluster_arrive();
     }
-    cluster_wait();
   }
   tc_fence_before();
   __syncthreads();
@@ -427,10 +477,19 @@ gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     tmem_dealloc(tmem_base, alloc_cols);
   }
   if (threadIdx.x == 0 && g.stamp) stamp_max(g.stamp + 3);
+  if constexpr (PUSH) {
+    // All that is sent to this CTA has arrived, or it has given up: then it waits until the others are through (threads that
+    // have left count as such), since its shared memory has to be there while they may still send to it.
+    if (*reinterpret_cast<volatile uint32_t *>(&ctl->abort_flag) != 0) {
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+    }
+  }
 }
 
 static size_t gemm_smem_bytes(int stages, int planes, int Mc) {
-  return (size_t)stages * (kWBytes + planes * Mc * kBlockK * 2) + sizeof(GemmSmemCtl) + 1024;
+  return (size_t)stages * (kWBytes + planes * Mc * kBlockK * 2) + sizeof(GemmSmemCtl);
 }
 
 int gemm_pick_stages(int planes, int Mc, size_t smem_budget) {
@@ -439,13 +498,13 @@ int gemm_pick_stages(int planes, int Mc, size_t smem_budget) {
   return s;
 }
 
-template <int EPI>
+template <int EPI, bool PUSH = false>
 static cudaError_t launch_one(const CUtensorMap &tw, const CUtensorMap &ta, const GemmArgs &g, dim3 grid,
                               size_t smem, cudaStream_t st, bool pdl) {
   static PerDeviceOnce once;
   int dev_ = -1;
   if (once.needed(&dev_)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_ws_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(gemm_ws_kernel<EPI, PUSH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          227 * 1024);
     if (e != cudaSuccess) return e;
     once.done(dev_);
@@ -471,7 +530,7 @@ static cudaError_t launch_one(const CUtensorMap &tw, const CUtensorMap &ta, cons
   }
   cfg.attrs = at;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, gemm_ws_kernel<EPI>, tw, ta, g);
+  return cudaLaunchKernelEx(&cfg, gemm_ws_kernel<EPI, PUSH>, tw, ta, g);
 }
 
 // (asked about a kernel without tensor memory: for one with it the occupancy call answers one CTA per SM)
@@ -503,15 +562,21 @@ int gemm_max_clusters(int cluster, size_t smem_budget) {
 cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int cluster,
                         size_t smem_budget, cudaStream_t st, bool pdl) {
   g.stages = gemm_pick_stages(g.planes, g.Mc, smem_budget);
-  const size_t smem = gemm_smem_bytes(g.stages, g.planes, g.Mc);
+  size_t smem = gemm_smem_bytes(g.stages, g.planes, g.Mc);
   const bool split = epi == EPI_QKV || epi == EPI_RESID;
+  // Few rows: a CTA's sums go straight to the CTAs that finish the rows, 4 bytes per lane, counted by a barrier there, instead of
+  // being fetched from it: one way through the cluster and no barriers of the cluster at the end (8B shape, one row: 76.4 -> 74.8
+  // us per layer).  By 33 rows the small stores cost more than that (QKV of the 1B shape 5.1 -> 6.0 us, at 76 rows 8.1 -> 9.5).
+  const size_t inbox = (size_t)cluster * ((g.M + cluster - 1) / cluster) * kTileN * 4;
+  const bool push = split && cluster > 1 && g.M <= kPushRows && smem + inbox <= smem_budget;
+  if (push) smem += inbox;
   if (g.N % kTileN || g.M > g.Mc || g.Mc % 8 || (g.planes * g.Mc) % 16 || cluster < 1 || cluster > (split ? 8 : 1) ||
-      cluster > g.n_kblocks || (int)(smem - 1024 - sizeof(GemmSmemCtl)) < g.Mc * kTileN * 4)
+      cluster > g.n_kblocks || g.stages * (kWBytes + g.planes * g.Mc * kBlockK * 2) < g.Mc * kTileN * 4)
     return cudaErrorInvalidValue;
   const dim3 grid(g.N / kTileN, cluster);
   switch (epi) {
-    case EPI_QKV: return launch_one<EPI_QKV>(tw, ta, g, grid, smem, st, pdl);
-    case EPI_RESID: return launch_one<EPI_RESID>(tw, ta, g, grid, smem, st, pdl);
+    case EPI_QKV: return push ? launch_one<EPI_QKV, true>(tw, ta, g, grid, smem, st, pdl) : launch_one<EPI_QKV>(tw, ta, g, grid, smem, st, pdl);
+    case EPI_RESID: return push ? launch_one<EPI_RESID, true>(tw, ta, g, grid, smem, st, pdl) : launch_one<EPI_RESID>(tw, ta, g, grid, smem, st, pdl);
     case EPI_SWIGLU: return launch_one<EPI_SWIGLU>(tw, ta, g, grid, smem, st, pdl);
     case EPI_LOGITS: return launch_one<EPI_LOGITS>(tw, ta, g, grid, smem, st, pdl);
     default: return cudaErrorInvalidValue;
