@@ -5,8 +5,9 @@
 // shared memory as the other.  The rows of a step are the N of the instruction, which comes in steps of 16: a step of 144 rows is
 // one chunk of 144, where the row-major kernel (gemm_rows_tcgen05.cu) works on two of 128 -- what a step of few more rows than a
 // multiple of 128 gains most (8B shape, per layer under the power cap: 144 rows 208 -> 148 us, 192 rows 229 -> 176, 288 rows 283 ->
-// 246).  The (hi, lo) bf16 planes of the activations are two instructions into the SAME sums.  The sums lie in tensor memory,
-// lane = weight row, column = activation row, in two sets: the loads and products of a pair's next tile run under the epilogue of
+// 246).  The (hi, lo) bf16 planes of the activations are two instructions into the SAME sums, or, in chunks of up to 128 rows, one
+// instruction into sums of their own, added in the epilogue as the weight-streaming kernel adds them.  The sums lie in tensor
+// memory, lane = weight row, column = activation row, in two sets: the loads and products of a pair's next tile run under the epilogue of
 // this one.  A k-block is 0.64 us at 256 rows (floor 0.52 at 1965 MHz), 0.35 at 144.
 //
 // The launch is persistent, at most one pair per two SMs.  Every pair has the same number of whole tiles; the tiles that are
@@ -38,6 +39,7 @@ struct __align__(8) PairSmemCtl {
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t last;               // this CTA completed the tile whose slab it wrote last
+  float rs[2][128];            // [item in turn][row]: 1 / rms of the input (where it is not normalised yet: g.ss)
 };
 static constexpr int kFoldAhead = 3;                       // slabs that are read at a time
 static constexpr int kPassRows = 16;                       // activation rows that an epilogue group stages at a time
@@ -91,8 +93,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_rank(), pair = blockIdx.x >> 1, P = gridDim.x >> 1;
   const int n_blocks = g.N / kBoxN;
+  const bool apart = g.planes == 2 && g.chunk_rows <= 128;   // the planes' sums in columns of their own
+  const int set_cols = apart ? 2 * g.chunk_rows : g.chunk_rows;
   uint32_t alloc_cols = 32;
-  while (alloc_cols < 2u * g.chunk_rows) alloc_cols <<= 1;
+  while (alloc_cols < 2u * set_cols) alloc_cols <<= 1;
 
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmap_w);
@@ -179,7 +183,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     bool ok = rank == 0;
     for (int j = 0; ok && pair_item(g, pair, P, j, t); ++j) {
       const int b = j & 1;
-      const uint32_t idesc = umma_idesc_bf16(2 * kBoxN, (uint32_t)t.rows), d = tmem_base + b * g.chunk_rows;
+      // (planes apart: a CTA's half of B is its half of the rows of the value plane, then the same of the remainder plane)
+      const uint32_t idesc = umma_idesc_bf16(2 * kBoxN, (uint32_t)(apart ? 2 * t.rows : t.rows)), d = tmem_base + b * set_cols;
+      const int instr = apart ? 1 : g.planes;
       const uint32_t lo16 = (uint32_t)(t.rows / 2 * kBlockK * 2) >> 4;   // from the value plane to the remainder plane
       // this set's previous sums have been read out
       if (j >= 2 && !__all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&ctl->acc_empty[b]), ((j >> 1) - 1) & 1))) {
@@ -198,7 +204,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         const uint64_t da = umma_desc_sw128(sa), db = umma_desc_sw128(sa + kBoxBytes);
         if (elect_one()) {
           // the value plane and the remainder plane of the activations into the same sums
-          for (int pl = 0; pl < g.planes; ++pl) {
+          for (int pl = 0; pl < instr; ++pl) {
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk)   // 16 bf16 along K = 32 bytes = 2 descriptor address units
               umma_bf16_pair(d, da + 2 * kk, db + pl * lo16 + 2 * kk, idesc, (it | kk | pl) != 0);
@@ -234,6 +240,16 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     PairItem t;
     for (int j = 0; pair_item(g, pair, P, j, t); ++j) {
       const int b = j & 1;
+      if constexpr (EPI == EPI_SWIGLU) {
+        const int r = (int)threadIdx.x - 64;
+        if (g.ss && r < t.rows && t.m0 + r < g.M) {
+          const float *p = g.ss + (size_t)(t.m0 + r) * g.ss_tiles;
+          float f = 0.f;
+#pragma unroll 8
+          for (int i = 0; i < g.ss_tiles; ++i) f += p[i];
+          ctl->rs[b][r] = rsqrtf(f * g.inv_d + g.eps);
+        }
+      }
       bool ok = __all_sync(0xffffffffu, mbar_wait_cluster(smem_u32(&ctl->acc_full[b]), (j >> 1) & 1));
       if (!ok && lane == 0) atomicExch(g.err, DEV_TIMEOUT_TMEM);
       tc_fence_after();
@@ -248,10 +264,16 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       if (!all_ok) break;
       const int blk = 2 * t.wt + rank, n = blk * kBoxN + lane * 4;   // this lane's features n .. n + 3 in the second pass
       const int rows = blk < n_blocks ? min(t.rows, g.M - t.m0) : 0;
-      const uint32_t tacc = taddr + b * g.chunk_rows;
+      const uint32_t tacc = taddr + b * set_cols;
       // what becomes of row r of the chunk, by a whole warp
-      auto finish = [&](int r, const float4 &v) {
+      auto finish = [&](int r, float4 v) {
         const int m = t.m0 + r;
+        if constexpr (EPI == EPI_SWIGLU) {
+          if (g.ss) {
+            const float f = ctl->rs[b][r];
+            v.x *= f; v.y *= f; v.z *= f; v.w *= f;
+          }
+        }
         if constexpr (EPI == EPI_PARTIAL) {
           *reinterpret_cast<float4 *>(g.out + ((size_t)t.slice * g.out_rows + m) * g.N + n) = v;
         } else if constexpr (EPI == EPI_LOGITS) {
@@ -286,8 +308,24 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       float *own = slab ? slab_at(t.slice) : nullptr;
       for (int c0 = grp * kPassRows; c0 < t.rows; c0 += 2 * kPassRows, buf ^= 1) {
         uint32_t r[16];
-        tmem_ld16(tacc + c0, r);
-        tmem_wait_ld();
+        if (apart) {
+          // rows of either half: value plane, then remainder plane (halves come in eights)
+          uint32_t a[8], b8[8], c[8], e[8];
+          const int h = t.rows >> 1, c1 = c0 + 8, k0 = c0 < h ? c0 : c0 + h, k1 = c1 < h ? c1 : c1 + h;
+          tmem_ld8(tacc + k0, a);
+          tmem_ld8(tacc + k0 + h, b8);
+          tmem_ld8(tacc + k1, c);
+          tmem_ld8(tacc + k1 + h, e);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            r[i] = __float_as_uint(__uint_as_float(a[i]) + __uint_as_float(b8[i]));
+            r[8 + i] = __float_as_uint(__uint_as_float(c[i]) + __uint_as_float(e[i]));
+          }
+        } else {
+          tmem_ld16(tacc + c0, r);
+          tmem_wait_ld();
+        }
         const uint32_t at = stg + buf * kPassBytes;   // (two buffers in turn: a barrier per pass)
 #pragma unroll
         for (int i = 0; i < 16; ++i) st_shared_f32(at + (i * kBoxN + q * 32 + lane) * 4, __uint_as_float(r[i]));
@@ -416,14 +454,17 @@ PairPlan plan_gemm_pair(int N, int M, int n_kblocks, int planes, bool fold, int 
   } else {
     const int q = p.tiles / pairs, r = p.tiles % pairs;
     const double out = 3.0 + 8.0 * r256;   // the last tile's way out
-    double best = r ? kb * n_kblocks + 1.0 : 0.0;    // of what comes on top of q whole tiles each
+    const double uncut = r ? kb * n_kblocks + 1.0 : 0.0;
+    double best = uncut;                             // of what comes on top of q whole tiles each
     for (int s = 2; r && s <= max_pieces && s <= n_kblocks / 4; ++s) {
       if ((size_t)r * s * 2 * p.rows * kBoxN > slab_room) break;
       // (a piece costs at least its sums' way out; what the adding takes beyond a whole tile's products shows as well)
       const int mine = (r * s + pairs - 1) / pairs;
       const double add = 10.0 * r256 * ((s + kFoldAhead - 1) / kFoldAhead) + 5.0 * r256 * mine;
       const double t = mine * std::max(kb * n_kblocks / s + 2.0, 6.0 * r256) + std::max(0.0, add - (q ? kb * n_kblocks : 0.0));
-      if (t < best - 1e-9) { best = t; p.pieces = s; }
+      // (slabs are traffic that the count above takes for hidden: not for a few per cent -- LM head of the 1B shape at 112 rows, 57
+      // tiles left for 74 pairs, 99 us uncut against 112)
+      if (t < best - 1e-9 && t < 0.75 * uncut) { best = t; p.pieces = s; }
     }
     if (p.pieces > 1) p.whole = q * pairs;
     p.us = q * (kb * n_kblocks + 0.5) + best + out;
@@ -436,6 +477,7 @@ PairPlan plan_gemm_pair(int N, int M, int n_kblocks, int planes, bool fold, int 
 // where plan.n_wide == plan.chunks).  N must be a multiple of 128.
 cudaError_t launch_gemm_pair(int epi, const CUtensorMap &tw, const CUtensorMap &ta, const CUtensorMap &ta_less, PairArgs g,
                              const PairPlan &plan, size_t smem_limit, cudaStream_t st, bool pdl) {
+  if (g.ss && plan.rows > 128) return cudaErrorInvalidValue;
   if (plan.pieces < 1 || plan.pieces > g.n_kblocks || g.N % kBoxN || plan.rows % 16 || plan.rows < 16 || plan.rows > 256 || plan.pairs < 1)
     return cudaErrorInvalidValue;
   g.chunk_rows = plan.rows;

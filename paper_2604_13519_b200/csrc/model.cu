@@ -441,7 +441,19 @@ ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUten
   return TS_OK;
 }
 
-// A projection of the weight-streaming kernel; `g` carries what its epilogue needs.
+// Whether gate-up or the LM head of a step that is the weight-streaming kernel's otherwise goes to the pair kernel.  From 41 rows on
+// that kernel's bytes of activations, loaded by every CTA, count for more than its second CTA per SM (1B shape, gate-up and LM
+// head at 48 rows 17.6 and 92.6 us against 15.0 and 83.3, at 64 19.1 and 97.9 against 15.4 and 87.8, at 33 the same).  The sums are the same bits as that kernel's as long as no tile is cut along K,
+// which steps of at most 64 rows need (a row's bits do not depend on what is verified beside it), so there the tiles have to
+// come out even on the pairs.  (One plane: the LM head past 64 rows, gate-up past 80, where a box of activations is as heavy as 40
+// rows of two: 8B shape at 76 rows 36.0 us against 38.0, at 96 39.8 against 39.2.)
+bool few_by_pairs(const ts_model *m, int epi, int N, int M) {
+  if (M > 64) return m->planes == 2 || epi == ts::EPI_LOGITS || M > 80;
+  const int tiles = (N + 255) / 256, rounds = (tiles + m->max_pairs - 1) / m->max_pairs;
+  return m->planes == 2 && M > 40 && rounds * m->max_pairs * 5 <= tiles * 6;
+}
+
+// A projection of at most kFewRows rows; `g` carries what its epilogue needs.
 ts_status run_gemm_ws(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M, ts::GemmArgs g) {
   const int mi = pick_mc_index(M, m->planes);
   g.N = N; g.K = K; g.M = M; g.Mc = box_rows(mi); g.planes = m->planes;
@@ -449,8 +461,20 @@ ts_status run_gemm_ws(ts_model *m, int epi, const CUtensorMap &tw, const CUtenso
   g.act_rows = m->L.rows_alloc; g.out_planes = m->planes;
   g.err = m->d_out() + m->L.o_err;
   g.stamp = m->stamp_slot();
-  const int cluster = (epi == ts::EPI_QKV || epi == ts::EPI_RESID) ? pick_cluster(m, N / 128, g.n_kblocks) : 1;
-  CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, cluster, m->gemm_smem_budget, m->st, m->use_pdl && !m->profiling));
+  const bool split = epi == ts::EPI_QKV || epi == ts::EPI_RESID, pdl = m->use_pdl && !m->profiling;
+  if (!split && few_by_pairs(m, epi, N, M)) {
+    ts::PairArgs p{};
+    static_cast<ts::GemmArgs &>(p) = g;
+    p.slab = (float *)m->WS(m->L.part);
+    p.n_done = (unsigned int *)m->WS(m->L.n_done);
+    const ts::PairPlan plan = ts::plan_gemm_pair(N, M, g.n_kblocks, m->planes, true, m->max_pairs, M > 64 ? kMaxPieces : 1,
+                                                 (size_t)m->L.part_rows * std::max(m->L.Nqkv, m->c.d_model));
+    const int box = plan.rows / 16 - 1;
+    CU_TRY(ts::launch_gemm_pair(epi, tw, ta[box], ta[std::max(0, box - 1)], p, plan, m->smem_optin, m->st, pdl));
+  } else {
+    const int cluster = split ? pick_cluster(m, N / 128, g.n_kblocks) : 1;
+    CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, cluster, m->gemm_smem_budget, m->st, pdl));
+  }
   m->launched(0);
   return TS_OK;
 }
