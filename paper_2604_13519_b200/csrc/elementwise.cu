@@ -46,7 +46,7 @@ norm_kernel(const int32_t *tokens, const __nv_bfloat16 *embed, const float *part
   float *xr = x + (size_t)m * d;
   float ss = 0.f;
   float4 keep = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (MODE == 0 && threadIdx.x == 0) amax[m] = 0ull;
+  if (MODE == 0 && threadIdx.x == 0) amax[(size_t)m * kAmaxStride] = 0ull;
   for (int c = c0; c < d; c += blockDim.x * 4) {
     float4 v;
     if (MODE == 0) {
@@ -332,7 +332,7 @@ accept_kernel(AcceptArgs a) {
   const int seq = blockIdx.x;
   const int r0 = a.in.cu_rows[seq], r1 = a.in.cu_rows[seq + 1];
   for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    a.argmax[r] = (int32_t)(0xFFFFFFFFu - (uint32_t)(a.amax[r] & 0xFFFFFFFFull));
+    a.argmax[r] = (int32_t)(0xFFFFFFFFu - (uint32_t)(a.amax[(size_t)r * kAmaxStride] & 0xFFFFFFFFull));
     // (a row's parent precedes it in its chunk; -1 marks the root)
     ts_in_range(a.in.ck, CHK_PARENT, (long long)a.in.parent[r] + 1, r - r0 + 1);
   }

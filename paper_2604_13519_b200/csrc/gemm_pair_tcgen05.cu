@@ -291,7 +291,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           }
           const uint32_t top = __reduce_max_sync(0xffffffffu, best);
           if (lane == __ffs(__ballot_sync(0xffffffffu, best == top)) - 1)
-            atomicMax(g.amax + m, ((unsigned long long)top << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)(n + bi)));
+            atomicMax(g.amax + (size_t)m * kAmaxStride, ((unsigned long long)top << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)(n + bi)));
         } else {  // EPI_SWIGLU: even feature row = gate_f, odd = up_f, f = n / 2
           __nv_bfloat16 h0, l0, h1, l1;
           split_bf16(v.x / (1.f + __expf(-v.x)) * v.y, h0, l0);

@@ -328,7 +328,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           // order-preserving map of the float to an unsigned word; ties resolve to the lowest id
           uint32_t u = __float_as_uint(best);
           u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-          atomicMax(g.amax + m, ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_n));
+          atomicMax(g.amax + (size_t)m * kAmaxStride, ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_n));
         }
       }
     }

@@ -49,6 +49,9 @@ struct StepIn {
 // the queries and appends K/V; RESID (O, down) adds to the residual stream and prepares the next projection's input.
 enum : int { EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_LOGITS = 2, EPI_QKV = 3, EPI_RESID = 4 };
 
+// A row's packed maximum (EPI_LOGITS) has a line of its own: with the rows' words side by side the LM head's thousand atomics
+// per row all went to a few lines of L2, one after the other at about 1 ns each: the launch grew by 0.45 us per row.
+constexpr int kAmaxStride = 16;   // 128 bytes
 struct GemmArgs {
   int N, K, M;          // output features, reduction length, valid activation rows
   int Mc;               // activation rows per CTA: the step's rows rounded up (weight-streaming kernel), 128 (many rows)
@@ -63,7 +66,7 @@ struct GemmArgs {
   __nv_bfloat16 *act_out;  // EPI_SWIGLU: [out_planes][act_rows][N/2]
   int act_rows;
   int out_planes;
-  unsigned long long *amax;  // EPI_LOGITS: [M] packed (ordered logit bits << 32 | ~token id), atomicMax
+  unsigned long long *amax;  // EPI_LOGITS: [M][kAmaxStride] packed (ordered logit bits << 32 | ~token id), atomicMax
   int *err;             // device status word
   unsigned long long *stamp;   // optional clock stamps of this launch (null = none)
   // ---- weight-streaming kernel only ----
@@ -200,7 +203,7 @@ struct HostOut {
 // per-row argmax over the LM-head tiles, longest accepted prefix per sequence, new lengths
 struct AcceptArgs {
   StepIn in;
-  const unsigned long long *amax;   // [M] packed per-row maxima written by the LM-head epilogue
+  const unsigned long long *amax;   // [M][kAmaxStride] packed per-row maxima written by the LM-head epilogue
   int32_t *argmax;         // [M]
   int32_t *accept_len;     // [B]
   int32_t *emitted;        // [B][k_max]
@@ -217,7 +220,7 @@ constexpr int kSampleSlices = 32;   // slices of a row whose sums of weights are
 struct SampleArgs {
   StepIn in;
   float *logits;                    // [M][V] (refused tokens are masked for the draw and restored)
-  const unsigned long long *amax;   // [M] packed per-row maxima (argmax is still reported)
+  const unsigned long long *amax;   // [M][kAmaxStride] packed per-row maxima (argmax is still reported)
   const float *uni;                 // [M] uniforms in [0, 1): row c of a chunk decides node c, the root row's draws the sample
   float *part;                      // [M][kSampleSlices] scratch: per-slice sums of exp((l - max) / T)
   int V;

@@ -163,7 +163,7 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->attn = take(planes * R * Nq * 2);
   L->act = take(planes * R * F * 2);
   L->logits = take(Rs * V * 4);
-  L->amax = take(R * 8);
+  L->amax = take(R * ts::kAmaxStride * 8);
   L->samp_stats = take(Rs * ts::kSampleSlices * 4);
   L->topk_cand = take(Rs * (uint64_t)((c.vocab + 4095) / 4096) * TS_TOPK * 8);
   L->rope = take((uint64_t)c.max_ctx * (hd / 2) * 8);

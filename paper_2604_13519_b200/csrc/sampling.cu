@@ -52,7 +52,7 @@ row_expsum_kernel(const float *logits, const unsigned long long *amax, int V, fl
   constexpr int kThreads = kStatThreads / PER;
   const int r = blockIdx.x, sl = blockIdx.y * PER + threadIdx.x / kThreads, tid = threadIdx.x % kThreads;
   const float *row = logits + (size_t)r * V;
-  const float mx = row_max_of(amax[r]);
+  const float mx = row_max_of(amax[(size_t)r * kAmaxStride]);
   const int per = slice_len(V), i0 = sl * per, i1 = min(V, i0 + per);
   float sum = 0.f;
 #pragma unroll 4
@@ -85,7 +85,7 @@ sample_accept_kernel(SampleArgs a) {
   const int r0 = a.in.cu_rows[seq], k = a.in.cu_rows[seq + 1] - r0;
   int32_t *path = a.path + (size_t)seq * a.k_max;
   for (int r = r0 + threadIdx.x; r < r0 + k; r += blockDim.x)
-    a.argmax[r] = (int32_t)(0xFFFFFFFFu - (uint32_t)(a.amax[r] & 0xFFFFFFFFull));
+    a.argmax[r] = (int32_t)(0xFFFFFFFFu - (uint32_t)(a.amax[(size_t)r * kAmaxStride] & 0xFFFFFFFFull));
   for (int c = warp; c < k; c += kSampleThreads / 32) {
     const float tot = warp_sum(a.part[(size_t)(r0 + c) * kStatSlices + lane]);   // total weight of node c's own row
     if (lane == 0) tot_node[c] = tot;
@@ -93,7 +93,7 @@ sample_accept_kernel(SampleArgs a) {
   if ((int)threadIdx.x < k) {
     const int c = threadIdx.x, par = a.in.parent[r0 + c];
     w_node[c] = par < 0 ? 0.f
-                        : __expf((a.logits[(size_t)(r0 + par) * a.V + a.in.tokens[r0 + c]] - row_max_of(a.amax[r0 + par])) * a.inv_t);
+                        : __expf((a.logits[(size_t)(r0 + par) * a.V + a.in.tokens[r0 + c]] - row_max_of(a.amax[(size_t)(r0 + par) * kAmaxStride])) * a.inv_t);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -122,7 +122,7 @@ sample_accept_kernel(SampleArgs a) {
   __syncthreads();
   const int l = sh_l, last = sh_last, nref = sh_nref;
   const float *row = a.logits + (size_t)(r0 + last) * a.V;
-  const float mx = row_max_of(a.amax[r0 + last]);
+  const float mx = row_max_of(a.amax[(size_t)(r0 + last) * kAmaxStride]);
   const int per = slice_len(a.V);
   if (threadIdx.x < kStatSlices) slice_sum[threadIdx.x] = a.part[(size_t)(r0 + last) * kStatSlices + threadIdx.x];
   __syncthreads();
