@@ -442,15 +442,20 @@ ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUten
 }
 
 // Whether gate-up or the LM head of a step that is the weight-streaming kernel's otherwise goes to the pair kernel.  From 41 rows on
-// that kernel's bytes of activations, loaded by every CTA, count for more than its second CTA per SM (1B shape, gate-up and LM
-// head at 48 rows 17.6 and 92.6 us against 15.0 and 83.3, at 64 19.1 and 97.9 against 15.4 and 87.8, at 33 the same).  The sums are the same bits as that kernel's as long as no tile is cut along K,
-// which steps of at most 64 rows need (a row's bits do not depend on what is verified beside it), so there the tiles have to
-// come out even on the pairs.  (One plane: the LM head past 64 rows, gate-up past 80, where a box of activations is as heavy as 40
-// rows of two: 8B shape at 76 rows 36.0 us against 38.0, at 96 39.8 against 39.2.)
+// that kernel's bytes of activations, loaded by every CTA, count for more than its second CTA per SM (1B shape, gate-up at 48
+// rows 17.6 us against 15.0, at 64 19.1 against 15.4, at 33 the same; LM head at 48 92.6 against 83.3, at 33 83.6 against 79.9,
+// at 20 the same).  The sums are the same bits as that kernel's as long as no tile is cut along K, which steps of at most 64
+// rows need (a row's bits do not depend on what is verified beside it), so there the tiles have to come out even on the pairs
+// (8B shape: 96 gate-up tiles on 74 pairs do not, and the 594 of its LM head, nine rounds where eight would nearly do, only from
+// 41 rows on: 189 us against 190 at 32, 216 against 199 at 48).  One plane: LM head at 64 rows 90.5 against 84.4, at 48 the same;
+// gate-up past 80, where a box of activations is as heavy as 40 rows of two (8B shape at 76 rows 36.0 against 38.0, at 96 39.8
+// against 39.2).
 bool few_by_pairs(const ts_model *m, int epi, int N, int M) {
-  if (M > 64) return m->planes == 2 || epi == ts::EPI_LOGITS || M > 80;
-  const int tiles = (N + 255) / 256, rounds = (tiles + m->max_pairs - 1) / m->max_pairs;
-  return m->planes == 2 && M > 40 && rounds * m->max_pairs * 5 <= tiles * 6;
+  const bool head = epi == ts::EPI_LOGITS;
+  if (M > 64) return m->planes == 2 || head || M > 80;
+  const int tiles = (N + 255) / 256, slots = (tiles + m->max_pairs - 1) / m->max_pairs * m->max_pairs;
+  if (m->planes == 1) return head && M > 48 && slots * 20 <= tiles * 21;
+  return (M > 40 && slots * 5 <= tiles * 6) || (head && M > 24 && slots * 20 <= tiles * 21);
 }
 
 // A projection of at most kFewRows rows; `g` carries what its epilogue needs.
