@@ -260,12 +260,13 @@ __device__ __forceinline__ void publish(const Args &a, int seq, int r0, int k, i
 }
 #endif
 
-// A row's Top-K straight to the host: kTopMax pairs, then the status word and a word that takes the call's number when all of
-// it is there, in pinned memory as the device sees it (null: not wanted).
+// Rows' Top-K straight to the host, in pinned memory as the device sees it (null: not wanted).  ends: one row, the last kernel of
+// a call: behind kTopMax pairs the status word and a word that takes the call's number when all of it is there.
 constexpr int kTopMax = 64;
 struct PairsOut {
   float *host;
   int32_t number;
+  bool ends;
 };
 
 // Cosine Top-K over datastore hidden states (retrieval.cu).  scores: [N + 2K] floats; the result pairs (index as int
@@ -275,7 +276,7 @@ cudaError_t launch_topk_cosine(const __nv_bfloat16 *H, int N, int d, const float
 
 // Row-wise Top-K (topk.cu): out[r][j] = (column as int bits, value) of the j-th largest entry of row r, lowest column
 // on ties.  cand: scratch of n_rows * ceil(n_cols / 4096) * K pairs.
-// po: one row only; err is published with it.
+// err is published with po where that ends the call.
 cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, float2 *cand, float *out, PairsOut po,
                              const int *err, cudaStream_t st);
 

@@ -683,7 +683,8 @@ ts_status run_step(ts_model *m) {
   int32_t *dout = m->d_out();
   if (m->last_flags & TS_FLAG_WANT_TOPK) {   // per-position Top-K of the logits, for the successor tables
     CU_TRY(ts::launch_topk_rows((const float *)m->WS(L.logits), M, c.vocab, TS_TOPK, (float2 *)m->WS(L.topk_cand),
-                                (float *)(dout + L.o_topk), ts::PairsOut{}, nullptr, m->st));
+                                (float *)(dout + L.o_topk),
+                                ts::PairsOut{m->publish ? (float *)(m->host_dev + L.in_ints + L.o_topk) : nullptr, 0, false}, nullptr, m->st));
     m->launched(5);
     m->launched(5);
   }
@@ -941,13 +942,13 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const size_t in_bytes = (m->last_units_at + (size_t)m->h_in()[I.o_cta_unit + m->last_ctas] * (sizeof(ts::AttnWork) / 4)) * 4;
   CU_TRY(cudaMemcpyAsync(m->d_in(), m->h_in(), in_bytes, cudaMemcpyHostToDevice, m->st));
   m->h2d += (int64_t)in_bytes;
-  // A step that ends in an acceptance kernel (and maybe the cache's compaction) publishes its results itself; prompts, the
-  // persistent kernel and per-position Top-K lists take a copy, as does the debug build, whose checks go on in the
+  // A step that ends in an acceptance kernel (and maybe the cache's compaction) publishes its results itself, its Top-K lists
+  // too; prompts and the persistent kernel take a copy, as does the debug build, whose checks go on in the
   // acceptance kernel's other blocks and in the compaction.
 #ifdef TS_DEBUG_BOUNDS
   const bool publishes = false;
 #else
-  const bool publishes = m->host_dev && !m->last_fused && !(flags & (TS_FLAG_SKIP_LM_HEAD | TS_FLAG_WANT_TOPK));
+  const bool publishes = m->host_dev && !m->last_fused && !(flags & TS_FLAG_SKIP_LM_HEAD);
 #endif
   m->publish = publishes;
   const bool flagged = publishes && !m->last_tree;   // (a tree's step ends with the compaction, which publishes nothing)
@@ -963,9 +964,10 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   const int32_t *ho = m->h_out();
   if (publishes) {
     // (see ts::publish: the status; per sequence length, pending id, accepted drafts and maybe the call's number; a row's
-    // argmax; emitted ids and path)
+    // argmax; emitted ids and path; a row's Top-K pairs)
     int64_t words = 1 + (3 + flagged) * (int64_t)B + M;
     for (int i = 0; i < B; ++i) words += 2 * (ho[L.o_accept + i] + 1);
+    if (flags & TS_FLAG_WANT_TOPK) words += 2 * TS_TOPK * (int64_t)M;
     m->d2h += 4 * words;
   } else {
     m->d2h += (int64_t)out_bytes;
@@ -2004,7 +2006,7 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
   if (m->inject_err) CU_TRY(write_injected(m));
   CU_TRY(ts::launch_topk_cosine((const __nv_bfloat16 *)hidden_dev, n_entries, m->c.d_model, query_dev, planes,
                                 (int)(m->L.rows_alloc * m->c.d_model), m->planes, K, scores_dev, m->n_sms,
-                                ts::PairsOut{res_dev, m->call_no}, m->d_out() + m->L.o_err, m->st));
+                                ts::PairsOut{res_dev, m->call_no, true}, m->d_out() + m->L.o_err, m->st));
   if (!res_dev) {
     CU_TRY(cudaMemcpyAsync(res, scores_dev + n_entries, 2 * (size_t)K * 4, cudaMemcpyDeviceToHost, m->st));
     CU_TRY(cudaMemcpyAsync(res + 2 * ts::kTopMax, m->d_out() + m->L.o_err, 4, cudaMemcpyDeviceToHost, m->st));

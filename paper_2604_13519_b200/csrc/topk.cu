@@ -6,10 +6,11 @@
 namespace ts {
 
 // Selection in two levels, both with the same rule (largest score, lowest index on ties).  First a CTA per slice of 4096
-// scores: every thread sorts its 16 in registers, every warp takes the K best of its 512 from the heads of its lanes' lists
-// in K rounds of two warp reductions (no barrier), and one warp merges the eight warps' lists the same way.  Then a CTA per
-// row merges the slices' lists.  (14 us cold for the two kernels, K = 10 of 100 000 scores; with a block-wide reduction over all scores per round 18,
-// with warp-wide rounds over unsorted registers 48.)
+// scores.  Up to kBoundK: the K-th largest of a warp's 32 lane maxima is a bound that at least K of its scores reach; the
+// largest bound of the CTA's warps leaves a few dozen of the slice, which are put in order by counting, for each, those above
+// it.  For larger K every thread sorts its 16 in registers, every warp takes the K best of its 512 from the heads of its lanes'
+// lists in K rounds of two warp reductions (no barrier), and one warp merges the eight warps' lists the same way.  Then a CTA
+// per row merges the slices' lists.
 // cand: [rows][slices][K] (column as int bits, value) pairs, best first; out: [rows][K] pairs.
 static constexpr int kSlice = 4096;
 static constexpr int kSelThreads = 256;
@@ -51,6 +52,85 @@ __device__ __forceinline__ void warp_merge(F next, int K, Entry *out) {
       second = next();
     }
   }
+}
+
+static constexpr int kBoundK = 16;      // most K of the bounded selection
+__global__ void __launch_bounds__(kSelThreads, 6)
+topk_bound_kernel(const float *x, int N, int K, float2 *cand) {
+  __shared__ Entry list[kSelThreads], best[kBoundK], of_warp[kSelWarps];
+  __shared__ uint32_t bound, count;
+  const float *scores = x + (size_t)blockIdx.y * N;          // this CTA's row
+  cand += ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * K;
+  const int lane = threadIdx.x & 31, base = blockIdx.x * kSlice + threadIdx.x;
+  if (threadIdx.x == 0) { bound = 1u; count = 0u; }
+  if (threadIdx.x < K) best[threadIdx.x] = 0ull;
+  pdl_launch_dependents();
+  pdl_wait();
+  uint32_t u[kPer], top = 0u;   // the scores as words of the same order, 0 = none
+  {
+    float v[kPer];
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) v[e] = base + e * kSelThreads < N ? scores[base + e * kSelThreads] : -INFINITY;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      u[e] = (uint32_t)(entry_of(v[e], 0) >> 32);
+      top = max(top, u[e]);
+    }
+  }
+  auto entry = [&](int e) { return u[e] ? ((Entry)u[e] << 32) | (uint32_t)~(base + e * kSelThreads) : 0ull; };
+  uint32_t mine = top, b = 0u;
+  for (int j = 0; j < K; ++j) {
+    b = __reduce_max_sync(0xffffffffu, mine);
+    if (lane == __ffs(__ballot_sync(0xffffffffu, mine == b)) - 1) mine = 0u;
+  }
+  __syncthreads();
+  if (lane == 0) atomicMax(&bound, b);   // (0 where the warp has fewer than K)
+  __syncthreads();
+  const uint32_t least = bound;
+  if (__any_sync(0xffffffffu, top >= least)) {
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      const uint32_t hit = __ballot_sync(0xffffffffu, u[e] >= least);
+      if (hit == 0u) continue;
+      uint32_t at = 0u;
+      if (lane == 0) at = atomicAdd(&count, (uint32_t)__popc(hit));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(hit & ((1u << lane) - 1u));
+      if (u[e] >= least && at < kSelThreads) list[at] = entry(e);
+    }
+  }
+  __syncthreads();
+  const int n = (int)count;
+  if (n <= kSelThreads) {
+    if ((int)threadIdx.x < n) {
+      const Entry e = list[threadIdx.x];
+      int above = 0;
+#pragma unroll 8
+      for (int i = 0; i < n; ++i) above += list[i] > e;
+      if (above < K) best[above] = e;   // (entries are unique)
+    }
+  } else {
+    // (hundreds of equal scores: one after the other, each the largest below the one before)
+    Entry last = ~0ull;
+    for (int j = 0; j < K; ++j) {
+      Entry e = 0ull;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const Entry t = entry(i);
+        if (t < last && t > e) e = t;
+      }
+      bool is_mine;
+      e = warp_max(e, is_mine);
+      if (lane == 0) of_warp[threadIdx.x >> 5] = e;
+      __syncthreads();
+      e = 0ull;
+      for (int w = 0; w < kSelWarps; ++w) e = max(e, of_warp[w]);
+      if (threadIdx.x == 0) best[j] = e;
+      last = e;
+      __syncthreads();
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < K) cand[threadIdx.x] = pair_of(best[threadIdx.x]);
 }
 
 __global__ void __launch_bounds__(kSelThreads)
@@ -111,6 +191,7 @@ topk_final_kernel(const float2 *cand, int n_lists, int K, float *out, PairsOut p
   out += (size_t)blockIdx.x * 2 * K;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int j = threadIdx.x; j < K; j += blockDim.x) lists[kSelWarps][j] = 0ull;   // (the K best so far)
+  pdl_launch_dependents();
   pdl_wait();
   // a thread per slice's list: every warp merges its 32, one warp the warps' lists and what earlier rounds left
   for (int l0 = 0; l0 < n_lists; l0 += kSelThreads) {
@@ -131,9 +212,14 @@ topk_final_kernel(const float2 *cand, int n_lists, int K, float *out, PairsOut p
     const float2 r = pair_of(lists[kSelWarps][threadIdx.x]);
     out[2 * threadIdx.x] = r.x;
     out[2 * threadIdx.x + 1] = r.y;
-    if (po.host) { po.host[2 * threadIdx.x] = r.x; po.host[2 * threadIdx.x + 1] = r.y; }
+    if (po.host) {
+      float *host = po.host + (size_t)blockIdx.x * 2 * K;
+      host[2 * threadIdx.x] = r.x;
+      host[2 * threadIdx.x + 1] = r.y;
+      if (!po.ends) __threadfence_system();   // (else raise_flag's)
+    }
   }
-  if (!po.host) return;
+  if (!po.host || !po.ends) return;
   int32_t *tail = reinterpret_cast<int32_t *>(po.host) + 2 * kTopMax;
   if (threadIdx.x == 0) tail[0] = *err;
   __syncthreads();
@@ -153,7 +239,7 @@ cudaError_t launch_topk_rows(const float *x, int n_rows, int n_cols, int K, floa
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, topk_slice_kernel, x, n_cols, K, cand);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, K <= kBoundK ? topk_bound_kernel : topk_slice_kernel, x, n_cols, K, cand);
   if (e != cudaSuccess) return e;
   cfg.gridDim = dim3(n_rows);
   return cudaLaunchKernelEx(&cfg, topk_final_kernel, (const float2 *)cand, slices, K, out, po, err);
