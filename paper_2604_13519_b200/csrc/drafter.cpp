@@ -155,20 +155,55 @@ static inline uint64_t gram_key(const int32_t *p) {  // hash of 5 ids
 
 }  // namespace ts
 
+// Postings come in order of (entry, m).  Many at once are dealt out by the leading bits of their keys, about one to a bucket (the
+// keys are hashes), and each bucket is put in order by itself: 70 000 postings of a thousand invocations 2.0 ms, by
+// comparisons alone 4.1 -- the first draft of a session with a fresh datastore waits for it.
+static constexpr size_t kFewPostings = 4096;
+
 void ts_datastore::ensure_index() const {
   if (indexed_entries == n_entries()) return;
-  size_t old = index.size();
-  for (int64_t e = indexed_entries; e < n_entries(); ++e) {
-    int32_t len;
-    const int32_t *p = entry((int32_t)e, &len);
-    for (int32_t m = 5; m < len; ++m) index.push_back({ts::gram_key(p + m - 5), (int32_t)e, m});
-  }
+  const size_t old = index.size();
+  size_t most = old;
+  for (int64_t e = indexed_entries; e < n_entries(); ++e) most += (size_t)std::max<int64_t>(0, offset[e + 1] - offset[e] - 5);
   auto cmp = [](const Posting &a, const Posting &b) {
     if (a.key != b.key) return a.key < b.key;
     if (a.entry != b.entry) return a.entry < b.entry;
     return a.m < b.m;
   };
-  std::sort(index.begin() + old, index.end(), cmp);
+  std::vector<Posting> fresh;
+  fresh.reserve(most - old);
+  for (int64_t e = indexed_entries; e < n_entries(); ++e) {
+    int32_t len;
+    const int32_t *p = entry((int32_t)e, &len);
+    for (int32_t m = 5; m < len; ++m) fresh.push_back({ts::gram_key(p + m - 5), (int32_t)e, m});
+  }
+  const size_t n = fresh.size();
+  index.resize(old + n);
+  if (n < kFewPostings) {
+    std::copy(fresh.begin(), fresh.end(), index.begin() + old);
+    std::sort(index.begin() + old, index.end(), cmp);
+  } else {
+    int bits = 12;
+    while (bits < 24 && ((size_t)1 << bits) < n) ++bits;
+    std::vector<uint32_t> at(((size_t)1 << bits) + 1, 0u);
+    for (const Posting &p : fresh) ++at[(p.key >> (64 - bits)) + 1];
+    for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
+    Posting *to = index.data() + old;
+    for (const Posting &p : fresh) to[at[p.key >> (64 - bits)]++] = p;   // (at[i] ends as the start of bucket i + 1)
+    for (size_t i = 0, lo = 0; i + 1 < at.size(); lo = at[i++]) {
+      const size_t hi = at[i];
+      if (hi - lo > 32) {   // (a 5-gram of the scaffolding, in every invocation: in order already, or nearly)
+        if (!std::is_sorted(to + lo, to + hi, cmp)) std::stable_sort(to + lo, to + hi, cmp);
+      } else {
+        for (size_t j = lo + 1; j < hi; ++j) {
+          const Posting p = to[j];
+          size_t k = j;
+          for (; k > lo && cmp(p, to[k - 1]); --k) to[k] = to[k - 1];
+          to[k] = p;
+        }
+      }
+    }
+  }
   std::inplace_merge(index.begin(), index.begin() + old, index.end(), cmp);
   indexed_entries = n_entries();
 }
