@@ -1,5 +1,6 @@
 // The dense projections of the verify step for MANY rows (batched steps and prompts: more than the weight-streaming kernel
-// takes, 80 rows or 96 with one plane of activations), where the work is bound by
+// takes, 80 rows or 96 with one plane of activations) whose row count and tiles suit it better than the pair kernel
+// (gemm_pair_tcgen05.cu; rows_plan in model.cu decides), where the work is bound by
 // the tensor cores and by the bytes an SM pulls from L2 per flop, no longer by streaming the weights:
 //     out[m][n] = sum_k act[m][k] * W[n][k]
 // Orientation: a CTA owns a chunk of 128 activation rows (operand A of the tensor-core instruction, its 128-row

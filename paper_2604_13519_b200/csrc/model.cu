@@ -49,10 +49,12 @@ constexpr int kMaxAttnSplits = ts::kAttnMaxSplits;
 // 14.9 at 8 rows.  Pair kernel: half of a chunk.  Many-rows kernel: 128.
 constexpr int kBoxes = 16;
 constexpr int box_rows(int i) { return 8 * (i + 1); }
-// Most rows of a step whose projections run on the weight-streaming kernel, with one and with two planes of activations.
-// With two planes a ring of three stages still fits twice on an SM at 80 rows and one of two at 88.  Measured, four sessions,
+// Most rows of a step whose projections run on the weight-streaming kernel (gate-up and the LM head of the larger ones on the
+// pair kernel, see few_by_pairs), with one and with two planes of activations.  With two planes a ring of three stages still fits twice on an SM at 80 rows and one of two at 88.  Measured, four sessions,
 // many-rows kernel against this one: 1B shape two planes 80 rows 1440 / 1281 us, 96 rows 1481 / 1518; 8B 5467 / 4684 and
-// 5511 / 5483; one plane 1B 96 rows 1267 / 1276, 112 rows 1297 / 1371, 8B 4547 / 4378 and 4672 / 4558.
+// 5511 / 5483; one plane 1B 96 rows 1267 / 1276, 112 rows 1297 / 1371, 8B 4547 / 4378 and 4672 / 4558.  (The pair kernel's QKV,
+// O and down at 80 rows are quicker, 1B shape 6.9, 5.9 and 9.7 us against 8.8, 8.5 and 13.9, but not with the norm and rotary
+// kernels that they need: a layer of 66.8 us against 65.1.)
 constexpr int kFewRows[2] = {96, 80};
 constexpr int kFusedMc[3] = {1, 3, 7};           // the persistent kernel's boxes: 16, 32, 64 rows
 constexpr int kPrefillRows = 1024;   // rows of a prompt that go through in one step

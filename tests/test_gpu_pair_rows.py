@@ -41,3 +41,25 @@ def test_rows_of_a_pair(name, rows, act_split):
             assert ((logits - lo) ** 2).sum() <= 4e-2 ** 2 * (lo ** 2).sum(), (name, rows, i)
         row += res.k
     gm.close()
+
+
+PAIRS = ModelShape("pairs-2l", 2, 2048, 32, 8, 64, 8192, 73 * 256, 500000.0, 1e-5)   # 64 gate-up tiles, 73 of the LM head
+
+
+def test_rows_are_the_same_bits_on_either_kernel():
+    """Steps of one session, 8 rows (weight-streaming kernel), 30 (LM head by pairs), 48 and 64 (gate-up too): a row's logits do
+    not depend on the chunk it is verified in."""
+    gm = ts.Model(PAIRS, max_pages=64, max_batch=1, k_max=64, max_rows=64, max_ctx=900)
+    gm.load_weights(synth.make_weights(PAIRS, gain_seed=3))
+    K, V = synth.make_synthetic_kv(PAIRS, 700)
+    s = ts.Session(gm, None, None)
+    for l in range(PAIRS.n_layers):
+        s.import_kv(l, K[l], V[l])
+    s.set_cache(700, 70)
+    draft = _rand_draft(PAIRS.vocab, 63, 5)
+    ts.ts_verify(gm, [s], [draft[:7]])
+    want = gm.read_logits(0, 8).copy()
+    for k in (30, 48, 64):
+        ts.ts_verify(gm, [s], [draft[:k - 1]])
+        assert (gm.read_logits(0, 8).view("u4") == want.view("u4")).all(), k
+    gm.close()
