@@ -467,7 +467,10 @@ PairPlan plan_gemm_pair(int N, int M, int n_kblocks, int planes, bool fold, int 
       if (t < best - 1e-9 && t < 0.75 * uncut) { best = t; p.pieces = s; }
     }
     if (p.pieces > 1) p.whole = q * pairs;
-    p.us = q * (kb * n_kblocks + 0.5) + best + out;
+    // (tiles of few k-blocks: an epilogue takes as long as the next tile's products, and memory from them; 1B shape, gate-up of 768
+    // rows 91 us against the row-major kernel's 89, of 475 54 against 61)
+    const double between = planes == 2 && n_kblocks < 48 ? 2.5 * r256 * r256 * std::max(0, q - (r ? 0 : 1)) : 0.0;
+    p.us = q * (kb * n_kblocks + 0.5) + between + best + out;
   }
   p.pairs = std::min(pairs, p.whole + (p.tiles - p.whole) * p.pieces);
   return p;

@@ -414,7 +414,11 @@ double gemm_rows_us(int N, int M, int n_kblocks, int planes, int n_splits, bool 
     const double work = rounds * ((planes == 2 ? 0.62 : 0.35) * n_kblocks / n_splits + 1.0);
     return std::max(work, stream) + 6.0 + rows_slab_us(M, N) * n_splits;
   }
-  return std::max((planes == 2 ? 0.68 : 0.39) * n_kblocks * pick_deal(blocks, chunks, 1, n_sms, true).rounds, stream) + 9.5;
+  // (a further round of tiles costs more than its k-blocks while they do not cover the epilogue of the one before: gate-up of the
+  // 1B shape, 32 k-blocks, 29 us at one round, 46 at 1.6, 59 at two; of the 8B shape, 64, 80 at 1.6 and 259 at 5.6)
+  const double rounds = pick_deal(blocks, chunks, 1, n_sms, true).rounds;
+  const double between = planes == 2 && rounds > 1.0 ? (rounds - 1.0) * std::max(0.0, 7.0 - 0.094 * n_kblocks) : 0.0;
+  return std::max((planes == 2 ? 0.68 : 0.39) * n_kblocks * rounds + between, stream) + 9.5;
 }
 
 // `ta` must be the activation map whose box holds 128 rows.  N must be a multiple of 128.
