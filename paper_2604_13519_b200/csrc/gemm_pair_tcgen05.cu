@@ -116,12 +116,15 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
   __syncwarp();
   if (warp == 1) {
     tmem_alloc_pair(smem_u32(&ctl->tmem_base), alloc_cols);
-    tmem_relinquish_pair();
   }
   tc_fence_before();
   __syncthreads();
   cluster_arrive();   // (both CTAs' barriers are set up before either's loads or products count on them)
   cluster_wait();
+  // The permit to allocate is the pair's: it goes back only when both CTAs hold their tensor memory.  (Given back behind the
+  // own allocation, it was gone for the CTA that came second, which then waited in its allocation for good: seen after some
+  // tens of steps back to back, 60 pairs of QKV of 640 rows, whose CTAs start under the embedding kernel's and so apart.)
+  if (warp == 1) tmem_relinquish_pair();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   if (threadIdx.x == 0) stamp_min(g.stamp);

@@ -3,6 +3,7 @@ rows that is a whole number of sixteens and one row more, one chunk and two, chu
 over and cut along K (8B layers: 96 gate-up tiles on 74 pairs); also on a shape all of whose matrices have an odd number of
 128-row blocks, so that a pair's second CTA has none in the last tile."""
 import pytest
+import torch
 
 import synth
 import paper_2604_13519_b200 as ts
@@ -62,4 +63,23 @@ def test_rows_are_the_same_bits_on_either_kernel():
     for k in (30, 48, 64):
         ts.ts_verify(gm, [s], [draft[:k - 1]])
         assert (gm.read_logits(0, 8).view("u4") == want.view("u4")).all(), k
+    gm.close()
+
+
+def test_pairs_that_start_apart_get_their_tensor_memory():
+    """Steps back to back, nothing waited for in between: QKV's pairs of CTAs then start while CTAs of the embedding kernel still run
+    on one SM of the pair and not on the other, and each CTA has to get its tensor memory whichever comes first."""
+    shape = ModelShape("apart", 1, 3072, 24, 8, 128, 1024, 4096, 10000.0, 1e-5)
+    gm = ts.Model(shape, max_pages=10 * 12, max_batch=10, k_max=64, max_rows=640, max_ctx=164, act_split=False)
+    gm.load_weights(synth.make_weights(shape))
+    gm.kv_pool_tensor().zero_()
+    sess = [ts.Session(gm, None, None) for _ in range(10)]
+    for s in sess:
+        s.set_cache(100, 70)
+    ts.ts_verify(gm, sess, [_rand_draft(shape.vocab, 63, i) for i in range(10)])
+    want = gm.read_logits(0, 640).copy()
+    for _ in range(500):
+        ts.ts_verify_replay(gm)
+    torch.cuda.synchronize()
+    assert (gm.read_logits(0, 640).view("u4") == want.view("u4")).all()
     gm.close()
