@@ -536,13 +536,25 @@ ts_status run_step_fused(ts_model *m) {
   return TS_OK;
 }
 
-// Test support (ts_debug_inject_device_error): leaves the status word that an expired device-side wait would have left.  In
-// the stream behind the last kernel that waits for anything and ahead of the acceptance kernel, which publishes the word with
-// the step's results as it would a real one.
+// What an expired device-side wait leaves behind, for whichever call meets its status word: the word, the counters that the
+// persistent kernel was in the middle of, and pieces of cut tiles that the pair kernel has counted and not added (the next
+// launch would take a tile for complete too soon, or never).
+void clear_device_error(ts_model *m) {
+  const Layout &L = m->L;
+  cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
+  cudaMemsetAsync(m->WS(L.sync), 0, (size_t)(8 + L.n_counters) * 4, m->st);
+  cudaMemsetAsync(m->WS(L.n_done), 0, (size_t)kMaxFusedCtas * 4, m->st);
+}
+
+// Test support (ts_debug_inject_device_error): leaves the status word that an expired device-side wait would have left, and
+// pieces counted by the pair kernel.  In the stream behind the last kernel that waits for anything and ahead of the acceptance
+// kernel, which publishes the word with the step's results as it would a real one.
 cudaError_t write_injected(ts_model *m) {
   int32_t *word = m->h_out() + m->L.o_err + 1;
   *word = m->inject_err;
   m->inject_err = 0;
+  const cudaError_t e = cudaMemsetAsync(m->WS(m->L.n_done), 1, (size_t)kMaxFusedCtas * 4, m->st);
+  if (e != cudaSuccess) return e;
   return cudaMemcpyAsync(m->d_out() + m->L.o_err, word, 4, cudaMemcpyHostToDevice, m->st);
 }
 
@@ -976,9 +988,7 @@ ts_status submit_step(ts_model *m, int B, int M, uint32_t flags) {
   }
   const int dev_err = ho[L.o_err];
   if (dev_err != 0) {
-    cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
-    cudaMemsetAsync(m->WS(L.sync), 0, (size_t)(8 + L.n_counters) * 4, m->st);   // the fused kernel left its counters mid-step
-    cudaMemsetAsync(m->WS(L.n_done), 0, (size_t)kMaxFusedCtas * 4, m->st);                       // and so may the pair kernel have
+    clear_device_error(m);
     if (dev_err >= ts::DEV_BOUNDS)
       return fail(TS_ERR_DEVICE_BOUNDS, "an index check of the debug build failed on the device (check %d)", dev_err - ts::DEV_BOUNDS);
     return fail(TS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired (code %d)", dev_err);
@@ -2018,7 +2028,7 @@ ts_status ts_topk_cosine(ts_model *m, const void *hidden_dev, int32_t n_entries,
   int dev_err;
   std::memcpy(&dev_err, res + 2 * ts::kTopMax, 4);
   if (dev_err != 0) {
-    cudaMemsetAsync(m->d_out() + m->L.o_err, 0, 4, m->st);
+    clear_device_error(m);
     return fail(TS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired (code %d)", dev_err);
   }
   for (int j = 0; j < K; ++j) {

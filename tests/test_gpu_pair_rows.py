@@ -66,6 +66,35 @@ def test_rows_are_the_same_bits_on_either_kernel():
     gm.close()
 
 
+def test_unfinished_tiles_are_forgotten_with_the_error_that_a_retrieval_reports():
+    """An expired wait in a replayed step, whose status nobody has looked at yet, is reported by whichever call comes next: by
+    a retrieval too the counts of tiles cut along K are cleared, so that the next step is the same bits as before it."""
+    shape = synth.SHAPES["8b-2l"]   # (96 gate-up tiles of 112 rows: 22 are left over by 74 pairs and cut)
+    gm = ts.Model(shape, max_pages=64, max_batch=2, k_max=56, max_rows=112, max_ctx=400)
+    gm.load_weights(synth.make_weights(shape))
+    gm.kv_pool_tensor().zero_()
+    sess = []
+    for i in range(2):
+        sess.append(ts.Session(gm, None, None))
+        sess[i].set_cache(200 + i, 70)
+    drafts = [[_rand_draft(shape.vocab, 55, 10 * j + i) for i in range(2)] for j in range(2)]
+
+    def logits(j):
+        ts.ts_verify(gm, sess, drafts[j])
+        return gm.read_logits(0, 112).copy()
+
+    want = logits(0)
+    assert not (logits(1) == want).all()
+    g = torch.Generator().manual_seed(1)
+    hidden = torch.randn(64, shape.d_model, generator=g).to(torch.bfloat16).cuda()
+    gm.inject_device_error(3)
+    with pytest.raises(ts.TsError) as e:
+        ts.ts_topk_cosine(gm, hidden, 4, query=torch.randn(shape.d_model, generator=g).cuda())
+    assert e.value.code == -6
+    assert (logits(0).view("u4") == want.view("u4")).all()
+    gm.close()
+
+
 def test_pairs_that_start_apart_get_their_tensor_memory():
     """Steps back to back, nothing waited for in between: QKV's pairs of CTAs then start while CTAs of the embedding kernel still run
     on one SM of the pair and not on the other, and each CTA has to get its tensor memory whichever comes first."""
