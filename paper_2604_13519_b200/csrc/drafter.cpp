@@ -160,10 +160,11 @@ static inline uint64_t gram_key(const int32_t *p) {  // hash of 5 ids
 // comparisons alone 4.1 -- the first draft of a session with a fresh datastore waits for it.
 static constexpr size_t kFewPostings = 4096;
 
+// (All that may fail for want of memory comes before the index changes -- what sorting and merging ask for they can do without --
+// so an attempt that is left by an exception leaves the index as it was, and the next one starts over.)
 void ts_datastore::ensure_index() const {
   if (indexed_entries == n_entries()) return;
-  const size_t old = index.size();
-  size_t most = old;
+  size_t most = 0;
   for (int64_t e = indexed_entries; e < n_entries(); ++e) most += (size_t)std::max<int64_t>(0, offset[e + 1] - offset[e] - 5);
   auto cmp = [](const Posting &a, const Posting &b) {
     if (a.key != b.key) return a.key < b.key;
@@ -171,24 +172,27 @@ void ts_datastore::ensure_index() const {
     return a.m < b.m;
   };
   std::vector<Posting> fresh;
-  fresh.reserve(most - old);
+  fresh.reserve(most);
   for (int64_t e = indexed_entries; e < n_entries(); ++e) {
     int32_t len;
     const int32_t *p = entry((int32_t)e, &len);
     for (int32_t m = 5; m < len; ++m) fresh.push_back({ts::gram_key(p + m - 5), (int32_t)e, m});
   }
-  const size_t n = fresh.size();
+  const size_t n = fresh.size(), old = index.size();
+  int bits = 0;
+  std::vector<uint32_t> at;
+  if (n >= kFewPostings) {
+    for (bits = 12; bits < 24 && ((size_t)1 << bits) < n;) ++bits;
+    at.assign(((size_t)1 << bits) + 1, 0u);
+  }
   index.resize(old + n);
+  Posting *to = index.data() + old;
   if (n < kFewPostings) {
-    std::copy(fresh.begin(), fresh.end(), index.begin() + old);
-    std::sort(index.begin() + old, index.end(), cmp);
+    std::copy(fresh.begin(), fresh.end(), to);
+    std::sort(to, to + n, cmp);
   } else {
-    int bits = 12;
-    while (bits < 24 && ((size_t)1 << bits) < n) ++bits;
-    std::vector<uint32_t> at(((size_t)1 << bits) + 1, 0u);
     for (const Posting &p : fresh) ++at[(p.key >> (64 - bits)) + 1];
     for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
-    Posting *to = index.data() + old;
     for (const Posting &p : fresh) to[at[p.key >> (64 - bits)]++] = p;   // (at[i] ends as the start of bucket i + 1)
     for (size_t i = 0, lo = 0; i + 1 < at.size(); lo = at[i++]) {
       const size_t hi = at[i];
@@ -204,6 +208,7 @@ void ts_datastore::ensure_index() const {
       }
     }
   }
+  std::vector<Posting>().swap(fresh);
   std::inplace_merge(index.begin(), index.begin() + old, index.end(), cmp);
   indexed_entries = n_entries();
 }
