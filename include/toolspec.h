@@ -403,9 +403,10 @@ ts_status ts_debug_timeline(ts_model *m, uint64_t *stamps, int32_t *classes, int
 /* Make the NEXT step or retrieval (ts_verify*, ts_prefill, ts_topk_cosine) report `code` (> 0) in its device status word,
  * as a bounded device-side wait that expired would: the word is written on the model's stream behind the step's last
  * kernel that waits for anything -- ahead of the acceptance kernel, which hands it to the host with its results; after the
- * last kernel where there is none; ahead of a retrieval's kernels, which do not read it -- so nothing is left waiting.  The
- * call then fails with TS_ERR_DEVICE_TIMEOUT (codes below 64) or TS_ERR_DEVICE_BOUNDS (64 + the number of a debug-build
- * index check; steps only), the library clears the word and the persistent kernel's counters, and later calls run normally.  For testing the
+ * last kernel where there is none; ahead of a retrieval's kernels, which do not read it -- so nothing is left waiting.  With it
+ * go counters of the persistent kernel that are not zero.  The call then fails with TS_ERR_DEVICE_TIMEOUT (codes below 64) or
+ * TS_ERR_DEVICE_BOUNDS (64 + the number of a debug-build index check; steps only), the library clears the word and the
+ * persistent kernel's counters, and later calls run normally.  For testing the
  * host's handling of a device timeout, or of a failed index check, without making a GPU wait or go out of range. */
 ts_status ts_debug_inject_device_error(ts_model *m, int32_t code);
 /* Counters: kernels launched since ts_init_model, bytes that steps have moved host->device and device->host since then

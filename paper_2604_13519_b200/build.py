@@ -9,7 +9,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtoolspec.so")
 # the same library with every device-side index check compiled in (TS_DEBUG_BOUNDS): for test runs, not for timing
 LIB_DEBUG = os.path.join(HERE, "libtoolspec_dbg.so")
-SOURCES = ["model.cu", "gemm_tcgen05.cu", "gemm_rows_tcgen05.cu", "gemm_pair_tcgen05.cu", "attention.cu", "attention_tc.cu", "elementwise.cu", "fused.cu", "attention_static.cu", "sampling.cu", "retrieval.cu", "topk.cu", "drafter.cpp"]
+SOURCES = ["model.cu", "gemm_tcgen05.cu", "gemm_rows_tcgen05.cu", "attention.cu", "attention_tc.cu", "elementwise.cu", "fused.cu", "attention_static.cu", "sampling.cu", "retrieval.cu", "topk.cu", "drafter.cpp"]
 
 
 def _stale(lib: str = LIB) -> bool:

@@ -1,6 +1,5 @@
 // The dense projections of the verify step for MANY rows (batched steps and prompts: more than the weight-streaming kernel
-// takes, 80 rows or 96 with one plane of activations) whose row count and tiles suit it better than the pair kernel
-// (gemm_pair_tcgen05.cu; rows_plan in model.cu decides), where the work is bound by
+// takes, 80 rows or 96 with one plane of activations), where the work is bound by
 // the tensor cores and by the bytes an SM pulls from L2 per flop, no longer by streaming the weights:
 //     out[m][n] = sum_k act[m][k] * W[n][k]
 // Orientation: a CTA owns a chunk of 128 activation rows (operand A of the tensor-core instruction, its 128-row
@@ -377,7 +376,7 @@ int gemm_rows_tiles(int N) { return (N + kTileN - 1) / kTileN; }
 // tiles narrow the CTAs end closer together.  The count of wide tiles, and how many narrow ones go to the CTAs that have
 // one wide tile less, with the earliest finish win; ties go to fewer narrow tiles.
 static constexpr double kNarrowCost = 0.6;
-struct Deal { int n_wide, narrow_short; double rounds; };
+struct Deal { int n_wide, narrow_short; };
 static Deal pick_deal(int blocks, int chunks, int splits, int G, bool mix) {
   static std::mutex mu;
   static std::map<std::tuple<int, int, int, int, bool>, Deal> memo;   // (a pure function of its key: shapes and SM count)
@@ -385,7 +384,7 @@ static Deal pick_deal(int blocks, int chunks, int splits, int G, bool mix) {
   const auto key = std::make_tuple(blocks, chunks, splits, G, mix);
   auto it = memo.find(key);
   if (it != memo.end()) return it->second;
-  Deal best{blocks / 2, 0, 0.0};
+  Deal best{blocks / 2, 0};
   double best_t = 1e30;
   const int x_max = blocks / 2, x_min = mix ? std::max(0, x_max - 2 * G / chunks) : x_max;
   for (int x = x_max; x >= x_min; --x) {
@@ -398,27 +397,10 @@ static Deal pick_deal(int blocks, int chunks, int splits, int G, bool mix) {
       if (t < t_x - 1e-9) { t_x = t; ns_x = ns; }
     }
     t_x += nW / G;
-    if (t_x < best_t - 1e-9) { best_t = t_x; best = {x, ns_x, t_x}; }
+    if (t_x < best_t - 1e-9) { best_t = t_x; best = {x, ns_x}; }
   }
   memo[key] = best;
   return best;
-}
-
-// (a k-block of a wide tile 0.62 us at the full clock, 0.68 in the longer launches that are not cut along K; set-up, first loads
-// and the last tile's way out 7 us, with SwiGLU or logits 9.5; with one plane of activations 0.35 and 0.39)
-double gemm_rows_us(int N, int M, int n_kblocks, int planes, int n_splits, bool partial, int n_sms) {
-  const int blocks = N / kBoxN, chunks = (M + kRowsM - 1) / kRowsM;
-  const double stream = (double)blocks * kBoxBytes * n_kblocks / 5.5e6;   // the weights at the rate these launches read them
-  if (partial) {
-    const int rounds = ((blocks + 1) / 2 * chunks * n_splits + n_sms - 1) / n_sms;
-    const double work = rounds * ((planes == 2 ? 0.62 : 0.35) * n_kblocks / n_splits + 1.0);
-    return std::max(work, stream) + 6.0 + rows_slab_us(M, N) * n_splits;
-  }
-  // (a further round of tiles costs more than its k-blocks while they do not cover the epilogue of the one before: gate-up of the
-  // 1B shape, 32 k-blocks, 29 us at one round, 46 at 1.6, 59 at two; of the 8B shape, 64, 80 at 1.6 and 259 at 5.6)
-  const double rounds = pick_deal(blocks, chunks, 1, n_sms, true).rounds;
-  const double between = planes == 2 && rounds > 1.0 ? (rounds - 1.0) * std::max(0.0, 7.0 - 0.094 * n_kblocks) : 0.0;
-  return std::max((planes == 2 ? 0.68 : 0.39) * n_kblocks * rounds + between, stream) + 9.5;
 }
 
 // `ta` must be the activation map whose box holds 128 rows.  N must be a multiple of 128.

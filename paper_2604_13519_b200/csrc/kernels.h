@@ -98,30 +98,6 @@ int gemm_rows_tiles(int N);
 cudaError_t launch_gemm_rows(int epi, const CUtensorMap &tw, const CUtensorMap &ta, GemmArgs g, int n_splits,
                              size_t smem_limit, int n_sms, cudaStream_t st, bool pdl);
 
-// The many-rows kernel's own estimate of a launch in us (splits: of EPI_PARTIAL, else 1), and what writing and reading back
-// one slab of partial sums costs (8 bytes per sum, most of them under other work; a load more for each row's kernel).
-double gemm_rows_us(int N, int M, int n_kblocks, int planes, int n_splits, bool partial, int n_sms);
-inline double rows_slab_us(int M, int N) { return 8.0 * M * N / 15e6 + 0.25; }
-
-// The same projections by pairs of CTAs (gemm_pair_tcgen05.cu): tiles of 256 weight rows x one chunk of activation rows.
-struct PairPlan {
-  int rows, n_wide, chunks;   // the first n_wide chunks have `rows` rows (a multiple of 16, at most 256), the others 16 less
-  int tiles, whole, pieces;   // tiles in all; of these done whole, by every pair the same number; K pieces of each of the others
-  int pairs;                  // of the launch
-  double us;                  // estimate
-};
-// fold: the kernel adds the pieces of a cut tile itself, slabs of up to slab_room floats; else (EPI_PARTIAL) all tiles are cut
-// alike and the next kernel adds the slabs.  pairs: that run at once.
-PairPlan plan_gemm_pair(int N, int M, int n_kblocks, int planes, bool fold, int pairs, int max_pieces, size_t slab_room);
-// (a type of its own: every byte of the other kernels' arguments is copied at each of a small step's launches)
-struct PairArgs : GemmArgs {   // n_wide and chunks are the plan's
-  int chunk_rows, n_tiles, n_whole, pieces;   // filled in by the launcher
-  float *slab;             // sums of the pieces of tiles cut along K
-  unsigned int *n_done;    // pieces of a cut tile that are there, per CTA of the pair (zero between launches)
-};
-cudaError_t launch_gemm_pair(int epi, const CUtensorMap &tw, const CUtensorMap &ta, const CUtensorMap &ta_less, PairArgs g,
-                             const PairPlan &plan, size_t smem_limit, cudaStream_t st, bool pdl);
-
 // x[m] = E[tokens[m]]; h = rmsnorm(x) * gain -> bf16 (hi[, lo])
 cudaError_t launch_embed_norm(const StepIn &in, const __nv_bfloat16 *embed, const float *gain, float eps,
                               int d, float *x, __nv_bfloat16 *h, int h_rows, int planes,

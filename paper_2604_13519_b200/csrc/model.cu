@@ -40,21 +40,18 @@ ts_status fail(ts_status code, const char *fmt, ...) {
 inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 constexpr int kMaxSplits = 12;
-constexpr int kMaxPieces = 6;    // K pieces of a left-over tile of the pair kernel
 constexpr int kMaxToolCandidates = 8;   // tool names verified in parallel while the name is open
 constexpr int kMaxAttnSplits = ts::kAttnMaxSplits;
-// Activation rows per TMA box: 8, 16, .. 128.  Weight-streaming kernel: the step's rows rounded up to 8 (16 with one plane of
+// activation rows per TMA box.  Weight-streaming kernel: the step's rows rounded up to 8 (16 with one plane of
 // activations: the tensor-core instruction's N, planes x rows, is a multiple of 16) -- a k-block of 33 rows in a box of
 // 64 takes as many bytes as its weights, which left three stages in the ring: gate-up of the 1B shape 24.5 us against
-// 14.9 at 8 rows.  Pair kernel: half of a chunk.  Many-rows kernel: 128.
-constexpr int kBoxes = 16;
-constexpr int box_rows(int i) { return 8 * (i + 1); }
-// Most rows of a step whose projections run on the weight-streaming kernel (gate-up and the LM head of the larger ones on the
-// pair kernel, see few_by_pairs), with one and with two planes of activations.  With two planes a ring of three stages still fits twice on an SM at 80 rows and one of two at 88.  Measured, four sessions,
+// 14.9 at 8 rows.  Many-rows kernel: 128.
+constexpr int kMcOptions[13] = {8, 16, 24, 32, 40, 48, 56, 64, 72, 80, 88, 96, 128};
+constexpr int kMcRows = 12;                      // index of the many-rows kernel's box
+// Most rows of a step whose projections run on the weight-streaming kernel, with one and with two planes of activations.
+// With two planes a ring of three stages still fits twice on an SM at 80 rows and one of two at 88.  Measured, four sessions,
 // many-rows kernel against this one: 1B shape two planes 80 rows 1440 / 1281 us, 96 rows 1481 / 1518; 8B 5467 / 4684 and
-// 5511 / 5483; one plane 1B 96 rows 1267 / 1276, 112 rows 1297 / 1371, 8B 4547 / 4378 and 4672 / 4558.  (The pair kernel's QKV,
-// O and down at 80 rows are quicker, 1B shape 6.9, 5.9 and 9.7 us against 8.8, 8.5 and 13.9, but not with the norm and rotary
-// kernels that they need: a layer of 66.8 us against 65.1.)
+// 5511 / 5483; one plane 1B 96 rows 1267 / 1276, 112 rows 1297 / 1371, 8B 4547 / 4378 and 4672 / 4558.
 constexpr int kFewRows[2] = {96, 80};
 constexpr int kFusedMc[3] = {1, 3, 7};           // the persistent kernel's boxes: 16, 32, 64 rows
 constexpr int kPrefillRows = 1024;   // rows of a prompt that go through in one step
@@ -83,7 +80,7 @@ struct Layout {
   // workspace (byte offsets)
   uint64_t x, h, part, q, attn_o, attn_ml, attn, act, logits, amax, rope, d_in, d_out, workspace_bytes;
   // fused single-kernel path
-  uint64_t maps, slab, ss_part, sync, n_done, phase_t, stamps;
+  uint64_t maps, slab, ss_part, sync, phase_t, stamps;
   int max_stamps;
   int n_maps, n_counters, n_phases;
   StepIo step_io, prompt_io;   // of a verification step, of a piece of a prompt
@@ -209,7 +206,6 @@ void make_layout(const ts_model_config &c, Layout *L) {
   L->ss_part = take((uint64_t)(d / 128) * R * 4);
   L->n_counters = (int)((L->Nqkv + 2 * d + 2 * F + V) / 128);
   L->sync = take((uint64_t)(8 + L->n_counters) * 4);
-  L->n_done = take((uint64_t)kMaxFusedCtas * 4);   // (pair kernel: fewer cut tiles than pairs of CTAs)
   L->n_phases = 6 * c.n_layers + 3;
   L->phase_t = take((uint64_t)3 * L->n_phases * 8);
   L->max_stamps = 9 * c.n_layers + 16;
@@ -247,7 +243,7 @@ struct ts_model {
   int leaf_len = 64;   // KV positions per attention leaf: a constant of the model (see AttnTcArgs), set by ts_init_model
   size_t gemm_smem_budget = 113 * 1024;   // two CTAs of the weight-streaming kernel per SM
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_d;
-  CUtensorMap tm_lm{}, tm_h[kBoxes]{}, tm_attn[kBoxes]{}, tm_act[kBoxes]{};
+  CUtensorMap tm_lm{}, tm_h[13]{}, tm_attn[13]{}, tm_act[13]{};
   std::vector<int32_t> free_pages;
   std::vector<ts_session *> sessions;   // live sessions over this model (detached on destroy)
   // last staged step
@@ -269,9 +265,6 @@ struct ts_model {
   bool last_sample = false;                    // the staged step accepts by speculative sampling
   float last_inv_t = 1.f;                      // 1 / temperature of that step
   size_t smem_optin = 0;
-  int max_pairs = 1;                           // pairs of CTAs of the pair kernel that run at once
-  struct RowsPlan { int N, K, M, splits; bool partial, by_pairs; ts::PairPlan pair; };
-  RowsPlan planned[5] = {};                    // of steps of the last number of rows
   int max_clusters[9] = {};                    // [c] = clusters of c CTAs of the weight-streaming kernel that fit at once
   // per-kernel timing pass (ts_profile_step): one event after every launch
   bool profiling = false;
@@ -350,9 +343,9 @@ ts_status weight_map(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t N
 }
 
 ts_status act_maps(EncodeTiledFn enc, CUtensorMap *out, void *base, uint64_t K, uint64_t rows, int planes) {
-  for (int i = 0; i < kBoxes; ++i) {
+  for (int i = 0; i < 13; ++i) {
     const uint64_t dims[3] = {K, rows, (uint64_t)planes};
-    const uint32_t box[3] = {64, (uint32_t)box_rows(i), (uint32_t)planes};
+    const uint32_t box[3] = {64, (uint32_t)kMcOptions[i], (uint32_t)planes};
     ts_status s = make_map(enc, &out[i], base, 3, dims, box);
     if (s) return s;
   }
@@ -395,93 +388,36 @@ int pick_splits_rows(const ts_model *m, int n_tiles, int m_chunks, int n_kblocks
   return best;
 }
 
-// Which kernel takes a projection of many rows, and how it is cut up: the quicker one by their estimates.  The pair kernel's rows
-// come in steps of 16, the row-major one's in steps of 128; that one has twice the tiles, and where they come out even on the
-// SMs it is the quicker one (8B shape, 384 rows, down: 58 us against 63; 256 rows: 42 against 42.7); within 0.7 us it keeps the work.
-const ts_model::RowsPlan &rows_plan(ts_model *m, int N, int K, int M, bool partial) {
-  // (a step's layers are all alike: four plans and the LM head's, each worked out once)
-  ts_model::RowsPlan *p = m->planned;
-  while (p < m->planned + 4 && p->M == M && (p->N != N || p->K != K || p->partial != partial)) ++p;
-  if (p->M == M && p->N == N && p->K == K && p->partial == partial) return *p;
-  const int Ma = (M + 127) / 128 * 128, kb = K / 64, room = std::min(kMaxSplits, m->L.part_rows / Ma);
-  *p = {};
-  p->N = N; p->K = K; p->M = M; p->partial = partial;
-  p->pair = ts::plan_gemm_pair(N, M, kb, m->planes, !partial, m->max_pairs, partial ? room : kMaxPieces,
-                               (size_t)m->L.part_rows * std::max(m->L.Nqkv, m->c.d_model));
-  p->splits = pick_splits_rows(m, ts::gemm_rows_tiles(N), Ma / 128, kb, partial, m->L.part_rows / Ma);
-  p->by_pairs = p->pair.us + 0.7 < ts::gemm_rows_us(N, M, kb, m->planes, p->splits, partial, m->n_sms);
-  if (p->by_pairs && partial) p->splits = p->pair.pieces;
-  return *p;
-}
-
-// A projection of more than kFewRows rows (bound by the tensor cores, their power and the bytes per flop an SM pulls from L2).
-// n_splits_out: split-K slabs written (EPI_PARTIAL).
+// A projection of the many-rows kernel (more than kFewRows rows: bound by the tensor cores and the bytes per flop an SM pulls
+// from L2).  n_splits_out: split-K slabs written (EPI_PARTIAL).
 ts_status run_gemm_rows(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M,
                         float *out, __nv_bfloat16 *act_out, unsigned long long *amax, int *n_splits_out) {
-  ts::PairArgs g{};
+  ts::GemmArgs g{};
   g.N = N; g.K = K; g.M = M; g.planes = m->planes;
   g.n_kblocks = K / 64;
   const int Ma = (M + 127) / 128 * 128;
-  const bool partial = epi == ts::EPI_PARTIAL;
-  const ts_model::RowsPlan &plan = rows_plan(m, N, K, M, partial);
+  const int splits = pick_splits_rows(m, ts::gemm_rows_tiles(N), Ma / 128, g.n_kblocks, epi == ts::EPI_PARTIAL, m->L.part_rows / Ma);
   g.out = out; g.out_rows = Ma;
   g.act_out = act_out; g.act_rows = m->L.rows_alloc; g.out_planes = m->planes;
   g.amax = amax;
-  g.slab = (float *)m->WS(m->L.part);
-  g.n_done = (unsigned int *)m->WS(m->L.n_done);
   g.err = m->d_out() + m->L.o_err;
   g.stamp = m->stamp_slot();
-  if (n_splits_out) *n_splits_out = plan.splits;
-  const bool pdl = m->use_pdl && !m->profiling;
-  if (plan.by_pairs) {
-    const int box = plan.pair.rows / 16 - 1;
-    CU_TRY(ts::launch_gemm_pair(epi, tw, ta[box], ta[std::max(0, box - 1)], g, plan.pair, m->smem_optin, m->st, pdl));
-  } else {
-    CU_TRY(ts::launch_gemm_rows(epi, tw, ta[kBoxes - 1], g, plan.splits, m->smem_optin, m->n_sms, m->st, pdl));
-  }
+  if (n_splits_out) *n_splits_out = splits;
+  CU_TRY(ts::launch_gemm_rows(epi, tw, ta[kMcRows], g, splits, m->smem_optin, m->n_sms, m->st, m->use_pdl && !m->profiling));
   m->launched(0);
   return TS_OK;
 }
 
-// Whether gate-up or the LM head of a step that is the weight-streaming kernel's otherwise goes to the pair kernel.  From 41 rows on
-// that kernel's bytes of activations, loaded by every CTA, count for more than its second CTA per SM (1B shape, gate-up at 48
-// rows 17.6 us against 15.0, at 64 19.1 against 15.4, at 33 the same; LM head at 48 92.6 against 83.3, at 33 83.6 against 79.9,
-// at 20 the same).  The sums are the same bits as that kernel's as long as no tile is cut along K, which steps of at most 64
-// rows need (a row's bits do not depend on what is verified beside it), so there the tiles have to come out even on the pairs
-// (8B shape: 96 gate-up tiles on 74 pairs do not, and the 594 of its LM head, nine rounds where eight would nearly do, only from
-// 41 rows on: 189 us against 190 at 32, 216 against 199 at 48).  One plane: LM head at 64 rows 90.5 against 84.4, at 48 the same;
-// gate-up past 80, where a box of activations is as heavy as 40 rows of two (8B shape at 76 rows 36.0 against 38.0, at 96 39.8
-// against 39.2).
-bool few_by_pairs(const ts_model *m, int epi, int N, int M) {
-  const bool head = epi == ts::EPI_LOGITS;
-  if (M > 64) return m->planes == 2 || head || M > 80;
-  const int tiles = (N + 255) / 256, slots = (tiles + m->max_pairs - 1) / m->max_pairs * m->max_pairs;
-  if (m->planes == 1) return head && M > 48 && slots * 20 <= tiles * 21;
-  return (M > 40 && slots * 5 <= tiles * 6) || (head && M > 24 && slots * 20 <= tiles * 21);
-}
-
-// A projection of at most kFewRows rows; `g` carries what its epilogue needs.
+// A projection of the weight-streaming kernel; `g` carries what its epilogue needs.
 ts_status run_gemm_ws(ts_model *m, int epi, const CUtensorMap &tw, const CUtensorMap *ta, int N, int K, int M, ts::GemmArgs g) {
   const int mi = pick_mc_index(M, m->planes);
-  g.N = N; g.K = K; g.M = M; g.Mc = box_rows(mi); g.planes = m->planes;
+  g.N = N; g.K = K; g.M = M; g.Mc = kMcOptions[mi]; g.planes = m->planes;
   g.n_kblocks = K / 64;
   g.act_rows = m->L.rows_alloc; g.out_planes = m->planes;
   g.err = m->d_out() + m->L.o_err;
   g.stamp = m->stamp_slot();
-  const bool split = epi == ts::EPI_QKV || epi == ts::EPI_RESID, pdl = m->use_pdl && !m->profiling;
-  if (!split && few_by_pairs(m, epi, N, M)) {
-    ts::PairArgs p{};
-    static_cast<ts::GemmArgs &>(p) = g;
-    p.slab = (float *)m->WS(m->L.part);
-    p.n_done = (unsigned int *)m->WS(m->L.n_done);
-    const ts::PairPlan plan = ts::plan_gemm_pair(N, M, g.n_kblocks, m->planes, true, m->max_pairs, M > 64 ? kMaxPieces : 1,
-                                                 (size_t)m->L.part_rows * std::max(m->L.Nqkv, m->c.d_model));
-    const int box = plan.rows / 16 - 1;
-    CU_TRY(ts::launch_gemm_pair(epi, tw, ta[box], ta[std::max(0, box - 1)], p, plan, m->smem_optin, m->st, pdl));
-  } else {
-    const int cluster = split ? pick_cluster(m, N / 128, g.n_kblocks) : 1;
-    CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, cluster, m->gemm_smem_budget, m->st, pdl));
-  }
+  const int cluster = (epi == ts::EPI_QKV || epi == ts::EPI_RESID) ? pick_cluster(m, N / 128, g.n_kblocks) : 1;
+  CU_TRY(ts::launch_gemm(epi, tw, ta[mi], g, cluster, m->gemm_smem_budget, m->st, m->use_pdl && !m->profiling));
   m->launched(0);
   return TS_OK;
 }
@@ -501,7 +437,7 @@ ts_status run_step_fused(ts_model *m) {
   a.in.parent = di + I.o_parent; a.in.anc = (const uint32_t *)(di + I.o_anc); a.in.slot = di + I.o_slot;
   a.in.row_tile = di + I.o_row_tile;
   a.in.B = m->last_B; a.in.M = m->last_M;
-  a.mc_index = m->last_M <= 16 ? 0 : (m->last_M <= 32 ? 1 : 2); a.Mc = box_rows(kFusedMc[a.mc_index]); a.planes = m->planes;
+  a.mc_index = m->last_M <= 16 ? 0 : (m->last_M <= 32 ? 1 : 2); a.Mc = kMcOptions[kFusedMc[a.mc_index]]; a.planes = m->planes;
   a.n_ctas = m->n_sms; a.skip_lm = (m->last_flags & TS_FLAG_SKIP_LM_HEAD) ? 1 : 0;
   a.k_max = c.k_max;
   a.n_attn_tiles = m->last_tiles128;
@@ -536,24 +472,22 @@ ts_status run_step_fused(ts_model *m) {
   return TS_OK;
 }
 
-// What an expired device-side wait leaves behind, for whichever call meets its status word: the word, the counters that the
-// persistent kernel was in the middle of, and pieces of cut tiles that the pair kernel has counted and not added (the next
-// launch would take a tile for complete too soon, or never).
+// What an expired device-side wait leaves behind, for whichever call meets its status word: the word, and the counters that the
+// persistent kernel was in the middle of.
 void clear_device_error(ts_model *m) {
   const Layout &L = m->L;
   cudaMemsetAsync(m->d_out() + L.o_err, 0, 4, m->st);
   cudaMemsetAsync(m->WS(L.sync), 0, (size_t)(8 + L.n_counters) * 4, m->st);
-  cudaMemsetAsync(m->WS(L.n_done), 0, (size_t)kMaxFusedCtas * 4, m->st);
 }
 
 // Test support (ts_debug_inject_device_error): leaves the status word that an expired device-side wait would have left, and
-// pieces counted by the pair kernel.  In the stream behind the last kernel that waits for anything and ahead of the acceptance
+// counters that are not zero.  In the stream behind the last kernel that waits for anything and ahead of the acceptance
 // kernel, which publishes the word with the step's results as it would a real one.
 cudaError_t write_injected(ts_model *m) {
   int32_t *word = m->h_out() + m->L.o_err + 1;
   *word = m->inject_err;
   m->inject_err = 0;
-  const cudaError_t e = cudaMemsetAsync(m->WS(m->L.n_done), 1, (size_t)kMaxFusedCtas * 4, m->st);
+  const cudaError_t e = cudaMemsetAsync(m->WS(m->L.sync), 1, (size_t)(8 + m->L.n_counters) * 4, m->st);
   if (e != cudaSuccess) return e;
   return cudaMemcpyAsync(m->d_out() + m->L.o_err, word, 4, cudaMemcpyHostToDevice, m->st);
 }
@@ -1274,8 +1208,6 @@ ts_status ts_init_model(const ts_model_config *cfg, const ts_buffers *bufs, void
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     m->smem_optin = (size_t)optin;
     for (int cl = 1; cl <= 8; ++cl) m->max_clusters[cl] = ts::gemm_max_clusters(cl, m->gemm_smem_budget);
-    // (one CTA per SM; asking about it costs a model's set-up 10 ms, and of two to an SM twice as many fit)
-    m->max_pairs = std::min(m->max_clusters[2] > 1 ? m->max_clusters[2] / 2 : m->n_sms / 2, kMaxFusedCtas / 2);
     m->fused_ok = coop != 0 && m->n_sms <= kMaxFusedCtas &&
                   ts::fused_ring_stages(m->planes, kFusedMaxRows, c.head_dim, m->smem_optin) >= 2;
   }

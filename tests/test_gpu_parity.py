@@ -455,6 +455,27 @@ def test_device_timeout_is_reported_and_survived(path):
     gm.close()
 
 
+@pytest.mark.parametrize("path", [1, 2])
+def test_error_that_a_retrieval_reports_is_survived(path):
+    """An expired wait in a replayed step, whose status nobody has looked at yet, is reported by whichever call comes next: a
+    retrieval too clears what it leaves behind, so that the next step is the same bits as before it."""
+    shape = synth.SHAPES["tiny"]
+    om, gm = make_pair(shape, k_max=16, max_ctx=512, path=path)
+    _, s, _ = synthetic_context(shape, om, gm, 200)
+    draft = _rand_draft(shape.vocab, 9, 31)
+    ts.ts_verify(gm, [s], [draft])
+    want = gm.read_logits(0, 10).copy()
+    g = torch.Generator().manual_seed(1)
+    hidden = torch.randn(64, shape.d_model, generator=g).to(torch.bfloat16).cuda()
+    gm.inject_device_error(3)
+    with pytest.raises(ts.TsError) as e:
+        ts.ts_topk_cosine(gm, hidden, 4, query=torch.randn(shape.d_model, generator=g).cuda())
+    assert e.value.code == -6
+    ts.ts_verify(gm, [s], [draft])
+    assert (gm.read_logits(0, 10).view("u4") == want.view("u4")).all()
+    gm.close()
+
+
 def test_device_index_check_is_reported_and_survived():
     """The host's handling of a failed index check of the debug build, exercised the same way (a status word written
     ahead of the acceptance kernel; the release build's kernels contain no checks): TS_ERR_DEVICE_BOUNDS with the check's
