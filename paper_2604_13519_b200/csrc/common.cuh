@@ -17,7 +17,7 @@ enum : int { DEV_OK = 0, DEV_TIMEOUT_FULL = 1, DEV_TIMEOUT_EMPTY = 2, DEV_TIMEOU
 // word and the access is skipped.  The host validates the same inputs before a step is staged, so no check is
 // expected to fail; the release build compiles the checks away.
 enum : int { CHK_TOKEN = 1, CHK_POSITION = 2, CHK_PAGE_APPEND = 3, CHK_PAGE_ATTN = 4, CHK_LEAVES = 5, CHK_PARENT = 6,
-             CHK_PAGE_COMPACT = 7, CHK_UNIT = 8 };
+             CHK_PAGE_COMPACT = 7, CHK_UNIT = 8, CHK_SMEM = 9 };
 struct BoundsCheck {
   int *err;                        // the step's status word (null: no checks)
   int vocab, max_pages, max_ctx;   // ranges of token ids, page ids and positions

@@ -55,8 +55,11 @@ template <int EPI, bool PUSH>
 __global__ void __launch_bounds__(192, 1)
 gemm_ws_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_a,
                const GemmArgs g) {
-  // 1024-byte alignment is required by the 128-byte swizzle pattern
+  // 1024-byte alignment is required by the 128-byte swizzle pattern: the declared one holds (no room is spent on rounding up)
   extern __shared__ __align__(1024) uint8_t smem[];
+#ifdef TS_DEBUG_BOUNDS
+  if (threadIdx.x == 0 && (smem_u32(smem) & 1023u)) atomicCAS(g.err, 0, DEV_BOUNDS + CHK_SMEM);
+#endif
   const int a_bytes = g.planes * g.Mc * kBlockK * 2;
   const int stage_bytes = kWBytes + a_bytes;
   GemmSmemCtl *ctl = reinterpret_cast<GemmSmemCtl *>(smem + (size_t)g.stages * stage_bytes);

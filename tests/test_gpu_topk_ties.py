@@ -1,6 +1,6 @@
 """Top-K where the bounded selection can go wrong: thousands of equal scores (more than it puts in order by counting), fewer
-valid scores than K in a slice, K at the most that it takes and one more, and as many lists as are put in order by counting and
-one more.  Entries are copies of a few vectors, so equal scores are equal bits and the order is known: best class first, lowest
+valid scores than K in a slice, K at the most that it takes and one more; and where the merge of the slices' lists goes wrong: as
+many lists as one round takes (256) and one more.  Entries are copies of a few vectors, so equal scores are equal bits and the order is known: best class first, lowest
 index within a class."""
 import pytest
 import torch
@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n,K,classes", [(9000, 10, [9000]), (9000, 16, [3, 8997]), (9000, 17, [3, 8997]), (4097, 16, [15, 4082]),
                                          (12288, 8, [300, 11988]), (64 * 4096, 16, [5, 40, 64 * 4096 - 45]),
-                                         (64 * 4096 + 1, 16, [5, 3, 64 * 4096 - 7]), (5, 5, [2, 3]), (4100, 1, [1, 4099])])
+                                         (64 * 4096 + 1, 16, [5, 3, 64 * 4096 - 7]), (256 * 4096, 16, [5, 40, 256 * 4096 - 45]),
+                                         (256 * 4096 + 1, 16, [5, 3, 256 * 4096 - 7]), (5, 5, [2, 3]), (4100, 1, [1, 4099])])
 def test_equal_scores_keep_their_order(n, K, classes):
     shape = synth.SHAPES["tiny"]
     g = torch.Generator().manual_seed(n + K)
