@@ -570,6 +570,8 @@ cudaError_t launch_gemm(int epi, const CUtensorMap &tw, const CUtensorMap &ta, G
   // Few rows: a CTA's sums go straight to the CTAs that finish the rows, 4 bytes per lane, counted by a barrier there, instead of
   // being fetched from it: one way through the cluster and no barriers of the cluster at the end (8B shape, one row: 76.4 -> 74.8
   // us per layer).  By 33 rows the small stores cost more than that (QKV of the 1B shape 5.1 -> 6.0 us, at 76 rows 8.1 -> 9.5).
+  // They lie in what the ring leaves of the budget: with two planes that holds the rows of all steps of up to 16, but for 6 to 8 with
+  // clusters of five and 8 with clusters of seven (two rows to a CTA beside boxes of eight), with one plane a row to a CTA.
   const size_t inbox = (size_t)cluster * ((g.M + cluster - 1) / cluster) * kTileN * 4;
   const bool push = split && cluster > 1 && g.M <= kPushRows && smem + inbox <= smem_budget;
   if (push) smem += inbox;
